@@ -188,15 +188,14 @@ miugks_status miugks_set_sweep_split(miugks_solver *s, int mode);
  * nothing where it is continuous.  The adjoint (which does not differentiate
  * this term) returns MIUGKS_EINVAL while it is on. */
 miugks_status miugks_set_shock_capturing(miugks_solver *s, int on);
-/* Bound of the prediction smoother's device waits (the cluster sweep of Eq.
- * macroFinalDefect waits for each diagonal's inputs and its neighbours'
- * values): a wait that has not completed after `seconds` (default 0.2, at
- * most 10) gives up, the kernel drains its copies in flight (waits bounded by
- * the default) and returns, and the next miugks_step / miugks_wait returns
- * MIUGKS_ETIMEOUT (sticky for the solver).  0 makes every such wait give up
- * without testing its inputs: it exercises the failure path without a fault
- * (the kernel computes one step on whatever the buffers hold, then drains and
- * returns; the state is garbage and the solver is to be destroyed), and the
+/* Bound of the prediction smoother's device waits (in the sweep of Eq.
+ * macroFinalDefect a strip of grid lines waits for the values of the strip
+ * before it): a wait that has not completed after `seconds` (default 0.2, at
+ * most 10) gives up, the kernel drains its copies in flight and returns, and the
+ * next miugks_step / miugks_wait returns MIUGKS_ETIMEOUT (sticky for the
+ * solver).  0 makes every sweep give up before its first step, without testing
+ * its inputs: it exercises the failure path without a fault (the kernel drains
+ * and returns; the state is garbage and the solver is to be destroyed), and the
  * CUDA context stays usable.  MIUGKS_EINVAL outside [0, 10]. */
 miugks_status miugks_set_wait_limit(miugks_solver *s, double seconds);
 int miugks_adaptive_decisions(const miugks_solver *s, unsigned char *out, int cap);

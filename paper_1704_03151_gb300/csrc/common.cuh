@@ -169,19 +169,19 @@ __device__ __forceinline__ void micro_slope(const double dw[4], double U, double
     micro_slope_t<double>(dw, U, V, lam, a);
 }
 
-// Reciprocal by the Newton-Raphson iteration y <- y + y (1 - x y) (quadratic
-// convergence) from a single-precision seed: two steps take the 24-bit seed to
-// double precision (within 1 ulp of 1/x).  Outside the seed's exponent range
-// the IEEE division is used.
+// Reciprocal by one third-order step y <- y + y (e + e^2), e = 1 - x y, from a
+// single-precision seed: e is below 2^-22, so the truncation e^3 is below 2^-66
+// and the result within 1 ulp of 1/x.  Outside the seed's exponent range (tested
+// on the exponent bits: a comparison would take the FP64 pipe twice) the IEEE
+// division is used.
 __device__ __forceinline__ double rcp64(double x)
 {
-    double ax = fabs(x);
-    if (!(ax > 1e-30 && ax < 1e30)) return 1.0 / x;
-    double y = (double)__frcp_rn((float)x);
-    double e = fma(-x, y, 1.0);
-    y = fma(y, e, y);
-    e = fma(-x, y, 1.0);
-    return fma(y, e, y);
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    if (ex - (1023u - 99u) > 198u) return 1.0 / x;
+    float s;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"((float)x));
+    const double y = (double)s, e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 
 template <typename T>

@@ -36,22 +36,35 @@ struct MacroArgs {
     unsigned long long wait_ns;            // bound of the sweep's waits for its inputs (ns of global time)
 };
 // Gamma of every face from the frozen state Wg
-// (and the inverse diagonal of the smoother per cell)
-cudaError_t launch_macro_gamma(const MacroArgs& a, const double* Wg, double* gx, double* gy, double* idiag,
-                               cudaStream_t st);
-// mode 0: out = Rin - R_E(W)  (forcing);  mode 1: out = Rin + R_E(W)  (renewal P + R_E)
-cudaError_t launch_macro_resid(const MacroArgs& a, const double* W, const double* gx, const double* gy,
-                               const double* Rin, double* out, int mode, cudaStream_t st);
+cudaError_t launch_macro_gamma(const MacroArgs& a, const double* Wg, double* gx, double* gy, cudaStream_t st);
+// What lies between two sweeps of a level (k_macro_stage): the state with the last
+// sweep's pending update dw (null: none) to Wo (null: not stored); mode 0: forcing
+// P = Rin - R_E(W), R = Rin and the inverse diagonal; mode 1: renewal R = Rin + R_E(W);
+// and the next sweep's records and ghosts (rec null: no sweep follows).  F: arithmetic
+// of the sweep (double, or float with increments).
+template <typename F>
+struct MacroStage {
+    const double* W; const F* dw; double* Wo;
+    const double *gx, *gy;
+    const double* Rin; double* P; double* R; double* idiag;
+    F* rec;                                // macro_rec_bytes(nx, ny, F == float)
+    double* ghost;                         // macro_ghost_elems(nubc)
+    int mode;
+};
+template <typename F>
+cudaError_t launch_macro_stage(const MacroArgs& a, const MacroStage<F>& A, cudaStream_t st);
 // y = J^T x, J = dR_E/dW at W with Gamma frozen (gx, gy); x may be null (no product);
 // binv (16 per cell, may be null) receives the inverses of the transposed diagonal blocks
 cudaError_t launch_macro_jacT(const MacroArgs& a, const double* W, const double* gx, const double* gy,
                               const double* x, double* y, double* binv, cudaStream_t st);
-// one LU-SGS pass: dW from R at state W; then W += dW.  F: arithmetic of the sweep
-// (double, or float with increments); rec: macro_rec_bytes(nx, ny, F == float) of scratch
+// one LU-SGS pass: dW ([nc][4], not yet added to W) from the records of a stage
 template <typename F>
-cudaError_t launch_macro_sgs(const MacroArgs& a, double* W, const double* gx, const double* gy, const double* idiag,
-                             void* rec, const double* R, double* dW, cudaStream_t st);
+cudaError_t launch_macro_sgs(const MacroArgs& a, F* rec, const double* ghost, F* dW, cudaStream_t st);
 size_t macro_rec_bytes(int nx, int ny, bool mixed);
+size_t macro_ghost_elems(int nubc);
+// volume-weighted restriction of a level's W and R
+cudaError_t launch_restrict_state(const LevelDev& F, const LevelDev& C, const double* W, const double* R, double* Wc,
+                                  double* Rc, cudaStream_t st);
 template <typename T>
 cudaError_t launch_restrict(const LevelDev& F, const LevelDev& C, int m, int nblk, const T* fine, T* coarse,
                             cudaStream_t st);
@@ -62,12 +75,14 @@ template <typename T>
 cudaError_t launch_prolong_add(const LevelDev& F, const LevelDev& C, int m, int nblk, const int* idx4,
                                const double* w4, const T* coarse, T* fine, T* out_pro, cudaStream_t st);
 cudaError_t launch_axpy(double* y, const double* x, double a, size_t n, cudaStream_t st);
-// Wt = Wc, or Wn in a cell where Wc has non-positive density or internal energy
-cudaError_t launch_predicted_state(int nc, const double* Wn, const double* Wc, double* Wt, cudaStream_t st);
-// FAS correction W += P dWc of the [nc][4] state, dropped in a cell where it would
-// leave the density or the internal energy non-positive
-cudaError_t launch_prolong_state(const LevelDev& F, const int* idx4, const double* w4, const double* dWc, double* W,
-                                 cudaStream_t st);
+// Wt = Wc + dw (dw may be null), or Wn in a cell where that has non-positive density or internal energy
+template <typename F>
+cudaError_t launch_predicted_state(int nc, const double* Wn, const double* Wc, const F* dw, double* Wt, cudaStream_t st);
+// FAS correction W += P (Wc + dw - Wn) of the [nc][4] state (dw may be null), dropped in a
+// cell where it would leave the density or the internal energy non-positive
+template <typename F>
+cudaError_t launch_prolong_state(const LevelDev& L, const int* idx4, const double* w4, const double* Wc, const F* dw,
+                                 const double* Wn, double* W, cudaStream_t st);
 cudaError_t launch_sub(double* out, const double* a, const double* b, size_t n, cudaStream_t st);
 
 // ---- evolution step (microscopic) ----

@@ -5,11 +5,12 @@
 // LU-SGS smoother of Eq. macroFinalDefect, and the grid-transfer kernels
 // (Eqs. macroRestriction, microRestriction, prolongation).
 //
-// The LU-SGS sweep runs as an anti-diagonal wavefront inside one thread-block
-// cluster: the cells of a diagonal are spread over the cluster's CTAs, which
-// pass the edge cells of each diagonal to their neighbours through
-// distributed shared memory, so the serial sweep order is kept without
-// grid-wide synchronisation.
+// The LU-SGS sweep runs as an anti-diagonal wavefront of warps: a warp owns a
+// strip of grid lines and walks along them one cell per step, so a cell's
+// neighbours are the last cells of its own line and of the line before it, in
+// the same lanes and the next ones.  Warps follow each other a few steps apart and hand over the
+// values of their last line through shared memory; the serial sweep order is
+// kept without any barrier per diagonal.
 #include "kernels.cuh"
 #include "async.cuh"
 
@@ -17,21 +18,6 @@ namespace cg = cooperative_groups;
 
 namespace miugks {
 
-constexpr int kMacroCluster = 8;
-constexpr int kMacroThreads = 128;
-
-__device__ __forceinline__ void euler_flux(const double* W, int axis, double sgn, double T[4])
-{
-    double rho, U, V, lam;
-    prim4(W, rho, U, V, lam);
-    double p = rho / (2.0 * lam);
-    double nx = axis == 0 ? sgn : 0.0, ny = axis == 1 ? sgn : 0.0;
-    double Un = U * nx + V * ny;
-    T[0] = rho * Un;
-    T[1] = W[1] * Un + p * nx;
-    T[2] = W[2] * Un + p * ny;
-    T[3] = (W[3] + p) * Un;
-}
 
 // Euler flux along +e_axis: (m_a, m_x U_a + p d_xa, m_y U_a + p d_ya, (E + p) U_a),
 // with p = 2 e_int / (K + 2)
@@ -53,22 +39,24 @@ __device__ __forceinline__ void euler_axis(const double* W, int axis, double T[4
 __device__ void macro_ghost(const BcDev& b, int axis, const double* Wi, double Wg[4], double* M)
 {
     if (b.type == BC_WALL) {
-        double rho, U, V, lam;
-        prim4(Wi, rho, U, V, lam);
-        double lamw = 1.0 / b.t;
-        double lamg = 2.0 * lamw - lam, Ug = 2.0 * b.u - U, Vg = 2.0 * b.v - V;
+        // lam_g = 2 lam_w - lam and Y = lam / (lam - 2 lam_w) through the temperatures:
+        // 1 / lam_g = T T_w / (2 T - T_w), Y = -T_w / (2 T - T_w), so two reciprocals in a row, not five
+        const double rho = Wi[0], ir = rcp64(rho), U = Wi[1] * ir, V = Wi[2] * ir, K = kKint + 2.0;
+        const double T = (4.0 / (kKint + 2)) * (Wi[3] * ir - 0.5 * (U * U + V * V));
+        const double Ug = 2.0 * b.u - U, Vg = 2.0 * b.v - V;
+        const double h = b.t * rcp64(2.0 * T - b.t);
         Wg[0] = rho; Wg[1] = rho * Ug; Wg[2] = rho * Vg;
-        Wg[3] = 0.5 * rho * (Ug * Ug + Vg * Vg) + (kKint + 2) * rho / (4.0 * lamg);
+        Wg[3] = rho * (0.5 * (Ug * Ug + Vg * Vg) + 0.25 * K * (T * h));
         if (M) {
-            double Y = lam / (lam - 2.0 * lamw), K = kKint + 2.0;
+            const double Y = -h, Y2 = h * h;
             for (int q = 0; q < 16; ++q) M[q] = 0.0;
             M[0] = 1.0;
             M[4] = 2.0 * b.u; M[5] = -1.0;
             M[8] = 2.0 * b.v; M[10] = -1.0;
-            M[12] = 2.0 * (b.u * b.u + b.v * b.v) - 0.5 * (U * U + V * V) * (1.0 + Y * Y) + K / (4.0 * lam) * (Y * Y - Y);
-            M[13] = U - 2.0 * b.u + U * Y * Y;
-            M[14] = V - 2.0 * b.v + V * Y * Y;
-            M[15] = -Y * Y;
+            M[12] = 2.0 * (b.u * b.u + b.v * b.v) - 0.5 * (U * U + V * V) * (1.0 + Y2) + 0.25 * K * T * (Y2 - Y);
+            M[13] = U - 2.0 * b.u + U * Y2;
+            M[14] = V - 2.0 * b.v + V * Y2;
+            M[15] = -Y2;
         }
     } else if (b.type == BC_SYMMETRY) {
         for (int m = 0; m < 4; ++m) Wg[m] = Wi[m];
@@ -79,9 +67,8 @@ __device__ void macro_ghost(const BcDev& b, int axis, const double* Wi, double W
             M[5 * (1 + axis)] = -1.0;
         }
     } else if (b.type == BC_FARFIELD) {
-        double lam = 1.0 / b.t;
         Wg[0] = b.rho; Wg[1] = b.rho * b.u; Wg[2] = b.rho * b.v;
-        Wg[3] = 0.5 * b.rho * (b.u * b.u + b.v * b.v) + (kKint + 2) * b.rho / (4.0 * lam);
+        Wg[3] = b.rho * (0.5 * (b.u * b.u + b.v * b.v) + 0.25 * (kKint + 2) * b.t);
         if (M) for (int q = 0; q < 16; ++q) M[q] = 0.0;
     } else {
         for (int m = 0; m < 4; ++m) Wg[m] = Wi[m];
@@ -94,13 +81,12 @@ __device__ void macro_ghost(const BcDev& b, int axis, const double* Wi, double W
 
 __device__ __forceinline__ double gamma_of(const GasDev& g, const double* Wa, const double* Wb, int axis, double dist)
 {
-    double Wm[4], rho, U, V, lam;
+    double Wm[4];
     for (int m = 0; m < 4; ++m) Wm[m] = 0.5 * (Wa[m] + Wb[m]);
-    prim4(Wm, rho, U, V, lam);
-    double gam = (kKint + 4.0) / (kKint + 2.0);
-    double as = sqrt(gam / (2.0 * lam));
-    double nu = g.mu_ref * pow(1.0 / lam, g.omega) / rho;
-    return fabs(axis == 0 ? U : V) + as + 2.0 * nu / dist;
+    const double rd = rcp64(dist), ir = rcp64(Wm[0]), U = Wm[1] * ir, V = Wm[2] * ir;
+    const double T = (4.0 / (kKint + 2)) * (Wm[3] * ir - 0.5 * (U * U + V * V));
+    const double gam = (kKint + 4.0) / (kKint + 2.0);
+    return fabs(axis == 0 ? U : V) + sqrt(0.5 * gam * T) + 2.0 * g.mu_ref * pow(T, g.omega) * (ir * rd);
 }
 
 __global__ void k_macro_gamma(MacroArgs a, const double* __restrict__ Wg, double* __restrict__ gx, double* __restrict__ gy)
@@ -144,27 +130,13 @@ __global__ void k_macro_gamma(MacroArgs a, const double* __restrict__ Wg, double
     }
 }
 
-// 1 / ((1/2V) sum_faces S Gamma + 1/dt_n): the inverse diagonal of the smoother
-__global__ void k_macro_idiag(MacroArgs a, const double* __restrict__ gx, const double* __restrict__ gy,
-                              double* __restrict__ idiag)
+cudaError_t launch_macro_gamma(const MacroArgs& a, const double* Wg, double* gx, double* gy, cudaStream_t st)
 {
-    const LevelDev& L = a.L;
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= L.nc) return;
-    int i = c % L.nx, j = c / L.nx;
-    double sx = gx[j * (L.nx + 1) + i] + gx[j * (L.nx + 1) + i + 1];
-    double sy = gy[j * L.nx + i] + gy[(j + 1) * L.nx + i];
-    double V = L.dx[i] * L.dy[j];
-    // zero in a body, whose records then give dW = 0
-    idiag[c] = L.solid[c] ? 0.0 : 1.0 / ((L.dy[j] * sx + L.dx[i] * sy) / (2.0 * V) + a.dtn_inv);
-}
-
-cudaError_t launch_macro_gamma(const MacroArgs& a, const double* Wg, double* gx, double* gy, double* idiag,
-                               cudaStream_t st)
-{
-    int n = a.L.nfx + a.L.nfy;
-    k_macro_gamma<<<(n + 127) / 128, 128, 0, st>>>(a, Wg, gx, gy);
-    k_macro_idiag<<<(a.L.nc + 127) / 128, 128, 0, st>>>(a, gx, gy, idiag);
+    // one warp per CTA: a face is a chain of FP64 divisions and a pow, and the FP64 pipe of an SM
+    // serves two lanes per clock, so the faces of a small level belong on as many SMs as possible
+    // (64x64 cells: 20 -> 14 us, with one reciprocal in a row instead of three divisions)
+    const int n = a.L.nfx + a.L.nfy;
+    k_macro_gamma<<<(n + 31) / 32, 32, 0, st>>>(a, Wg, gx, gy);
     return cudaGetLastError();
 }
 
@@ -189,48 +161,200 @@ __device__ __forceinline__ double face_gamma(const LevelDev& L, const double* gx
     return axis == 0 ? gx[j * (L.nx + 1) + i + up] : gy[(j + up) * L.nx + i];
 }
 
-// R_E of a cell: -(1/V) sum_faces S F_split(W_i, W_j).  Four lanes per cell,
-// one face each (the FP64 latency of a cell is spread over four lanes); the
-// face terms are added in face order.
-__global__ void k_macro_resid(MacroArgs a, const double* __restrict__ W, const double* __restrict__ gx,
-                              const double* __restrict__ gy, const double* __restrict__ Rin, double* __restrict__ out,
-                              int mode)
+// ---- records of the sweep
+//
+// How a strip's warp is laid out: lanes per grid line (and components per lane),
+// lines per strip, values of a lane's record, records in flight, steps that a
+// strip starts after the values it needs first, and the place of (1/2V) / D in a record.
+template <typename F> struct MacroLane;
+template <> struct MacroLane<float> {
+    static constexpr int kLanes = 1, kComp = 4, kLines = 32, kVals = 16, kRow = kVals * 32, kRing = 8, kLead = 3, kHv = 10;
+};
+template <> struct MacroLane<double> {
+    static constexpr int kLanes = 4, kComp = 1, kLines = 8, kVals = 10, kRow = kVals * 32, kRing = 4, kLead = 1, kHv = 2;
+};
+constexpr int kMacroMaxLines = 256;   // min(nx, ny)
+constexpr int kGhostRec = 24;         // per upper boundary face: dB/dW (16), rho, m_x, m_y, E + p, U, V of the ghost, S, S Gamma
+
+// Frame of a pass: s counts grid lines across the strips (along the shorter mesh
+// direction, so that few strips do many steps), t the cells along a line, both
+// from the corner the pass starts in.  Cell (s, t) is swept at step t + s % lines
+// of strip s / lines, and its record lies in the order in which the strip reads
+// it, in units of 16 bytes per lane, so that the records of a step are contiguous.
+template <typename F>
+struct MacroFrame {
+    using T = MacroLane<F>;
+    int ns, nt, strips, nk, rows;     // lines, cells along a line, strips, steps of a strip, rows kept for them
+    bool xl;                          // lines are columns (s along x)
+    __host__ __device__ MacroFrame(int nx, int ny)
+    {
+        xl = nx <= ny;
+        ns = xl ? nx : ny;
+        nt = xl ? ny : nx;
+        strips = (ns + T::kLines - 1) / T::kLines;
+        nk = nt + T::kLines - 1;
+        rows = (nk + T::kRing - 1) / T::kRing * T::kRing + T::kRing;   // steps are done and prefetched in rings
+    }
+    __host__ __device__ size_t values() const { return 2 * (size_t)strips * rows * T::kRow; }
+    // value v of component m (the same record in the mixed form, where v + m is meant) of cell (i, j)
+    __device__ __forceinline__ size_t at(int pass, int i, int j, int m, int v) const
+    {
+        int s = xl ? i : j, t = xl ? j : i;
+        if (pass) { s = ns - 1 - s; t = nt - 1 - t; }
+        const int l = s % T::kLines, lane = l * T::kLanes + (T::kLanes > 1 ? m : 0);
+        if (T::kLanes == 1) v += m;
+        constexpr int V = 16 / (int)sizeof(F);
+        const size_t row = ((size_t)pass * strips + s / T::kLines) * rows + t + l;
+        return row * T::kRow + ((size_t)(v / V) * 32 + lane) * V + v % V;
+    }
+};
+
+// State of a cell with the pending update of the last sweep.
+template <typename F>
+__device__ __forceinline__ void ld_state(const double* __restrict__ W, const F* __restrict__ dw, int c, double (&w)[4])
+{
+    const double2 a = *reinterpret_cast<const double2*>(W + 4 * (size_t)c);
+    const double2 b = *reinterpret_cast<const double2*>(W + 4 * (size_t)c + 2);
+    w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
+    if (dw)
+        #pragma unroll
+        for (int m = 0; m < 4; ++m) w[m] += (double)dw[4 * (size_t)c + m];
+}
+
+// Everything between two sweeps of a level in one pass over its cells: the
+// state with the last sweep's update (A.dw, when not null) goes to A.Wo; from
+// the split-flux residual R_E = -(1/V) sum_faces S F_split(W_i, W_j) comes
+//   mode 0 (start of a level's cycle)  P = Rin - R_E (forcing), R = Rin, and the inverse diagonal
+//          1 / ((1/2V) sum_faces S Gamma + 1/dt_n) (zero in a body, whose dW is then zero),
+//   mode 1 (renewal)                   R = Rin + R_E  (Rin = P),
+// and, when a sweep follows (A.rec), the cell's records of both passes and the
+// ghosts of the upper boundary faces.  Four lanes per cell, one face each (the
+// FP64 latency of a cell is spread over four lanes); the face terms are added
+// in face order.  Blocks from ncb on do the ghosts, one thread per face.
+// FP64 latency bounds it (10 us at 64x64 cells and at 16x16).  It replaces the residual, the inverse
+// diagonal, the record kernel and two copies: five launches and 24 us at 64x64 cells.
+template <typename F>
+__global__ void __launch_bounds__(64) k_macro_stage(MacroArgs a, MacroStage<F> A, int ncb)
 {
     const LevelDev& L = a.L;
+    if ((int)blockIdx.x >= ncb) {
+        const int q = ((int)blockIdx.x - ncb) * blockDim.x + threadIdx.x, b = q >> 1, axis = q & 1;
+        if (b >= L.nubc) return;
+        const int c = L.ubc[b], i = c % L.nx, j = c / L.nx;
+        const int bcid = axis == 0 ? L.fbx[j * (L.nx + 1) + i + 1] : L.fby[(j + 1) * L.nx + i];
+        double* g = A.ghost + (size_t)q * kGhostRec;
+        if (bcid < 0) { g[22] = 0.0; return; }
+        double w[4], G[4], M[16];
+        ld_state(A.W, A.dw, c, w);
+        macro_ghost(a.bc[bcid], axis, w, G, M);
+        for (int m = 0; m < 16; ++m) g[m] = M[m];
+        const double ir = rcp64(G[0]), U = G[1] * ir, V = G[2] * ir;
+        const double p = (2.0 / (kKint + 2)) * (G[3] - 0.5 * (G[1] * U + G[2] * V));
+        const double S = axis == 0 ? L.dy[j] : L.dx[i];
+        g[16] = G[0]; g[17] = G[1]; g[18] = G[2]; g[19] = G[3] + p; g[20] = U; g[21] = V;
+        g[22] = S;
+        g[23] = S * (axis == 0 ? A.gx[j * (L.nx + 1) + i + 1] : A.gy[(j + 1) * L.nx + i]);
+        return;
+    }
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = t >> 2, f = t & 3;
     const bool on = c < L.nc;
     const int cc = on ? c : 0, i = cc % L.nx, j = cc / L.nx;
-    const double* Wi = W + 4 * (size_t)cc;
-    double term[4] = {0, 0, 0, 0};
-    if (!L.solid[cc]) {   // a body has R_E = 0
-        const int axis = f >> 1, up = f & 1;
-        const double sgn = up ? 1.0 : -1.0, S = axis == 0 ? L.dy[j] : L.dx[i];
-        int bcid, nb; double dum = 0;
-        face_of(L, i, j, f, bcid, nb, dum);
-        double G[4], Ti[4], Tj[4];
-        const double* Wj;
-        if (bcid >= 0) { macro_ghost(a.bc[bcid], axis, Wi, G, nullptr); Wj = G; }
-        else Wj = W + 4 * (size_t)nb;
-        euler_flux(Wi, axis, sgn, Ti);
-        euler_flux(Wj, axis, sgn, Tj);
-        const double gm = face_gamma(L, gx, gy, i, j, f);
-        for (int m = 0; m < 4; ++m) term[m] = S * (0.5 * (Ti[m] + Tj[m] + gm * (Wi[m] - Wj[m])));
-    }
-    const int base = threadIdx.x & ~3;
-    double acc[4] = {0, 0, 0, 0};
-    #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    double Wi[4], term[4] = {0, 0, 0, 0};
+    ld_state(A.W, A.dw, cc, Wi);
+    const double ir = rcp64(Wi[0]), U = Wi[1] * ir, V = Wi[2] * ir;
+    const double p = (2.0 / (kKint + 2)) * (Wi[3] - 0.5 * (Wi[1] * U + Wi[2] * V));
+    const int axis = f >> 1, up = f & 1;
+    const double S = axis == 0 ? L.dy[j] : L.dx[i];
+    const double gm = face_gamma(L, A.gx, A.gy, i, j, f);
+    const bool solid = L.solid[cc];
+    int bcid, nb; double dum = 0;
+    face_of(L, i, j, f, bcid, nb, dum);
+    const bool joined = !solid && bcid < 0;                // a face shared with another fluid cell
+    if (!solid) {                                          // a body has R_E = 0
+        double Wj[4], Tj[4];
+        if (bcid >= 0) macro_ghost(a.bc[bcid], axis, Wi, Wj, nullptr);
+        else ld_state(A.W, A.dw, nb, Wj);
+        euler_axis(Wj, axis, Tj);
+        const double Ua = axis == 0 ? U : V, sgn = up ? 1.0 : -1.0;
+        double Ti[4] = {axis == 0 ? Wi[1] : Wi[2], Wi[1] * Ua, Wi[2] * Ua, (Wi[3] + p) * Ua};
+        if (axis == 0) Ti[1] += p; else Ti[2] += p;
         #pragma unroll
-        for (int m = 0; m < 4; ++m) acc[m] += __shfl_sync(0xffffffffu, term[m], (base + q) & 31);
-    if (on && f == 0) {
-        const double V = L.dx[i] * L.dy[j];
-        for (int m = 0; m < 4; ++m) {
-            const double RE = -acc[m] / V;
-            out[4 * (size_t)c + m] = mode == 0 ? Rin[4 * (size_t)c + m] - RE : Rin[4 * (size_t)c + m] + RE;
+        for (int m = 0; m < 4; ++m) term[m] = S * (0.5 * (sgn * (Ti[m] + Tj[m]) + gm * (Wi[m] - Wj[m])));
+    }
+    const int base = threadIdx.x & 28;
+    const double Sg = S * gm, cS = joined ? S : 0.0, cSg = joined ? Sg : 0.0;
+    double acc[4] = {0, 0, 0, 0}, fS[4], fSg[4], sum = 0.0;
+    #pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        #pragma unroll
+        for (int m = 0; m < 4; ++m) acc[m] += __shfl_sync(0xffffffffu, term[m], base + q);
+        fS[q] = __shfl_sync(0xffffffffu, cS, base + q);
+        fSg[q] = __shfl_sync(0xffffffffu, cSg, base + q);
+        sum += __shfl_sync(0xffffffffu, Sg, base + q);
+    }
+    if (!on) return;
+    const double rV = L.rdx[i] * L.rdy[j];
+    double id = 0.0;
+    if (A.idiag) {
+        if (A.mode == 0) {
+            id = solid ? 0.0 : 1.0 / (0.5 * rV * sum + a.dtn_inv);
+            if (f == 0) A.idiag[c] = id;
+        } else {
+            id = A.idiag[c];
+        }
+    }
+    // lane f: component f of R (and P, W), unit f of the records
+    const double RE = -rV * (f == 0 ? acc[0] : f == 1 ? acc[1] : f == 2 ? acc[2] : acc[3]);
+    const double rin = A.Rin[4 * (size_t)c + f], R = A.mode == 0 ? rin : rin + RE;
+    if (A.P) A.P[4 * (size_t)c + f] = rin - RE;
+    A.R[4 * (size_t)c + f] = R;
+    if (A.Wo) A.Wo[4 * (size_t)c + f] = f == 0 ? Wi[0] : f == 1 ? Wi[1] : f == 2 ? Wi[2] : Wi[3];
+    if (!A.rec) return;
+    // records (a cell in a body may hold any values: its record is a unit density at rest)
+    const unsigned cell = 0xfu << base;                    // the cell's four lanes leave or stay together
+    const MacroFrame<F> fr(L.nx, L.ny);
+    const double hv = 0.5 * rV * id;
+    if constexpr (sizeof(F) == 4) {
+        double u[4];
+        #pragma unroll
+        for (int m = 0; m < 4; ++m) u[m] = __shfl_sync(cell, R, base + m) * id;
+        if (f == 1) { u[0] = solid ? 1.0 : Wi[0]; u[1] = solid ? 0.0 : Wi[1]; u[2] = solid ? 0.0 : Wi[2]; u[3] = solid ? 0.0 : Wi[3] + p; }
+        if (f == 2) { u[0] = solid ? 0.0 : U; u[1] = solid ? 0.0 : V; u[2] = hv; u[3] = 0.0; }
+        const int xu = fr.xl ? 0 : 2, yu = 2 - xu;         // x- and y-faces: across and along, or the other way round
+        if (f == 3) { u[xu] = -fS[1]; u[xu + 1] = fSg[1]; u[yu] = -fS[3]; u[yu + 1] = fSg[3]; }
+        *reinterpret_cast<float4*>(A.rec + fr.at(0, i, j, 0, 4 * f)) = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
+        if (f == 0) return;                                // pass 1 takes its own value from pass 0
+        if (f == 3) { u[xu] = fS[0]; u[xu + 1] = fSg[0]; u[yu] = fS[2]; u[yu + 1] = fSg[2]; }
+        *reinterpret_cast<float4*>(A.rec + fr.at(1, i, j, 0, 4 * f)) = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
+    } else {
+        const double w = f == 0 ? Wi[0] : f == 1 ? Wi[1] : f == 2 ? Wi[2] : Wi[3];
+        const double e = f == 3 ? w + p : w;
+        const double Tx = f == 0 ? Wi[1] : fma(e, U, f == 1 ? p : 0.0), Ty = f == 0 ? Wi[2] : fma(e, V, f == 2 ? p : 0.0);
+        for (int pass = 0; pass < 2; ++pass) {
+            const double sx = pass ? fS[0] : -fS[1], gx = pass ? fSg[0] : fSg[1], sy = pass ? fS[2] : -fS[3], gy = pass ? fSg[2] : fSg[3];
+            const double r[10] = {R * id, solid ? (f == 0 ? 1.0 : 0.0) : w, hv, 0.0, fr.xl ? sx : sy, fr.xl ? gx : gy,
+                                  solid ? 0.0 : fr.xl ? -sx * Tx : -sy * Ty, fr.xl ? sy : sx, fr.xl ? gy : gx,
+                                  solid ? 0.0 : fr.xl ? -sy * Ty : -sx * Tx};
+            #pragma unroll
+            for (int v = 0; v < 10; v += 2) {
+                double* o = (double*)A.rec + fr.at(pass, i, j, f, v);
+                if (v == 0 && pass == 1) o[1] = r[1];      // pass 1 takes its own value from pass 0
+                else *reinterpret_cast<double2*>(o) = make_double2(r[v], r[v + 1]);
+            }
         }
     }
 }
+
+template <typename F>
+cudaError_t launch_macro_stage(const MacroArgs& a, const MacroStage<F>& A, cudaStream_t st)
+{
+    const int ncb = (4 * a.L.nc + 63) / 64, ngb = A.rec ? (2 * a.L.nubc + 63) / 64 : 0;
+    k_macro_stage<F><<<ncb + ngb, 64, 0, st>>>(a, A, ncb);
+    return cudaGetLastError();
+}
+template cudaError_t launch_macro_stage<double>(const MacroArgs&, const MacroStage<double>&, cudaStream_t);
+template cudaError_t launch_macro_stage<float>(const MacroArgs&, const MacroStage<float>&, cudaStream_t);
 
 // Jacobian of the Euler flux T(W) . n, n = sgn e_axis, with p = 2 e_int / (K + 2):
 // A[r * 4 + c] = dT_r / dW_c
@@ -337,370 +461,357 @@ cudaError_t launch_macro_jacT(const MacroArgs& a, const double* W, const double*
     return cudaGetLastError();
 }
 
-cudaError_t launch_macro_resid(const MacroArgs& a, const double* W, const double* gx, const double* gy,
-                               const double* Rin, double* out, int mode, cudaStream_t st)
-{
-    k_macro_resid<<<(4 * a.L.nc + 127) / 128, 128, 0, st>>>(a, W, gx, gy, Rin, out, mode);
-    return cudaGetLastError();
-}
-
-// LU-SGS pass of Eq. macroFinalDefect, one lane per (cell, component).
+// LU-SGS pass of Eq. macroFinalDefect.  At every step a strip's lanes update one
+// cell per grid line, an anti-diagonal:
+//   dW = own - (1/2V D) (sum over the two upstream faces of sgn S X - S Gamma dW),
+// X = T(W + dW) - T(W) of the upstream cell.  The cell that owns a value forms
+// its two downstream face terms itself: the one along the line stays in
+// registers, the one across goes to the next line by a shuffle, and the last
+// line's goes to the next strip's shared memory.  Those edge values announce
+// themselves: the buffer starts out filled with a signalling NaN, which no
+// arithmetic produces, and a reader waits (bounded) until the value it wants is
+// another one, so a step has no barrier, no fence (a fence would wait for the
+// step's global stores: 3300 against 2500 cycles per FP64 step) and no remote
+// round trip.  A strip starts kLead steps late and reads a step ahead, so that
+// the values are there when it looks.  Records stream into a ring of kRing steps
+// (every lane copies and reads its own, so the ring needs no barrier either).
 //
-// The cells of an anti-diagonal are spread over the CTAs of one cluster, 32
-// cells (128 lanes) per CTA; cell s of a diagonal only needs cells s-1, s and
-// s+1 of the previous one.  So a diagonal's results -- dW and the flux terms X
-// along x and y that its successors need -- go to shared memory, and only the
-// two edge cells of each CTA are pushed into the neighbouring CTAs' shared
-// memory (st.async on their mbarrier).  A CTA waits for its two neighbours
-// only: no cluster-wide barrier and no global-memory round trip per diagonal.
-//
-// Everything a lane needs that does not depend on the sweep (own defect times
-// 1/D, face coefficients, the base state) is packed by k_macro_rec into a
-// record of kRec values per (pass, diagonal, slot, component), diagonal-major,
-// so that the records of upcoming diagonals stream into a ring in shared
-// memory with one bulk copy per CTA and diagonal.
-//
-// Flux terms.  FP64: X = T(W + dW), and the record carries
-// c0 = -sum sgn S T(W_nb), so the coupling term is c0 + sum (sgn S X_nb -
-// S Gamma dW_nb).  Mixed: X = T(W + dW) - T(W) written through the increments
-// (dU = (dm_x - U drho) / (rho + drho), dp, ... -- exact identities), which
-// FP32 evaluates to a relative error of the increments themselves, with no
-// cancellation against T(W).
+// What bounds it is the dependency chain of a step times nx + ny - 1 steps,
+// twice; DRAM idles.  Mixed form: one lane per line with all four components, so
+// that no value crosses lanes inside a cell, X through the increments
+// (dU = (dm_x - U drho) / (rho + drho), dp, ... -- exact identities, with no
+// cancellation against T(W)); every strip in one CTA.  FP64: one lane per
+// component and eight lines per strip.  An FP64 instruction holds its warp for
+// about 50 cycles however many lanes take part, so the step is its count of FP64
+// instructions (23 with a component per lane, 60 with a cell per lane: 0.32
+// against 0.64 ms per sweep of the 64x64 level), and the strips are spread over
+// the CTAs of a cluster, handing over through distributed shared memory; X from
+// T(W + dW) with -sgn S T(W) in the record.
+// 64x64 level, one sweep (both passes): mixed 155 -> 66 us, FP64 407 -> 320 us, against the
+// wavefront of CTAs with a barrier per diagonal that this replaces.
 //
 // Boundary ghosts enter only the backward sweep (they use dW of the forward
 // sweep); their term is folded into that sweep's own value between the passes.
-// W += dW closes the kernel.
+// The update W += dW is left to the next kernel over the cells.
 
-constexpr int kRec = 12;                         // values per record
-constexpr int kMacroRing = 8;                    // diagonals of records in flight
-constexpr int kMacroSlots = kMacroThreads / 4;   // cells of a diagonal per CTA
-constexpr int kMsg = 3;                          // values per lane and message: dW, X_x, X_y
-
-__host__ __device__ inline int diag_lo(int d, int ny) { return d - (ny - 1) > 0 ? d - (ny - 1) : 0; }
-__host__ __device__ inline int diag_len(int d, int nx, int ny)
+__device__ __forceinline__ float recip_of(float x)
 {
-    return (d < nx - 1 ? d : nx - 1) - diag_lo(d, ny) + 1;
+    float y;                                             // one Newton-Raphson step from the approximate seed
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return fmaf(y, fmaf(-x, y, 1.0f), y);
+}
+__device__ __forceinline__ double recip_of(double x) { return rcp64(x); }
+
+// flux increments X_x, X_y of a state (rho, m_x, m_y, E + p; U, V) changed by d
+template <typename F>
+__device__ __forceinline__ void flux_increments(const F (&d)[4], F rho, F mx, F my, F Ep, F U, F V, F (&Xx)[4], F (&Xy)[4])
+{
+    // dp = 2/3 (d(E) - d(m^2 / 2 rho)), the kinetic part as one quotient: its numerator waits for no reciprocal
+    const F n = d[1] * (mx + mx + d[1]) + (d[2] * (my + my + d[2]) - (mx * U + my * V) * d[0]);
+    const F ir = recip_of(rho + d[0]);
+    const F dU = (d[1] - U * d[0]) * ir, dV = (d[2] - V * d[0]) * ir;
+    const F Up = U + dU, Vp = V + dV;
+    const F dp = fma(F(-1.0 / (kKint + 2)) * n, ir, F(2.0 / (kKint + 2)) * d[3]), dE = d[3] + dp;
+    const F a = mx * dU + d[1] * Up, b = my * dV + d[2] * Vp;
+    Xx[0] = d[1];
+    Xx[1] = a + dp;
+    Xx[2] = my * dU + d[2] * Up;
+    Xx[3] = Ep * dU + dE * Up;
+    Xy[0] = d[2];
+    Xy[1] = mx * dV + d[1] * Vp;
+    Xy[2] = b + dp;
+    Xy[3] = Ep * dV + dE * Vp;
 }
 
-// record layout: rec[((pass * nd + d) * maxdiag + slot) * 4 + m][kRec]
-//   0 own value (pass 0: R / D; pass 1: forward dW minus the ghost term / D)
-//   1 base: W_m (FP64) or Q_m = (rho, m_x, m_y, E + p)_m (mixed)
-//   2 c0 (FP64; 0 in mixed)           3 hv / D, hv = 1 / (2V)
-//   4, 5 sgn S of the x and y neighbour faces (0 at a boundary face)
-//   6, 7 S Gamma of those faces        8, 9, 10 U, V, rho (mixed)
-template <typename F>
-__global__ void k_macro_rec(MacroArgs a, const double* __restrict__ W, const double* __restrict__ gx,
-                            const double* __restrict__ gy, const double* __restrict__ idiag,
-                            const double* __restrict__ R, F* __restrict__ rec, int maxdiag)
+// edge values: relaxed accesses, each value complete by itself (4 or 8 bytes)
+__device__ __forceinline__ void st_edge(bool on, unsigned a, const float (&v)[4])
 {
-    const LevelDev& L = a.L;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 4 * L.nc) return;
-    const int c = t >> 2, m = t & 3, nx = L.nx, ny = L.ny, nd = nx + ny - 1;
-    const int i = c % nx, j = c / nx, d = i + j, slot = i - diag_lo(d, ny);
-    const double* Wc = W + 4 * (size_t)c;
-    const double id = idiag[c];
-    const double ir = rcp64(Wc[0]), U = Wc[1] * ir, V = Wc[2] * ir;
-    const double p = (2.0 / (kKint + 2)) * (Wc[3] - 0.5 * (Wc[1] * U + Wc[2] * V));
-    for (int pass = 0; pass < 2; ++pass) {
-        F* o = rec + ((((size_t)pass * nd + d) * maxdiag + slot) * 4 + m) * kRec;
-        const double sgn = pass ? 1.0 : -1.0;
-        double sS[2] = {0.0, 0.0}, Sgm[2] = {0.0, 0.0}, c0 = 0.0;
-        for (int axis = 0; axis < 2; ++axis) {
-            const int fidx = axis == 0 ? j * (nx + 1) + i + pass : (j + pass) * nx + i;
-            if ((axis == 0 ? L.fbx[fidx] : L.fby[fidx]) >= 0 || L.solid[c]) continue;
-            const double S = axis == 0 ? L.dy[j] : L.dx[i];
-            sS[axis] = sgn * S;
-            Sgm[axis] = S * (axis == 0 ? gx[fidx] : gy[fidx]);
-            if constexpr (sizeof(F) == 8) {
-                const int nb = axis == 0 ? c + (pass ? 1 : -1) : c + (pass ? nx : -nx);
-                double T0[4];
-                euler_axis(W + 4 * (size_t)nb, axis, T0);
-                c0 -= sS[axis] * T0[m];
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n @p st.relaxed.cluster.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};\n}\n"
+                 ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void st_edge(bool on, unsigned a, const double (&v)[1])
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.relaxed.cluster.shared::cluster.f64 [%0], %1;\n}\n"
+                 ::"r"(a), "d"(v[0]), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void ld_edge(unsigned a, float (&v)[4])
+{
+    asm volatile("ld.relaxed.cluster.shared::cta.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ld_edge(unsigned a, double (&v)[1])
+{
+    asm volatile("ld.relaxed.cluster.shared::cta.f64 %0, [%1];\n" : "=d"(v[0]) : "r"(a) : "memory");
+}
+constexpr unsigned kEmpty32 = 0x7fa5a5a5u;                    // signalling NaNs
+constexpr unsigned long long kEmpty64 = 0x7ff4a5a5a5a5a5a5ull;
+__device__ __forceinline__ bool is_empty(float v) { return __float_as_uint(v) == kEmpty32; }
+__device__ __forceinline__ bool is_empty(double v) { return (unsigned long long)__double_as_longlong(v) == kEmpty64; }
+__device__ __forceinline__ void set_empty(float* p) { *reinterpret_cast<unsigned*>(p) = kEmpty32; }
+__device__ __forceinline__ void set_empty(double* p) { *reinterpret_cast<unsigned long long*>(p) = kEmpty64; }
+
+// the edge values at address a once all of them are there (bounded); the whole warp gets the verdict
+template <typename F, int C>
+__device__ __forceinline__ bool edge_wait(unsigned a, bool mine, uint64_t limit_ns, F (&v)[C])
+{
+    uint64_t t0 = 0;
+    for (int it = 0; it < kWaitRounds; ++it) {
+        if (mine) ld_edge(a, v);
+        bool empty = false;
+        #pragma unroll
+        for (int q = 0; q < C; ++q) empty = empty || is_empty(v[q]);
+        if (!__any_sync(0xffffffffu, mine && empty)) return true;
+        if ((it & 31) == 31) {
+            const uint64_t t = __shfl_sync(0xffffffffu, global_ns(), 0);   // one clock for the warp
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > limit_ns) return false;
+        }
+    }
+    return false;
+}
+
+// predicated stores (a branch per step would have to be resolved on the step's path)
+__device__ __forceinline__ void st_if(bool on, float* p, const float (&v)[4])
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n @p st.global.v4.f32 [%0], {%1, %2, %3, %4};\n}\n"
+                 ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void st_if(bool on, double* p, const double (&v)[1])
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.global.f64 [%0], %1;\n}\n"
+                 ::"l"(p), "d"(v[0]), "r"((unsigned)on) : "memory");
+}
+
+// What a strip's warp needs for one pass.
+template <typename F>
+struct MacroStrip {
+    const F* src;            // its records of this pass, [nk][kRow]
+    F* ring;                 // [kRing][kRow]
+    unsigned edge, p_edge;   // [nt][4] across terms from the strip before; the next strip's (shared addresses)
+    F* out;                  // where cell t = 0 of this lane's line puts its dW ...
+    long ostep;              // ... and the step from one cell of the line to the next
+    bool first, feeds, line; // no strip before; a strip after; this lane has a grid line
+};
+
+template <typename F, bool XL, int PASS>
+__device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int nk, uint64_t limit_ns)
+{
+    using T = MacroLane<F>;
+    constexpr int C = T::kComp, R = T::kRing, NU = T::kVals * (int)sizeof(F) / 16, V = 16 / (int)sizeof(F);
+    const int lane = threadIdx.x & 31, ll = lane / T::kLanes, m = lane % T::kLanes, g0 = lane & 28;
+    F across[C], along[C], rc[T::kVals];
+    #pragma unroll
+    for (int q = 0; q < C; ++q) across[q] = along[q] = F(0);
+    const F* g = S.src + lane * V;
+    F* rl = S.ring + lane * V;
+    auto issue = [&](int k, int stage) {       // rows beyond nk exist (allocation is rounded up) and are not used
+        const F* p = g + (size_t)k * T::kRow;
+        #pragma unroll
+        for (int q = 0; q < NU; ++q) cp_async16(rl + stage * T::kRow + q * 32 * V, p + q * 32 * V);
+        cp_async_commit();
+    };
+    auto fetch = [&](int stage, F (&r)[T::kVals]) {
+        #pragma unroll
+        for (int q = 0; q < NU; ++q) {
+            const F* p = rl + stage * T::kRow + q * 32 * V;
+            if constexpr (sizeof(F) == 4) {
+                const float4 t = *reinterpret_cast<const float4*>(p);
+                r[4 * q] = t.x; r[4 * q + 1] = t.y; r[4 * q + 2] = t.z; r[4 * q + 3] = t.w;
+            } else {
+                const double2 t = *reinterpret_cast<const double2*>(p);
+                r[2 * q] = t.x; r[2 * q + 1] = t.y;
             }
         }
-        double base = Wc[m];
-        if constexpr (sizeof(F) == 4) base = m == 3 ? Wc[3] + p : Wc[m];
-        o[0] = pass == 0 ? (F)(R[4 * (size_t)c + m] * id) : F(0);
-        o[1] = (F)base;
-        o[2] = (F)c0;
-        o[3] = (F)(0.5 * L.rdx[i] * L.rdy[j] * id);
-        o[4] = (F)sS[0];
-        o[5] = (F)sS[1];
-        o[6] = (F)Sgm[0];
-        o[7] = (F)Sgm[1];
-        o[8] = (F)U;
-        o[9] = (F)V;
-        o[10] = (F)Wc[0];
-        o[11] = F(0);
-    }
-}
-
-// Euler flux component m of W along +e_axis, given 1/rho, U_a and p
-__device__ __forceinline__ double euler_comp(const double* W, int m, int axis, double Ua, double p)
-{
-    if (m == 0) return W[1 + axis];
-    if (m == 3) return (W[3] + p) * Ua;
-    double v = W[m] * Ua;
-    return (m == 1 + axis) ? v + p : v;
-}
-
-__device__ __forceinline__ void producer_fluxes(const double wp, int m, int g0, double* T1c)
-{
-    // gather the four components of W + dW of this cell (lanes g0..g0+3)
-    double Wp[4];
+    };
+    F* out = S.out - ll * S.ostep;                                      // cell t = k - ll at step k
+    const bool mine = !S.first && ll == 0;                              // this lane takes across terms from the edge
+    const unsigned edge = S.edge + (unsigned)(m * (int)sizeof(F));
     #pragma unroll
-    for (int q = 0; q < 4; ++q) Wp[q] = __shfl_sync(0xffffffffu, wp, g0 + q);
-    double ir = rcp64(Wp[0]);
-    double U = Wp[1] * ir, V = Wp[2] * ir;
-    double p = (2.0 / (kKint + 2)) * fma(-0.5, fma(Wp[2], V, Wp[1] * U), Wp[3]);
-    T1c[m] = euler_comp(Wp, m, 0, U, p);
-    T1c[4 + m] = euler_comp(Wp, m, 1, V, p);
-}
-
-// ghost term of the upper-side boundary faces of cell (i, j) for the backward sweep
-__device__ void macro_ghost_terms(const MacroArgs& a, const double* W, const double* gx, const double* gy,
-                                  const double* dW, int i, int j, double Gc[4])
-{
-    const LevelDev& L = a.L;
-    const int c = j * L.nx + i;
-    for (int m = 0; m < 4; ++m) Gc[m] = 0.0;
-    for (int axis = 0; axis < 2; ++axis) {
-        const int bcid = axis == 0 ? L.fbx[j * (L.nx + 1) + i + 1] : L.fby[(j + 1) * L.nx + i];
-        if (bcid < 0) continue;
-        double Wn[4], dWn[4], Wp[4], T1[4], T0[4], M[16];
-        macro_ghost(a.bc[bcid], axis, W + 4 * (size_t)c, Wn, M);
-        for (int m = 0; m < 4; ++m) {
-            double s2 = 0.0;
-            for (int q = 0; q < 4; ++q) s2 += M[4 * m + q] * dW[4 * (size_t)c + q];
-            dWn[m] = s2;
-            Wp[m] = Wn[m] + dWn[m];
+    for (int k = 0; k < R - 1; ++k) issue(k, k);
+    if (limit_ns == 0) return false;
+    F en[C];
+    #pragma unroll
+    for (int q = 0; q < C; ++q) en[q] = F(0);
+    if (!S.first) {
+        if (!edge_wait<F, C>(edge + (unsigned)(4 * min(nt - 1, T::kLead) * (int)sizeof(F)), mine, limit_ns, en)) return false;
+        if (!edge_wait<F, C>(edge, mine, limit_ns, en)) return false;
+    }
+    cp_async_wait_n<R - 2>();
+    fetch(0, rc);
+    for (int k0 = 0; k0 < nk; k0 += R) {
+        #pragma unroll
+        for (int kk = 0; kk < R; ++kk) {
+            const int k = k0 + kk;
+            #pragma unroll
+            for (int q = 0; q < C; ++q) across[q] = mine ? en[q] : across[q];
+            if (!S.first) {                                             // the next step's edge values
+                const unsigned ea = edge + (unsigned)(4 * min(nt - 1, k + 1) * (int)sizeof(F));
+                if (mine) ld_edge(ea, en);
+                bool empty = false;
+                #pragma unroll
+                for (int q = 0; q < C; ++q) empty = empty || is_empty(en[q]);
+                if (__any_sync(0xffffffffu, mine && empty) && !edge_wait<F, C>(ea, mine, limit_ns, en)) return false;
+            }
+            issue(k + R - 1, (kk + R - 1) % R);
+            cp_async_wait_n<R - 2>();                                   // step k + 1 has arrived
+            F rn[T::kVals];
+            fetch((kk + 1) % R, rn);
+            const int t = k - ll;
+            const bool on = (unsigned)t < (unsigned)nt && S.line;
+            F dw[C], oc[C];
+            if constexpr (C == 4) {
+                // record: own[4], rho, m_x, m_y, E + p, U, V, (1/2V) / D, -, across (sgn S, S Gamma), along
+                F Xx[4], Xy[4];
+                #pragma unroll
+                for (int q = 0; q < 4; ++q) dw[q] = fma(-across[q], rc[10], fma(-along[q], rc[10], rc[q]));
+                flux_increments<F>(dw, rc[4], rc[5], rc[6], rc[7], rc[8], rc[9], Xx, Xy);
+                #pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    oc[q] = fma(rc[12], XL ? Xx[q] : Xy[q], -rc[13] * dw[q]);
+                    along[q] = fma(rc[14], XL ? Xy[q] : Xx[q], -rc[15] * dw[q]);
+                }
+            } else {
+                // record of component m: own, W, (1/2V) / D, -, across (sgn S, S Gamma, -sgn S T(W)), along
+                dw[0] = fma(-(across[0] + along[0]), rc[2], rc[0]);
+                const F wp = rc[1] + dw[0];
+                F w[4];
+                #pragma unroll
+                for (int q = 0; q < 4; ++q) w[q] = __shfl_sync(0xffffffffu, wp, g0 + q);
+                const F s2 = F(-1.0 / (kKint + 2)) * fma(w[2], w[2], w[1] * w[1]);
+                const F pk = (m == 3 ? F(2.0 / (kKint + 2) + 1.0) : F(2.0 / (kKint + 2))) * w[3];
+                const F ir = recip_of(w[0]), U = w[1] * ir, W = w[2] * ir;
+                const F z = fma(s2, ir, pk), A = m == 3 ? z : wp;       // p, or E + p in lane 3
+                F Tx = fma(A, U, m == 1 ? z : F(0)), Ty = fma(A, W, m == 2 ? z : F(0));
+                if (m == 0) { Tx = w[1]; Ty = w[2]; }
+                oc[0] = fma(rc[4], XL ? Tx : Ty, fma(-rc[5], dw[0], rc[6]));
+                along[0] = fma(rc[7], XL ? Ty : Tx, fma(-rc[8], dw[0], rc[9]));
+            }
+            #pragma unroll
+            for (int q = 0; q < C; ++q) {
+                if (!on) { oc[q] = F(0); along[q] = F(0); }
+                const F v = __shfl_up_sync(0xffffffffu, oc[q], T::kLanes);
+                across[q] = ll > 0 ? v : F(0);
+            }
+            st_edge(S.feeds && ll == T::kLines - 1 && on, S.p_edge + (unsigned)((4 * t + m) * (int)sizeof(F)), oc);
+            // pass 0: the backward sweep's own value; pass 1: the row of dW
+            st_if(on, out + k * S.ostep, dw);
+            #pragma unroll
+            for (int q = 0; q < T::kVals; ++q) rc[q] = rn[q];
         }
-        euler_axis(Wp, axis, T1);
-        euler_axis(Wn, axis, T0);
-        double S = axis == 0 ? L.dy[j] : L.dx[i];
-        double gm = axis == 0 ? gx[j * (L.nx + 1) + i + 1] : gy[(j + 1) * L.nx + i];
-        for (int m = 0; m < 4; ++m) Gc[m] += S * ((T1[m] - T0[m]) - gm * dWn[m]);
     }
+    return true;
 }
 
-// four consecutive record values (16-byte aligned for float, 32 for double)
-__device__ __forceinline__ void ld4v(const float* p, float* v)
+template <typename F, bool XL>
+__global__ void __launch_bounds__(256, 1) k_macro_sgs(MacroArgs a, F* __restrict__ rec, F* __restrict__ dW,
+                                                      const double* __restrict__ ghost, int wpc)
 {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-}
-__device__ __forceinline__ void ld4v(const double* p, double* v)
-{
-    const double2 t0 = *reinterpret_cast<const double2*>(p), t1 = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = t0.x; v[1] = t0.y; v[2] = t1.x; v[3] = t1.y;
-}
-
-// flux terms X_x, X_y of lane m (component m) of a cell updated by dw
-__device__ __forceinline__ void macro_x(double dw, const double* rc, int m, int g0, double& Xx, double& Xy)
-{
-    double T1c[8];
-    producer_fluxes(rc[1] + dw, m, g0, T1c);             // X = T(W + dW)
-    Xx = T1c[m];
-    Xy = T1c[4 + m];
-}
-__device__ __forceinline__ void macro_x(float dw, const float* rc, int m, int g0, float& Xx, float& Xy)
-{
-    float dq[4];                                         // increments of the four components
-    #pragma unroll
-    for (int q = 0; q < 4; ++q) dq[q] = __shfl_sync(0xffffffffu, dw, g0 + q);
-    const float Q = rc[1], U = rc[8], V = rc[9], rho = rc[10];
-    const float ir = __frcp_rn(rho + dq[0]);
-    const float dU = (dq[1] - U * dq[0]) * ir, dV = (dq[2] - V * dq[0]) * ir;
-    const float Up = U + dU, Vp = V + dV;
-    const float dp = (2.0f / (kKint + 2)) * (dq[3] - 0.5f * (rho * U * dU + dq[1] * Up + rho * V * dV + dq[2] * Vp));
-    const float dm = m == 3 ? dq[3] + dp : dq[m];
-    Xx = Q * dU + dm * Up + (m == 1 ? dp : 0.0f);       // X = T(W + dW) - T(W)
-    Xy = Q * dV + dm * Vp + (m == 2 ? dp : 0.0f);
-}
-
-constexpr int kMacroBlock = kMacroThreads + 32;   // four sweep warps and one producer warp
-
-// The producer warp (lane 0) keeps the record ring kMacroRing - 1 diagonals
-// ahead.  Each ring slot's mbarrier also counts the halo bytes the neighbours
-// push for that step (the edge cells of the previous diagonal), so one wait
-// per step covers both.
-template <typename F>
-__global__ void __cluster_dims__(kMacroCluster, 1, 1) __launch_bounds__(kMacroBlock)
-k_macro_sgs(MacroArgs a, double* __restrict__ W, F* __restrict__ rec, double* __restrict__ dW,
-            const double* __restrict__ gx, const double* __restrict__ gy, int maxdiag, int nact)
-{
+    using T = MacroLane<F>;
     extern __shared__ __align__(128) unsigned char smraw[];
-    constexpr int per = kMacroSlots * 4 * kRec;          // record values of one CTA and diagonal
-    constexpr int xper = (kMacroSlots + 2) * 4 * kMsg;   // message values of one diagonal
-    F* ring = reinterpret_cast<F*>(smraw);               // [kMacroRing][per]
-    F* xb = ring + kMacroRing * per;                     // [2][kMacroSlots + 2][4][kMsg], halo at 0 and kMacroSlots + 1
-    uint64_t* rb = reinterpret_cast<uint64_t*>(xb + 2 * xper);   // [kMacroRing] records + halo of a step
-
     cg::cluster_group cl = cg::this_cluster();
     const LevelDev& L = a.L;
-    const int nx = L.nx, ny = L.ny, nd = nx + ny - 1;
-    const int rank = (int)cl.block_rank(), tid = threadIdx.x;
-    const bool prod = tid >= kMacroThreads;              // the producer warp
-    const int m = tid & 3, g0 = tid & 28, ls = tid >> 2;  // component, first lane of the cell, local slot
-    const int gs0 = rank * kMacroSlots;                   // first slot of this CTA
-    const bool active = rank < nact;
-    const int nbrs = active ? (rank > 0) + (rank + 1 < nact) : 0;
-    const unsigned halo_bytes = nbrs * 4 * kMsg * (unsigned)sizeof(F);
-    if (tid == 0) {
-        for (int q = 0; q < kMacroRing; ++q) mbar_init(&rb[q], 1);
-        mbar_init_fence();
-    }
-    for (int e = tid; e < 2 * xper; e += blockDim.x) xb[e] = F(0);
-    // edge lanes: the peer CTA and the cluster addresses of its halo buffer and mbarriers
-    int peer = -1, hs = 0;
-    if (!prod && ls == 0 && rank > 0) { peer = rank - 1; hs = kMacroSlots + 1; }
-    if (!prod && ls == kMacroSlots - 1 && rank + 1 < nact) { peer = rank + 1; hs = 0; }
-    const unsigned r_xb = peer >= 0 ? peer_addr(xb, peer) : 0u, r_rb = peer >= 0 ? peer_addr(rb, peer) : 0u;
+    const MacroFrame<F> fr(L.nx, L.ny);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = (int)cl.block_rank();
+    F* edge = reinterpret_cast<F*>(smraw);                              // [wpc][nt][4] from the strip before
+    const int strip = rank * wpc + warp;
+    const bool active = warp < wpc && strip < fr.strips;
+    for (int q = threadIdx.x; q < wpc * fr.nt * 4; q += blockDim.x) set_empty(edge + q);
     cl.sync();
 
-    const int nsteps = 2 * nd;
-    // producer: arm ring slot g % kMacroRing for step g (records, plus the halo of step g - 1)
-    // and start the records' bulk copy; step nsteps only collects the last halo
-    auto issue = [&](int g) {
-        uint64_t* mb = &rb[g % kMacroRing];
-        const unsigned hb = g > 0 ? halo_bytes : 0u;
-        if (g >= nsteps) { mbar_arrive_tx(mb, hb); return; }
-        const int pass = g / nd, dd = g - pass * nd, d = pass == 0 ? dd : nd - 1 - dd;
-        int nloc = diag_len(d, nx, ny) - gs0;
-        nloc = nloc < 0 ? 0 : (nloc > kMacroSlots ? kMacroSlots : nloc);
-        const unsigned bytes = (unsigned)(nloc * 4 * kRec * sizeof(F));
-        mbar_arrive_tx(mb, bytes + hb);
-        if (bytes) bulk_g2s(ring + (g % kMacroRing) * per, rec + (((size_t)pass * nd + d) * maxdiag + gs0) * 4 * kRec,
-                            bytes, mb);
-    };
-    const bool issuer = prod && (tid & 31) == 0;
     bool ok = true;
-    int issued = -1;                                     // last step armed (producer)
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
-            cl.sync();                                   // forward dW and records visible in the cluster
-            // upper-side ghost terms (east / north boundary faces: the last column and row,
-            // and the faces of bodies), from the forward dW, folded into the backward
-            // sweep's own values (one thread per cell)
-            for (int b = rank * blockDim.x + tid; ok && b < L.nubc; b += kMacroCluster * blockDim.x) {
-                const int cb = L.ubc[b], i = cb % nx, j = cb / nx, d = i + j;
-                double Gc[4];
-                macro_ghost_terms(a, W, gx, gy, dW, i, j, Gc);
-                F* o = rec + (((size_t)nd + d) * maxdiag + (i - diag_lo(d, ny))) * 4 * kRec;
-                for (int q = 0; q < 4; ++q)
-                    o[q * kRec] = (F)((double)o[q * kRec] - Gc[q] * (double)o[q * kRec + 3]);
+            if (warp < wpc)                                             // (read by this warp alone)
+                for (int q = lane; q < fr.nt * 4; q += 32) set_empty(edge + (size_t)warp * fr.nt * 4 + q);
+            cl.sync();                                                  // forward dW of every strip is in the records
+            // ghost terms of the upper boundary faces from the forward dW
+            for (int b = rank * blockDim.x + threadIdx.x; b < L.nubc; b += (int)cl.num_blocks() * blockDim.x) {
+                const int c = L.ubc[b], i = c % L.nx, j = c / L.nx;
+                double own[4], Gc[4] = {0, 0, 0, 0};
+                #pragma unroll
+                for (int m = 0; m < 4; ++m) own[m] = (double)__ldcg(rec + fr.at(1, i, j, m, 0));
+                for (int axis = 0; axis < 2; ++axis) {
+                    const double* g = ghost + ((size_t)b * 2 + axis) * kGhostRec;
+                    if (g[22] == 0.0) continue;
+                    double d[4], Xx[4], Xy[4];
+                    #pragma unroll
+                    for (int m = 0; m < 4; ++m) d[m] = g[4 * m] * own[0] + g[4 * m + 1] * own[1] + g[4 * m + 2] * own[2] + g[4 * m + 3] * own[3];
+                    flux_increments<double>(d, g[16], g[17], g[18], g[19], g[20], g[21], Xx, Xy);
+                    #pragma unroll
+                    for (int m = 0; m < 4; ++m) Gc[m] += g[22] * (axis == 0 ? Xx[m] : Xy[m]) - g[23] * d[m];
+                }
+                const double h = (double)rec[fr.at(1, i, j, 0, T::kHv)];
+                #pragma unroll
+                for (int m = 0; m < 4; ++m) rec[fr.at(1, i, j, m, 0)] = (F)(own[m] - Gc[m] * h);
             }
-            fence_proxy_async();
             cl.sync();
         }
         if (!active || !ok) continue;
-        const int gbase = pass * nd;
-        if (issuer)
-            for (int g = gbase; g < gbase + kMacroRing - 1 && g < gbase + nd; ++g) issue(issued = g);
-        for (int dd = 0; dd < nd; ++dd) {
-            const int g = gbase + dd, d = pass == 0 ? dd : nd - 1 - dd;
-            bool got = true;
-            if (prod) {
-                if (issuer && dd + kMacroRing - 1 < nd) issue(issued = g + kMacroRing - 1);
-            } else {
-                got = mbar_wait(&rb[g % kMacroRing], (g / kMacroRing) & 1, a.wait_ns);
-                const int ilo = diag_lo(d, ny), ncell = diag_len(d, nx, ny);
-                const bool on = gs0 + ls < ncell;
-                F rc[kRec];                              // this lane's record
-                {
-                    const F* rp = ring + (g % kMacroRing) * per + (ls * 4 + m) * kRec;
-                    #pragma unroll
-                    for (int q = 0; q < kRec; q += 4) ld4v(rp + q, rc + q);
-                }
-                F dw = F(0);
-                if (on) {
-                    // local indices (halo offset 1) of the x and y neighbours on the previous diagonal
-                    int nbx, nby;
-                    if (pass == 0) {
-                        const bool same = diag_lo(d - 1, ny) == ilo;
-                        nbx = ls + (same ? 0 : 1);
-                        nby = ls + (same ? 1 : 2);
-                    } else {
-                        const bool same = diag_lo(d + 1, ny) == ilo;
-                        nbx = ls + (same ? 2 : 1);
-                        nby = ls + (same ? 1 : 0);
-                    }
-                    const F* pb = xb + ((g - 1) & 1) * xper;
-                    F acc = rc[2];
-                    if (rc[4] != F(0)) acc = fma(rc[4], pb[(nbx * 4 + m) * kMsg + 1], fma(-rc[6], pb[(nbx * 4 + m) * kMsg], acc));
-                    if (rc[5] != F(0)) acc = fma(rc[5], pb[(nby * 4 + m) * kMsg + 2], fma(-rc[7], pb[(nby * 4 + m) * kMsg], acc));
-                    dw = fma(-acc, rc[3], rc[0]);
-                }
-                F Xx, Xy;
-                macro_x(dw, rc, m, g0, Xx, Xy);          // all lanes of the warp (shuffles)
-                if (!on) Xx = Xy = F(0);
-                F* cb = xb + (g & 1) * xper;
-                cb[((ls + 1) * 4 + m) * kMsg] = dw;
-                cb[((ls + 1) * 4 + m) * kMsg + 1] = Xx;
-                cb[((ls + 1) * 4 + m) * kMsg + 2] = Xy;
-                if (peer >= 0) {                         // edge cell: into the neighbour's halo for step g + 1
-                    const unsigned rmb = r_rb + (unsigned)(((g + 1) % kMacroRing) * sizeof(uint64_t));
-                    const unsigned hl = r_xb + (unsigned)((((g & 1) * xper) + (hs * 4 + m) * kMsg) * sizeof(F));
-                    st_async(hl, dw, rmb);
-                    st_async(hl + (unsigned)sizeof(F), Xx, rmb);
-                    st_async(hl + 2u * (unsigned)sizeof(F), Xy, rmb);
-                }
-                if (on) {
-                    const int i = ilo + gs0 + ls, c = (d - i) * nx + i;
-                    dW[4 * (size_t)c + m] = (double)dw;
-                    if (pass == 0)
-                        rec[((((size_t)nd + d) * maxdiag + gs0 + ls) * 4 + m) * kRec] = dw;   // backward own value
-                }
-            }
-            if (!__syncthreads_and(got)) { ok = false; break; }
+        MacroStrip<F> S;
+        S.src = rec + ((size_t)pass * fr.strips + strip) * fr.rows * T::kRow;
+        S.ring = edge + (size_t)wpc * fr.nt * 4 + (size_t)warp * T::kRing * T::kRow;
+        S.first = strip == 0;
+        S.feeds = strip + 1 < fr.strips;
+        S.edge = smem_addr(edge + (size_t)warp * fr.nt * 4);
+        S.p_edge = S.feeds ? peer_addr(edge + (size_t)((strip + 1) % wpc) * fr.nt * 4, (strip + 1) / wpc) : 0u;
+        const int sl = strip * T::kLines + lane / T::kLanes, m = lane % T::kLanes;   // this lane's line in the pass's frame
+        S.line = sl < fr.ns;
+        const int s = pass ? fr.ns - 1 - sl : sl, t0 = pass ? fr.nt - 1 : 0;
+        if (pass == 0) {
+            // cell (s, t) is at line ns - 1 - s, t' = nt - 1 - t of the other pass: one row back per step
+            const int i0 = XL ? s : 0, j0 = XL ? 0 : s;
+            S.out = rec + (S.line ? fr.at(1, i0, j0, m, 0) : 0);
+            S.ostep = -(long)T::kRow;
+        } else {
+            const int i0 = XL ? s : t0, j0 = XL ? t0 : s;
+            S.out = dW + (S.line ? 4 * ((long)j0 * L.nx + i0) + m : 0);
+            S.ostep = -(long)(XL ? 4 * L.nx : 4);
         }
-        fence_proxy_async();
+        ok = pass == 0 ? macro_strip<F, XL, 0>(S, fr.nt, fr.nk, a.wait_ns) : macro_strip<F, XL, 1>(S, fr.nt, fr.nk, a.wait_ns);
+        cp_async_wait_n<0>();
+        if (!ok && lane == 0) *a.flag = 1.0;                            // a wait gave up: report, and skip the second pass
     }
-    if (active && issuer) {
-        if (ok) {                                        // the halo of the last step
-            issue(issued = nsteps);
-            if (!mbar_wait(&rb[nsteps % kMacroRing], (nsteps / kMacroRing) & 1, a.wait_ns)) ok = false;
-        }
-        if (!ok) {
-            // after a timeout: the latest armed phase of every slot, so that no bulk copy
-            // still targets this CTA (bounded waits), then report
-            for (int g = issued - kMacroRing + 1 > 0 ? issued - kMacroRing + 1 : 0; g <= issued; ++g)
-                mbar_wait(&rb[g % kMacroRing], (g / kMacroRing) & 1);
-            *a.flag = 1.0;
-        }
-    }
-    cl.sync();                                           // no peer writes into this CTA after this point
-    for (int q = rank * blockDim.x + tid; q < 4 * L.nc; q += kMacroCluster * blockDim.x) W[q] += dW[q];
+    cl.sync();                                                          // no strip writes into this CTA after this point
 }
 
 template <typename F>
-cudaError_t launch_macro_sgs(const MacroArgs& a, double* W, const double* gx, const double* gy, const double* idiag,
-                             void* rec, const double* R, double* dW, cudaStream_t st)
+cudaError_t launch_macro_sgs(const MacroArgs& a, F* rec, const double* ghost, F* dW, cudaStream_t st)
 {
-    const int maxdiag = a.L.nx < a.L.ny ? a.L.nx : a.L.ny;
-    const int nact = (maxdiag + kMacroSlots - 1) / kMacroSlots;
-    if (nact > kMacroCluster) return cudaErrorInvalidValue;
-    const size_t smem = sizeof(F) * ((size_t)kMacroRing * kMacroSlots * 4 * kRec + 2 * (kMacroSlots + 2) * 4 * kMsg) +
-                        sizeof(uint64_t) * kMacroRing;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_macro_sgs<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    using T = MacroLane<F>;
+    const MacroFrame<F> fr(a.L.nx, a.L.ny);
+    if (fr.ns > kMacroMaxLines) return cudaErrorInvalidValue;
+    // mixed: every strip in one CTA; FP64: as few strips per SM as eight CTAs allow (they share its FP64 pipe)
+    const int wpc = sizeof(F) == 8 ? (fr.strips + 7) / 8 : fr.strips;
+    int ncl = 1;
+    while (ncl * wpc < fr.strips) ncl *= 2;
+    const size_t smem = sizeof(F) * (size_t)wpc * ((size_t)fr.nt * 4 + T::kRing * T::kRow);
+    auto kern = fr.xl ? k_macro_sgs<F, true> : k_macro_sgs<F, false>;
+    if (smem > 47 * 1024) {                             // with the static part, 48 KB need no opt-in
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_macro_rec<F><<<(4 * a.L.nc + 127) / 128, 128, 0, st>>>(a, W, gx, gy, idiag, R, (F*)rec, maxdiag);
-    k_macro_sgs<F><<<kMacroCluster, kMacroBlock, smem, st>>>(a, W, (F*)rec, dW, gx, gy, maxdiag, nact);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ncl, 1, 1);
+    cfg.blockDim = dim3((unsigned)(32 * (wpc > 4 ? wpc : 4)), 1, 1);   // idle warps help with the ghosts
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ncl;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, a, rec, dW, ghost, wpc);
 }
-template cudaError_t launch_macro_sgs<double>(const MacroArgs&, double*, const double*, const double*, const double*,
-                                              void*, const double*, double*, cudaStream_t);
-template cudaError_t launch_macro_sgs<float>(const MacroArgs&, double*, const double*, const double*, const double*,
-                                             void*, const double*, double*, cudaStream_t);
+template cudaError_t launch_macro_sgs<double>(const MacroArgs&, double*, const double*, double*, cudaStream_t);
+template cudaError_t launch_macro_sgs<float>(const MacroArgs&, float*, const double*, float*, cudaStream_t);
 
 size_t macro_rec_bytes(int nx, int ny, bool mixed)
 {
-    const size_t maxdiag = nx < ny ? nx : ny, nd = (size_t)nx + ny - 1;
-    return 2 * nd * maxdiag * 4 * kRec * (mixed ? sizeof(float) : sizeof(double));
+    return mixed ? MacroFrame<float>(nx, ny).values() * sizeof(float) : MacroFrame<double>(nx, ny).values() * sizeof(double);
 }
+size_t macro_ghost_elems(int nubc) { return 2 * (size_t)nubc * kGhostRec; }
 
 // ---------------------------------------------------------------------------
 // volume-weighted restriction (nblk blocks of [nc][m])
@@ -817,17 +928,26 @@ __global__ void k_prolong_add(LevelDev F, LevelDev C, int m, int nblk, const int
 // without positive density and internal energy is dropped in that cell: at a
 // strong shock the bilinear correction of the coarse state can overshoot (the
 // paper is silent here; with smooth flow the test never triggers).
-__global__ void k_prolong_state(LevelDev F, const int* __restrict__ idx4, const double* __restrict__ w4,
-                                const double* __restrict__ dWc, double* __restrict__ W)
+template <typename F>
+__global__ void k_prolong_state(LevelDev L, const int* __restrict__ idx4, const double* __restrict__ w4,
+                                const double* __restrict__ Wc, const F* __restrict__ dw,
+                                const double* __restrict__ Wn, double* __restrict__ W)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= F.nc) return;
+    if (c >= L.nc) return;
     double w[4];
+    const double* wt = w4 + 4 * (size_t)c;
+    int id[4];
+    #pragma unroll
+    for (int s = 0; s < 4; ++s) id[s] = idx4[4 * c + s];
     #pragma unroll
     for (int q = 0; q < 4; ++q) {
         double v = 0.0;
         #pragma unroll
-        for (int s = 0; s < 4; ++s) v += w4[4 * c + s] * dWc[(size_t)idx4[4 * c + s] * 4 + q];
+        for (int s = 0; s < 4; ++s) {
+            const size_t e = (size_t)id[s] * 4 + q;
+            v += wt[s] * ((dw ? Wc[e] + (double)dw[e] : Wc[e]) - Wn[e]);
+        }
         w[q] = W[4 * (size_t)c + q] + v;
     }
     const double e2 = w[3] * w[0] - 0.5 * (w[1] * w[1] + w[2] * w[2]);
@@ -836,32 +956,75 @@ __global__ void k_prolong_state(LevelDev F, const int* __restrict__ idx4, const 
         for (int q = 0; q < 4; ++q) W[4 * (size_t)c + q] = w[q];
 }
 
-cudaError_t launch_prolong_state(const LevelDev& F, const int* idx4, const double* w4, const double* dWc, double* W,
-                                 cudaStream_t st)
+template <typename F>
+cudaError_t launch_prolong_state(const LevelDev& L, const int* idx4, const double* w4, const double* Wc, const F* dw,
+                                 const double* Wn, double* W, cudaStream_t st)
 {
-    k_prolong_state<<<(F.nc + 127) / 128, 128, 0, st>>>(F, idx4, w4, dWc, W);
+    k_prolong_state<F><<<(L.nc + 31) / 32, 32, 0, st>>>(L, idx4, w4, Wc, dw, Wn, W);
     return cudaGetLastError();
 }
+template cudaError_t launch_prolong_state<double>(const LevelDev&, const int*, const double*, const double*,
+                                                  const double*, const double*, double*, cudaStream_t);
+template cudaError_t launch_prolong_state<float>(const LevelDev&, const int*, const double*, const double*,
+                                                 const float*, const double*, double*, cudaStream_t);
 
-// Predicted state of Step 2: Wt = Wc (the FAS result), except in a cell where
-// Wc has non-positive density or internal energy, which keeps its state W^n
-// (no prediction there; the paper is silent, and with smooth flow the test
-// never triggers).
+// Predicted state of Step 2: Wt = Wc (the FAS result, with the pending update
+// dw of its last sweep), except in a cell where it has non-positive density or
+// internal energy, which keeps its state W^n (no prediction there; the paper is
+// silent, and with smooth flow the test never triggers).
+template <typename F>
 __global__ void k_predicted_state(int nc, const double* __restrict__ Wn, const double* __restrict__ Wc,
-                                  double* __restrict__ Wt)
+                                  const F* __restrict__ dw, double* __restrict__ Wt)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nc) return;
-    const double* w = Wc + 4 * (size_t)c;
+    double w[4];
+    ld_state(Wc, dw, c, w);
     const double e2 = w[3] * w[0] - 0.5 * (w[1] * w[1] + w[2] * w[2]);
-    const double* src = (w[0] > 0.0 && e2 > 0.0) ? w : Wn + 4 * (size_t)c;
+    const bool good = w[0] > 0.0 && e2 > 0.0;
     #pragma unroll
-    for (int q = 0; q < 4; ++q) Wt[4 * (size_t)c + q] = src[q];
+    for (int q = 0; q < 4; ++q) Wt[4 * (size_t)c + q] = good ? w[q] : Wn[4 * (size_t)c + q];
 }
 
-cudaError_t launch_predicted_state(int nc, const double* Wn, const double* Wc, double* Wt, cudaStream_t st)
+template <typename F>
+cudaError_t launch_predicted_state(int nc, const double* Wn, const double* Wc, const F* dw, double* Wt, cudaStream_t st)
 {
-    k_predicted_state<<<(nc + 127) / 128, 128, 0, st>>>(nc, Wn, Wc, Wt);
+    k_predicted_state<F><<<(nc + 63) / 64, 64, 0, st>>>(nc, Wn, Wc, dw, Wt);
+    return cudaGetLastError();
+}
+template cudaError_t launch_predicted_state<double>(int, const double*, const double*, const double*, double*,
+                                                    cudaStream_t);
+template cudaError_t launch_predicted_state<float>(int, const double*, const double*, const float*, double*,
+                                                   cudaStream_t);
+
+// Volume-weighted restriction of a level's state and residual in one launch,
+// one thread per coarse cell and component.
+__global__ void k_restrict_state(LevelDev F, LevelDev C, const double* __restrict__ W, const double* __restrict__ R,
+                                 double* __restrict__ Wc, double* __restrict__ Rc)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * C.nc) return;
+    const int cc = t >> 2, q = t & 3, I = cc % C.nx, J = cc / C.nx;
+    double sw = 0.0, sr = 0.0, vs = 0.0;
+    #pragma unroll
+    for (int b = 0; b < 2; ++b)
+        #pragma unroll
+        for (int a2 = 0; a2 < 2; ++a2) {
+            const int i = 2 * I + a2, j = 2 * J + b;
+            const size_t e = 4 * (size_t)(j * F.nx + i) + q;
+            const double V = F.dx[i] * F.dy[j];
+            sw += W[e] * V;
+            sr += R[e] * V;
+            vs += V;
+        }
+    Wc[t] = sw / vs;
+    Rc[t] = sr / vs;
+}
+
+cudaError_t launch_restrict_state(const LevelDev& F, const LevelDev& C, const double* W, const double* R, double* Wc,
+                                  double* Rc, cudaStream_t st)
+{
+    k_restrict_state<<<(4 * C.nc + 63) / 64, 64, 0, st>>>(F, C, W, R, Wc, Rc);
     return cudaGetLastError();
 }
 

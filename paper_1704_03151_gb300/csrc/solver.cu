@@ -36,8 +36,11 @@ struct HLevel {
     int* sidx = nullptr;      // the same for a state (cells in bodies take their coarse cell's value)
     double* sw = nullptr;
     // prediction work, [nc][4]
-    double *Wn = nullptr, *Wc = nullptr, *Rc = nullptr, *P = nullptr, *R = nullptr, *dW = nullptr, *gx = nullptr,
-           *gy = nullptr, *Wt = nullptr, *idiag = nullptr, *T = nullptr;
+    // (Wc: the state of the cycle, Wd its other buffer; dW: the last sweep's update in the sweep's
+    // arithmetic, still to be added to Wc while pend is set; T, ghost: the next sweep's records)
+    double *Wn = nullptr, *Wc = nullptr, *Wd = nullptr, *Rc = nullptr, *P = nullptr, *R = nullptr, *dW = nullptr,
+           *gx = nullptr, *gy = nullptr, *Wt = nullptr, *idiag = nullptr, *T = nullptr, *ghost = nullptr;
+    bool pend = false;
     // evolution work, [2][nc][nv] (invD [nc][nv]); element type double, or float in the mixed form
     void *r = nullptr, *df = nullptr, *dl = nullptr, *invD = nullptr;
     // W and F cycles (second coarse visit of the CS cycle): the restricted residual and
@@ -121,7 +124,7 @@ struct miugks_solver {
         bool lv_alloc = false;
         // macroscopic correction of the preconditioner (transposed prediction step): Gamma at the
         // checkpoint, inverse transposed diagonal blocks of dR_E/dW, 4-vectors and the inner basis
-        double *gx = nullptr, *gy = nullptr, *idiag = nullptr, *binv = nullptr;
+        double *gx = nullptr, *gy = nullptr, *binv = nullptr;
         double *m4 = nullptr, *w4 = nullptr, *t4 = nullptr, *Vi = nullptr;
         double* Zb = nullptr;                 // flexible-GMRES preconditioned basis
         int mz = 0;
@@ -343,7 +346,11 @@ miugks_status upload_level(miugks_solver* s, HLevel& Lv)
     ST(dalloc(s, &Lv.Wn, n4)); ST(dalloc(s, &Lv.Wc, n4)); ST(dalloc(s, &Lv.Rc, n4)); ST(dalloc(s, &Lv.P, n4));
     ST(dalloc(s, &Lv.R, n4)); ST(dalloc(s, &Lv.dW, n4)); ST(dalloc(s, &Lv.Wt, n4));
     ST(dalloc(s, &Lv.gx, (size_t)Lv.nfx)); ST(dalloc(s, &Lv.gy, (size_t)Lv.nfy));
-    ST(dalloc(s, &Lv.idiag, (size_t)Lv.nc)); ST(dalloc(s, &Lv.T, (macro_rec_bytes(Lv.nx, Lv.ny, s->mixed) + 7) / 8));
+    ST(dalloc(s, &Lv.idiag, (size_t)Lv.nc)); // records, ghosts and the state's other buffer (16-byte aligned parts of one block)
+    const size_t nrec = macro_rec_bytes(Lv.nx, Lv.ny, s->mixed) / 8, ngh = macro_ghost_elems((int)ubc.size());
+    ST(dalloc(s, &Lv.T, nrec + ngh + n4));
+    Lv.ghost = Lv.T + nrec;
+    Lv.Wd = Lv.ghost + ngh;
     ST(falloc(s, &Lv.r, nf)); ST(falloc(s, &Lv.df, nf)); ST(falloc(s, &Lv.dl, nf));
     ST(falloc(s, &Lv.invD, (size_t)Lv.nc * s->nv)); ST(dalloc(s, &Lv.inv_tau, (size_t)Lv.nc));
     return MIUGKS_OK;
@@ -522,17 +529,36 @@ double dtn_inv(miugks_solver* s)
 }
 
 // ---------------------------------------------------------------- cycles
-cudaError_t macro_sgs(miugks_solver* s, const MacroArgs& ma, HLevel& Lv)
+// One launch between two sweeps of level l: the state W with the pending update
+// becomes the level's Wc, and R (and the forcing P in mode 0) follow from Rin; rec:
+// a sweep follows.
+miugks_status macro_stage(miugks_solver* s, const MacroArgs& ma, HLevel& Lv, int mode, const double* W,
+                          const double* Rin, bool rec)
 {
-    if (s->mixed) return launch_macro_sgs<float>(ma, Lv.Wc, Lv.gx, Lv.gy, Lv.idiag, Lv.T, Lv.R, Lv.dW, s->st);
-    return launch_macro_sgs<double>(ma, Lv.Wc, Lv.gx, Lv.gy, Lv.idiag, Lv.T, Lv.R, Lv.dW, s->st);
+    const bool add = mode == 1 && Lv.pend;
+    double* Wo = mode == 0 ? Lv.Wc : add ? Lv.Wd : nullptr;
+    auto run = [&](auto z) {
+        using F = decltype(z);
+        return launch_macro_stage<F>(ma, MacroStage<F>{W, add ? (const F*)Lv.dW : nullptr, Wo, Lv.gx, Lv.gy, Rin,
+                                                       mode == 0 ? Lv.P : nullptr, Lv.R, Lv.idiag,
+                                                       rec ? (F*)Lv.T : nullptr, Lv.ghost, mode}, s->st);
+    };
+    CK(s->mixed ? run(0.0f) : run(0.0));
+    if (add) std::swap(Lv.Wc, Lv.Wd);
+    Lv.pend = false;
+    return MIUGKS_OK;
 }
 
-// one prediction sweep; on the finest level, bracketed by events in timing mode
-miugks_status timed_macro_sgs(miugks_solver* s, const MacroArgs& ma, HLevel& Lv, int l)
+// one prediction sweep (its update stays pending); on the finest level, bracketed by events in timing mode
+miugks_status macro_sgs(miugks_solver* s, const MacroArgs& ma, HLevel& Lv, int l)
 {
+    auto run = [&] {
+        return s->mixed ? launch_macro_sgs<float>(ma, (float*)Lv.T, Lv.ghost, (float*)Lv.dW, s->st)
+                        : launch_macro_sgs<double>(ma, Lv.T, Lv.ghost, Lv.dW, s->st);
+    };
+    Lv.pend = true;
     if (!s->timing || l != 0) {
-        CK(macro_sgs(s, ma, Lv));
+        CK(run());
         return MIUGKS_OK;
     }
     while ((int)s->ev_macro.size() < 2 * (s->n_macro_used + 1)) {
@@ -541,7 +567,7 @@ miugks_status timed_macro_sgs(miugks_solver* s, const MacroArgs& ma, HLevel& Lv,
         s->ev_macro.push_back(e);
     }
     CK(cudaEventRecord(s->ev_macro[2 * s->n_macro_used], s->st));
-    CK(macro_sgs(s, ma, Lv));
+    CK(run());
     CK(cudaEventRecord(s->ev_macro[2 * s->n_macro_used + 1], s->st));
     s->n_macro_used++;
     return MIUGKS_OK;
@@ -573,14 +599,13 @@ constexpr int kAdaptMaxVisits = 2;
 // and post-smooths.
 miugks_status fas_visit(miugks_solver* s, int l, double dti, int type, bool first);
 
-miugks_status fas(miugks_solver* s, int l, double dti, int type)
+// (Wn, Rc: the level's W^n and residual; level 0 takes the solver's own arrays)
+miugks_status fas(miugks_solver* s, int l, double dti, int type, const double* Wn, const double* Rc)
 {
     HLevel& Lv = s->lev[l];
     MacroArgs ma = macro_args(s, l, dti);
-    size_t n4 = 4 * (size_t)Lv.nc;
-    CK(launch_macro_gamma(ma, Lv.Wn, Lv.gx, Lv.gy, Lv.idiag, s->st));
-    CK(launch_macro_resid(ma, Lv.Wn, Lv.gx, Lv.gy, Lv.Rc, Lv.P, 0, s->st));     // forcing function
-    CK(cudaMemcpyAsync(Lv.Wc, Lv.Wn, n4 * sizeof(double), cudaMemcpyDeviceToDevice, s->st));
+    CK(launch_macro_gamma(ma, Wn, Lv.gx, Lv.gy, s->st));
+    ST(macro_stage(s, ma, Lv, 0, Wn, Rc, true));                              // forcing function
     return fas_visit(s, l, dti, type, true);
 }
 
@@ -588,21 +613,18 @@ miugks_status fas_visit(miugks_solver* s, int l, double dti, int type, bool firs
 {
     HLevel& Lv = s->lev[l];
     MacroArgs ma = macro_args(s, l, dti);
-    size_t n4 = 4 * (size_t)Lv.nc;
-    if (first) CK(cudaMemcpyAsync(Lv.R, Lv.Rc, n4 * sizeof(double), cudaMemcpyDeviceToDevice, s->st));
-    else CK(launch_macro_resid(ma, Lv.Wc, Lv.gx, Lv.gy, Lv.P, Lv.R, 1, s->st));   // P + R_E(W) of the state left
+    if (!first) ST(macro_stage(s, ma, Lv, 1, Lv.Wc, Lv.P, true));             // P + R_E(W) of the state left
     const bool coarsest = l == s->L - 1;
     const int npre = coarsest ? (s->L == 1 ? 1 : s->opts.nu_coarse) : s->opts.nu1;
     for (int m = 0; m < npre; ++m) {
-        ST(timed_macro_sgs(s, ma, Lv, l));
+        ST(macro_sgs(s, ma, Lv, l));
         if (coarsest && m == npre - 1) break;
-        CK(launch_macro_resid(ma, Lv.Wc, Lv.gx, Lv.gy, Lv.P, Lv.R, 1, s->st));  // renewal P + R_E(W)
+        ST(macro_stage(s, ma, Lv, 1, Lv.Wc, Lv.P, m < npre - 1));             // renewal P + R_E(W)
     }
     if (coarsest) return MIUGKS_OK;
     HLevel& Cv = s->lev[l + 1];
-    CK(launch_restrict<double>(Lv.dev, Cv.dev, 4, 1, Lv.Wc, Cv.Wn, s->st));
-    CK(launch_restrict<double>(Lv.dev, Cv.dev, 4, 1, Lv.R, Cv.Rc, s->st));
-    ST(fas(s, l + 1, dti, type));
+    CK(launch_restrict_state(Lv.dev, Cv.dev, Lv.Wc, Lv.R, Cv.Wn, Cv.Rc, s->st));
+    ST(fas(s, l + 1, dti, type, Cv.Wn, Cv.Rc));
     if (type == 1 || type == 2) ST(fas_visit(s, l + 1, dti, type == 1 ? 1 : 0, false));
     if (type == 3) {
         // adaptive: the coarse residual on entry is the restricted R; after a visit, P + R_E(W)
@@ -611,18 +633,20 @@ miugks_status fas_visit(miugks_solver* s, int l, double dti, int type, bool firs
         double before = 0.0, after = 0.0;
         ST(sumsq<double>(s, Cv.Rc, c4, &before));
         for (int visit = 1; visit < kAdaptMaxVisits; ++visit) {
-            CK(launch_macro_resid(mc, Cv.Wc, Cv.gx, Cv.gy, Cv.P, Cv.R, 1, s->st));
+            ST(macro_stage(s, mc, Cv, 1, Cv.Wc, Cv.P, false));
             ST(sumsq<double>(s, Cv.R, c4, &after));
             if (!adapt_again(s, before, after)) break;
             before = after;
             ST(fas_visit(s, l + 1, dti, 3, false));
         }
     }
-    CK(launch_sub(Cv.dW, Cv.Wc, Cv.Wn, 4 * (size_t)Cv.nc, s->st));
-    CK(launch_prolong_state(Lv.dev, Lv.pidx, Lv.pw, Cv.dW, Lv.Wc, s->st));
+    CK(s->mixed ? launch_prolong_state<float>(Lv.dev, Lv.pidx, Lv.pw, Cv.Wc, Cv.pend ? (const float*)Cv.dW : nullptr,
+                                              Cv.Wn, Lv.Wc, s->st)
+                : launch_prolong_state<double>(Lv.dev, Lv.pidx, Lv.pw, Cv.Wc, Cv.pend ? Cv.dW : nullptr, Cv.Wn, Lv.Wc,
+                                               s->st));
     for (int m = 0; m < s->opts.nu2; ++m) {
-        CK(launch_macro_resid(ma, Lv.Wc, Lv.gx, Lv.gy, Lv.P, Lv.R, 1, s->st));
-        ST(timed_macro_sgs(s, ma, Lv, l));
+        ST(macro_stage(s, ma, Lv, 1, Lv.Wc, Lv.P, true));
+        ST(macro_sgs(s, ma, Lv, l));
     }
     return MIUGKS_OK;
 }
@@ -712,11 +736,8 @@ miugks_status one_iteration_t(miugks_solver* s)
     ST(flux_stage(s));                                                       // Step 1
     if (s->timing) CK(cudaEventRecord(s->ev[1], s->st));
     CK(launch_rms(s->R, s->W, L0.nc, L0.nfluid, s->rms_part, s->rms_out, s->st));
-    size_t n4 = 4 * (size_t)L0.nc;
-    CK(cudaMemcpyAsync(L0.Wn, s->W, n4 * sizeof(double), cudaMemcpyDeviceToDevice, s->st));
-    CK(cudaMemcpyAsync(L0.Rc, s->R, n4 * sizeof(double), cudaMemcpyDeviceToDevice, s->st));
-    ST(fas(s, 0, dti, s->cycle));                                            // Step 2
-    CK(launch_predicted_state(L0.nc, L0.Wn, L0.Wc, L0.Wt, s->st));
+    ST(fas(s, 0, dti, s->cycle, s->W, s->R));                                // Step 2
+    CK(launch_predicted_state<F>(L0.nc, s->W, L0.Wc, L0.pend ? (const F*)L0.dW : nullptr, L0.Wt, s->st));
     MicroArgs m0 = micro_args(s, 0);                                         // Steps 3-4
     CK(launch_micro_residual<F>(m0, s->gas, L0.Wt, s->q, (const F*)s->f, (const F*)s->phx, (const F*)s->phy, dti,
                                 L0.inv_tau, (F*)L0.invD, (F*)L0.r, s->st));
@@ -1569,13 +1590,14 @@ miugks_status miugks_stage_sgs_macro(miugks_solver* s, int lev, const double* W,
     ST(check_level(s, lev));
     HLevel& Lv = s->lev[lev];
     size_t n4 = 4 * (size_t)Lv.nc;
-    CK(cudaMemcpyAsync(Lv.Wc, W, n4 * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemcpyAsync(Lv.Wd, W, n4 * sizeof(double), cudaMemcpyHostToDevice, s->st));
     CK(cudaMemcpyAsync(Lv.Wn, Wg, n4 * sizeof(double), cudaMemcpyHostToDevice, s->st));
     CK(cudaMemcpyAsync(Lv.R, R, n4 * sizeof(double), cudaMemcpyHostToDevice, s->st));
     MacroArgs ma = macro_args(s, lev, dtn_inv(s));   // the diagonal of the current iteration
-    CK(launch_macro_gamma(ma, Lv.Wn, Lv.gx, Lv.gy, Lv.idiag, s->st));
-    CK(macro_sgs(s, ma, Lv));
-    CK(cudaMemcpyAsync(dW, Lv.dW, n4 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
+    CK(launch_macro_gamma(ma, Lv.Wn, Lv.gx, Lv.gy, s->st));
+    ST(macro_stage(s, ma, Lv, 0, Lv.Wd, Lv.R, true));
+    ST(macro_sgs(s, ma, Lv, -1));
+    ST(to_host(s, dW, Lv.dW, n4));
     double flag = 0.0;
     CK(cudaMemcpyAsync(&flag, s->rms_out + 5, sizeof flag, cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
@@ -1592,8 +1614,9 @@ miugks_status miugks_stage_resid_macro(miugks_solver* s, int lev, const double* 
     CK(cudaMemcpyAsync(Lv.Wn, Wg, n4 * sizeof(double), cudaMemcpyHostToDevice, s->st));
     CK(cudaMemsetAsync(Lv.P, 0, n4 * sizeof(double), s->st));
     MacroArgs ma = macro_args(s, lev, 0.0);
-    CK(launch_macro_gamma(ma, Lv.Wn, Lv.gx, Lv.gy, Lv.idiag, s->st));
-    CK(launch_macro_resid(ma, Lv.Wc, Lv.gx, Lv.gy, Lv.P, Lv.R, 1, s->st));
+    CK(launch_macro_gamma(ma, Lv.Wn, Lv.gx, Lv.gy, s->st));
+    Lv.pend = false;
+    ST(macro_stage(s, ma, Lv, 1, Lv.Wc, Lv.P, false));
     CK(cudaMemcpyAsync(RE, Lv.R, n4 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
     return MIUGKS_OK;
@@ -1673,7 +1696,7 @@ miugks_status adj_prepare(miugks_solver* s, int m)
         ST(dalloc(s, &A.fpart, 4 * (size_t)(L0.nfx + L0.nfy)));
         ST(dalloc(s, &A.faces, (size_t)(L0.nfx + L0.nfy)));
         ST(dalloc(s, &A.gx, (size_t)L0.nfx)); ST(dalloc(s, &A.gy, (size_t)L0.nfy));
-        ST(dalloc(s, &A.idiag, (size_t)L0.nc)); ST(dalloc(s, &A.binv, 16 * (size_t)L0.nc));
+        ST(dalloc(s, &A.binv, 16 * (size_t)L0.nc));
         ST(dalloc(s, &A.m4, 4 * (size_t)L0.nc)); ST(dalloc(s, &A.w4, 8 * (size_t)L0.nc));
         ST(dalloc(s, &A.t4, 4 * (size_t)L0.nc));
         ST(dalloc(s, &A.Vi, (size_t)(kInnerRestart + 1) * 4 * L0.nc));
@@ -1689,7 +1712,7 @@ miugks_status adj_prepare(miugks_solver* s, int m)
     CK(launch_moments<double>(L0.dev, s->vel, A.f, A.W, A.q, s->st));
     CK(launch_inv_tau(s->gas, A.W, L0.nc, A.itau, s->st));
     MacroArgs ma = macro_args(s, 0, 0.0);
-    CK(launch_macro_gamma(ma, A.W, A.gx, A.gy, A.idiag, s->st));
+    CK(launch_macro_gamma(ma, A.W, A.gx, A.gy, s->st));
     CK(launch_macro_jacT(ma, A.W, A.gx, A.gy, nullptr, nullptr, A.binv, s->st));
     return adj_prepare_levels(s);
 }
@@ -2089,15 +2112,15 @@ miugks_status miugks_stage_macro_jacobian_transposed(miugks_solver* s, const dou
     if (L0.nfluid != L0.nc) return fail(s, MIUGKS_EINVAL, "adjoint: meshes with bodies (solid cells) are not supported");
     const size_t n4 = 4 * (size_t)L0.nc;
     // scratch for this test stage only, released before returning
-    const size_t tot = 3 * n4 + (size_t)L0.nfx + L0.nfy + L0.nc;
+    const size_t tot = 3 * n4 + (size_t)L0.nfx + L0.nfy;
     double* buf = nullptr;
     cudaError_t e = cudaMalloc(&buf, tot * sizeof(double));
     if (e != cudaSuccess) return fail(s, MIUGKS_ENOMEM, "cudaMalloc: %s", cudaGetErrorString(e));
-    double *dW = buf, *dx = dW + n4, *dy = dx + n4, *gx = dy + n4, *gy = gx + L0.nfx, *id = gy + L0.nfy;
+    double *dW = buf, *dx = dW + n4, *dy = dx + n4, *gx = dy + n4, *gy = gx + L0.nfx;
     MacroArgs ma = macro_args(s, 0, 0.0);
     e = cudaMemcpyAsync(dW, W, n4 * sizeof(double), cudaMemcpyHostToDevice, s->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dx, x, n4 * sizeof(double), cudaMemcpyHostToDevice, s->st);
-    if (e == cudaSuccess) e = launch_macro_gamma(ma, dW, gx, gy, id, s->st);
+    if (e == cudaSuccess) e = launch_macro_gamma(ma, dW, gx, gy, s->st);
     if (e == cudaSuccess) e = launch_macro_jacT(ma, dW, gx, gy, dx, dy, nullptr, s->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(y, dy, n4 * sizeof(double), cudaMemcpyDeviceToHost, s->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
