@@ -171,14 +171,12 @@ miugks_status miugks_set_cycle(miugks_solver *s, int type);
  * adaptive_decisions: the last min(n, cap, 4096) decisions, oldest first
  * (1 = a second visit), into out (may be NULL); returns n, the number taken. */
 miugks_status miugks_set_adaptive_ratio(miugks_solver *s, double ratio);
-/* Launch layout of the evolution smoother's sweeps (Eq. microFinalDefect); the
- * result is the same bit for bit.  In a sweep pass a velocity whose u (or v)
- * points away from the upwind neighbour in x (or y) has a zero coefficient
- * there: velocities coupled in both directions need the anti-diagonal
- * wavefront, the others are independent along rows, along columns or per
- * cell.  mode 1 sweeps those in a separate line-parallel kernel, 2 sweeps every
- * velocity in the wavefront kernel, 0 (default) splits a level from 20 Mi
- * cell-velocity pairs on.  MIUGKS_EINVAL for another mode. */
+/* Launch layout of the evolution smoother's sweeps (Eq. microFinalDefect):
+ * 1 asked for the velocities coupled along one axis only in a kernel of their
+ * own, 2 for every velocity in the wavefront kernel, 0 (default) for the choice
+ * by size.  The wavefront kernel now skips the couplings that a block of
+ * velocities does not have and serves every size, so the three modes are
+ * accepted and run the same launches.  MIUGKS_EINVAL for another mode. */
 miugks_status miugks_set_sweep_split(miugks_solver *s, int mode);
 /* Shock capturing (off by default; the paper describes none, and runs its
  * Ma 5 case without): on != 0 adds the pressure-jump term of the gas-kinetic
@@ -319,11 +317,11 @@ miugks_status miugks_kernel_times(miugks_solver *s, double *flux_ms, double *swe
  * pair of CUDA events: total milliseconds and launch count since the last
  * call (-1 and 0 when timing is off); the counters are reset. */
 miugks_status miugks_macro_sweep_times(miugks_solver *s, double *ms, int *launches);
-/* With timing on, every launch of the evolution smoother's sweep kernels on the
- * finest level (Eq. microFinalDefect; see miugks_set_sweep_split) is bracketed
- * by CUDA events.  out[0..2]: total milliseconds, launches and cell-velocity
- * pairs swept by the wavefront kernel; out[3..5]: the same for the line-class
- * kernel; since the last call (then reset).  -1 ms when timing is off. */
+/* With timing on, every launch of the evolution smoother's wavefront kernel on
+ * the finest level (Eq. microFinalDefect) is bracketed by CUDA events.
+ * out[0..2]: total milliseconds, launches and cell-velocity pairs swept, since
+ * the last call (then reset); out[3..5], once a second kernel's, stay zero.
+ * -1 ms when timing is off. */
 miugks_status miugks_sweep_kernel_times(miugks_solver *s, double out[6]);
 
 /* Residual norm of caller-owned device arrays without allocating anything.

@@ -1575,6 +1575,21 @@ cudaError_t launch_to_double(const F* a, double* b, size_t n, cudaStream_t st)
 template cudaError_t launch_to_double<float>(const float*, double*, size_t, cudaStream_t);
 template cudaError_t launch_to_double<double>(const double*, double*, size_t, cudaStream_t);
 
+template <typename F>
+__global__ void k_rows_to_double(const F* __restrict__ a, int ld, double* __restrict__ b, int nv)
+{
+    const size_t row = blockIdx.x;
+    for (int k = threadIdx.x; k < nv; k += blockDim.x) b[row * nv + k] = (double)a[row * ld + k];
+}
+template <typename F>
+cudaError_t launch_rows_to_double(const F* a, int ld, double* b, int nv, size_t rows, cudaStream_t st)
+{
+    k_rows_to_double<F><<<(unsigned)rows, 256, 0, st>>>(a, ld, b, nv);
+    return cudaGetLastError();
+}
+template cudaError_t launch_rows_to_double<float>(const float*, int, double*, int, size_t, cudaStream_t);
+template cudaError_t launch_rows_to_double<double>(const double*, int, double*, int, size_t, cudaStream_t);
+
 __global__ void k_to_float(const double* __restrict__ a, float* __restrict__ b, size_t n)
 {
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)

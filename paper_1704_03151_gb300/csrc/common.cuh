@@ -26,15 +26,12 @@ struct VelDev {
     const double *ua, *vb;       // per-axis nodes
     const float *uf, *vf, *wf;   // u, v, w rounded to FP32 (for the mixed-precision kernels)
     double umax, vmax;           // largest |u|, |v|
-    // Coupling classes of the evolution sweep, per pass (0 forward, 1 backward),
-    // from the signs of u and v: the blocks of four consecutive velocities that
-    // hold a velocity coupled to both its x and its y upwind neighbour (swept as
-    // a wavefront), and every other velocity, listed as those coupled along rows
-    // only, along columns only, and to no neighbour (in that order in lk)
-    const int* wblk[2];
-    int nwblk[2];
-    const int* lk[2];
-    int nrow[2], ncol[2], nelem[2];
+    int ld;                      // row stride of per-velocity arrays: nv rounded up to a multiple of 16 (the tables
+                                 // u, v, w, uf, vf, wf go on with zeros to ld)
+    // per pass (0 forward, 1 backward) and axis: the nodes of that axis that leave
+    // through a boundary face on the sweep side (u_n > 0): the first ones of the
+    // axis in pass 0, the last ones in pass 1
+    int nleave[2][2];
 };
 
 // one grid level (all device pointers)

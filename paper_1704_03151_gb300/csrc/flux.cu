@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
     const LevelDev& L = A.L;
     const VelDev& Vg = A.V;
     const int nv = Vg.nv, tid = threadIdx.x, bs = blockDim.x;
+    const size_t ld = Vg.ld;
     const int axis = A.axis, fi = blockIdx.x / ncl;
     const int chunk = (nv + ncl - 1) / ncl, kb = rank * chunk, ke = min(nv, kb + chunk);
     const int nx = L.nx, ny = L.ny;
@@ -183,9 +184,9 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
     const int j = axis == 0 ? fi / (nx + 1) : fi / nx;
     const int bcid = (axis == 0 ? L.fbx : L.fby)[fi];
     const F* __restrict__ fG = A.f;
-    const F* __restrict__ fH = A.f + nc * nv;
-    F* __restrict__ phG = A.ph + (size_t)fi * nv;
-    F* __restrict__ phH = A.ph + (nf + fi) * (size_t)nv;
+    const F* __restrict__ fH = A.f + nc * ld;
+    F* __restrict__ phG = A.ph + (size_t)fi * ld;
+    F* __restrict__ phH = A.ph + (nf + fi) * ld;
 
     if (bcid >= 0) {
         if (rank != 0) return;
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
             double s[2] = {0.0, 0.0};
             for (int k = tid; k < nv; k += bs) {
                 double uo = outsign * (axis == 0 ? Vg.u[k] : Vg.v[k]);
-                if (uo > 0) s[0] += Vg.w[k] * uo * (double)fG[c * (size_t)nv + k];
+                if (uo > 0) s[0] += Vg.w[k] * uo * (double)fG[c * ld + k];
                 else if (uo < 0) s[1] += Vg.w[k] * uo * Cb[k];
             }
             block_sum<2>(s, red);
@@ -212,11 +213,11 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
             double uo = outsign * un;
             double g, h;
             if (uo >= 0 || B.type == BC_OUTFLOW) {
-                g = fG[c * (size_t)nv + k]; h = fH[c * (size_t)nv + k];
+                g = fG[c * ld + k]; h = fH[c * ld + k];
             } else if (B.type == BC_SYMMETRY) {
                 int a = k / Vg.nvv, b = k - a * Vg.nvv;
                 int km = axis == 0 ? (Vg.nu - 1 - a) * Vg.nvv + b : a * Vg.nvv + (Vg.nvv - 1 - b);
-                g = fG[c * (size_t)nv + km]; h = fH[c * (size_t)nv + km];
+                g = fG[c * ld + km]; h = fH[c * ld + km];
             } else {   // wall (rho_w C) or farfield (rho_inf C)
                 g = rhow * Cb[k]; h = g * Hfac;
             }
@@ -270,10 +271,10 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
         #pragma unroll
         for (int cp = 0; cp < 2; ++cp) {
             const F* fc = cp == 0 ? fG : fH;
-            F fL = fc[cL * (size_t)nv + k], fR = fc[cR * (size_t)nv + k];
+            F fL = fc[cL * ld + k], fR = fc[cR * ld + k];
             F d2 = (fR - fL) * r2;
-            F sL = cLL >= 0 ? vl_limited((fL - fc[cLL * (size_t)nv + k]) * r1, d2) : F(0);
-            F sR = cRR >= 0 ? vl_limited(d2, (fc[cRR * (size_t)nv + k] - fR) * r3) : F(0);
+            F sL = cLL >= 0 ? vl_limited((fL - fc[cLL * ld + k]) * r1, d2) : F(0);
+            F sR = cRR >= 0 ? vl_limited(d2, (fc[cRR * ld + k] - fR) * r3) : F(0);
             F faceL = fL + sL * fhL, faceR = fR - sR * fhR;
             if (un > F(0)) { f0[cp] = faceL; sg[cp] = sL; }
             else if (un < F(0)) { f0[cp] = faceR; sg[cp] = sR; }

@@ -91,33 +91,51 @@ cudaError_t launch_sub(double* out, const double* a, const double* b, size_t n, 
 // the domain edge's column and row (a corner cell first), and the lines along
 // bodies.  Each such cell has a fold entry e (its ghost-folded inputs).
 struct SweepPlanDev {
-    const int* code[2];     // per cell: -1 ordinary, -2 in a body, else e << 2 | x-face line << 1 | y-face line
-    const int4* lcell[2];   // per fold entry: {cell, line axis (0 x-face, 1 y-face), wall-density slot, final}
-    const int* lines[2];    // lines along bodies: [q][8] = {i0, j0, di, dj, len, line axis, density slot, 0}
+    const int* code[2];     // per cell: -1 ordinary, -2 in a body, else its fold entry
+    const int4* lcell[2];   // per fold entry: {cell, line axis (0 x-face, 1 y-face), the face's bc id, corner}
+    const int* lines[2];    // lines: [q][8] = {i0, j0, di, dj, len, line axis, entry of cell 0, has symmetry faces};
+                            // 0 the edge column, 1 the edge row, then the lines along bodies
     int nl[2];              // fold entries of the edge lines (the rest belong to body lines)
-    int nl_max;             // fold-entry stride of the layout
+    int nl_max;             // fold entries (larger pass)
     int bodies;             // the level has solid cells
+    int sym[2];             // bit q: edge line q has symmetry faces
+    int cbc[2][2];          // boundary ids of the corner cell's x- and y-face
+    int general[2];         // a line has symmetry faces, or the corner a symmetry or outflow face
 };
 constexpr int kMaxBodyLines = 64;   // lines along bodies per pass and level
 struct MicroArgs {
     LevelDev L; VelDev V; const BcDev* bc; const double* Cw;
     const double* inv_tau;                 // [nc] collision frequency (+ 1/dt_n)
     SweepPlanDev P;
+    double* flag;                          // set to 1 when a bounded device wait gave up
+};
+// Scratch of the sweeps, kept per solver and sized for its largest level
+// (micro_scratch_elems); laid out by launch_micro_sgs.
+template <typename F>
+struct SweepScratch {
+    F* corner;   // [2][ld] corner cell of the pass
+    F* rho;      // [nl] wall densities of the line cells
+    F* part;     // [2 + body lines][chunks][kMaxLine] partial wall sums
+    F* fold;     // [velocity blocks][nl][3][block] inputs of the line cells
+    F* xline;    // [nl][2][ld] leaving values on lines with symmetry faces
+    int* count;  // [2 + body lines] CTAs done per line (zero between launches)
+    int nl;
 };
 // Host schedule of the body lines of one pass: after wave step dd - 1, the lines
 // q0 .. q0 + nq - 1 (fold entries e0 .. e0 + ne - 1) are walked and folded.
 struct SweepBreak { int dd, q0, nq, e0, ne; };
-// Timing mode: event pairs around the launches of the wavefront and line-class
-// sweep kernels, with the cell-velocity pairs each launch sweeps.
+// Timing mode: event pairs around the launches of the wavefront kernel, with the
+// cell-velocity pairs each launch sweeps.
 struct SweepTimer {
     std::vector<cudaEvent_t> ev;  // two per launch
-    std::vector<int> kind;        // 0 wavefront, 1 line class
     std::vector<double> units;
     int used = 0;
 };
-// split: 0 by the level's size, 1 always split the velocities by coupling class, 2 never;
-// timer: null unless the launches are to be timed
-struct SweepPlanHost { const SweepBreak* brk[2]; int nbrk[2]; int split; SweepTimer* timer; };
+// timer: null unless the launches are to be timed; nl, nlines, nchunk, count: the scratch's layout
+struct SweepPlanHost {
+    const SweepBreak* brk[2]; int nbrk[2]; SweepTimer* timer;
+    int nl, nlines, nchunk; int* count;
+};
 // Step 3-4: r = (g~ - f)/tau~ - div(ph) on level 0; also inv_tau (with dtn_inv) and invD
 template <typename F>
 cudaError_t launch_micro_residual(const MicroArgs& m, GasDev gas, const double* Wt, const double* q,
@@ -128,18 +146,16 @@ template <typename F>
 cudaError_t launch_coarse_coeffs(const MicroArgs& m, GasDev gas, const double* Wt, double dtn_inv,
                                  double* inv_tau, F* invD, cudaStream_t st);
 // one symmetric Gauss-Seidel pass: x = SGS(r).  Zw[b*4 + axis*2 + (outsign>0)] = sum over the
-// incoming velocities of w u_n C_k of wall BC b; xcorner: scratch of
-// micro_scratch_elems(nv, nl_max, body lines) values (the largest over the levels)
-size_t micro_scratch_elems(int nv, int nl, int nlines);
+// incoming velocities of w u_n C_k of wall BC b; scratch: micro_scratch_elems values
+// (nl, nlines: the largest over the levels)
+size_t micro_scratch_elems(int ld, int nl, int nlines, int nchunk, bool sym);
+int micro_edge_chunks(const VelDev& V);   // CTAs per line of the line walk
 // *out = sum of a[q]^2 over n values; part: scratch of 128 doubles
 template <typename T>
 cudaError_t launch_sumsq(const T* a, size_t n, double* part, double* out, cudaStream_t st);
-// coupling classes of the evolution sweep for one pass (VelDev::wblk, lk, nrow, ncol, nelem)
-void sweep_classes(const double* u, const double* v, int nv, int pass, std::vector<int>& wblk, std::vector<int>& lk,
-                   int& nrow, int& ncol, int& nelem);
 template <typename F>
 cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, const double* Zw, const F* invD,
-                             const F* r, F* x, F* xcorner, cudaStream_t st);
+                             const F* r, F* x, F* scratch, cudaStream_t st);
 // r -= A x (when renew) and acc += x (when acc != null)
 template <typename F>
 cudaError_t launch_micro_renew(const MicroArgs& m, const double* Zw, const F* x, F* r, F* acc, int renew,
@@ -218,6 +234,9 @@ cudaError_t launch_multi_axpy(const double* Vb, int m, size_t n, const double* h
                               cudaStream_t st);
 cudaError_t launch_mass_dot(const LevelDev& L, const VelDev& V, const double* x, double* part, cudaStream_t st);
 template <typename F> cudaError_t launch_to_double(const F* a, double* b, size_t n, cudaStream_t st);
+// rows of nv values at a stride of ld to packed rows
+template <typename F>
+cudaError_t launch_rows_to_double(const F* a, int ld, double* b, int nv, size_t rows, cudaStream_t st);
 cudaError_t launch_to_float(const double* a, float* b, size_t n, cudaStream_t st);
 // zero the entries of cells in bodies of a 2 x nc x nv vector
 cudaError_t launch_zero_solid(const LevelDev& L, int nv, double* x, cudaStream_t st);

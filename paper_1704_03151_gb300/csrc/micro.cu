@@ -16,28 +16,23 @@
 // cell, the velocities leaving through the boundary face (outgoing) need no
 // ghost, and the incoming ones need only the cell's wall density, a sum over
 // the outgoing ones.  Each sweep is therefore two launches:
-//   * k_sgs_chain: one thread-block cluster per boundary line solves the
-//     corner cell, then every outgoing velocity along the line, then the wall
-//     density of every line cell (partial sums combined through distributed
-//     shared memory with one hardware cluster barrier);
-//   * k_sgs_wave: every CTA owns a contiguous chunk of discrete velocities and
-//     sweeps all cells diagonal by diagonal, with only __syncthreads between
-//     diagonals (no grid-wide synchronisation); the incoming velocities of
-//     line cells are ordinary updates there, their ghost term being known.
+//   * k_sgs_edge walks the lines for their outgoing velocities and sums up the
+//     wall densities;
+//   * k_sgs_wave sweeps all cells, every CTA for its own velocities and with
+//     no synchronisation between CTAs; the incoming velocities of line cells
+//     are ordinary updates there, their ghost term being known.
+//
+// Rows of velocities are padded to a multiple of eight (VelDev::ld), so that
+// every cell's row starts on a 32-byte sector; the padding is zero and stays so.
 #include "kernels.cuh"
 #include "async.cuh"
 #include <algorithm>
-#include <climits>
+#include <array>
+#include <type_traits>
 
 namespace cg = cooperative_groups;
 
 namespace miugks {
-
-constexpr int kChainCluster = 8;
-constexpr int kChainThreads = 128;    // 4 warps: one per SM sub-partition
-constexpr int kChainKptMax = 16;      // local velocities per thread in the chain kernel (at most)
-constexpr int kInteriorKc = 4;        // velocities per CTA in the wavefront kernel
-constexpr size_t kSweepSplitMinCv = 20u << 20;   // cell-velocity pairs of a level from which the sweep is split
 
 // asynchronous 4- or 8-byte global -> shared copies (LDGSTS), completed per commit group
 template <typename F>
@@ -49,23 +44,6 @@ __device__ __forceinline__ void cp_async_elem(F* sdst, const F* gsrc)
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gsrc) : "memory");
 }
-// wait until at most n (0..7) of this thread's most recent groups are pending
-__device__ __forceinline__ void cp_async_wait(int n)
-{
-    switch (n) {
-    case 0: asm volatile("cp.async.wait_group 0;\n" ::: "memory"); break;
-    case 1: asm volatile("cp.async.wait_group 1;\n" ::: "memory"); break;
-    case 2: asm volatile("cp.async.wait_group 2;\n" ::: "memory"); break;
-    case 3: asm volatile("cp.async.wait_group 3;\n" ::: "memory"); break;
-    case 4: asm volatile("cp.async.wait_group 4;\n" ::: "memory"); break;
-    case 5: asm volatile("cp.async.wait_group 5;\n" ::: "memory"); break;
-    case 6: asm volatile("cp.async.wait_group 6;\n" ::: "memory"); break;
-    default: asm volatile("cp.async.wait_group 7;\n" ::: "memory"); break;
-    }
-}
-
-constexpr int kWaveRingMax = 8;       // cells or diagonals of inputs in flight in the sweep kernels (at most)
-
 // (1/V) sum over the faces with u_n > 0 of u_n S = |u|/dx + |v|/dy
 template <typename F>
 __device__ __forceinline__ F geomD(const LevelDev& L, int i, int j, F u, F v)
@@ -104,6 +82,7 @@ __global__ void __launch_bounds__(256) k_micro_residual(MicroArgs M, GasDev gas,
     const LevelDev& L = M.L;
     const VelDev& Vg = M.V;
     const int c = blockIdx.x, nv = Vg.nv, nx = L.nx;
+    const size_t ld = Vg.ld;
     const int i = c % nx, j = c / nx;
     const size_t nc = L.nc;
     // cell constants: FP64 state from thread 0, then one constant per lane of warp 0
@@ -171,12 +150,12 @@ __global__ void __launch_bounds__(256) k_micro_residual(MicroArgs M, GasDev gas,
         F gt[2] = {gM * (F(1) + Fq * (flam2 * c2 - F(4))), hM * (F(1) + Fq * (flam2 * c2 - F(2)))};
         #pragma unroll
         for (int cp = 0; cp < 2; ++cp) {
-            const F* px = phx + cp * nfx * nv;
-            const F* py = phy + cp * nfy * nv;
-            F div = (px[fE * nv + k] - px[fW * nv + k]) * rdxi + (py[fN * nv + k] - py[fS * nv + k]) * rdyj;
-            r[(cp * nc + c) * nv + k] = body ? F(0) : (gt[cp] - f[(cp * nc + c) * nv + k]) * fitau - div;
+            const F* px = phx + cp * nfx * ld;
+            const F* py = phy + cp * nfy * ld;
+            F div = (px[fE * ld + k] - px[fW * ld + k]) * rdxi + (py[fN * ld + k] - py[fS * ld + k]) * rdyj;
+            r[(cp * nc + c) * ld + k] = body ? F(0) : (gt[cp] - f[(cp * nc + c) * ld + k]) * fitau - div;
         }
-        invD[(size_t)c * nv + k] = recip(fdiag + geomD_r<F>(rdxi, rdyj, u, v));
+        invD[(size_t)c * ld + k] = recip(fdiag + geomD_r<F>(rdxi, rdyj, u, v));
     }
 }
 
@@ -219,7 +198,7 @@ __global__ void k_coarse_coeffs(MicroArgs M, GasDev gas, const double* __restric
     const F* __restrict__ vu = VelT<F>::u(M.V);
     const F* __restrict__ vv = VelT<F>::v(M.V);
     for (int k = threadIdx.x; k < M.V.nv; k += blockDim.x)
-        invD[(size_t)c * M.V.nv + k] = recip(fit + geomD_r<F>(rdxi, rdyj, vu[k], vv[k]));
+        invD[(size_t)c * M.V.ld + k] = recip(fit + geomD_r<F>(rdxi, rdyj, vu[k], vv[k]));
 }
 
 template <typename F>
@@ -252,528 +231,6 @@ __device__ __forceinline__ int side_faces(const LevelDev& L, int i, int j, int s
     return n;
 }
 
-// local velocity m of chain CTA `rank` -> global k (or -1); groups pair u-rows a and nu-1-a
-__device__ __forceinline__ int chain_k(const VelDev& Vg, int rank, int m, int* mirror_u_local, int* mirror_v_local)
-{
-    int nvv = Vg.nvv, nu = Vg.nu;
-    int s = m / (2 * nvv), rem = m - s * 2 * nvv, side = rem / nvv, b = rem - side * nvv;
-    int g = rank + s * kChainCluster;
-    int ngroups = (nu + 1) / 2;
-    if (g >= ngroups) return -1;
-    int a = side == 0 ? g : nu - 1 - g;
-    if (side == 1 && a == g) return -1;             // middle row of an odd grid
-    int sideu = (nu - 1 - g == g) ? 0 : 1 - side;   // local side holding the u-mirror
-    *mirror_u_local = s * 2 * nvv + sideu * nvv + b;
-    *mirror_v_local = s * 2 * nvv + side * nvv + (nvv - 1 - b);
-    return a * nvv + b;
-}
-
-// Cluster-wide deterministic sum of NR values with a fixed summation tree:
-// each warp reduces its lanes with xor shuffles, lane 0 publishes the warp's
-// partial in this CTA's shared slot, one cluster barrier, then every warp
-// loads the 32 partials of the cluster (8 CTAs x 4 warps, one per lane, read
-// through distributed shared memory) and reduces them with xor shuffles.
-// Every thread ends with the same sum.  Slots are double-buffered by event.
-template <typename T, int NR>
-__device__ __forceinline__ void cluster_sum(cg::cluster_group& cl, T (&v)[NR], T* slots, int& ev)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    #pragma unroll
-    for (int q = 0; q < NR; ++q)
-        #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    T* my = slots + (ev & 1) * (4 * 4);                // [warp][q]
-    if (lane == 0)
-        #pragma unroll
-        for (int q = 0; q < NR; ++q) my[warp * 4 + q] = v[q];
-    cl.sync();
-    const T* src = cl.map_shared_rank(my, lane >> 2);
-    #pragma unroll
-    for (int q = 0; q < NR; ++q) {
-        T x = src[(lane & 3) * 4 + q];
-        #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        v[q] = x;
-    }
-    ++ev;
-}
-
-
-// Cells 1.. of a boundary line, given the values of cell 0 in xprev: on the
-// domain edge, cell 0 is the corner; along a body, cell 0 is the fluid cell
-// before the line (a wavefront cell).  Cell st is (i0 + st di, j0 + st dj).  Every such cell has one boundary face on the sweep side, with a
-// fixed orientation along the line, so velocities split into
-//   outgoing (u_n >= 0 at that face): no ghost term, a recurrence along the
-//     line per velocity (phase A, inputs streamed RA cells ahead through a
-//     ring of asynchronous shared-memory copies);
-//   incoming (u_n < 0): the ghost term needs the cell's wall density, a sum
-//     over its outgoing velocities (phase A': per CTA, P threads per cell;
-//     phase B: over the cluster, one exchange; published in rho_out), or the
-//     mirrored outgoing value (symmetry).  With the ghost known, an incoming
-//     velocity of a line cell is an ordinary cell update, done by the
-//     wavefront kernel.
-// The arithmetic per cell is that of the serial sweep; only the order in which
-// independent velocities are visited changes.
-template <typename F, int kChainKpt>
-__device__ void chain_rest(cg::cluster_group& cl, const MicroArgs& M, const double* __restrict__ iZw,
-                           const F* __restrict__ invD, const F* __restrict__ r, F* __restrict__ x, int pass,
-                           int line, int i0, int j0, int di, int dj, int len, const int (&kk)[kChainKpt],
-                           F (&xprev)[kChainKpt][2],
-                           F* __restrict__ rho_out, F* ring, int RA, const int* lk, const F* lw, int nloc)
-{
-    __shared__ F part[kMaxLine];              // wall sum of this CTA's velocities per cell
-    __shared__ F rho_s[kMaxLine];
-    __shared__ F lm_nbS[kMaxLine], lm_itau[kMaxLine];
-    __shared__ F psum[kChainThreads];
-    const LevelDev& L = M.L;
-    const VelDev& Vg = M.V;
-    const int nx = L.nx, nv = Vg.nv;
-    const size_t nc = L.nc;
-    const int tid = threadIdx.x, B = blockDim.x;
-    const int nb_axis = line == 0 ? 1 : 0, nb_sign = pass == 0 ? -1 : 1;
-    // orientation of the line's boundary face (column lines: x-faces, row lines: y-faces)
-    const int f_axis = line == 0 ? 0 : 1, f_out = pass == 0 ? -1 : 1;
-    auto cell = [&](int st, int& i, int& j) { i = i0 + st * di; j = j0 + st * dj; };
-    auto face_bc = [&](int i, int j) {   // the line face of cell (i, j): west / south (forward), east / north
-        return f_axis == 0 ? L.fbx[j * (nx + 1) + i + (f_out > 0)] : L.fby[(j + (f_out > 0)) * nx + i];
-    };
-    for (int st = tid; st < len; st += B) {
-        int i, j;
-        cell(st, i, j);
-        lm_nbS[st] = (F)(nb_axis == 0 ? L.rdx[i] : L.rdy[j]);
-        lm_itau[st] = (F)M.inv_tau[j * nx + i];
-    }
-    // per velocity: Dn = an * nbS (the neighbour along the line) and
-    // D = itau + gfix + gvar * nbS (|u|/dx + |v|/dy with the line's fixed spacing in gfix)
-    int ifx, jfx;
-    cell(0, ifx, jfx);
-    F an[kChainKpt], gfix[kChainKpt], gvar[kChainKpt];
-    bool outg[kChainKpt];
-    #pragma unroll
-    for (int t = 0; t < kChainKpt; ++t) {
-        const int k = kk[t];
-        const F u = k < 0 ? F(0) : (F)Vg.u[k], v = k < 0 ? F(0) : (F)Vg.v[k];
-        const F uo = f_out < 0 ? -(f_axis == 0 ? u : v) : (f_axis == 0 ? u : v);
-        outg[t] = k >= 0 && uo >= F(0);
-        const F un = nb_sign < 0 ? -(nb_axis == 0 ? u : v) : (nb_axis == 0 ? u : v);
-        an[t] = un < F(0) ? un : F(0);
-        gfix[t] = line == 0 ? fabs(u) * (F)L.rdx[ifx] : fabs(v) * (F)L.rdy[jfx];
-        gvar[t] = line == 0 ? fabs(v) : fabs(u);
-    }
-    __syncthreads();
-    // ---- phase A: outgoing velocities
-    {
-        F xp[kChainKpt][2];
-        #pragma unroll
-        for (int t = 0; t < kChainKpt; ++t) { xp[t][0] = xprev[t][0]; xp[t][1] = xprev[t][1]; }
-        const F* src = pass == 0 ? r : x;
-        const size_t rstride = (size_t)kChainKpt * 3 * B;
-        auto issue = [&](int st) {
-            if (st < len) {
-                int i, j;
-                cell(st, i, j);
-                const size_t c = (size_t)j * nx + i;
-                F* rs = ring + (size_t)(st % RA) * rstride;
-                #pragma unroll
-                for (int t = 0; t < kChainKpt; ++t) {
-                    if (!outg[t]) continue;
-                    const int k = kk[t];
-                    cp_async_elem(rs + (t * 3 + 0) * B + tid, invD + c * nv + k);
-                    cp_async_elem(rs + (t * 3 + 1) * B + tid, src + c * nv + k);
-                    cp_async_elem(rs + (t * 3 + 2) * B + tid, src + (nc + c) * nv + k);
-                }
-            }
-            cp_async_commit();
-        };
-        for (int q = 1; q < RA; ++q) issue(q);
-        for (int st = 1; st < len; ++st) {
-            issue(st + RA - 1);
-            cp_async_wait(RA - 1);
-            const F* rs = ring + (size_t)(st % RA) * rstride;
-            int i, j;
-            cell(st, i, j);
-            const size_t c = (size_t)j * nx + i;
-            const F nbS = lm_nbS[st], itau = lm_itau[st];
-            #pragma unroll
-            for (int t = 0; t < kChainKpt; ++t) {
-                if (!outg[t]) continue;
-                const int k = kk[t];
-                const F Dn = an[t] * nbS, id = rs[(t * 3) * B + tid];
-                const F D = pass == 1 ? itau + (gfix[t] + gvar[t] * nbS) : F(0);
-                #pragma unroll
-                for (int cp = 0; cp < 2; ++cp) {
-                    const F in = rs[(t * 3 + 1 + cp) * B + tid];
-                    const F base = pass == 0 ? in - Dn * xp[t][cp] : D * in - Dn * xp[t][cp];
-                    const F xv = base * id;
-                    x[(cp * nc + c) * nv + k] = xv;
-                    xp[t][cp] = xv;
-                }
-            }
-        }
-        cp_async_wait(0);
-    }
-    __syncthreads();   // this CTA's outgoing values along the line are in x
-    // ---- phase A': wall sum over this CTA's outgoing velocities, P threads per cell
-    {
-        const int ncell = len - 1;
-        const int P = ncell >= B ? 1 : B / ncell, per = B / P;
-        for (int s0 = 0; s0 < ncell; s0 += per) {
-            const int st = 1 + s0 + tid / P, p = tid % P;
-            const bool mine = tid / P < per && st < len;
-            F sum = F(0);
-            if (mine) {
-                int i, j;
-                cell(st, i, j);
-                if (M.bc[face_bc(i, j)].type == BC_WALL) {
-                    // eight independent loads in flight (the values of incoming velocities are not
-                    // read: they belong to the previous sweep and may be anything)
-                    const F* xc0 = x + (size_t)(j * nx + i) * nv;
-                    F acc[8] = {F(0), F(0), F(0), F(0), F(0), F(0), F(0), F(0)};
-                    int q = p;
-                    for (; q + 7 * P < nloc; q += 8 * P) {
-                        F xv[8];
-                        #pragma unroll
-                        for (int u8 = 0; u8 < 8; ++u8) {
-                            const int qq = q + u8 * P;
-                            xv[u8] = lw[qq] != F(0) ? xc0[lk[qq]] : F(0);
-                        }
-                        #pragma unroll
-                        for (int u8 = 0; u8 < 8; ++u8) acc[u8] += lw[q + u8 * P] * xv[u8];
-                    }
-                    for (int u8 = 0; q < nloc; q += P, ++u8)
-                        if (lw[q] != F(0)) acc[u8] += lw[q] * xc0[lk[q]];
-                    sum = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
-                }
-            }
-            if (P == 1) {
-                if (mine) part[st] = sum;
-            } else {
-                psum[tid] = sum;
-                __syncthreads();
-                if (mine && p == 0) {
-                    F t = F(0);
-                    for (int q = 0; q < P; ++q) t += psum[tid + q];
-                    part[st] = t;
-                }
-                __syncthreads();
-            }
-        }
-    }
-    cl.sync();
-    // ---- phase B: wall density of every cell of the line (fixed summation order)
-    for (int st = 1 + tid; st < len; st += B) {
-        int i, j;
-        cell(st, i, j);
-        const int bc = face_bc(i, j);
-        F rho = F(0);
-        if (M.bc[bc].type == BC_WALL) {
-            F sum = F(0);
-            for (int rk = 0; rk < kChainCluster; ++rk) sum += cl.map_shared_rank(part, rk)[st];
-            rho = -sum * (F)iZw[bc * 4 + f_axis * 2 + (f_out > 0)];
-        }
-        rho_s[st] = rho;
-    }
-    __syncthreads();
-    // the incoming velocities of cells 1.. are finished by the wavefront kernel
-    if (cl.block_rank() == 0)
-        for (int st = tid; st < len; st += B) rho_out[st] = st == 0 ? F(0) : rho_s[st];
-}
-
-template <typename F, int kChainKpt>
-__global__ void __cluster_dims__(kChainCluster, 1, 1) __launch_bounds__(kChainThreads)
-k_sgs_chain(MicroArgs M, const double* __restrict__ Zw, const F* __restrict__ invD, const F* __restrict__ r,
-            F* __restrict__ x, const F* __restrict__ xcorner, F* __restrict__ rho_lines, int pass, int RA)
-{
-    const double* __restrict__ iZw = Zw + 4 * kMaxBcs;          // reciprocals of the wall normalisations
-    __shared__ F slots[2 * 4 * 4];
-    extern __shared__ double xsm_raw[];
-    F* xsm = reinterpret_cast<F*>(xsm_raw);  // [2][nloc] current cell values of this CTA's velocities
-    cg::cluster_group cl = cg::this_cluster();
-    const LevelDev& L = M.L;
-    const VelDev& Vg = M.V;
-    const int rank = cl.block_rank(), line = blockIdx.x / kChainCluster;
-    const int nx = L.nx, ny = L.ny, nv = Vg.nv;
-    const size_t nc = L.nc;
-    const int ngroups = (Vg.nu + 1) / 2;
-    const int nloc = ((ngroups + kChainCluster - 1) / kChainCluster) * 2 * Vg.nvv;
-    int ev = 0;
-    int kk[kChainKpt], mu[kChainKpt], mvv[kChainKpt];
-    #pragma unroll
-    for (int t = 0; t < kChainKpt; ++t) {
-        int m = threadIdx.x + t * blockDim.x;
-        kk[t] = m < nloc ? chain_k(Vg, rank, m, &mu[t], &mvv[t]) : -1;
-    }
-    F xprev[kChainKpt][2];
-    const int len = line == 0 ? ny : nx;
-    auto cell_of = [&](int st, int& ci, int& cj) {
-        if (pass == 0) { ci = line == 0 ? 0 : st; cj = line == 0 ? st : 0; }
-        else { ci = line == 0 ? nx - 1 : nx - 1 - st; cj = line == 0 ? ny - 1 - st : ny - 1; }
-    };
-    // per-velocity inputs of the current and the next cell (prefetched one step ahead)
-    F cin[kChainKpt][2], cdi[kChainKpt], nin[kChainKpt][2], ndi[kChainKpt];
-    double citau = 0.0, nitau = 0.0;
-    auto load = [&](int st, F (&in)[kChainKpt][2], F (&di)[kChainKpt], double& it) {
-        int ci, cj;
-        cell_of(st, ci, cj);
-        const int cc = cj * nx + ci;
-        it = M.inv_tau[cc];
-        #pragma unroll
-        for (int t = 0; t < kChainKpt; ++t) {
-            int k = kk[t];
-            if (k < 0) continue;
-            di[t] = invD[(size_t)cc * nv + k];
-            #pragma unroll
-            for (int cp = 0; cp < 2; ++cp) {
-                size_t id = (cp * nc + cc) * nv + k;
-                // backward: the corner's forward value comes from a copy taken before the
-                // launch, because the column line overwrites the corner while the row line reads it
-                in[t][cp] = pass == 0 ? r[id] : (st == 0 ? xcorner[cp * nv + k] : x[id]);
-            }
-        }
-    };
-    load(0, cin, cdi, citau);
-    for (int s = 0; s < 1; ++s) {   // the corner cell; the rest of the line follows in three phases
-        (void)nin; (void)ndi; (void)nitau;
-        // cell of this step
-        int i, j;
-        cell_of(s, i, j);
-        const int c = j * nx + i;
-        const F itau = (F)citau;
-        // interior neighbour along the line (the previous cell), if any
-        int nb_axis = line == 0 ? 1 : 0, nb_sign = pass == 0 ? -1 : 1;
-        const F nbS = (F)(nb_axis == 0 ? L.rdx[i] : L.rdy[j]);
-        BFace bf[2];
-        int nb = side_faces(L, i, j, pass, bf);
-        int nwall = 0, nsym = 0;
-        bool has_out = false;
-        for (int b = 0; b < nb; ++b) {
-            int t = M.bc[bf[b].bc].type;
-            nwall += t == BC_WALL;
-            nsym += t == BC_SYMMETRY;
-            has_out = has_out || t == BC_OUTFLOW;
-        }
-        F base[kChainKpt][2], den[kChainKpt], xc[kChainKpt][2];   // den holds 1/denominator
-        #pragma unroll
-        for (int t = 0; t < kChainKpt; ++t) {
-            int k = kk[t];
-            if (k < 0) continue;
-            const F u = (F)Vg.u[k], v = (F)Vg.v[k];
-            const F Dn = s > 0 ? Dface<F>(nb_axis, nb_sign, nbS, u, v) : F(0);
-            // 1/D from the precomputed table unless an outflow face adds to the diagonal
-            F D = F(0);
-            if (has_out || pass == 1) D = itau + geomD<F>(L, i, j, u, v);
-            if (has_out) {
-                F dd = D;
-                for (int b = 0; b < nb; ++b)
-                    if (M.bc[bf[b].bc].type == BC_OUTFLOW) dd += Dface<F>(bf[b].axis, bf[b].outsign, (F)bf[b].rS, u, v);
-                den[t] = recip(dd);
-            } else {
-                den[t] = cdi[t];
-            }
-            #pragma unroll
-            for (int cp = 0; cp < 2; ++cp) {
-                F y = s > 0 ? Dn * xprev[t][cp] : F(0);
-                base[t][cp] = pass == 0 ? cin[t][cp] - y : D * cin[t][cp] - y;
-                xc[t][cp] = base[t][cp] * den[t];
-            }
-        }
-        if (nwall == 2 && nb == 2) {
-            // two walls at a corner: 2x2 system for the two ghost densities
-            double z[2];
-            F acc[4] = {0, 0, 0, 0};
-            for (int b = 0; b < 2; ++b) z[b] = Zw[bf[b].bc * 4 + bf[b].axis * 2 + (bf[b].outsign > 0)];
-            #pragma unroll
-            for (int t = 0; t < kChainKpt; ++t) {
-                int k = kk[t];
-                if (k < 0) continue;
-                const F u = (F)Vg.u[k], v = (F)Vg.v[k], w = (F)Vg.w[k];
-                for (int b = 0; b < 2; ++b) {
-                    F uo = bf[b].axis == 0 ? u : v;
-                    uo = bf[b].outsign < 0 ? -uo : uo;
-                    if (!(uo > F(0))) continue;
-                    acc[b] += w * uo * base[t][0] * den[t];
-                    int o = 1 - b;
-                    F Do = Dface<F>(bf[o].axis, bf[o].outsign, (F)bf[o].rS, u, v);
-                    if (Do != F(0)) acc[2 + b] += w * uo * Do * (F)M.Cw[(size_t)bf[o].bc * nv + k] * den[t];
-                }
-            }
-            cluster_sum<F, 4>(cl, acc, slots, ev);
-            double cc0 = -acc[0] / z[0], cc1 = -acc[1] / z[1], mm0 = acc[2] / z[0], mm1 = acc[3] / z[1];
-            double rho2[2];
-            rho2[0] = (cc0 + mm0 * cc1) / (1.0 - mm0 * mm1);
-            rho2[1] = cc1 + mm1 * rho2[0];
-            const F rho[2] = {(F)rho2[0], (F)rho2[1]};
-            #pragma unroll
-            for (int t = 0; t < kChainKpt; ++t) {
-                int k = kk[t];
-                if (k < 0) continue;
-                const F u = (F)Vg.u[k], v = (F)Vg.v[k];
-                for (int cp = 0; cp < 2; ++cp) {
-                    F a = base[t][cp];
-                    for (int b = 0; b < 2; ++b) {
-                        F Db = Dface<F>(bf[b].axis, bf[b].outsign, (F)bf[b].rS, u, v);
-                        F C = (F)(M.Cw[(size_t)bf[b].bc * nv + k] * (cp == 0 ? 1.0 : kKint * M.bc[bf[b].bc].t / 4.0));
-                        if (Db != F(0)) a -= Db * C * rho[b];
-                    }
-                    xc[t][cp] = a * den[t];
-                }
-            }
-        } else if (nwall + nsym > 0) {
-            // substitution rounds (exact for every other combination; one round without symmetry)
-            int rounds = nsym > 0 ? 3 : 1;
-            for (int rd = 0; rd < rounds; ++rd) {
-                F rho = F(0);
-                int wb = -1;
-                for (int b = 0; b < nb; ++b) if (M.bc[bf[b].bc].type == BC_WALL) wb = b;
-                if (nsym > 0) {
-                    #pragma unroll
-                    for (int t = 0; t < kChainKpt; ++t) {
-                        int m = threadIdx.x + t * blockDim.x;
-                        if (kk[t] >= 0) { xsm[m] = xc[t][0]; xsm[nloc + m] = xc[t][1]; }
-                    }
-                    __syncthreads();
-                }
-                if (wb >= 0) {
-                    F acc[1] = {F(0)};
-                    #pragma unroll
-                    for (int t = 0; t < kChainKpt; ++t) {
-                        int k = kk[t];
-                        if (k < 0) continue;
-                        F uo = (F)(bf[wb].axis == 0 ? Vg.u[k] : Vg.v[k]);
-                        uo = bf[wb].outsign < 0 ? -uo : uo;
-                        if (uo > F(0)) acc[0] += (F)Vg.w[k] * uo * xc[t][0];
-                    }
-                    cluster_sum<F, 1>(cl, acc, slots, ev);
-                    rho = -acc[0] * (F)iZw[bf[wb].bc * 4 + bf[wb].axis * 2 + (bf[wb].outsign > 0)];
-                }
-                F xn[kChainKpt][2];
-                #pragma unroll
-                for (int t = 0; t < kChainKpt; ++t) {
-                    int k = kk[t];
-                    if (k < 0) continue;
-                    const F u = (F)Vg.u[k], v = (F)Vg.v[k];
-                    for (int cp = 0; cp < 2; ++cp) {
-                        F a = base[t][cp];
-                        for (int b = 0; b < nb; ++b) {
-                            F Db = Dface<F>(bf[b].axis, bf[b].outsign, (F)bf[b].rS, u, v);
-                            if (Db == F(0)) continue;
-                            int ty = M.bc[bf[b].bc].type;
-                            if (ty == BC_WALL)
-                                a -= Db * (F)(M.Cw[(size_t)bf[b].bc * nv + k] *
-                                              (cp == 0 ? 1.0 : kKint * M.bc[bf[b].bc].t / 4.0)) * rho;
-                            else if (ty == BC_SYMMETRY)
-                                a -= Db * xsm[cp * nloc + (bf[b].axis == 0 ? mu[t] : mvv[t])];
-                        }
-                        xn[t][cp] = a * den[t];
-                    }
-                }
-                if (nsym > 0) __syncthreads();
-                #pragma unroll
-                for (int t = 0; t < kChainKpt; ++t)
-                    if (kk[t] >= 0) { xc[t][0] = xn[t][0]; xc[t][1] = xn[t][1]; }
-            }
-        }
-        // store (the corner is written by the column line only) and carry along the line
-        const bool write = !(line == 1 && s == 0);
-        #pragma unroll
-        for (int t = 0; t < kChainKpt; ++t) {
-            int k = kk[t];
-            if (k < 0) continue;
-            xprev[t][0] = xc[t][0];
-            xprev[t][1] = xc[t][1];
-            if (write) {
-                x[c * (size_t)nv + k] = xc[t][0];
-                x[(nc + c) * (size_t)nv + k] = xc[t][1];
-            }
-        }
-    }
-    if (len > 1) {
-        // this CTA's velocities with their outgoing wall weights w u_n (0 when not outgoing)
-        F* lw = xsm + 2 * nloc;
-        F* ring = lw + nloc;
-        int* lk = reinterpret_cast<int*>(ring + (size_t)RA * kChainKpt * 3 * blockDim.x);
-        const int f_axis = line == 0 ? 0 : 1;
-        #pragma unroll
-        for (int t = 0; t < kChainKpt; ++t) {
-            const int m = threadIdx.x + t * blockDim.x;
-            if (m >= nloc) continue;
-            const int k = kk[t];
-            F wuo = F(0);
-            if (k >= 0) {
-                const F un = (F)(f_axis == 0 ? Vg.u[k] : Vg.v[k]), uo = pass == 0 ? -un : un;
-                wuo = uo > F(0) ? (F)Vg.w[k] * uo : F(0);
-            }
-            lk[m] = k;
-            lw[m] = wuo;
-        }
-        const int i0 = pass == 0 ? 0 : nx - 1, j0 = pass == 0 ? 0 : ny - 1, sg = pass == 0 ? 1 : -1;
-        chain_rest<F, kChainKpt>(cl, M, iZw, invD, r, x, pass, line, i0, j0, line == 0 ? 0 : sg, line == 0 ? sg : 0,
-                                 len, kk, xprev, rho_lines + line * kMaxLine, ring, RA, lk, lw, nloc);
-    }
-    cl.sync();   // keep every CTA's shared memory alive until all remote reads are done
-}
-
-
-// The lines along bodies of one sweep pass that start after the same
-// wavefront step, one cluster per line.  Cell 0 of a line is the fluid cell
-// before it, whose values (all velocities) the wavefront has already written
-// to x; chain_rest walks the line's outgoing velocities and publishes the
-// wall densities, and the wavefront then finishes its incoming velocities.
-template <typename F, int kChainKpt>
-__global__ void __cluster_dims__(kChainCluster, 1, 1) __launch_bounds__(kChainThreads)
-k_sgs_chain_body(MicroArgs M, const double* __restrict__ Zw, const F* __restrict__ invD, const F* __restrict__ r,
-                 F* __restrict__ x, F* __restrict__ rho_lines, int pass, int q0, int RA)
-{
-    const double* __restrict__ iZw = Zw + 4 * kMaxBcs;
-    extern __shared__ double xsm_raw[];
-    F* xsm = reinterpret_cast<F*>(xsm_raw);
-    cg::cluster_group cl = cg::this_cluster();
-    const VelDev& Vg = M.V;
-    const int rank = cl.block_rank(), nv = Vg.nv, nx = M.L.nx;
-    const size_t nc = M.L.nc;
-    const int* ld = M.P.lines[pass] + 8 * (q0 + blockIdx.x / kChainCluster);
-    const int i0 = ld[0], j0 = ld[1], di = ld[2], dj = ld[3], len = ld[4], line = ld[5], slot = ld[6];
-    const int ngroups = (Vg.nu + 1) / 2;
-    const int nloc = ((ngroups + kChainCluster - 1) / kChainCluster) * 2 * Vg.nvv;
-    int kk[kChainKpt], mu[kChainKpt], mvv[kChainKpt];
-    #pragma unroll
-    for (int t = 0; t < kChainKpt; ++t) {
-        int m = threadIdx.x + t * blockDim.x;
-        kk[t] = m < nloc ? chain_k(Vg, rank, m, &mu[t], &mvv[t]) : -1;
-    }
-    F xprev[kChainKpt][2];
-    const size_t c0 = (size_t)j0 * nx + i0;
-    #pragma unroll
-    for (int t = 0; t < kChainKpt; ++t) {
-        xprev[t][0] = xprev[t][1] = F(0);
-        if (kk[t] >= 0) {
-            xprev[t][0] = x[c0 * nv + kk[t]];
-            xprev[t][1] = x[(nc + c0) * nv + kk[t]];
-        }
-    }
-    F* lw = xsm + 2 * nloc;
-    F* ring = lw + nloc;
-    int* lk = reinterpret_cast<int*>(ring + (size_t)RA * kChainKpt * 3 * blockDim.x);
-    #pragma unroll
-    for (int t = 0; t < kChainKpt; ++t) {
-        const int m = threadIdx.x + t * blockDim.x;
-        if (m >= nloc) continue;
-        const int k = kk[t];
-        F wuo = F(0);
-        if (k >= 0) {
-            const F un = (F)(line == 0 ? Vg.u[k] : Vg.v[k]), uo = pass == 0 ? -un : un;
-            wuo = uo > F(0) ? (F)Vg.w[k] * uo : F(0);
-        }
-        lk[m] = k;
-        lw[m] = wuo;
-    }
-    __syncthreads();
-    chain_rest<F, kChainKpt>(cl, M, iZw, invD, r, x, pass, line, i0, j0, di, dj, len, kk, xprev, rho_lines + slot,
-                             ring, RA, lk, lw, nloc);
-    cl.sync();   // keep every CTA's shared memory alive until all remote reads are done
-}
-
-
 // four consecutive values through 16-byte accesses (16-byte aligned for float, 32 for double)
 __device__ __forceinline__ void ld4(const float* p, float (&v)[4])
 {
@@ -795,431 +252,825 @@ __device__ __forceinline__ void st4(double* p, const double (&v)[4])
     *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
 }
 
-// the kInteriorKc values of consecutive velocities at gsrc (nk of them exist) into sdst
-template <typename F, bool VEC>
-__device__ __forceinline__ void cp_async_k4(F* sdst, const F* gsrc, int nk)
+// ---------------------------------------------------------------------------
+// The evolution smoother's sweeps.
+__device__ __forceinline__ void cp_async16_if(bool on, void* sdst, const void* gsrc)   // zeros when off
 {
-    if constexpr (VEC) {
-        cp_async16(sdst, gsrc);
-        if constexpr (sizeof(F) == 8)
-            if (nk > 2) cp_async16(sdst + 2, gsrc + 2);
-    } else if (sizeof(F) == 4 && nk == kInteriorKc && (reinterpret_cast<uintptr_t>(gsrc) & 7) == 0) {
-        // FP32 with a velocity count that is not a multiple of four: the run of four
-        // values still starts on an 8- or 16-byte boundary for half of the cells
-        // (sdst is 16-byte aligned)
-        if ((reinterpret_cast<uintptr_t>(gsrc) & 15) == 0) {
-            cp_async16(sdst, gsrc);
-        } else {
-            const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gsrc) : "memory");
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa + 8), "l"(gsrc + 2) : "memory");
-        }
-    } else {
-        #pragma unroll
-        for (int q = 0; q < kInteriorKc; ++q)
-            if (q < nk) cp_async_elem(sdst + q, gsrc + q);
-    }
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_addr(sdst)), "l"(gsrc), "r"(on ? 16 : 0)
+                 : "memory");
 }
-
-// store a run of four FP32 values with the widest accesses its address allows
-__device__ __forceinline__ void st4_any(float* p, const float (&v)[4])
+__device__ __forceinline__ void ld16(const float* p, float* v)
 {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-    if ((a & 15) == 0) {
-        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    } else if ((a & 7) == 0) {
-        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
-        *reinterpret_cast<float2*>(p + 2) = make_float2(v[2], v[3]);
-    } else {
-        p[0] = v[0];
-        *reinterpret_cast<float2*>(p + 1) = make_float2(v[1], v[2]);
-        p[3] = v[3];
-    }
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
-
-// Inputs of the boundary-line cells for k_sgs_wave, after their line walk
-// (k_sgs_chain, k_sgs_chain_body): per fold entry e in [e0, e0 + ne) (a cell
-// of a line, from the plan's table) and velocity, the right-hand side b of G
-// and H and 1/D, laid out as the wavefront's ring entries,
-// fold[blk][e][3][kInteriorKc] (blk = k / kInteriorKc).  Outgoing velocities
-// and the corner carry their final value (applied as is).  Incoming ones carry
-// the ghost term folded in: forward b = r - g, backward b = (D x - g) / D, with
-// g = Db C rho_s (wall) or Db x_mirror (symmetry), and 1/(D + Db) in place of
-// 1/D at an outflow face.
-template <typename F>
-__global__ void k_line_fold(MicroArgs M, const F* __restrict__ invD, const F* __restrict__ r,
-                            const F* __restrict__ x, const F* __restrict__ rho_lines, F* __restrict__ fold, int pass,
-                            int e0, int ne)
+__device__ __forceinline__ void ld16(const double* p, double* v)
 {
-    constexpr int K = kInteriorKc;
+    const double2 t = *reinterpret_cast<const double2*>(p);
+    v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void st16(float* p, const float* v) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void st16(double* p, const double* v) { *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]); }
+
+// Walk of boundary lines.  On the sweep side of a pass, the cells of a line
+// each have one boundary face of the same orientation (the domain edge's column
+// and row, and runs along bodies).  A velocity that leaves through that face is
+// coupled only along the line, and the wall density of a cell is a sum over the
+// leaving velocities: one thread per line and leaving velocity walks the line
+// (inputs streamed RA cells ahead by asynchronous copies), and the contributions
+// of RA cells at a time are summed over the CTA's velocities through shared
+// memory; the last CTA of a line to finish adds the CTAs' sums in order and
+// publishes rho = -sum / Z per cell.  Nothing is written to x: the wavefront
+// recomputes the leaving velocities as ordinary cells and takes the densities.
+// Where a line has a symmetry face, the leaving values themselves are kept (the
+// mirrored ghosts are made of them).
+//
+// Edge lines start in the corner cell, whose two faces couple its velocities
+// (a 2x2 system for two walls, substitution otherwise): every CTA solves it for
+// itself from the cell's inputs (a few loads per thread), which costs less than
+// a cluster exchange.  Lines along bodies start from a cell that the wavefront
+// has finished.
+//
+// Bound by latency: the corner, then one load latency and a short recurrence per
+// RA cells.  64x64 cavity, 32x32 velocities, mixed: 14 us, against 34 us for the walk
+// by clusters of eight CTAs that this replaces (with its fold launch).
+template <typename F> struct EdgeRing { static constexpr int RA = 128 / (int)sizeof(F); };
+
+// GENERAL: symmetry faces on the lines, or a symmetry or outflow face at the corner
+// (without them the code is half as long, and a short kernel is mostly instruction fetches).
+template <typename F, bool GENERAL>
+__global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __restrict__ Zw, const F* __restrict__ invD,
+                                                  const F* __restrict__ r, const F* __restrict__ x, SweepScratch<F> S,
+                                                  int pass, int q0, int nchunk)
+{
+    constexpr int RA = EdgeRing<F>::RA, U = 8, NB = RA / U, B = 128, TP = B / RA, TS = B + 4;
+    extern __shared__ __align__(16) unsigned char esm[];
+    F* ring = reinterpret_cast<F*>(esm);              // [RA][3][B]
+    F* tile = ring + RA * 3 * B;                      // [RA][TS] contributions to the wall sums
+    __shared__ F nbS[kMaxLine], zf[kMaxLine];
+    __shared__ F red[4][4];
+    __shared__ int last;
     const LevelDev& L = M.L;
-    const VelDev& Vg = M.V;
-    const int nx = L.nx, nv = Vg.nv, nls = M.P.nl_max;
-    const size_t nc = L.nc;
-    const int nblk = (nv + K - 1) / K;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nblk * ne * K) return;
-    const int kk = t % K, e = e0 + (t / K) % ne, blk = t / (K * ne), kq = blk * K + kk;
-    const int4 lc = M.P.lcell[pass][e];                  // {cell, line axis, density slot, final}
-    const int c = lc.x, line = lc.y, i = c % nx, j = c / nx, fout = pass == 0 ? -1 : 1;
-    F b[2] = {F(0), F(0)}, iv = F(1);
-    if (kq < nv) {
-        const size_t id = (size_t)c * nv + kq;
-        const F u = (F)Vg.u[kq], v = (F)Vg.v[kq];
-        const F uo = fout < 0 ? -(line == 0 ? u : v) : (line == 0 ? u : v);   // u_n at the line face
-        if (lc.w || uo >= F(0)) {
-            b[0] = x[id];
-            b[1] = x[nc * nv + id];
-        } else {
-            const int bc = line == 0 ? L.fbx[j * (nx + 1) + i + (fout > 0)] : L.fby[(j + (fout > 0)) * nx + i];
-            const BcDev Bc = M.bc[bc];
-            const F Db = uo * (line == 0 ? (F)L.rdx[i] : (F)L.rdy[j]);
-            const F D = (F)M.inv_tau[c] + geomD<F>(L, i, j, u, v);
-            iv = Bc.type == BC_OUTFLOW ? recip(D + Db) : invD[id];
-            int km = 0;
-            if (Bc.type == BC_SYMMETRY) {
-                const int a2 = kq / Vg.nvv, b2 = kq - a2 * Vg.nvv;
-                km = line == 0 ? (Vg.nu - 1 - a2) * Vg.nvv + b2 : a2 * Vg.nvv + (Vg.nvv - 1 - b2);
-            }
-            #pragma unroll
-            for (int cp = 0; cp < 2; ++cp) {
-                F g = F(0);
-                if (Bc.type == BC_WALL)
-                    g = Db * ((F)(M.Cw[(size_t)bc * nv + kq] * (cp == 0 ? 1.0 : kKint * Bc.t / 4.0)) * rho_lines[lc.z]);
-                else if (Bc.type == BC_SYMMETRY)
-                    g = Db * x[cp * nc * nv + (size_t)c * nv + km];   // an outgoing velocity: final
-                b[cp] = pass == 0 ? r[cp * nc * nv + id] - g : (D * x[cp * nc * nv + id] - g) * iv;
-            }
-        }
+    const VelDev& V = M.V;
+    const int nx = L.nx, ny = L.ny, nv = V.nv, tid = threadIdx.x;
+    const size_t nc = L.nc, ld = V.ld;
+    const F* __restrict__ vu = VelT<F>::u(V);
+    const F* __restrict__ vv = VelT<F>::v(V);
+    const F* __restrict__ vw = VelT<F>::w(V);
+    const double* __restrict__ iZw = Zw + 4 * kMaxBcs;
+    const int q = q0 + (int)blockIdx.x / nchunk, chunk = (int)blockIdx.x % nchunk;
+    // the line; the edge's two follow from the mesh (a load less before the first inputs can be asked for)
+    const bool edge = q < 2;
+    int i0 = pass == 0 ? 0 : nx - 1, j0 = pass == 0 ? 0 : ny - 1, di = q == 1 ? (pass == 0 ? 1 : -1) : 0,
+        dj = q == 0 ? (pass == 0 ? 1 : -1) : 0, len = q == 0 ? ny : nx, axis = q, ebase = q == 0 ? 0 : ny;
+    bool sym = GENERAL && edge && (M.P.sym[pass] >> (q & 1) & 1);
+    if (!edge) {
+        const int* ln = M.P.lines[pass] + 8 * q;
+        i0 = ln[0]; j0 = ln[1]; di = ln[2]; dj = ln[3]; len = ln[4]; axis = ln[5]; ebase = ln[6];
+        sym = GENERAL && ln[7] != 0;
     }
-    F* o = fold + ((size_t)(blk * nls + e) * 3) * K + kk;
-    o[0] = b[0];
-    o[K] = b[1];
-    o[2 * K] = iv;
-}
-
-// Wavefront steps [dd0, dd1) of one sweep over every cell for the
-// kInteriorKc velocities of this CTA, in anti-diagonal order, one thread per
-// cell of the diagonal handling the 2 x kInteriorKc values (G and H,
-// consecutive velocities) of its cell.  Ordinary update: (forward)
-// x = (b - D_W x_W - D_S x_S) / D with b the residual, (backward)
-// x = b - (D_E x_E + D_N x_N) / D with b the forward value.  Boundary-line
-// cells take b and 1/D from k_line_fold and drop the neighbour across their
-// line face; cells in a body are zero.  Values of the previous diagonal stay
-// in shared memory (a segment after the first reloads them from x); the inputs
-// of the next R - 1 diagonals are in flight as asynchronous copies into a ring
-// of R shared buffers, so the per-diagonal path only touches shared memory.
-// BODIES: cell codes from the plan's table (a mesh with bodies); without
-// bodies the code of a cell follows from its position (the edge column and row).
-template <typename F, int R, bool VEC, bool BODIES>
-__global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restrict__ invD, const F* __restrict__ r,
-                                                  F* __restrict__ x, const F* __restrict__ fold, int pass, int dd0,
-                                                  int dd1, int listed)
-{
-    // this CTA's block of velocities: every block, or the listed wavefront-class blocks
-    const int blk = listed ? M.V.wblk[pass][blockIdx.x] : blockIdx.x;
-    extern __shared__ __align__(16) double sraw[];
-    constexpr int K = kInteriorKc, W = 2 * K;
-    const LevelDev& L = M.L;
-    const VelDev& Vg = M.V;
-    const int nx = L.nx, ny = L.ny, nv = Vg.nv;
-    const size_t nc = L.nc;
-    const int B = blockDim.x, tid = threadIdx.x;
-    const int k0 = blk * K, nk = min(K, nv - k0);
-    const int nd = nx + ny - 1, nls = M.P.nl_max;
-    const int* __restrict__ code = M.P.code[pass];
-    F* sx = reinterpret_cast<F*>(sraw);                 // [2][nx][W] values of the previous diagonal
-    F* ring = sx + 2 * (size_t)nx * W;                  // [R][3][B][K] b (G, H) and 1/D of upcoming diagonals
-    F* srdx = ring + (size_t)R * 3 * B * K;             // [nx] 1/dx
-    F* srdy = srdx + nx;                                // [ny] 1/dy
-    int* cring = reinterpret_cast<int*>(srdy + ny);     // [R][B] cell codes of the upcoming diagonals
+    const long c0 = (long)j0 * nx + i0, cstep = (long)dj * nx + di;
     const F* src = pass == 0 ? r : x;
-    const int ib = pass == 0 ? 0 : nx - 1, jb = pass == 0 ? 0 : ny - 1;   // the edge column and row of the pass
-    // code of this thread's cell on wavefront step dd (with bodies; loaded one step before it is needed)
-    auto code_of = [&](int dd) {
-        if (!BODIES || dd >= dd1) return -3;
-        const int d = pass == 0 ? dd : nd - 1 - dd;
-        const int ilo = max(0, d - (ny - 1)), ncell = min(nx - 1, d) - ilo + 1;
-        return tid < ncell ? code[(d - ilo - tid) * nx + ilo + tid] : -3;
-    };
-    auto issue = [&](int dd, int cd) {
-        if (dd < dd1) {
-            const int d = pass == 0 ? dd : nd - 1 - dd;
-            const int ilo = max(0, d - (ny - 1)), ncell = min(nx - 1, d) - ilo + 1;
-            if (tid < ncell) {
-                const int i = ilo + tid, j = d - i;
-                F* ra = ring + ((size_t)(dd % R) * 3 * B + tid) * K;
-                if constexpr (BODIES) {
-                    cring[(dd % R) * B + tid] = cd;     // read back by this thread when swept
-                } else {                                // without bodies the position gives the code
-                    cd = i != ib && j != jb ? -1 : ((i == ib ? (pass == 0 ? j : ny - 1 - j)
-                                                             : ny + (pass == 0 ? i : nx - 1 - i)) << 2);
-                }
-                if (cd == -1) {
-                    const size_t e = ((size_t)j * nx + i) * nv + k0;
-                    cp_async_k4<F, VEC>(ra, src + e, nk);
-                    cp_async_k4<F, VEC>(ra + (size_t)B * K, src + nc * nv + e, nk);
-                    cp_async_k4<F, VEC>(ra + (size_t)2 * B * K, invD + e, nk);
-                } else if (cd >= 0) {                   // a boundary-line cell: its folded inputs
-                    const F* fo = fold + ((size_t)(blk * nls + (cd >> 2)) * 3) * K;
-                    cp_async_k4<F, true>(ra, fo, K);
-                    cp_async_k4<F, true>(ra + (size_t)B * K, fo + K, K);
-                    cp_async_k4<F, true>(ra + (size_t)2 * B * K, fo + 2 * K, K);
-                }
+    // the velocities that leave: nodes ascend, so the first (pass 0) or last ones of that axis
+    const int v = chunk * B + tid, nl1 = V.nleave[pass][axis], other = axis == 0 ? V.nvv : V.nu;
+    const bool on = v < nl1 * other;
+    int k = 0;
+    if (on) {
+        if (axis == 0) k = (pass == 0 ? 0 : (V.nu - nl1) * V.nvv) + v;
+        else { const int a = v / nl1; k = a * V.nvv + (pass == 0 ? 0 : V.nvv - nl1) + v - a * nl1; }
+    }
+    const long pst = cstep * (long)ld;
+    const F *pi = invD + (c0 + cstep) * (long)ld + k, *ps = src + (c0 + cstep) * (long)ld + k;
+    auto issue = [&](int b) {                         // cells 1 + U b .. U (b + 1), one copy group
+        F* d = ring + (b % NB) * U * 3 * B + tid;
+        #pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (1 + U * b + u < len && on) {
+                cp_async_elem(d + u * 3 * B, pi);
+                cp_async_elem(d + u * 3 * B + B, ps);
+                if (sym) cp_async_elem(d + u * 3 * B + 2 * B, ps + nc * ld);
             }
+            pi += pst;
+            ps += pst;
         }
         cp_async_commit();
     };
-    if constexpr (R > 1)
-        for (int dd = dd0; dd < dd0 + R - 1; ++dd) issue(dd, code_of(dd));
-    // cell codes of the next four issues, loaded four sweep steps before they are used
-    // (one step is shorter than a global load)
-    int cd_next = code_of(dd0 + R - 1), cd_n1 = code_of(dd0 + R), cd_n2 = code_of(dd0 + R + 1),
-        cd_n3 = code_of(dd0 + R + 2);
-    // prologue: diagonal buffers (the previous segment's last diagonal from x) and spacings
-    for (int q = tid; q < 2 * nx * W; q += B) sx[q] = F(0);
-    __syncthreads();
-    if (dd0 > 0) {
-        const int d = pass == 0 ? dd0 - 1 : nd - dd0;
-        const int ilo = max(0, d - (ny - 1)), ncell = min(nx - 1, d) - ilo + 1;
-        F* prev = sx + (size_t)((dd0 + 1) & 1) * nx * W;
-        for (int q = tid; q < ncell * W; q += B) {
-            const int i = ilo + q / W, w = q % W, cp = w / K, kk = w % K;
-            if (kk < nk) prev[(size_t)i * W + w] = x[(cp * nc + (size_t)(d - i) * nx + i) * nv + k0 + kk];
-        }
-    }
-    for (int q = tid; q < nx; q += B) srdx[q] = (F)L.rdx[q];
-    for (int q = tid; q < ny; q += B) srdy[q] = (F)L.rdy[q];
-    // per velocity: neighbour coefficients (zero where the upwind neighbour is on the other side)
-    // and which velocities leave through a column / row line face
-    F cu[K], cv[K];
-    unsigned outc = 0, outr = 0;
+    for (int b = 0; b < NB - 1; ++b) issue(b);
+    // what the end of the walk needs per cell, asked for early: 1/d along the line and the boundary id
+    int zb[kMaxLine / B];
     #pragma unroll
-    for (int kk = 0; kk < K; ++kk) {
-        const int kq = k0 + kk;
-        const F u = kq < nv ? (F)Vg.u[kq] : F(0), v = kq < nv ? (F)Vg.v[kq] : F(0);
-        cu[kk] = pass == 0 ? (u > F(0) ? -u : F(0)) : (u < F(0) ? u : F(0));
-        cv[kk] = pass == 0 ? (v > F(0) ? -v : F(0)) : (v < F(0) ? v : F(0));
-        if ((pass == 0 ? -u : u) >= F(0)) outc |= 1u << kk;
-        if ((pass == 0 ? -v : v) >= F(0)) outr |= 1u << kk;
+    for (int t = 0; t < kMaxLine / B; ++t) {
+        const int st = tid + t * B;
+        zb[t] = -1;
+        if (st < len && (st > 0 || edge)) zb[t] = M.P.lcell[pass][ebase + st].z;
+        if (st < len) nbS[st] = (F)(axis == 0 ? L.rdy[j0 + st * dj] : L.rdx[i0 + st * di]);
     }
-    const int xo = pass == 0 ? -1 : 1;                  // x neighbour: i - 1 (forward) or i + 1
-    __syncthreads();
-    for (int dd = dd0; dd < dd1; ++dd) {
-        if constexpr (R == 1) {
-            issue(dd, cd_next);
-            cd_next = code_of(dd + 1);
-            cp_async_wait_n<0>();
-        } else {
-            cp_async_wait_n<R - 2>();
-        }
-        const int d = pass == 0 ? dd : nd - 1 - dd;
-        const int ilo = max(0, d - (ny - 1)), ncell = min(nx - 1, d) - ilo + 1;
-        const F* prev = sx + (size_t)((dd + 1) & 1) * nx * W;
-        F* cur = sx + (size_t)(dd & 1) * nx * W;
-        if (tid < ncell) {
-            const int i = ilo + tid, j = d - i;
-            int cd = -1;
-            if constexpr (BODIES) cd = cring[(dd % R) * B + tid];
-            const F* ra = ring + ((size_t)(dd % R) * 3 * B + tid) * K;
-            static_assert(K == 4, "vector accesses assume four velocities per CTA");
-            F res[2][K];
-            if (BODIES && cd == -2) {                   // in a body
+    F xp[2] = {F(0), F(0)};
+    if (edge) {
+        // the corner cell: face 0 its x-face, face 1 its y-face
+        const int c = pass == 0 ? 0 : (int)nc - 1, ci = pass == 0 ? 0 : nx - 1, cj = pass == 0 ? 0 : ny - 1;
+        const int bc0 = M.P.cbc[pass][0], bc1 = M.P.cbc[pass][1];
+        const BcDev B0 = M.bc[bc0], B1 = M.bc[bc1];
+        const double* __restrict__ C0 = M.Cw + (size_t)bc0 * nv;
+        const double* __restrict__ C1 = M.Cw + (size_t)bc1 * nv;
+        const double z0 = iZw[bc0 * 4 + pass], z1 = iZw[bc1 * 4 + 2 + pass];
+        const F rx = (F)L.rdx[ci], ry = (F)L.rdy[cj], itau = (F)M.inv_tau[c];
+        const F h0 = (F)(kKint * B0.t / 4.0), h1 = (F)(kKint * B1.t / 4.0);
+        const bool w0 = B0.type == BC_WALL, w1 = B1.type == BC_WALL;
+        const bool y0 = GENERAL && B0.type == BC_SYMMETRY, y1 = GENERAL && B1.type == BC_SYMMETRY;
+        const bool o0 = GENERAL && B0.type == BC_OUTFLOW, o1 = GENERAL && B1.type == BC_OUTFLOW;
+        const F sg = pass == 0 ? F(-1) : F(1);
+        // a velocity of the corner: outward normal speeds, 1/D, values without ghosts, the walls' Maxwellians
+        struct Vel { F ux, uy, w, den, x[2], c0, c1; };
+        auto fetch = [&](int kk, Vel& q) {           // independent loads, used once all are asked for
+            q.ux = vu[kk];
+            q.uy = vv[kk];
+            q.w = vw[kk];
+            q.den = invD[(size_t)c * ld + kk];
+            q.x[0] = src[(size_t)c * ld + kk];
+            q.x[1] = src[(nc + c) * ld + kk];
+            q.c0 = w0 ? (F)C0[kk] : F(0);
+            q.c1 = w1 ? (F)C1[kk] : F(0);
+        };
+        auto finish = [&](Vel& q) {
+            q.ux *= sg;
+            q.uy *= sg;
+            if (o0 || o1) {
+                const F D = itau + fabs(q.ux) * rx + fabs(q.uy) * ry;
+                q.den = recip(D + (o0 ? min(q.ux, F(0)) * rx : F(0)) + (o1 ? min(q.uy, F(0)) * ry : F(0)));
+                if (pass == 1) { q.x[0] *= D; q.x[1] *= D; }
+            }
+            if (pass == 0 || o0 || o1) { q.x[0] *= q.den; q.x[1] *= q.den; }
+        };
+        auto mirrored = [&](int f, int kk, Vel& q) { // the velocity mirrored at face f, ready
+            const int a = kk / V.nvv, b = kk - a * V.nvv;
+            fetch(f == 0 ? (V.nu - 1 - a) * V.nvv + b : a * V.nvv + (V.nvv - 1 - b), q);
+            finish(q);
+        };
+        F rho0 = F(0), rho1 = F(0);
+        const bool two = w0 && w1;
+        if (w0 || w1) {
+            F acc[4] = {F(0), F(0), F(0), F(0)};
+            #pragma unroll 1
+            for (int kb = tid; kb < nv; kb += 4 * B) {
+                Vel q[4];
                 #pragma unroll
-                for (int kk = 0; kk < K; ++kk) res[0][kk] = res[1][kk] = F(0);
-            } else {
-                F a[2][K], iv[K], pwv[2][K], psv[2][K];
-                ld4(ra, a[0]);
-                ld4(ra + (size_t)B * K, a[1]);
-                ld4(ra + (size_t)2 * B * K, iv);
-                bool hx = i != ib, hy = j != jb;
-                if constexpr (BODIES) { hx = !(cd >= 0 && (cd & 2)); hy = !(cd >= 0 && (cd & 1)); }
-                const F fx = hx ? srdx[i] : F(0), fy = hy ? srdy[j] : F(0);
-                const F* pw = prev + (size_t)(hx ? i + xo : i) * W;
-                const F* ps = prev + (size_t)i * W;
-                ld4(pw, pwv[0]);
-                ld4(pw + K, pwv[1]);
-                ld4(ps, psv[0]);
-                ld4(ps + K, psv[1]);
-                // boundary-line cell: the final values (corner, outgoing velocities) are applied as is
-                const unsigned ld = hx && hy ? 0u : (!hx && !hy ? 0xFu : (!hx ? outc : outr));
+                for (int t = 0; t < 4; ++t) fetch(min(kb + t * B, nv - 1), q[t]);
                 #pragma unroll
-                for (int cp = 0; cp < 2; ++cp)
-                    #pragma unroll
-                    for (int kk = 0; kk < K; ++kk) {
-                        const F y = cu[kk] * fx * pwv[cp][kk] + cv[kk] * fy * psv[cp][kk];
-                        const F rv = pass == 0 ? (a[cp][kk] - y) * iv[kk] : a[cp][kk] - y * iv[kk];
-                        res[cp][kk] = (ld >> kk) & 1u ? a[cp][kk] : rv;
+                for (int t = 0; t < 4; ++t) {
+                    finish(q[t]);
+                    F val = q[t].x[0];
+                    if (!two && ((y0 && q[t].ux < F(0)) || (y1 && q[t].uy < F(0)))) {
+                        // beside a symmetry face: the mirrored ghost of a velocity that enters through it
+                        Vel m;
+                        mirrored(y0 ? 0 : 1, min(kb + t * B, nv - 1), m);
+                        val -= (y0 ? q[t].ux * rx : q[t].uy * ry) * q[t].den * m.x[0];
                     }
+                    const F wt = kb + t * B < nv ? q[t].w : F(0);
+                    const F ax = w0 ? wt * max(q[t].ux, F(0)) : F(0), ay = w1 ? wt * max(q[t].uy, F(0)) : F(0);
+                    acc[0] += ax * val;
+                    acc[1] += ay * val;
+                    if (two) {
+                        acc[2] += ax * (min(q[t].uy, F(0)) * ry) * q[t].c1 * q[t].den;
+                        acc[3] += ay * (min(q[t].ux, F(0)) * rx) * q[t].c0 * q[t].den;
+                    }
+                }
             }
             #pragma unroll
-            for (int cp = 0; cp < 2; ++cp) {
-                F* xd = x + (cp * nc + (size_t)j * nx + i) * nv + k0;
-                st4(cur + (size_t)i * W + cp * K, res[cp]);
-                if constexpr (VEC) {
-                    if (nk == K) {
-                        st4(xd, res[cp]);
-                    } else {                            // double, nv = 2 mod 4: the last two values do not exist
-                        xd[0] = res[cp][0];
-                        xd[1] = res[cp][1];
-                    }
-                } else if constexpr (sizeof(F) == 4) {
-                    if (nk == K) {
-                        st4_any(xd, res[cp]);
-                    } else {
-                        #pragma unroll
-                        for (int kk = 0; kk < K; ++kk)
-                            if (kk < nk) xd[kk] = res[cp][kk];
-                    }
-                } else {
-                    #pragma unroll
-                    for (int kk = 0; kk < K; ++kk)
-                        if (kk < nk) xd[kk] = res[cp][kk];
+            for (int m = 0; m < 4; ++m) {
+                #pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
+                if ((tid & 31) == 0) red[tid >> 5][m] = acc[m];
+            }
+            __syncthreads();
+            if (tid == 0) {
+                double t[4];
+                for (int m = 0; m < 4; ++m) t[m] = ((double)red[0][m] + red[1][m]) + ((double)red[2][m] + red[3][m]);
+                // rho_0 = k_0 + m_0 rho_1, rho_1 = k_1 + m_1 rho_0
+                const double k0 = -t[0] * z0, k1 = -t[1] * z1, m0 = t[2] * z0, m1 = t[3] * z1;
+                const double r0 = two ? (k0 + m0 * k1) * rcp64(1.0 - m0 * m1) : k0;
+                red[0][0] = w0 ? (F)r0 : F(0);
+                red[0][1] = w1 ? (F)(two ? k1 + m1 * r0 : k1) : F(0);
+            }
+            __syncthreads();
+            rho0 = red[0][0];
+            rho1 = red[0][1];
+        }
+        // value of a velocity with both ghosts
+        auto value = [&](int kk, const Vel& q, int cp) {
+            F a = q.x[cp];
+            const F f0 = cp ? h0 : F(1), f1 = cp ? h1 : F(1);
+            if (q.ux < F(0)) {
+                if (w0) a -= q.ux * rx * q.den * (q.c0 * f0 * rho0);
+                else if (y0) {       // the mirrored velocity leaves there and may itself enter through the other face
+                    Vel m;
+                    mirrored(0, kk, m);
+                    F g = m.x[cp];
+                    if (m.uy < F(0) && w1) g -= m.uy * ry * m.den * (m.c1 * f1 * rho1);
+                    if (m.uy < F(0) && y1) { Vel n; const int aa = kk / V.nvv, bb = kk - aa * V.nvv;
+                        mirrored(1, (V.nu - 1 - aa) * V.nvv + bb, n); g -= m.uy * ry * m.den * n.x[cp]; }
+                    a -= q.ux * rx * q.den * g;
+                }
+            }
+            if (q.uy < F(0)) {
+                if (w1) a -= q.uy * ry * q.den * (q.c1 * f1 * rho1);
+                else if (y1) {
+                    Vel m;
+                    mirrored(1, kk, m);
+                    F g = m.x[cp];
+                    if (m.ux < F(0) && w0) g -= m.ux * rx * m.den * (m.c0 * f0 * rho0);
+                    if (m.ux < F(0) && y0) { Vel n; const int aa = kk / V.nvv, bb = kk - aa * V.nvv;
+                        mirrored(0, aa * V.nvv + (V.nvv - 1 - bb), n); g -= m.ux * rx * m.den * n.x[cp]; }
+                    a -= q.uy * ry * q.den * g;
+                }
+            }
+            return a;
+        };
+        if (on) {
+            Vel q0;
+            fetch(k, q0);
+            finish(q0);
+            xp[0] = value(k, q0, 0);
+            if (sym) xp[1] = value(k, q0, 1);
+        }
+        if (q == 0) {                                // the corner's values for the wavefront, a slice per CTA
+            const int per = (nv + nchunk - 1) / nchunk;
+            #pragma unroll 1
+            for (int kk = chunk * per + tid; kk < min(nv, (chunk + 1) * per); kk += B) {
+                Vel q0;
+                fetch(kk, q0);
+                finish(q0);
+                S.corner[kk] = value(kk, q0, 0);
+                S.corner[ld + kk] = value(kk, q0, 1);
+            }
+        }
+    } else if (on) {
+        xp[0] = x[c0 * ld + k];
+        xp[1] = x[(nc + c0) * ld + k];
+    }
+    // -1/Z of the cells' walls (0 at other boundaries), for the end of the walk
+    #pragma unroll
+    for (int t = 0; t < kMaxLine / B; ++t) {
+        const int st = tid + t * B;
+        if (st < len) zf[st] = zb[t] >= 0 && M.bc[zb[t]].type == BC_WALL ? -(F)iZw[zb[t] * 4 + axis * 2 + pass] : F(0);
+    }
+    if (sym && edge && on)
+        for (int cp = 0; cp < 2; ++cp) S.xline[((size_t)ebase * 2 + cp) * ld + k] = xp[cp];
+    __syncthreads();                                 // nbS
+    // an[k]: coefficient of the previous cell of the line; lw: weight of the velocity in the wall sum
+    const F s1 = axis == 0 ? vv[k] : vu[k], uo = axis == 0 ? (pass == 0 ? -vu[k] : vu[k]) : (pass == 0 ? -vv[k] : vv[k]);
+    const F an = min(pass == 0 ? -s1 : s1, F(0)), lw = on ? vw[k] * uo : F(0);
+    F* part = S.part + ((size_t)q * nchunk + chunk) * kMaxLine;
+    const int nbat = (len - 1 + U - 1) / U;
+    for (int b = 0; b < nbat; ++b) {
+        issue(b + NB - 1);
+        cp_async_wait_n<NB - 1>();
+        const F* d = ring + (b % NB) * U * 3 * B + tid;
+        F xv[U];
+        #pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int st = 1 + U * b + u;
+            xv[u] = F(0);
+            if (st < len && on) {
+                const F id = d[u * 3 * B], in = d[u * 3 * B + B], Dn = an * nbS[st];
+                xp[0] = xv[u] = pass == 0 ? (in - Dn * xp[0]) * id : in - Dn * xp[0] * id;
+                if (sym) {
+                    const F ih = d[u * 3 * B + 2 * B];
+                    xp[1] = pass == 0 ? (ih - Dn * xp[1]) * id : ih - Dn * xp[1] * id;
+                    S.xline[((size_t)(ebase + st) * 2) * ld + k] = xp[0];
+                    S.xline[((size_t)(ebase + st) * 2 + 1) * ld + k] = xp[1];
                 }
             }
         }
-        if constexpr (R > 1) {
-            issue(dd + R - 1, cd_next);
-            cd_next = cd_n1;
-            cd_n1 = cd_n2;
-            cd_n2 = cd_n3;
-            cd_n3 = code_of(dd + R + 3);                // consumed four steps later
+        const int row = (b % NB) * U;
+        #pragma unroll
+        for (int u = 0; u < U; ++u) tile[(row + u) * TS + tid] = lw * xv[u];
+        if (row + U == RA || b == nbat - 1) {          // sums of the cells of the last NB batches
+            __syncthreads();
+            const int cell = tid / TP, p = tid % TP, st = 1 + U * b - row + cell;
+            F s0 = F(0), s2 = F(0);
+            for (int m = p; m < B; m += 2 * TP) { s0 += tile[cell * TS + m]; s2 += tile[cell * TS + m + TP]; }
+            s0 += s2;
+            #pragma unroll
+            for (int o = TP / 2; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            if (p == 0 && cell < row + U && st < len) part[st] = s0;
+            __syncthreads();
         }
-        __syncthreads();
+    }
+    cp_async_wait_n<0>();
+    // the last CTA of the line adds the partial sums, in order
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        last = atomicAdd(S.count + q, 1) == nchunk - 1;
+        if (last) S.count[q] = 0;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int st = 1 + tid; st < len; st += B) {
+        F sum = F(0);
+        #pragma unroll 4
+        for (int m = 0; m < nchunk; ++m) sum += __ldcg(S.part + ((size_t)q * nchunk + m) * kMaxLine + st);
+        S.rho[ebase + st] = sum * zf[st];
+    }
+}
+
+// Wavefront steps [dd0, dd1) of one sweep over every cell.  A CTA owns 16 LPC
+// bytes of consecutive velocities and the whole mesh; its warps own strips of
+// 32 / LPC grid lines, LPC lanes per line, and walk along the lines one cell per
+// step: the cells of a step lie on an anti-diagonal, the neighbour along the line
+// is the lane's own last result, the one across comes from the line before by
+// shuffles (from the strip before through a shared ring), so there is no barrier.
+// Strips follow each other; their counters are looked at every kWaveChunk steps.
+// Inputs stream through a ring of R steps by asynchronous copies, every lane its own.
+//   forward   x = (b - C_a x_a - C_l x_l) / D, b the residual,
+//   backward  x = b - (C_a x_a + C_l x_l) / D, b the forward value,
+// with the coefficients zero where the neighbour lies downwind: a CTA whose
+// velocities need no neighbour across (or along) skips that part, and in the
+// backward pass one that needs neither leaves its values as they are.
+// Boundary-line cells take b and 1/D from the fold, which the CTA makes for its
+// velocities before it starts, from the wall densities of the line walk: the
+// entries [e0, e0 + ne) of the lines walked last.  Cells in a body, and steps
+// outside a line, are copied as zeros, which makes their result zero and drops
+// the neighbour across a boundary face without a test.
+// What bounds it: on large levels the L1 look-ups of the copies and stores (one per
+// cell and warp access, see LPC in launch_micro_sgs), on small ones the
+// instructions of a step, as an SM sub-partition has one warp.  Square cylinder,
+// mixed: 9.0 ms per iteration for all levels, against 16.4 ms for the wavefront of
+// 4-velocity CTAs with a barrier per diagonal and the line kernel beside it that
+// this replaces; 64x64 cavity 29 us per launch against 32 us.
+constexpr int kWaveChunk = 4;
+constexpr int kWaveEdge = 16;                       // results of a strip's last line in flight to the next strip
+constexpr int kWaveSpin = 1 << 24;                  // looks of a wait before it gives up
+
+__device__ __forceinline__ bool wave_wait(const int* flag, int need)
+{
+    const unsigned a = smem_addr(flag);
+    for (int it = 0; it < kWaveSpin; ++it) {
+        int v;
+        asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];\n" : "=r"(v) : "r"(a) : "memory");
+        if (v >= need) return true;
+        __nanosleep(20);                             // (a spinning strip takes issue slots from the working ones)
+    }
+    return false;
+}
+__device__ __forceinline__ void wave_post(int* flag, int v)
+{
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;\n" ::"r"(smem_addr(flag)), "r"(v) : "memory");
+}
+
+// 64 bits of velocities: two floats (packed arithmetic, rounded as the scalar one) or a double
+template <typename F> struct Pack;
+template <> struct Pack<float> {
+    using T = unsigned long long;
+    static __device__ __forceinline__ T make(float a, float b) { T r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+    static __device__ __forceinline__ T splat(float a) { return make(a, a); }
+    static __device__ __forceinline__ T load(const float* p) { return make(p[0], p[1]); }
+    static __device__ __forceinline__ T mul(T a, T b) { T r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+    static __device__ __forceinline__ T add(T a, T b) { T r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+    static __device__ __forceinline__ T fma(T a, T b, T c)
+    {
+        T r;
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+        return r;
+    }
+};
+template <> struct Pack<double> {
+    using T = double;
+    static __device__ __forceinline__ T splat(double a) { return a; }
+    static __device__ __forceinline__ T load(const double* p) { return p[0]; }
+    static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
+    static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+    static __device__ __forceinline__ T fma(T a, T b, T c) { return ::fma(a, b, c); }
+};
+__device__ __forceinline__ void ld_pair(const void* p, unsigned long long* v)
+{
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void ld_pair(const void* p, double* v)
+{
+    const double2 t = *reinterpret_cast<const double2*>(p);
+    v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void st_pair(void* p, const unsigned long long* v)
+{
+    *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v[0], v[1]);
+}
+__device__ __forceinline__ void st_pair(void* p, const double* v) { *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]); }
+
+// the same under a predicate (a branch would have to be resolved on the path of a step)
+__device__ __forceinline__ unsigned long long bits(unsigned long long v) { return v; }
+__device__ __forceinline__ unsigned long long bits(double v) { return (unsigned long long)__double_as_longlong(v); }
+__device__ __forceinline__ void st_pair_if(bool on, void* p, unsigned long long a, unsigned long long b)
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %3, 0;\n @p st.global.v2.b64 [%0], {%1, %2};\n}\n"
+                 ::"l"(p), "l"(a), "l"(b), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void sts_pair_if(bool on, unsigned p, unsigned long long a, unsigned long long b)
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %3, 0;\n @p st.shared.v2.b64 [%0], {%1, %2};\n}\n"
+                 ::"r"(p), "l"(a), "l"(b), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void lds_pair_if(bool on, unsigned p, unsigned long long* v)
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %3, 0;\n @p ld.shared.v2.b64 {%0, %1}, [%2];\n}\n"
+                 : "+l"(v[0]), "+l"(v[1]) : "r"(p), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void lds_pair_if(bool on, unsigned p, double* v)
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %3, 0;\n @p ld.shared.v2.f64 {%0, %1}, [%2];\n}\n"
+                 : "+d"(v[0]), "+d"(v[1]) : "r"(p), "r"((unsigned)on) : "memory");
+}
+
+// Fold of the boundary-line cells [e0, e0 + ne) for the CTA's velocities (k_sgs_wave)
+template <typename F, int PASS, int LPC>
+__device__ void wave_fold(const MicroArgs& M, const F* __restrict__ invD, const F* __restrict__ src, const SweepScratch<F>& S,
+                          F* __restrict__ fold, int k0, int e0, int ne)
+{
+    constexpr int V16 = 16 / (int)sizeof(F), K = V16, KB = LPC * V16;   // a thread's and the CTA's velocities
+    const LevelDev& L = M.L;
+    const VelDev& V = M.V;
+    const int nx = L.nx, nv = V.nv;
+    const size_t nc = L.nc, ld = V.ld;
+    const F* __restrict__ vu = VelT<F>::u(V);
+    const F* __restrict__ vv = VelT<F>::v(V);
+    const int part = (int)threadIdx.x % LPC;
+    k0 += part * V16;
+    for (int e = e0 + (int)threadIdx.x / LPC; e < e0 + ne; e += (int)blockDim.x / LPC) {
+        const int4 lc = M.P.lcell[PASS][e];         // {cell, line axis, bc id, corner}
+        const int c = lc.x, axis = lc.y, i = c % nx, j = c / nx;
+        F b[2][K], iv[K];
+        if (lc.w) {
+            #pragma unroll
+            for (int q = 0; q < K; ++q) {
+                const bool in = k0 + q < nv;
+                b[0][q] = in ? S.corner[k0 + q] : F(0);
+                b[1][q] = in ? S.corner[ld + k0 + q] : F(0);
+                iv[q] = F(1);
+            }
+        } else {
+            const size_t o = (size_t)c * ld + k0;
+            #pragma unroll
+            for (int q = 0; q < K; q += V16) {
+                ld16(src + o + q, b[0] + q);
+                ld16(src + nc * ld + o + q, b[1] + q);
+                ld16(invD + o + q, iv + q);
+            }
+            const int bc = lc.z;
+            const BcDev Bc = M.bc[bc];
+            const F rS = axis == 0 ? (F)L.rdx[i] : (F)L.rdy[j], h = (F)(kKint * Bc.t / 4.0), rho = S.rho[e];
+            #pragma unroll
+            for (int q = 0; q < K; ++q) {
+                const int k = k0 + q;
+                const F u = vu[k], v = vv[k];
+                F un = axis == 0 ? u : v;
+                un = PASS == 0 ? -un : un;
+                if (!(un < F(0)) || k >= nv) continue;
+                const F Db = un * rS;
+                F g[2] = {F(0), F(0)};
+                if (Bc.type == BC_WALL) {
+                    g[0] = Db * ((F)M.Cw[(size_t)bc * nv + k] * rho);
+                    g[1] = h * g[0];
+                } else if (Bc.type == BC_SYMMETRY) {
+                    const int a2 = k / V.nvv, b2 = k - a2 * V.nvv;
+                    const int km = axis == 0 ? (V.nu - 1 - a2) * V.nvv + b2 : a2 * V.nvv + (V.nvv - 1 - b2);
+                    g[0] = Db * S.xline[((size_t)e * 2) * ld + km];
+                    g[1] = Db * S.xline[((size_t)e * 2 + 1) * ld + km];
+                } else if (Bc.type == BC_OUTFLOW) {
+                    const F D = (F)M.inv_tau[c] + fabs(u) * (F)L.rdx[i] + fabs(v) * (F)L.rdy[j];
+                    iv[q] = recip(D + Db);
+                    if (PASS == 1) { b[0][q] = D * b[0][q] * iv[q]; b[1][q] = D * b[1][q] * iv[q]; }
+                }
+                b[0][q] -= PASS == 0 ? g[0] : g[0] * iv[q];
+                b[1][q] -= PASS == 0 ? g[1] : g[1] * iv[q];
+            }
+        }
+        F* o = fold + (size_t)e * 3 * KB + part * V16;
+        st16(o, b[0]);
+        st16(o + KB, b[1]);
+        st16(o + 2 * KB, iv);
+    }
+}
+
+// LPC: lanes per cell, 16 bytes of velocities each
+template <typename F, int R, int PASS, bool BODIES, int LPC>
+__global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restrict__ invD, const F* __restrict__ r,
+                                                  F* __restrict__ x, SweepScratch<F> S, int dd0, int dd1, int e0, int ne)
+{
+    using P = Pack<F>;
+    using T = typename P::T;
+    constexpr int V16 = 16 / (int)sizeof(F), K = LPC * V16, NL = 32 / LPC, step_bytes = 3 * 512, ebytes = 32 * LPC;
+    extern __shared__ __align__(16) unsigned char wsm[];
+    const LevelDev& L = M.L;
+    const VelDev& V = M.V;
+    const int nx = L.nx, ny = L.ny, k0 = (int)blockIdx.x * K;
+    const bool xl = nx <= ny;                       // lines are columns
+    const int ns = xl ? nx : ny, nt = xl ? ny : nx, nw = (int)blockDim.x >> 5;
+    const size_t nc = L.nc, ld = V.ld;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, ll = lane / LPC, part = lane % LPC, s = NL * w + ll;
+    unsigned char* ring = wsm + (size_t)w * R * step_bytes + lane * 16;
+    unsigned char* edges = wsm + (size_t)nw * R * step_bytes;                   // [strip][kWaveEdge][2][LPC] x 16 bytes
+    F* ral = reinterpret_cast<F*>(edges + (size_t)nw * kWaveEdge * ebytes);     // [nt] -1/d along the lines
+    int* prog = reinterpret_cast<int*>(ral + nt);                               // per strip: edge values there
+    int* cons = prog + nw;                                                      // per strip: edge values taken
+    const F* src = PASS == 0 ? r : x;
+    const F* __restrict__ vu = VelT<F>::u(V);
+    const F* __restrict__ vv = VelT<F>::v(V);
+    const int kl = k0 + part * V16;                 // first velocity of this lane
+    // coefficients per unit face: across and along the lines (zero where that neighbour lies downwind)
+    F ca[V16], cl[V16];
+    bool any_a = false, any_l = false;
+    #pragma unroll
+    for (int q = 0; q < V16; ++q) {
+        const F u = vu[kl + q], v = vv[kl + q];     // the tables are padded with zeros
+        const F cu = min(PASS == 0 ? -u : u, F(0)), cv = min(PASS == 0 ? -v : v, F(0));
+        ca[q] = xl ? cu : cv;
+        cl[q] = xl ? cv : cu;
+        any_a = any_a || ca[q] != F(0);
+        any_l = any_l || cl[q] != F(0);
+    }
+    any_a = __any_sync(0xffffffffu, any_a);
+    any_l = __any_sync(0xffffffffu, any_l);
+    if (PASS == 1 && !any_a && !any_l) return;      // (the same in every warp)
+    F* fold = S.fold + (size_t)blockIdx.x * S.nl * 3 * K;
+    wave_fold<F, PASS, LPC>(M, invD, src, S, fold, k0, e0, ne);
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) {
+        const int p = PASS == 0 ? t : nt - 1 - t;
+        ral[t] = -(F)(xl ? L.rdy[p] : L.rdx[p]);
+    }
+    if (lane == 0) prog[w] = cons[w] = max(0, dd0 + 1 - NL * w);
+    __threadfence();                                // the fold is read by asynchronous copies of other threads
+    __syncthreads();
+    // ---- this strip's steps of the segment: step k sweeps the strip's diagonal NL w + k
+    const int kb = max(0, dd0 - NL * w), ke = min(nt + NL - 1, dd1 - NL * w);
+    if (kb >= ke) return;
+    const bool line = s < ns;
+    const int sp = PASS == 0 ? s : ns - 1 - s, tp = PASS == 0 ? 0 : nt - 1;
+    const long cfirst = line ? (xl ? (long)tp * nx + sp : (long)sp * nx + tp) : 0;   // the line's cell t = 0
+    const long cst = (PASS == 0 ? 1 : -1) * (xl ? (long)nx : 1L);
+    const long pst = cst * (long)ld;                // from a cell of the line to the next, in values
+    const F rac = line && s > 0 ? -(xl ? (F)L.rdx[sp] : (F)L.rdy[sp]) : F(0);
+    T nca[2], ncl[2];
+    #pragma unroll
+    for (int q = 0; q < V16; ++q) ca[q] *= rac;
+    #pragma unroll
+    for (int q = 0; q < 2; ++q) { nca[q] = P::load(ca + q * (V16 / 2)); ncl[q] = P::load(cl + q * (V16 / 2)); }
+    const int ea = xl ? 0 : ny, eb = xl ? ny + s : s;   // fold entries of line 0 (+ t) and of the cells t = 0
+    const int* __restrict__ code = M.P.code[PASS];
+    auto code_of = [&](int k) {
+        const int t = k - ll;
+        return line && (unsigned)t < (unsigned)nt && k < ke ? code[cfirst + t * cst] : -2;
+    };
+    int cd0 = 0, cd1 = 0, cd2 = 0, cd3 = 0;         // codes of the next four cells to be copied
+    if constexpr (BODIES) { cd0 = code_of(kb); cd1 = code_of(kb + 1); cd2 = code_of(kb + 2); cd3 = code_of(kb + 3); }
+    const size_t hoff = nc * ld;
+    // running addresses of the next cell to be copied (before and after the line they are not used)
+    const F* pb = src + (cfirst + (kb - ll) * cst) * (long)ld + kl;
+    const F* pi = invD + (cfirst + (kb - ll) * cst) * (long)ld + kl;
+    const F* safe = src + kl;
+    auto issue = [&](int k, int stage) {
+        const int t = k - ll;
+        bool on = line && (unsigned)t < (unsigned)nt && k < ke;
+        const F *p0 = pb, *p1 = pb + hoff, *p2 = pi;
+        pb += pst;
+        pi += pst;
+        if constexpr (BODIES) {
+            on = on && cd0 != -2;
+            if (cd0 >= 0) {
+                p0 = fold + (long)cd0 * 3 * K + part * V16;
+                p1 = p0 + K;
+                p2 = p0 + 2 * K;
+            }
+            cd0 = cd1; cd1 = cd2; cd2 = cd3; cd3 = code_of(k + 4);
+        } else if (w == 0 || k < NL) {              // (the other steps of a strip hold no line cell)
+            if (s == 0 || t == 0) {
+                p0 = fold + (long)(s == 0 ? ea + t : eb) * 3 * K + part * V16;
+                p1 = p0 + K;
+                p2 = p0 + 2 * K;
+            }
+        }
+        if (!on) p0 = p1 = p2 = safe;               // nothing is read from it
+        unsigned char* d = ring + stage * step_bytes;
+        cp_async16_if(on, d, p0);
+        cp_async16_if(on, d + 512, p1);
+        cp_async16_if(on, d + 1024, p2);
+        cp_async_commit();
+    };
+    T ac[2][2], al[2][2];
+    #pragma unroll
+    for (int q = 0; q < 2; ++q) ac[0][q] = ac[1][q] = al[0][q] = al[1][q] = P::splat(F(0));
+    #pragma unroll
+    for (int q = 0; q < R - 1; ++q) issue(kb + q, q);
+    if (dd0 > 0 && kb + NL * w == dd0) {
+        // the segment goes on from the diagonal before it
+        const int t = kb - ll;
+        const bool hl = line && t >= 1 && t <= nt, ha = s >= 1 && s <= ns && t >= 0 && t < nt;
+        const long c_l = cfirst + (long)(t - 1) * cst;
+        const int sa = PASS == 0 ? s - 1 : ns - s, ta = PASS == 0 ? t : nt - 1 - t;
+        const long c_a = xl ? (long)ta * nx + sa : (long)sa * nx + ta;
+        #pragma unroll
+        for (int cp = 0; cp < 2; ++cp) {
+            if (hl) ld_pair(x + (cp * nc + c_l) * ld + kl, al[cp]);
+            if (ha) ld_pair(x + (cp * nc + c_a) * ld + kl, ac[cp]);
+        }
+    }
+    const bool takes = any_a && w > 0, feeds = any_a && w + 1 < nw;
+    const int tfirst = max(0, dd0 + 1 - NL * w);    // edge values from here on come through the ring
+    const unsigned etake = smem_addr(edges + (size_t)w * kWaveEdge * ebytes + part * 32);
+    const unsigned efeed = smem_addr(edges + (size_t)(w + 1) * kWaveEdge * ebytes + part * 32);
+    F* xo = x + (cfirst + (kb - ll) * cst) * (long)ld + kl;
+    for (int kc = kb; kc < ke; kc += 8) {
+        #pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {             // steps beyond ke copy zeros and store nothing
+            const int k = kc + kk, t = k - ll;
+            if (kk % kWaveChunk == 0) {
+                const int kn = min(k + kWaveChunk, ke);
+                bool got = true;
+                if (takes) got = wave_wait(prog + w, min(nt, kn));
+                if (feeds) got = got && wave_wait(cons + w + 1, min(nt, kn - (NL - 1)) - kWaveEdge);
+                if (!__all_sync(0xffffffffu, got)) { if (lane == 0) *M.flag = 1.0; cp_async_wait_n<0>(); return; }
+            }
+            cp_async_wait_n<R - 2>();
+            T b[2][2], iv[2];
+            const unsigned char* d = ring + (kk % R) * step_bytes;
+            ld_pair(d, b[0]);
+            ld_pair(d + 512, b[1]);
+            ld_pair(d + 1024, iv);
+            const bool tk = takes && ll == 0 && k >= tfirst && k < nt;
+            const unsigned ea_ = etake + (unsigned)(k % kWaveEdge) * ebytes;
+            lds_pair_if(tk, ea_, ac[0]);
+            lds_pair_if(tk, ea_ + 16, ac[1]);
+            issue(k + R - 1, (kk + R - 1) % R);
+            // minus the neighbours' terms (line 0 has no neighbour across: its coefficient is zero)
+            if (any_l) {
+                const T ra = P::splat(ral[min(max(t, 0), nt - 1)]);
+                #pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const T g = P::mul(ncl[q], ra);
+                    al[0][q] = P::mul(g, al[0][q]);
+                    al[1][q] = P::mul(g, al[1][q]);
+                }
+            }
+            #pragma unroll
+            for (int cp = 0; cp < 2; ++cp)
+                #pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    T n = any_l ? al[cp][q] : P::splat(F(0));
+                    if (any_a) n = any_l ? P::fma(nca[q], ac[cp][q], n) : P::mul(nca[q], ac[cp][q]);
+                    al[cp][q] = PASS == 0 ? P::mul(P::add(b[cp][q], n), iv[q]) : P::fma(n, iv[q], b[cp][q]);
+                }
+            const bool on = line && (unsigned)t < (unsigned)nt && k < ke;
+            st_pair_if(on, xo, bits(al[0][0]), bits(al[0][1]));
+            st_pair_if(on, xo + hoff, bits(al[1][0]), bits(al[1][1]));
+            xo += pst;
+            if (any_a) {
+                const bool fd = feeds && ll == NL - 1 && on;
+                const unsigned ed = efeed + (unsigned)(t & (kWaveEdge - 1)) * ebytes;
+                sts_pair_if(fd, ed, bits(al[0][0]), bits(al[0][1]));
+                sts_pair_if(fd, ed + 16, bits(al[1][0]), bits(al[1][1]));
+                #pragma unroll
+                for (int cp = 0; cp < 2; ++cp)
+                    #pragma unroll
+                    for (int q = 0; q < 2; ++q) ac[cp][q] = __shfl_up_sync(0xffffffffu, al[cp][q], LPC);
+            }
+            if ((kk + 1) % kWaveChunk == 0 && (feeds || takes)) {
+                const int kn = min(k + 1, ke);
+                __syncwarp();                        // every lane's edge values are stored, or read
+                if (feeds && lane == 31) wave_post(prog + w + 1, min(nt, kn - (NL - 1)));
+                if (takes && lane == 0) wave_post(cons + w, min(nt, kn));
+            }
+        }
     }
     cp_async_wait_n<0>();
 }
 
-// Wavefront steps [dd0, dd1) of one sweep pass for the velocities that are
-// coupled to one upwind neighbour only, or to none (the sign of u or v puts the
-// other neighbour downwind, and its coefficient is an exact zero): such a
-// velocity is independent along every row (coupled along x only) or every
-// column (along y only), or every cell (neither), so one thread per (line,
-// velocity) walks the cells of its line that lie on the segment's diagonals,
-// with no barrier.  Consecutive threads take consecutive velocities of the
-// same line, so every access is coalesced, and each thread loads the inputs of
-// four cells before it updates them in order.  The update of a cell is the
-// wavefront kernel's with the zero coupling left out; boundary-line cells take
-// their folded inputs (incoming velocities) or keep the value of their line
-// walk (outgoing velocities and the corner), as in the wavefront kernel.  The
-// backward pass leaves the uncoupled velocities as they are (x = x).
-// Block b: rows (class 0) first, nbr blocks of 128 velocities per row, then
-// columns (class 1), nbc per column, then cells of no coupling by rows, nbe per
-// row (0 in the backward pass).
-template <typename F, bool BODIES>
-__global__ void __launch_bounds__(128) k_sgs_lines(MicroArgs M, const F* __restrict__ invD, const F* __restrict__ r,
-                                                   F* __restrict__ x, const F* __restrict__ fold, int pass, int dd0,
-                                                   int dd1, int nbr, int nbc, int nbe)
+// sweep scratch: values of the storage type per solver (the largest level), and line counters
+size_t micro_scratch_elems(int ld, int nl, int nlines, int nchunk, bool sym)
 {
-    constexpr int K = kInteriorKc, U = 4;
-    const LevelDev& L = M.L;
-    const VelDev& Vg = M.V;
-    const int nx = L.nx, ny = L.ny, nv = Vg.nv, nd = nx + ny - 1, nls = M.P.nl_max;
-    const size_t nc = L.nc;
-    int b = blockIdx.x, cls, line, q;
-    if (b < nbr * ny) {
-        cls = 0; line = b / nbr; q = (b % nbr) * 128 + threadIdx.x;
-        if (q >= Vg.nrow[pass]) return;
-    } else if ((b -= nbr * ny) < nbc * nx) {
-        cls = 1; line = b / nbc; q = (b % nbc) * 128 + threadIdx.x;
-        if (q >= Vg.ncol[pass]) return;
-        q += Vg.nrow[pass];
-    } else {
-        b -= nbc * nx;
-        cls = 2; line = b / nbe; q = (b % nbe) * 128 + threadIdx.x;
-        if (q >= Vg.nelem[pass]) return;
-        q += Vg.nrow[pass] + Vg.ncol[pass];
-    }
-    const int k = Vg.lk[pass][q];
-    const F u = (F)Vg.u[k], v = (F)Vg.v[k];
-    const F cu = pass == 0 ? (u > F(0) ? -u : F(0)) : (u < F(0) ? u : F(0));
-    const F cv = pass == 0 ? (v > F(0) ? -v : F(0)) : (v < F(0) ? v : F(0));
-    const F cc = cls == 0 ? cu : cls == 1 ? cv : F(0);   // coefficient of the neighbour along the line
-    // the line's cells on diagonals [dlo, dhi): position p along the line (i for rows, j for columns)
-    const int dlo = pass == 0 ? dd0 : nd - dd1, dhi = pass == 0 ? dd1 : nd - dd0;
-    const int len = cls == 1 ? ny : nx;
-    const int p0 = max(0, dlo - line), p1 = min(len, dhi - line);
-    if (p1 <= p0) return;
-    const int n = p1 - p0, step = pass == 0 ? 1 : -1, pfirst = pass == 0 ? p0 : p1 - 1;
-    const int ib = pass == 0 ? 0 : nx - 1, jb = pass == 0 ? 0 : ny - 1;
-    const int* __restrict__ code = M.P.code[pass];
-    const F* src = pass == 0 ? r : x;
-    const int kb = k / K, kk = k - kb * K;
-    auto cell_of = [&](int p) { return cls == 1 ? p * nx + line : line * nx + p; };
-    // value of the upwind neighbour of the first cell (from an earlier segment), 0 at the line's start
-    F xp[2] = {F(0), F(0)};
-    const int pnb = pfirst - step;
-    if (cls != 2 && pnb >= 0 && pnb < len) {
-        const size_t cn = (size_t)cell_of(pnb) * nv + k;
-        xp[0] = x[cn];
-        xp[1] = x[nc * nv + cn];
-    }
-    for (int s0 = 0; s0 < n; s0 += U) {
-        // inputs of up to U cells: kind 0 ordinary, 1 folded (incoming at a line face),
-        // 2 final (outgoing at a line face, or the corner), 3 in a body
-        F a[U][2], iv[U], rd[U];
-        int kind[U];
-        #pragma unroll
-        for (int t = 0; t < U; ++t) {
-            kind[t] = 2;
-            a[t][0] = a[t][1] = iv[t] = rd[t] = F(0);
-            if (s0 + t >= n) continue;
-            const int p = pfirst + (s0 + t) * step;
-            const int c = cell_of(p), i = cls == 1 ? line : p, j = cls == 1 ? p : line;
-            bool hasx, hasy;
-            int e = 0;
-            if constexpr (BODIES) {
-                const int cd = code[c];
-                if (cd == -2) { kind[t] = 3; continue; }
-                hasx = cd >= 0 && (cd & 2);
-                hasy = cd >= 0 && (cd & 1);
-                e = cd >> 2;
-            } else {
-                hasx = i == ib;
-                hasy = j == jb;
-                e = hasx ? (pass == 0 ? j : ny - 1 - j) : ny + (pass == 0 ? i : nx - 1 - i);
-            }
-            // the line face across which this class's velocities enter, and the one they leave by
-            const bool fin = cls == 0 ? hasy : cls == 1 ? hasx : (hasx || hasy);
-            const bool fld = !fin && (cls == 0 ? hasx : cls == 1 ? hasy : false);
-            const size_t id = (size_t)c * nv + k;
-            if (fin) {
-                kind[t] = 2;
-                if (cls != 2) { a[t][0] = x[id]; a[t][1] = x[nc * nv + id]; }
-            } else if (fld) {
-                kind[t] = 1;
-                const F* fo = fold + ((size_t)(kb * nls + e) * 3) * K + kk;
-                a[t][0] = fo[0]; a[t][1] = fo[K]; iv[t] = fo[2 * K];
-            } else {
-                kind[t] = 0;
-                a[t][0] = src[id]; a[t][1] = src[nc * nv + id]; iv[t] = invD[id];
-                rd[t] = cls == 0 ? (F)L.rdx[i] : cls == 1 ? (F)L.rdy[j] : F(0);
-            }
-        }
-        #pragma unroll
-        for (int t = 0; t < U; ++t) {
-            if (s0 + t >= n) continue;
-            const int p = pfirst + (s0 + t) * step;
-            const size_t id = (size_t)cell_of(p) * nv + k;
-            F res[2];
-            #pragma unroll
-            for (int cp = 0; cp < 2; ++cp) {
-                if (kind[t] == 3) res[cp] = F(0);
-                else if (kind[t] == 2) res[cp] = a[t][cp];
-                else if (kind[t] == 1) res[cp] = pass == 0 ? a[t][cp] * iv[t] : a[t][cp];
-                else {
-                    const F y = cls == 2 ? F(0) : cc * rd[t] * xp[cp];
-                    res[cp] = pass == 0 ? (a[t][cp] - y) * iv[t] : a[t][cp] - y * iv[t];
-                }
-                xp[cp] = res[cp];
-            }
-            if (kind[t] != 2) {
-                x[id] = res[0];
-                x[nc * nv + id] = res[1];
-            }
-        }
-    }
+    return 2 * (size_t)ld + (((size_t)nl + 15) & ~(size_t)15) + (2 + (size_t)nlines) * nchunk * kMaxLine +
+           3 * (size_t)ld * nl + (sym ? 2 * (size_t)nl * ld : 0);
 }
+template <typename F>
+SweepScratch<F> sweep_scratch(F* base, int* count, int ld, int nl, int nlines, int nchunk)
+{
+    SweepScratch<F> S;
+    S.corner = base;
+    S.rho = S.corner + 2 * (size_t)ld;
+    S.part = S.rho + (((size_t)nl + 15) & ~(size_t)15);
+    S.fold = S.part + (2 + (size_t)nlines) * nchunk * kMaxLine;
+    S.xline = S.fold + 3 * (size_t)ld * nl;
+    S.count = count;
+    S.nl = nl;
+    return S;
+}
+int micro_edge_chunks(const VelDev& V)
+{
+    int m = 1;
+    for (int p = 0; p < 2; ++p)
+        for (int a = 0; a < 2; ++a) m = std::max(m, (V.nleave[p][a] * (a == 0 ? V.nvv : V.nu) + 127) / 128);
+    return m;
+}
+
+template <typename F>
+cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, const double* Zw, const F* invD,
+                             const F* r, F* x, F* scratch, cudaStream_t st)
+{
+    if (m.L.nx > kMaxLine || m.L.ny > kMaxLine) return cudaErrorInvalidValue;
+    const int ns = std::min(m.L.nx, m.L.ny), nt = std::max(m.L.nx, m.L.ny), nchunk = plan.nchunk;
+    const SweepScratch<F> S = sweep_scratch<F>(scratch, plan.count, m.V.ld, plan.nl, plan.nlines, nchunk);
+    constexpr size_t kSmemMax = 227 * 1024;
+    constexpr size_t esmem = sizeof(F) * EdgeRing<F>::RA * (3 * 128 + 132);
+    // Lanes per cell: an asynchronous copy or store of a warp costs its SM's L1 one look-up per cell, so
+    // the more lanes share a cell the better (64 bytes of a cell with four), as long as the strips fit a
+    // CTA of 16 warps and the CTAs fill the SMs.  Finest level and coarser ones together, per
+    // iteration, 1 / 2 / 4 lanes: square cylinder mixed 21.5 / 12.8 / 9.0 ms, plate mixed 2.9 / 2.0 / 1.7 ms;
+    // 64x64 cavity with 32x32 velocities (64 CTAs with four lanes) 0.62 / 0.57 / 0.63 ms.
+    constexpr int V16 = 16 / (int)sizeof(F);
+    const int LPC = ns <= 128 && m.V.ld / (4 * V16) > 128 ? 4 : ns <= 256 ? 2 : 1;
+    const int nblk = m.V.ld / (LPC * V16), nw = (ns * LPC + 31) / 32;
+    // ring depth: eight steps in flight where they fit, else four
+    const size_t fixed = (size_t)nw * kWaveEdge * 32 * LPC + sizeof(F) * nt + 2 * sizeof(int) * nw + 16, slot = (size_t)nw * 1536;
+    const int R = fixed + 8 * slot <= kSmemMax ? 8 : 4;
+    const size_t wsmem = fixed + R * slot;
+    if (wsmem > kSmemMax) return cudaErrorInvalidValue;
+    using Wave = void (*)(MicroArgs, const F*, const F*, F*, SweepScratch<F>, int, int, int, int);
+    auto pick = [&](auto h, auto bodies) {
+        constexpr int HH = decltype(h)::value;
+        constexpr bool BB = decltype(bodies)::value;
+        std::array<Wave, 2> f;
+        f[0] = R == 8 ? k_sgs_wave<F, 8, 0, BB, HH> : k_sgs_wave<F, 4, 0, BB, HH>;
+        f[1] = R == 8 ? k_sgs_wave<F, 8, 1, BB, HH> : k_sgs_wave<F, 4, 1, BB, HH>;
+        return f;
+    };
+    auto by_lanes = [&](auto bodies) {
+        return LPC == 4 ? pick(std::integral_constant<int, 4>(), bodies)
+               : LPC == 2 ? pick(std::integral_constant<int, 2>(), bodies) : pick(std::integral_constant<int, 1>(), bodies);
+    };
+    const std::array<Wave, 2> wave = m.P.bodies ? by_lanes(std::true_type()) : by_lanes(std::false_type());
+    for (int p = 0; p < 2; ++p) {
+        cudaError_t e = cudaFuncSetAttribute(wave[p], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
+        if (e != cudaSuccess) return e;
+    }
+    using Edge = void (*)(MicroArgs, const double*, const F*, const F*, const F*, SweepScratch<F>, int, int, int);
+    const Edge walk[2] = {k_sgs_edge<F, false>, k_sgs_edge<F, true>};
+    cudaError_t e = cudaSuccess;
+    for (int g = 0; g < 2; ++g)
+        if ((e = cudaFuncSetAttribute(walk[g], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esmem)) != cudaSuccess) return e;
+    // timing mode: an event pair around a launch, with the cell-velocity pairs it sweeps
+    auto timed = [&](double units, auto&& launch) {
+        SweepTimer* T = plan.timer;
+        if (!T) { launch(); return cudaGetLastError(); }
+        while ((int)T->ev.size() < 2 * (T->used + 1)) {
+            cudaEvent_t ev;
+            cudaError_t ce = cudaEventCreate(&ev);
+            if (ce != cudaSuccess) return ce;
+            T->ev.push_back(ev);
+        }
+        if ((int)T->units.size() <= T->used) T->units.resize(T->used + 1);
+        cudaError_t ce = cudaEventRecord(T->ev[2 * T->used], st);
+        if (ce != cudaSuccess) return ce;
+        launch();
+        if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+        if ((ce = cudaEventRecord(T->ev[2 * T->used + 1], st)) != cudaSuccess) return ce;
+        T->units[T->used] = units;
+        T->used++;
+        return cudaSuccess;
+    };
+    const int nd = m.L.nx + m.L.ny - 1;
+    for (int pass = 0; pass < 2; ++pass) {
+        walk[m.P.general[pass]]<<<2 * nchunk, 128, esmem, st>>>(m, Zw, invD, r, x, S, pass, 0, nchunk);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        // wavefront segments between the body lines' walks
+        int dd = 0, e0 = 0, ne = m.P.nl[pass];
+        for (int b = 0; b <= plan.nbrk[pass]; ++b) {
+            const int end = b < plan.nbrk[pass] ? plan.brk[pass][b].dd : nd;
+            double cells = 0.0;                        // cells on the segment's diagonals
+            for (int q = dd; q < end; ++q) {
+                const int d = pass == 0 ? q : nd - 1 - q;
+                cells += std::min(m.L.nx - 1, d) - std::max(0, d - (m.L.ny - 1)) + 1;
+            }
+            if ((e = timed(cells * m.V.nv, [&] {
+                    wave[pass]<<<nblk, 32 * nw, wsmem, st>>>(m, invD, r, x, S, dd, end, e0, ne);
+                })) != cudaSuccess)
+                return e;
+            dd = end;
+            if (b < plan.nbrk[pass]) {
+                const SweepBreak& k = plan.brk[pass][b];
+                walk[m.P.general[pass]]<<<k.nq * nchunk, 128, esmem, st>>>(m, Zw, invD, r, x, S, pass, 2 + k.q0, nchunk);
+                if ((e = cudaGetLastError()) != cudaSuccess) return e;
+                e0 = k.e0;
+                ne = k.ne;
+            }
+        }
+    }
+    return cudaSuccess;
+}
+template cudaError_t launch_micro_sgs<double>(const MicroArgs&, const SweepPlanHost&, const double*, const double*,
+                                              const double*, double*, double*, cudaStream_t);
+template cudaError_t launch_micro_sgs<float>(const MicroArgs&, const SweepPlanHost&, const double*, const float*,
+                                             const float*, float*, float*, cudaStream_t);
 
 // Sum of squares of n values (deterministic: fixed grid, fixed per-thread order,
 // fixed reduction tree), for the decisions of the adaptive multigrid cycle.
@@ -1254,212 +1105,6 @@ cudaError_t launch_sumsq(const T* a, size_t n, double* part, double* out, cudaSt
 template cudaError_t launch_sumsq<float>(const float*, size_t, double*, double*, cudaStream_t);
 template cudaError_t launch_sumsq<double>(const double*, size_t, double*, double*, cudaStream_t);
 
-// Coupling classes of one pass (0 forward, 1 backward) for the velocity nodes
-// (u_k, v_k): the wavefront blocks and the lists of the other velocities.
-void sweep_classes(const double* u, const double* v, int nv, int pass, std::vector<int>& wblk, std::vector<int>& lk,
-                   int& nrow, int& ncol, int& nelem)
-{
-    const int K = kInteriorKc, nblk = (nv + K - 1) / K;
-    auto cx = [&](int k) { return pass == 0 ? u[k] > 0.0 : u[k] < 0.0; };
-    auto cy = [&](int k) { return pass == 0 ? v[k] > 0.0 : v[k] < 0.0; };
-    std::vector<int> rows, cols, elem;
-    wblk.clear();
-    for (int b = 0; b < nblk; ++b) {
-        bool wave = false;
-        for (int k = b * K; k < std::min(nv, b * K + K); ++k) wave = wave || (cx(k) && cy(k));
-        if (wave) { wblk.push_back(b); continue; }
-        for (int k = b * K; k < std::min(nv, b * K + K); ++k)
-            (cx(k) ? rows : cy(k) ? cols : elem).push_back(k);
-    }
-    nrow = (int)rows.size(); ncol = (int)cols.size(); nelem = (int)elem.size();
-    lk = rows;
-    lk.insert(lk.end(), cols.begin(), cols.end());
-    lk.insert(lk.end(), elem.begin(), elem.end());
-}
-
-// sweep scratch (elements of the storage type): corner copy, wall densities of
-// the edge lines and the body lines, folded line inputs
-size_t micro_fold_offset(int nv, int nlines) { return ((2 * (size_t)nv + (2 + (size_t)nlines) * kMaxLine + 3) / 4) * 4; }
-size_t micro_scratch_elems(int nv, int nl, int nlines)
-{
-    return micro_fold_offset(nv, nlines) + (size_t)((nv + kInteriorKc - 1) / kInteriorKc) * nl * 3 * kInteriorKc;
-}
-
-template <typename F>
-cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, const double* Zw, const F* invD,
-                             const F* r, F* x, F* xcorner, cudaStream_t st)
-{
-    int nlines = 0;
-    for (int p = 0; p < 2; ++p)
-        for (int b = 0; b < plan.nbrk[p]; ++b)
-            nlines = std::max(nlines, plan.brk[p][b].q0 + plan.brk[p][b].nq);
-    F* rho_lines = xcorner + 2 * (size_t)m.V.nv;       // (2 + body lines) x kMaxLine wall densities
-    F* fold = xcorner + micro_fold_offset(m.V.nv, nlines);
-    const int ngroups = (m.V.nu + 1) / 2;
-    const int nloc = ((ngroups + kChainCluster - 1) / kChainCluster) * 2 * m.V.nvv;
-    if (nloc > kChainKptMax * kChainThreads) return cudaErrorInvalidValue;
-    if (m.L.nx > kMaxLine || m.L.ny > kMaxLine) return cudaErrorInvalidValue;
-    const int kpt = (nloc + kChainThreads - 1) / kChainThreads;
-    const size_t rslot = sizeof(F) * (size_t)(kpt <= 1 ? 1 : kpt <= 2 ? 2 : kpt <= 4 ? 4 : kpt <= 8 ? 8 : 16) * 3 *
-                         kChainThreads;
-    int RA = (int)((96 * 1024) / rslot);
-    RA = RA < 1 ? 1 : (RA > kWaveRingMax ? kWaveRingMax : RA);
-    size_t smem = sizeof(F) * 2 * nloc + (sizeof(F) + sizeof(int)) * (size_t)nloc + rslot * RA;
-    void (*chain)(MicroArgs, const double*, const F*, const F*, F*, const F*, F*, int, int) =
-        kpt <= 1 ? k_sgs_chain<F, 1> : kpt <= 2 ? k_sgs_chain<F, 2> : kpt <= 4 ? k_sgs_chain<F, 4>
-                 : kpt <= 8 ? k_sgs_chain<F, 8> : k_sgs_chain<F, 16>;
-    void (*chain_b)(MicroArgs, const double*, const F*, const F*, F*, F*, int, int, int) =
-        kpt <= 1 ? k_sgs_chain_body<F, 1> : kpt <= 2 ? k_sgs_chain_body<F, 2> : kpt <= 4 ? k_sgs_chain_body<F, 4>
-                 : kpt <= 8 ? k_sgs_chain_body<F, 8> : k_sgs_chain_body<F, 16>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        if (nlines > 0) {
-            e = cudaFuncSetAttribute(chain_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-    }
-    const int nblk = (m.V.nv + kInteriorKc - 1) / kInteriorKc;
-    const int maxdiag = m.L.nx < m.L.ny ? m.L.nx : m.L.ny;
-    const int nthr = ((maxdiag + 31) / 32) * 32;       // one thread per cell of the longest diagonal
-    const bool vec = (m.V.nv * sizeof(F)) % 16 == 0;
-    const size_t nl = (size_t)m.L.nx + m.L.ny;
-    const size_t fixed = sizeof(F) * (2 * (size_t)m.L.nx * 2 * kInteriorKc + nl);
-    const size_t slot = sizeof(F) * 3 * (size_t)nthr * kInteriorKc + sizeof(int) * (size_t)nthr;
-    constexpr size_t kSmemMax = 227 * 1024;
-    if (fixed + slot > kSmemMax) return cudaErrorInvalidValue;
-    const size_t rfit = (kSmemMax - fixed) / slot;
-    // On a large level the wavefront kernel takes only the blocks of velocities coupled in
-    // both directions and the line-class kernel the rest; on a small one the wavefront's
-    // dependency chain, not its traffic, sets the time and one wavefront launch over every
-    // block is faster than two launches.
-    const bool split = plan.split == 1 || (plan.split == 0 && (size_t)m.L.nc * m.V.nv >= kSweepSplitMinCv);
-    // Ring depth: the deepest of 8, 4, 2 stages whose shared memory lets the launch's CTAs
-    // be resident in the fewest rounds (a CTA's time is the dependency chain of its steps,
-    // so a second round of CTAs doubles the launch).
-    int R = rfit >= 8 ? 8 : rfit >= 4 ? 4 : rfit >= 2 ? 2 : 1;
-    {
-        static int nsm = 0, smem_sm = 0, resv = 0;
-        if (nsm == 0) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-            cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-            cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-        }
-        const long grid = split ? std::max(m.V.nwblk[0], m.V.nwblk[1]) : nblk;
-        auto rounds = [&](int r) -> long {
-            const long per = std::min<long>((long)smem_sm / (long)(fixed + slot * r + resv), 2048 / nthr);
-            return per > 0 ? (grid + per * nsm - 1) / (per * nsm) : LONG_MAX;
-        };
-        if (nsm > 0 && smem_sm > 0 && R >= 2) {
-            int best = R;
-            for (int r = R / 2; r >= 2; r /= 2)
-                if (rounds(r) < rounds(best)) best = r;
-            R = best;
-        }
-    }
-    void (*wave)(MicroArgs, const F*, const F*, F*, const F*, int, int, int, int);
-    if (m.P.bodies) {
-        if (vec) wave = R == 8 ? k_sgs_wave<F, 8, true, true> : R == 4 ? k_sgs_wave<F, 4, true, true> : R == 2 ? k_sgs_wave<F, 2, true, true> : k_sgs_wave<F, 1, true, true>;
-        else wave = R == 8 ? k_sgs_wave<F, 8, false, true> : R == 4 ? k_sgs_wave<F, 4, false, true> : R == 2 ? k_sgs_wave<F, 2, false, true> : k_sgs_wave<F, 1, false, true>;
-    } else {
-        if (vec) wave = R == 8 ? k_sgs_wave<F, 8, true, false> : R == 4 ? k_sgs_wave<F, 4, true, false> : R == 2 ? k_sgs_wave<F, 2, true, false> : k_sgs_wave<F, 1, true, false>;
-        else wave = R == 8 ? k_sgs_wave<F, 8, false, false> : R == 4 ? k_sgs_wave<F, 4, false, false> : R == 2 ? k_sgs_wave<F, 2, false, false> : k_sgs_wave<F, 1, false, false>;
-    }
-    const size_t wsmem = fixed + slot * R;
-    if (wsmem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(wave, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
-        if (e != cudaSuccess) return e;
-    }
-    void (*lines)(MicroArgs, const F*, const F*, F*, const F*, int, int, int, int, int, int) =
-        m.P.bodies ? k_sgs_lines<F, true> : k_sgs_lines<F, false>;
-    // one segment (split: see above)
-    // timing mode: an event pair around a launch, with the cell-velocity pairs it sweeps
-    auto timed = [&](int kind, double units, auto&& launch) {
-        SweepTimer* T = plan.timer;
-        if (!T) { launch(); return cudaGetLastError(); }
-        while ((int)T->ev.size() < 2 * (T->used + 1)) {
-            cudaEvent_t e;
-            cudaError_t ce = cudaEventCreate(&e);
-            if (ce != cudaSuccess) return ce;
-            T->ev.push_back(e);
-        }
-        if ((int)T->kind.size() <= T->used) { T->kind.resize(T->used + 1); T->units.resize(T->used + 1); }
-        cudaError_t e = cudaEventRecord(T->ev[2 * T->used], st);
-        if (e != cudaSuccess) return e;
-        launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(T->ev[2 * T->used + 1], st)) != cudaSuccess) return e;
-        T->kind[T->used] = kind;
-        T->units[T->used] = units;
-        T->used++;
-        return cudaSuccess;
-    };
-    auto segment = [&](int pass, int dd, int end) {
-        const int nw = split ? m.V.nwblk[pass] : nblk;
-        const int nbr = (m.V.nrow[pass] + 127) / 128, nbc = (m.V.ncol[pass] + 127) / 128;
-        const int nbe = pass == 0 ? (m.V.nelem[pass] + 127) / 128 : 0;
-        const int nb = split ? nbr * m.L.ny + nbc * m.L.nx + nbe * m.L.ny : 0;
-        double cells = 0.0;                            // cells on the segment's diagonals
-        for (int q = dd; q < end; ++q) {
-            const int d = pass == 0 ? q : m.L.nx + m.L.ny - 2 - q;
-            cells += std::min(m.L.nx - 1, d) - std::max(0, d - (m.L.ny - 1)) + 1;
-        }
-        const double kl = (double)m.V.nrow[pass] + m.V.ncol[pass] + (pass == 0 ? m.V.nelem[pass] : 0);
-        const double kw = std::min((double)nw * kInteriorKc, (double)m.V.nv);
-        cudaError_t e = cudaSuccess;
-        if (nb > 0 && (e = timed(1, cells * kl, [&] {
-                lines<<<nb, 128, 0, st>>>(m, invD, r, x, fold, pass, dd, end, nbr, nbc, nbe);
-            })) != cudaSuccess)
-            return e;
-        if (nw > 0 && (e = timed(0, cells * kw, [&] {
-                wave<<<nw, nthr, wsmem, st>>>(m, invD, r, x, fold, pass, dd, end, split ? 1 : 0);
-            })) != cudaSuccess)
-            return e;
-        return cudaSuccess;
-    };
-    auto fold_range = [&](int pass, int e0, int ne) {
-        const int n = nblk * ne * kInteriorKc;
-        if (n > 0) k_line_fold<F><<<(n + 255) / 256, 256, 0, st>>>(m, invD, r, x, rho_lines, fold, pass, e0, ne);
-        return cudaGetLastError();
-    };
-    const size_t nc = m.L.nc, nv = m.V.nv, corner = (size_t)m.L.nc - 1;
-    const int nd = m.L.nx + m.L.ny - 1;
-    for (int pass = 0; pass < 2; ++pass) {
-        if (pass == 1)
-            for (int cp = 0; cp < 2; ++cp) {
-                cudaError_t e = cudaMemcpyAsync(xcorner + cp * nv, x + (cp * nc + corner) * nv, nv * sizeof(F),
-                                                cudaMemcpyDeviceToDevice, st);
-                if (e != cudaSuccess) return e;
-            }
-        chain<<<2 * kChainCluster, kChainThreads, smem, st>>>(m, Zw, invD, r, x, xcorner, rho_lines, pass, RA);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        if ((e = fold_range(pass, 0, m.P.nl[pass])) != cudaSuccess) return e;
-        // wavefront segments between the body lines' walks
-        int dd = 0;
-        for (int b = 0; b <= plan.nbrk[pass]; ++b) {
-            const int end = b < plan.nbrk[pass] ? plan.brk[pass][b].dd : nd;
-            if (end > dd) {
-                if ((e = segment(pass, dd, end)) != cudaSuccess) return e;
-                dd = end;
-            }
-            if (b < plan.nbrk[pass]) {
-                const SweepBreak& k = plan.brk[pass][b];
-                chain_b<<<k.nq * kChainCluster, kChainThreads, smem, st>>>(m, Zw, invD, r, x, rho_lines, pass, k.q0, RA);
-                if ((e = cudaGetLastError()) != cudaSuccess) return e;
-                if ((e = fold_range(pass, k.e0, k.ne)) != cudaSuccess) return e;
-            }
-        }
-    }
-    return cudaSuccess;
-}
-template cudaError_t launch_micro_sgs<double>(const MicroArgs&, const SweepPlanHost&, const double*, const double*,
-                                              const double*, double*, double*, cudaStream_t);
-template cudaError_t launch_micro_sgs<float>(const MicroArgs&, const SweepPlanHost&, const double*, const float*,
-                                             const float*, float*, float*, cudaStream_t);
-
 // ---------------------------------------------------------------------------
 // r -= A x (full operator with every neighbour and ghost), acc += x
 template <typename F>
@@ -1469,7 +1114,7 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
     __shared__ double red[32 * 4];
     const LevelDev& L = M.L;
     const VelDev& Vg = M.V;
-    const int c = blockIdx.x, nx = L.nx, nv = Vg.nv, i = c % nx, j = c / nx;
+    const int c = blockIdx.x, nx = L.nx, nv = Vg.ld, i = c % nx, j = c / nx;   // rows with their padding
     const size_t nc = L.nc;
     const bool vec = sizeof(F) == 4 && (nv & 3) == 0;   // 16-byte accesses over four velocities
     if (acc) {
@@ -1511,7 +1156,7 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
     for (int b = 0; b < nb; ++b) nwall += M.bc[bf[b].bc].type == BC_WALL;
     if (nwall > 0) {
         Acc<F> sa[4];
-        for (int k = threadIdx.x; k < nv; k += blockDim.x)
+        for (int k = threadIdx.x; k < Vg.nv; k += blockDim.x)
             for (int b = 0; b < nb; ++b) {
                 if (M.bc[bf[b].bc].type != BC_WALL) continue;
                 F uo = bf[b].axis == 0 ? vu[k] : vv[k];
@@ -1612,7 +1257,7 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
     for (int cp = 0; cp < 2; ++cp) {
         const F* xb = x + cp * nc * nv;
         F* rb = r + cp * nc * nv;
-        for (int k = threadIdx.x; k < nv; k += blockDim.x) {
+        for (int k = threadIdx.x; k < Vg.nv; k += blockDim.x) {
             const F u = vu[k], v = vv[k];
             size_t id = (size_t)c * nv + k;
             F a = (itau + geomD_r<F>(rdxi, rdyj, u, v)) * xb[id];
@@ -1625,7 +1270,7 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
                 if (Db == F(0)) continue;
                 int ty = M.bc[bf[b].bc].type;
                 if (ty == BC_WALL)
-                    a += Db * (F)(M.Cw[(size_t)bf[b].bc * nv + k] * (cp == 0 ? 1.0 : kKint * M.bc[bf[b].bc].t / 4.0)) * rho[b];
+                    a += Db * (F)(M.Cw[(size_t)bf[b].bc * Vg.nv + k] * (cp == 0 ? 1.0 : kKint * M.bc[bf[b].bc].t / 4.0)) * rho[b];
                 else if (ty == BC_SYMMETRY) {
                     int aa = k / Vg.nvv, bb = k - aa * Vg.nvv;
                     int km = bf[b].axis == 0 ? (Vg.nu - 1 - aa) * Vg.nvv + bb : aa * Vg.nvv + (Vg.nvv - 1 - bb);
@@ -1659,10 +1304,10 @@ __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F
 {
     __shared__ double red[32 * 4];
     const int c = blockIdx.x, nv = Vg.nv;
-    const size_t nc = L.nc;
+    const size_t nc = L.nc, ld = Vg.ld;
     __shared__ F sUV[2];
-    F* fG = f + (size_t)c * nv;
-    F* fH = f + (nc + c) * (size_t)nv;
+    F* fG = f + (size_t)c * ld;
+    F* fH = f + (nc + c) * ld;
     const F* __restrict__ vu = VelT<F>::u(Vg);
     const F* __restrict__ vv = VelT<F>::v(Vg);
     const F* __restrict__ vw = VelT<F>::w(Vg);
@@ -1679,8 +1324,8 @@ __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F
             if (k < nv) {
                 g[q] = fG[k]; h[q] = fH[k];
                 if (df) {
-                    g[q] = g[q] + df[(size_t)c * nv + k];
-                    h[q] = h[q] + df[(nc + c) * (size_t)nv + k];
+                    g[q] = g[q] + df[(size_t)c * ld + k];
+                    h[q] = h[q] + df[(nc + c) * ld + k];
                 }
             }
         }
@@ -1709,7 +1354,7 @@ __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F
                     const int k = k0 + q * bs;
                     if (k < nv) {
                         g[q] = fG[k]; h[q] = fH[k];
-                        dg[q] = df[(size_t)c * nv + k]; dh[q] = df[(nc + c) * (size_t)nv + k];
+                        dg[q] = df[(size_t)c * ld + k]; dh[q] = df[(nc + c) * ld + k];
                     }
                 }
                 #pragma unroll
@@ -1793,13 +1438,13 @@ __global__ void __launch_bounds__(256) k_state_fallback(LevelDev L, VelDev Vg, i
 {
     __shared__ double red[32 * 4];
     const int c = blockIdx.x, nv = Vg.nv, i = c % L.nx, j = c / L.nx;
-    const size_t nc = L.nc, cc = (size_t)(j / 2) * ncx + i / 2;
+    const size_t nc = L.nc, ld = Vg.ld, cc = (size_t)(j / 2) * ncx + i / 2;
     const F* __restrict__ vu = VelT<F>::u(Vg);
     const F* __restrict__ vv = VelT<F>::v(Vg);
     const F* __restrict__ vw = VelT<F>::w(Vg);
     Acc<F> sa[4];
     for (int k = threadIdx.x; k < nv; k += blockDim.x) {
-        const F g = f[(size_t)c * nv + k], h = f[(nc + c) * (size_t)nv + k], u = vu[k], v = vv[k], w = vw[k];
+        const F g = f[(size_t)c * ld + k], h = f[(nc + c) * ld + k], u = vu[k], v = vv[k], w = vw[k];
         sa[0].add(w * g); sa[1].add(w * u * g); sa[2].add(w * v * g);
         sa[3].add(w * (F(0.5) * (u * u + v * v) * g + h));
     }
@@ -1807,8 +1452,8 @@ __global__ void __launch_bounds__(256) k_state_fallback(LevelDev L, VelDev Vg, i
     block_total<4>(sa, red, s);
     if (s[0] > 0.0 && s[3] * s[0] - 0.5 * (s[1] * s[1] + s[2] * s[2]) > 0.0) return;
     for (int k = threadIdx.x; k < nv; k += blockDim.x) {
-        f[(size_t)c * nv + k] = fc[cc * nv + k];
-        f[(nc + c) * (size_t)nv + k] = fc[(ncc + cc) * nv + k];
+        f[(size_t)c * ld + k] = fc[cc * ld + k];
+        f[(nc + c) * ld + k] = fc[(ncc + cc) * ld + k];
     }
 }
 template <typename F>
@@ -1831,7 +1476,7 @@ __global__ void k_init_maxwell(LevelDev L, VelDev Vg, const double* __restrict__
 {
     extern __shared__ double etab[];      // [nu] rho lam/pi e^{-lam (u_a - U)^2}, [nvv] e^{-lam (v_b - V)^2}
     const int c = blockIdx.x, nv = Vg.nv, nu = Vg.nu, nvv = Vg.nvv, tid = threadIdx.x, bs = blockDim.x;
-    const size_t nc = L.nc;
+    const size_t nc = L.nc, ld = Vg.ld;
     const double rho = prim[4 * c], U = prim[4 * c + 1], V = prim[4 * c + 2], lam = 1.0 / prim[4 * c + 3];
     const double hfac = kKint / (4.0 * lam);
     for (int e = tid; e < nu + nvv; e += bs) {
@@ -1850,8 +1495,8 @@ __global__ void k_init_maxwell(LevelDev L, VelDev Vg, const double* __restrict__
     for (int k = tid; k < nv; k += bs, a += sa, b += sb) {
         if (b >= nvv) { b -= nvv; ++a; }
         const double g = etab[a] * etab[nu + b];
-        f[(size_t)c * nv + k] = (F)g;
-        f[(nc + c) * (size_t)nv + k] = (F)(g * hfac);
+        f[(size_t)c * ld + k] = (F)g;
+        f[(nc + c) * ld + k] = (F)(g * hfac);
     }
 }
 template <typename F>
@@ -1873,7 +1518,7 @@ __global__ void k_wall_quantities(LevelDev L, VelDev Vg, const BcDev* __restrict
     const int code = faces[blockIdx.x];
     const int axis = code >> 30, fi = code & ((1 << 30) - 1);
     const int nx = L.nx, nv = Vg.nv;
-    const size_t nc = L.nc;
+    const size_t nc = L.nc, ld = Vg.ld;
     int i = axis == 0 ? fi % (nx + 1) : fi % nx, j = axis == 0 ? fi / (nx + 1) : fi / nx;
     int outsign, c;
     bface_side(L, axis, i, j, c, outsign);
@@ -1882,7 +1527,7 @@ __global__ void k_wall_quantities(LevelDev L, VelDev Vg, const BcDev* __restrict
     double s[2] = {0, 0};
     for (int k = threadIdx.x; k < nv; k += blockDim.x) {
         double uo = outsign * (axis == 0 ? Vg.u[k] : Vg.v[k]);
-        if (uo > 0) s[0] += Vg.w[k] * uo * (double)f[(size_t)c * nv + k];
+        if (uo > 0) s[0] += Vg.w[k] * uo * (double)f[(size_t)c * ld + k];
         else if (uo < 0) s[1] += Vg.w[k] * uo * Cb[k];
     }
     block_sum<2>(s, red);
@@ -1893,7 +1538,7 @@ __global__ void k_wall_quantities(LevelDev L, VelDev Vg, const BcDev* __restrict
         double u = Vg.u[k], v = Vg.v[k];
         double uo = outsign * (axis == 0 ? u : v), ut = axis == 0 ? v : u;
         double g, h;
-        if (uo >= 0) { g = f[(size_t)c * nv + k]; h = f[(nc + c) * (size_t)nv + k]; }
+        if (uo >= 0) { g = f[(size_t)c * ld + k]; h = f[(nc + c) * ld + k]; }
         else { g = rhow * Cb[k]; h = g * kKint * B.t / 4.0; }
         double du = u - B.u, dv = v - B.v;
         t[0] += Vg.w[k] * uo * uo * g;

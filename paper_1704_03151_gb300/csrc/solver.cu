@@ -57,11 +57,11 @@ struct miugks_solver {
     cudaStream_t st = nullptr;
     std::vector<void*> allocs;
     int L = 1, nu = 0, nvv = 0, nv = 0, nbc = 0;
+    int ld = 0;                             // row stride of the per-velocity arrays (VelDev::ld)
     double umax = 0, vmax = 0;
     GasDev gas{};
     std::vector<BcDev> bch;
     std::vector<double> uh, vh, wh, uah, vbh;
-    std::vector<float> ufh, vfh, wfh;
     VelDev vel{};
     BcDev* bc = nullptr;
     double *Cw = nullptr, *Zw = nullptr;
@@ -70,7 +70,9 @@ struct miugks_solver {
     // finest-level state (f, face fluxes and the corner scratch in the per-velocity type)
     bool mixed = false;
     size_t fsz = sizeof(double);
-    void *f = nullptr, *phx = nullptr, *phy = nullptr, *xcorner = nullptr;
+    void *f = nullptr, *phx = nullptr, *phy = nullptr, *scratch = nullptr;
+    int* line_count = nullptr;
+    int sw_nl = 0, sw_nlines = 0, sw_nchunk = 1;   // layout of the sweep scratch
     double* fgeo[2] = {nullptr, nullptr};   // finest level: mesh constants of the interface flux per face
     double *W = nullptr, *q = nullptr, *R = nullptr, *Fx = nullptr, *Fy = nullptr;
     double *rms_part = nullptr, *rms_out = nullptr;
@@ -83,13 +85,12 @@ struct miugks_solver {
     long adapt_n = 0;
     std::vector<unsigned char> adapt_log = std::vector<unsigned char>(4096);
     double* nrm = nullptr;                      // device: 128 partial sums and the total
-    int sweep_split = 0;                        // evolution sweep: 0 by size, 1 split by coupling class, 2 never
     bool shock = false;                         // pressure-jump collision time at interior faces
     unsigned long long wait_ns = 200000000ull;  // bound of the prediction sweep's device waits
-    // timing mode: the finest level's wavefront and line-class sweep launches; totals since the last read
+    // timing mode: the finest level's wavefront launches; totals since the last read
     SweepTimer sweep_timer;
-    double t_sweepk[2] = {0, 0}, u_sweepk[2] = {0, 0};
-    long n_sweepk[2] = {0, 0};
+    double t_sweepk = 0, u_sweepk = 0;
+    long n_sweepk = 0;
     bool initialised = false;
     bool timing = false;
     cudaEvent_t ev[6] = {};
@@ -204,10 +205,13 @@ std::vector<double> flux_face_geometry(const HLevel& L, int axis, double cfl, do
 }
 
 // per-velocity array of count elements of the solver's storage type
+// (zeroed: the padding of the rows of velocities is zero and stays so)
 miugks_status falloc(miugks_solver* s, void** p, size_t count)
 {
-    if (s->mixed) return dalloc(s, (float**)p, count);
-    return dalloc(s, (double**)p, count);
+    if (s->mixed) ST(dalloc(s, (float**)p, count));
+    else ST(dalloc(s, (double**)p, count));
+    if (s->ld != s->nv) CK(cudaMemsetAsync(*p, 0, count * s->fsz, s->st));
+    return MIUGKS_OK;
 }
 
 template <typename T>
@@ -342,7 +346,7 @@ miugks_status upload_level(miugks_solver* s, HLevel& Lv)
     ST(upload(s, &ubcd, ubc));
     Lv.dev = LevelDev{Lv.nx, Lv.ny, Lv.nc, Lv.nfx, Lv.nfy, xn, yn, xc, yc, dx, dy, fbx, fby, rdx, rdy, solid,
                       ubcd, (int)ubc.size()};
-    size_t n4 = 4 * (size_t)Lv.nc, nf = 2 * (size_t)Lv.nc * s->nv;
+    size_t n4 = 4 * (size_t)Lv.nc, nf = 2 * (size_t)Lv.nc * s->ld;
     ST(dalloc(s, &Lv.Wn, n4)); ST(dalloc(s, &Lv.Wc, n4)); ST(dalloc(s, &Lv.Rc, n4)); ST(dalloc(s, &Lv.P, n4));
     ST(dalloc(s, &Lv.R, n4)); ST(dalloc(s, &Lv.dW, n4)); ST(dalloc(s, &Lv.Wt, n4));
     ST(dalloc(s, &Lv.gx, (size_t)Lv.nfx)); ST(dalloc(s, &Lv.gy, (size_t)Lv.nfy));
@@ -352,20 +356,20 @@ miugks_status upload_level(miugks_solver* s, HLevel& Lv)
     Lv.ghost = Lv.T + nrec;
     Lv.Wd = Lv.ghost + ngh;
     ST(falloc(s, &Lv.r, nf)); ST(falloc(s, &Lv.df, nf)); ST(falloc(s, &Lv.dl, nf));
-    ST(falloc(s, &Lv.invD, (size_t)Lv.nc * s->nv)); ST(dalloc(s, &Lv.inv_tau, (size_t)Lv.nc));
+    ST(falloc(s, &Lv.invD, (size_t)Lv.nc * s->ld)); ST(dalloc(s, &Lv.inv_tau, (size_t)Lv.nc));
     return MIUGKS_OK;
 }
 
 MicroArgs micro_args(miugks_solver* s, int l)
 {
-    return MicroArgs{s->lev[l].dev, s->vel, s->bc, s->Cw, s->lev[l].inv_tau, s->lev[l].plan};
+    return MicroArgs{s->lev[l].dev, s->vel, s->bc, s->Cw, s->lev[l].inv_tau, s->lev[l].plan, s->rms_out + 5};
 }
 
 SweepPlanHost sweep_plan(const miugks_solver* s, const HLevel& Lv)
 {
     SweepPlanHost h{};
     for (int p = 0; p < 2; ++p) { h.brk[p] = Lv.brk[p].data(); h.nbrk[p] = (int)Lv.brk[p].size(); }
-    h.split = s->sweep_split;
+    h.nl = s->sw_nl; h.nlines = s->sw_nlines; h.nchunk = s->sw_nchunk; h.count = s->line_count;
     h.timer = s->timing && &Lv == &s->lev[0] ? const_cast<SweepTimer*>(&s->sweep_timer) : nullptr;
     return h;
 }
@@ -393,14 +397,14 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
         for (int st = 0; st < ny; ++st) {
             int i = ie, j = je + sg * st, c = j * nx + i;
             if (Lv.solid[c]) return fail(s, MIUGKS_EINVAL, "level with %dx%d cells: the cells on the domain edge must be fluid", nx, ny);
-            lcell.insert(lcell.end(), {c, 0, st, st == 0});
-            code[c] = (st << 2) | 2 | (st == 0 ? 1 : 0);
+            lcell.insert(lcell.end(), {c, 0, Lv.fbx[j * (nx + 1) + i + p], st == 0});
+            code[c] = st;
         }
         for (int st = 0; st < nx; ++st) {
             int i = ie + sg * st, j = je, c = j * nx + i;
             if (Lv.solid[c]) return fail(s, MIUGKS_EINVAL, "level with %dx%d cells: the cells on the domain edge must be fluid", nx, ny);
-            lcell.insert(lcell.end(), {c, 1, kMaxLine + st, st == 0});
-            if (st > 0) code[c] = ((ny + st) << 2) | 1;
+            lcell.insert(lcell.end(), {c, 1, Lv.fby[(j + p) * nx + i], st == 0});
+            if (st > 0) code[c] = ny + st;
         }
         Lv.plan.nl[p] = nx + ny;
         // every other fluid cell: at most one sweep-side boundary face
@@ -440,16 +444,27 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
         }
         std::stable_sort(runs.begin(), runs.end(), [](const Run& x, const Run& y) { return x.dd < y.dd; });
         if ((int)runs.size() > kMaxBodyLines) return fail(s, MIUGKS_EINVAL, "too many body lines (%d > %d)", (int)runs.size(), kMaxBodyLines);
-        std::vector<int> lines;
+        // the line's faces on the sweep side: does one belong to a symmetry plane
+        auto has_sym = [&](int i, int j, int di, int dj, int first, int len, int axis) {
+            for (int st = first; st < len; ++st) {
+                const int a = i + st * di, b = j + st * dj;
+                const int id = axis == 0 ? Lv.fbx[b * (nx + 1) + a + p] : Lv.fby[(b + p) * nx + a];
+                if (id >= 0 && s->bch[id].type == MIUGKS_BC_SYMMETRY) return 1;
+            }
+            return 0;
+        };
+        std::vector<int> lines = {ie, je, 0, sg, ny, 0, 0, has_sym(ie, je, 0, sg, 0, ny, 0),
+                                  ie, je, sg, 0, nx, 1, ny, has_sym(ie, je, sg, 0, 0, nx, 1)};
         Lv.brk[p].clear();
         for (int q = 0; q < (int)runs.size(); ++q) {
             const Run& R = runs[q];
-            const int slot = (2 + q) * kMaxLine, e0 = (int)lcell.size() / 4;
-            lines.insert(lines.end(), {R.i0, R.j0, R.di, R.dj, R.len, R.axis, slot, 0});
+            const int e0 = (int)lcell.size() / 4;
+            lines.insert(lines.end(), {R.i0, R.j0, R.di, R.dj, R.len, R.axis, e0 - 1,
+                                       has_sym(R.i0, R.j0, R.di, R.dj, 1, R.len, R.axis)});
             for (int st = 1; st < R.len; ++st) {
                 int i = R.i0 + st * R.di, j = R.j0 + st * R.dj, c = j * nx + i;
-                code[c] = (((int)lcell.size() / 4) << 2) | (R.axis == 0 ? 2 : 1);
-                lcell.insert(lcell.end(), {c, R.axis, slot + st, 0});
+                code[c] = (int)lcell.size() / 4;
+                lcell.insert(lcell.end(), {c, R.axis, R.axis == 0 ? Lv.fbx[j * (nx + 1) + i + p] : Lv.fby[(j + p) * nx + i], 0});
             }
             const int ne = (int)lcell.size() / 4 - e0;
             if (!Lv.brk[p].empty() && Lv.brk[p].back().dd == R.dd) {
@@ -463,15 +478,24 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
         nl_max = std::max(nl_max, (int)lcell.size() / 4);
         int* dcode;
         int4* dl;
-        int* dlines = nullptr;
+        int* dlines;
         ST(upload(s, &dcode, code));
         std::vector<int4> l4(lcell.size() / 4);
         for (size_t e = 0; e < l4.size(); ++e) l4[e] = make_int4(lcell[4 * e], lcell[4 * e + 1], lcell[4 * e + 2], lcell[4 * e + 3]);
         ST(upload(s, &dl, l4));
-        if (!lines.empty()) ST(upload(s, &dlines, lines));
+        ST(upload(s, &dlines, lines));
         Lv.plan.code[p] = dcode;
         Lv.plan.lcell[p] = dl;
         Lv.plan.lines[p] = dlines;
+        Lv.plan.sym[p] = lines[7] | lines[15] << 1;
+        Lv.plan.cbc[p][0] = Lv.fbx[je * (nx + 1) + ie + p];
+        Lv.plan.cbc[p][1] = Lv.fby[(je + p) * nx + ie];
+        Lv.plan.general[p] = 0;
+        for (size_t q = 7; q < lines.size(); q += 8) Lv.plan.general[p] |= lines[q];
+        for (int f = 0; f < 2; ++f) {
+            const int type = s->bch[Lv.plan.cbc[p][f]].type;
+            Lv.plan.general[p] |= type == MIUGKS_BC_SYMMETRY || type == MIUGKS_BC_OUTFLOW;
+        }
     }
     Lv.plan.nl_max = nl_max;
     Lv.plan.bodies = Lv.nfluid != Lv.nc;
@@ -659,8 +683,8 @@ miugks_status cs(miugks_solver* s, int l, int type)
 {
     HLevel& Lv = s->lev[l];
     MicroArgs mi = micro_args(s, l);
-    size_t n = 2 * (size_t)Lv.nc * s->nv;
-    F *r = (F*)Lv.r, *df = (F*)Lv.df, *dl = (F*)Lv.dl, *invD = (F*)Lv.invD, *xc = (F*)s->xcorner;
+    size_t n = 2 * (size_t)Lv.nc * s->ld;
+    F *r = (F*)Lv.r, *df = (F*)Lv.df, *dl = (F*)Lv.dl, *invD = (F*)Lv.invD, *xc = (F*)s->scratch;
     CK(cudaMemsetAsync(df, 0, n * sizeof(F), s->st));
     const bool coarsest = l == s->L - 1;
     const int npre = coarsest ? (s->L == 1 ? 1 : s->opts.nu_coarse) : s->opts.nu1;
@@ -671,8 +695,8 @@ miugks_status cs(miugks_solver* s, int l, int type)
         if (last) return MIUGKS_OK;
     }
     HLevel& Cv = s->lev[l + 1];
-    const size_t nC = 2 * (size_t)Cv.nc * s->nv;
-    CK(launch_restrict<F>(Lv.dev, Cv.dev, s->nv, 2, r, (F*)Cv.r, s->st));
+    const size_t nC = 2 * (size_t)Cv.nc * s->ld;
+    CK(launch_restrict<F>(Lv.dev, Cv.dev, s->ld, 2, r, (F*)Cv.r, s->st));
     if (type != 0) CK(cudaMemcpyAsync(Cv.r0, Cv.r, nC * sizeof(F), cudaMemcpyDeviceToDevice, s->st));
     ST(cs<F>(s, l + 1, type));
     if (type == 3) {
@@ -700,7 +724,7 @@ miugks_status cs(miugks_solver* s, int l, int type)
         ST(cs<F>(s, l + 1, type == 1 ? 1 : 0));
         CK(launch_micro_renew<F>(mc, s->Zw, (F*)Cv.acc, (F*)Cv.r, (F*)Cv.df, 0, s->st)); // df_H += first correction
     }
-    CK(launch_prolong_add<F>(Lv.dev, Cv.dev, s->nv, 2, Lv.pidx, Lv.pw, (F*)Cv.df, df, dl, s->st));
+    CK(launch_prolong_add<F>(Lv.dev, Cv.dev, s->ld, 2, Lv.pidx, Lv.pw, (F*)Cv.df, df, dl, s->st));
     for (int m = 0; m < s->opts.nu2; ++m) {
         CK(launch_micro_renew<F>(mi, s->Zw, dl, r, nullptr, 1, s->st));
         CK(launch_micro_sgs<F>(mi, sweep_plan(s, Lv), s->Zw, invD, r, dl, xc, s->st));
@@ -765,7 +789,7 @@ miugks_status read_residual(miugks_solver* s, double res_out[4])
     CK(cudaMemcpyAsync(h, s->rms_out, sizeof h, cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
     if (res_out) memcpy(res_out, h, 4 * sizeof(double));
-    if (h[5] != 0.0) return fail(s, MIUGKS_ETIMEOUT, "a bounded wait of the macro sweep gave up at iteration %d", s->iter);
+    if (h[5] != 0.0) return fail(s, MIUGKS_ETIMEOUT, "a bounded wait of a sweep gave up at iteration %d", s->iter);
     bool bad = h[4] > 0;
     for (int m = 0; m < 4; ++m) bad = bad || !std::isfinite(h[m]);
     if (bad) return fail(s, MIUGKS_EDIVERGED, "diverged at iteration %d (%.0f unphysical cells)", s->iter, h[4]);
@@ -800,10 +824,57 @@ miugks_status to_host(miugks_solver* s, double* dst, const void* src, size_t n)
     return MIUGKS_OK;
 }
 
+// the same for rows of nv velocities, kept on the device at a stride of ld
+miugks_status rows_to_device(miugks_solver* s, void* dst, const double* src, size_t rows)
+{
+    const size_t nv = s->nv, ld = s->ld;
+    if (nv == ld) return to_device(s, dst, src, rows * nv);
+    if (!s->mixed) {
+        CK(cudaMemcpy2DAsync(dst, ld * sizeof(double), src, nv * sizeof(double), nv * sizeof(double), rows,
+                             cudaMemcpyHostToDevice, s->st));
+        CK(cudaStreamSynchronize(s->st));
+        return MIUGKS_OK;
+    }
+    std::vector<float> h(rows * ld, 0.0f);
+    for (size_t q = 0; q < rows; ++q)
+        for (size_t k = 0; k < nv; ++k) h[q * ld + k] = (float)src[q * nv + k];
+    CK(cudaMemcpyAsync(dst, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, s->st));
+    CK(cudaStreamSynchronize(s->st));
+    return MIUGKS_OK;
+}
+
+miugks_status rows_to_host(miugks_solver* s, double* dst, const void* src, size_t rows)
+{
+    const size_t nv = s->nv, ld = s->ld;
+    if (nv == ld) return to_host(s, dst, src, rows * nv);
+    if (!s->mixed) {
+        CK(cudaMemcpy2DAsync(dst, nv * sizeof(double), src, ld * sizeof(double), nv * sizeof(double), rows,
+                             cudaMemcpyDeviceToHost, s->st));
+        CK(cudaStreamSynchronize(s->st));
+        return MIUGKS_OK;
+    }
+    std::vector<float> h(rows * ld);
+    CK(cudaMemcpyAsync(h.data(), src, h.size() * sizeof(float), cudaMemcpyDeviceToHost, s->st));
+    CK(cudaStreamSynchronize(s->st));
+    for (size_t q = 0; q < rows; ++q)
+        for (size_t k = 0; k < nv; ++k) dst[q * nv + k] = h[q * ld + k];
+    return MIUGKS_OK;
+}
+
 miugks_status moments_now(miugks_solver* s)
 {
     if (s->mixed) CK(launch_moments<float>(s->lev[0].dev, s->vel, (const float*)s->f, s->W, s->q, s->st));
     else CK(launch_moments<double>(s->lev[0].dev, s->vel, (const double*)s->f, s->W, s->q, s->st));
+    return MIUGKS_OK;
+}
+
+// did a bounded wait of a sweep give up (waits for the stream)
+miugks_status sweep_status(miugks_solver* s)
+{
+    double flag = 0.0;
+    CK(cudaMemcpyAsync(&flag, s->rms_out + 5, sizeof flag, cudaMemcpyDeviceToHost, s->st));
+    CK(cudaStreamSynchronize(s->st));
+    if (flag != 0.0) return fail(s, MIUGKS_ETIMEOUT, "a bounded wait of a sweep gave up");
     return MIUGKS_OK;
 }
 
@@ -823,7 +894,7 @@ __global__ void k_invD_from_itau(LevelDev L, VelDev Vg, const double* it, F* inv
     int c = blockIdx.x, i = c % L.nx, j = c / L.nx;
     for (int k = threadIdx.x; k < Vg.nv; k += blockDim.x) {
         double g = fabs(Vg.u[k]) * L.rdx[i] + fabs(Vg.v[k]) * L.rdy[j];
-        invD[(size_t)c * Vg.nv + k] = (F)(1.0 / (it[c] + g));
+        invD[(size_t)c * Vg.ld + k] = (F)(1.0 / (it[c] + g));
     }
 }
 } // namespace
@@ -890,6 +961,7 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
             break;
         }
         s->nu = vg->nu; s->nvv = vg->nv; s->nv = vg->nu * vg->nv;
+        s->ld = (s->nv + 15) / 16 * 16;
         s->uah = ua; s->vbh = vb;
         s->uh.resize(s->nv); s->vh.resize(s->nv); s->wh.resize(s->nv);
         for (int a = 0; a < s->nu; ++a)
@@ -990,27 +1062,27 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
         if (nloc > 8 * 256) { st = bad("velocity grid too large for the boundary-line kernel (%d local > 2048)", nloc); break; }
         // device data (on the caller's stream, or the legacy default stream when none is given)
         upload_series_coefficients();
-        if ((st = upload(s, (double**)&s->vel.u, s->uh)) != MIUGKS_OK) break;
-        if ((st = upload(s, (double**)&s->vel.v, s->vh)) != MIUGKS_OK) break;
-        if ((st = upload(s, (double**)&s->vel.w, s->wh)) != MIUGKS_OK) break;
+        {
+            auto pad = [&](const std::vector<double>& h) { std::vector<double> p(h); p.resize(s->ld, 0.0); return p; };
+            auto single = [](const std::vector<double>& h) { return std::vector<float>(h.begin(), h.end()); };
+            const std::vector<double> pu = pad(s->uh), pv = pad(s->vh), pw = pad(s->wh);
+            if ((st = upload(s, (double**)&s->vel.u, pu)) != MIUGKS_OK) break;
+            if ((st = upload(s, (double**)&s->vel.v, pv)) != MIUGKS_OK) break;
+            if ((st = upload(s, (double**)&s->vel.w, pw)) != MIUGKS_OK) break;
+            if ((st = upload(s, (float**)&s->vel.uf, single(pu))) != MIUGKS_OK) break;
+            if ((st = upload(s, (float**)&s->vel.vf, single(pv))) != MIUGKS_OK) break;
+            if ((st = upload(s, (float**)&s->vel.wf, single(pw))) != MIUGKS_OK) break;
+            if (cudaStreamSynchronize(s->st) != cudaSuccess) { st = fail(s, MIUGKS_ECUDA, "velocity tables"); break; }
+        }
         if ((st = upload(s, (double**)&s->vel.ua, s->uah)) != MIUGKS_OK) break;
         if ((st = upload(s, (double**)&s->vel.vb, s->vbh)) != MIUGKS_OK) break;
-        s->ufh.assign(s->uh.begin(), s->uh.end());
-        s->vfh.assign(s->vh.begin(), s->vh.end());
-        s->wfh.assign(s->wh.begin(), s->wh.end());
-        if ((st = upload(s, (float**)&s->vel.uf, s->ufh)) != MIUGKS_OK) break;
-        if ((st = upload(s, (float**)&s->vel.vf, s->vfh)) != MIUGKS_OK) break;
-        if ((st = upload(s, (float**)&s->vel.wf, s->wfh)) != MIUGKS_OK) break;
         s->vel.nu = s->nu; s->vel.nvv = s->nvv; s->vel.nv = s->nv; s->vel.umax = s->umax; s->vel.vmax = s->vmax;
-        for (int p = 0; p < 2 && st == MIUGKS_OK; ++p) {
-            std::vector<int> wb, lk;
-            sweep_classes(s->uh.data(), s->vh.data(), s->nv, p, wb, lk, s->vel.nrow[p], s->vel.ncol[p], s->vel.nelem[p]);
-            s->vel.nwblk[p] = (int)wb.size();
-            if (wb.empty()) wb.push_back(0);        // keep a valid pointer
-            if (lk.empty()) lk.push_back(0);
-            if ((st = upload(s, (int**)&s->vel.wblk[p], wb)) != MIUGKS_OK) break;
-            st = upload(s, (int**)&s->vel.lk[p], lk);
-        }
+        s->vel.ld = s->ld;
+        for (int p = 0; p < 2; ++p)
+            for (int a = 0; a < 2; ++a) {
+                const std::vector<double>& n = a == 0 ? ua : vb;
+                s->vel.nleave[p][a] = (int)std::count_if(n.begin(), n.end(), [&](double z) { return p == 0 ? z < 0.0 : z > 0.0; });
+            }
         if (st != MIUGKS_OK) break;
         if ((st = upload(s, &s->bc, s->bch)) != MIUGKS_OK) break;
         s->Cwh.assign((size_t)n_bcs * s->nv, 0.0);
@@ -1040,7 +1112,7 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
             st = upload(s, &F.pw, w);
         }
         if (st != MIUGKS_OK) break;
-        size_t nc = L0.nc, nv = s->nv;
+        size_t nc = L0.nc, nv = s->ld;
         if ((st = falloc(s, &s->f, 2 * nc * nv)) != MIUGKS_OK) break;
         if ((st = dalloc(s, &s->W, 4 * nc)) != MIUGKS_OK) break;
         if ((st = dalloc(s, &s->q, 2 * nc)) != MIUGKS_OK) break;
@@ -1055,14 +1127,16 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
         if ((st = dalloc(s, &s->rms_out, 8)) != MIUGKS_OK) break;
         if ((st = dalloc(s, &s->nrm, 129)) != MIUGKS_OK) break;
         if (cudaMemset(s->rms_out, 0, 8 * sizeof(double)) != cudaSuccess) { st = fail(s, MIUGKS_ECUDA, "cudaMemset"); break; }
-        {
-            int nlines = 0, nlm = 0;
-            for (int l = 0; l < s->L; ++l) {
-                nlines = std::max(nlines, s->lev[l].nlines);
-                nlm = std::max(nlm, s->lev[l].plan.nl_max);
-            }
-            if ((st = falloc(s, &s->xcorner, micro_scratch_elems(nv, nlm, nlines))) != MIUGKS_OK) break;
+        for (int l = 0; l < s->L; ++l) {
+            s->sw_nlines = std::max(s->sw_nlines, s->lev[l].nlines);
+            s->sw_nl = std::max(s->sw_nl, s->lev[l].plan.nl_max);
         }
+        s->sw_nchunk = micro_edge_chunks(s->vel);
+        bool any_sym = false;
+        for (const BcDev& B : s->bch) any_sym = any_sym || B.type == MIUGKS_BC_SYMMETRY;
+        if ((st = falloc(s, &s->scratch, micro_scratch_elems(s->ld, s->sw_nl, s->sw_nlines, s->sw_nchunk, any_sym))) != MIUGKS_OK) break;
+        if ((st = dalloc(s, &s->line_count, 2 + (size_t)s->sw_nlines)) != MIUGKS_OK) break;
+        if (cudaMemsetAsync(s->line_count, 0, (2 + (size_t)s->sw_nlines) * sizeof(int), s->st) != cudaSuccess) { st = fail(s, MIUGKS_ECUDA, "cudaMemset"); break; }
         // smallest interior physical time step (for the numerical time step)
         s->dtp_min = 1e300;
         for (int i = 1; i < L0.nx; ++i) s->dtp_min = std::fmin(s->dtp_min, opts->cfl * std::fmin(L0.dx[i - 1], L0.dx[i]) / s->umax);
@@ -1166,9 +1240,9 @@ static miugks_status enqueue_iterations(miugks_solver* s, int n_iter)
                 for (int q = 0; q < T.used; ++q) {
                     float t = 0;
                     CK(cudaEventElapsedTime(&t, T.ev[2 * q], T.ev[2 * q + 1]));
-                    s->t_sweepk[T.kind[q]] += t;
-                    s->u_sweepk[T.kind[q]] += T.units[q];
-                    s->n_sweepk[T.kind[q]]++;
+                    s->t_sweepk += t;
+                    s->u_sweepk += T.units[q];
+                    s->n_sweepk++;
                 }
                 T.used = 0;
             }
@@ -1257,13 +1331,13 @@ miugks_status miugks_get_macro(miugks_solver* s, double* rho, double* u, double*
 miugks_status miugks_get_f(miugks_solver* s, double* f)
 {
     if (!s || !f) return MIUGKS_EINVAL;
-    return to_host(s, f, s->f, 2 * (size_t)s->lev[0].nc * s->nv);
+    return rows_to_host(s, f, s->f, 2 * (size_t)s->lev[0].nc);
 }
 
 miugks_status miugks_set_f(miugks_solver* s, const double* f)
 {
     if (!s || !f) return MIUGKS_EINVAL;
-    ST(to_device(s, s->f, f, 2 * (size_t)s->lev[0].nc * s->nv));
+    ST(rows_to_device(s, s->f, f, 2 * (size_t)s->lev[0].nc));
     ST(moments_now(s));
     CK(cudaStreamSynchronize(s->st));
     s->initialised = true;
@@ -1305,14 +1379,14 @@ miugks_status miugks_init_from_coarse(miugks_solver* s, const miugks_solver* c)
         if (std::fabs(C0.yn[j] - F1.yn[j]) > 1e-12 * (1.0 + std::fabs(F1.yn[j])))
             return fail(s, MIUGKS_EINVAL, "init_from_coarse: y nodes differ");
     HLevel& L0 = s->lev[0];
-    const size_t n = 2 * (size_t)L0.nc * s->nv;
+    const size_t n = 2 * (size_t)L0.nc * s->ld;
     CK(cudaStreamSynchronize(c->st));                      // the coarse state is complete
     CK(cudaMemsetAsync(s->f, 0, n * s->fsz, s->st));
     if (s->mixed)
-        CK(launch_prolong_add<float>(L0.dev, F1.dev, s->nv, 2, L0.sidx, L0.sw, (const float*)c->f, (float*)s->f,
+        CK(launch_prolong_add<float>(L0.dev, F1.dev, s->ld, 2, L0.sidx, L0.sw, (const float*)c->f, (float*)s->f,
                                      (float*)nullptr, s->st));
     else
-        CK(launch_prolong_add<double>(L0.dev, F1.dev, s->nv, 2, L0.sidx, L0.sw, (const double*)c->f, (double*)s->f,
+        CK(launch_prolong_add<double>(L0.dev, F1.dev, s->ld, 2, L0.sidx, L0.sw, (const double*)c->f, (double*)s->f,
                                       (double*)nullptr, s->st));
     // cells whose prolonged state is unphysical take their coarse cell's f
     if (s->mixed)
@@ -1343,7 +1417,7 @@ miugks_status miugks_copy_state(miugks_solver* s, const miugks_solver* src)
         if (s->uh[k] != src->uh[k] || s->vh[k] != src->vh[k] || s->wh[k] != src->wh[k])
             return fail(s, MIUGKS_EINVAL, "copy_state: velocity grids differ");
     if (!src->initialised) return fail(s, MIUGKS_ESTATE, "copy_state: the source solver has no state");
-    const size_t n = 2 * (size_t)A.nc * s->nv;
+    const size_t n = 2 * (size_t)A.nc * s->ld;
     CK(cudaStreamSynchronize(src->st));                    // the source state is complete
     if (s->mixed == src->mixed) CK(cudaMemcpyAsync(s->f, src->f, n * s->fsz, cudaMemcpyDeviceToDevice, s->st));
     else if (!s->mixed) CK(launch_to_double<float>((const float*)src->f, (double*)s->f, n, s->st));
@@ -1362,7 +1436,7 @@ miugks_status miugks_set_cycle(miugks_solver* s, int type)
     if (type != 0)
         for (int l = 1; l < s->L; ++l) {
             HLevel& Cv = s->lev[l];
-            const size_t n = 2 * (size_t)Cv.nc * s->nv;
+            const size_t n = 2 * (size_t)Cv.nc * s->ld;
             if (!Cv.r0) ST(falloc(s, &Cv.r0, n));
             if (!Cv.acc) ST(falloc(s, &Cv.acc, n));
         }
@@ -1382,16 +1456,7 @@ miugks_status miugks_set_sweep_split(miugks_solver* s, int mode)
 {
     if (!s) return MIUGKS_EINVAL;
     if (mode < 0 || mode > 2) return fail(s, MIUGKS_EINVAL, "sweep split mode %d: 0 by size, 1 always, 2 never", mode);
-    if (mode != s->sweep_split && s->gexec) {
-        // the captured iteration holds the old launch sequence
-        CK(cudaStreamSynchronize(s->st));
-        cudaGraphExecDestroy(s->gexec);
-        if (s->graph) cudaGraphDestroy(s->graph);
-        s->gexec = nullptr;
-        s->graph = nullptr;
-    }
-    s->sweep_split = mode;
-    return MIUGKS_OK;
+    return MIUGKS_OK;                          // one layout serves every size
 }
 
 miugks_status miugks_set_wait_limit(miugks_solver* s, double seconds)
@@ -1511,13 +1576,13 @@ miugks_status miugks_macro_sweep_times(miugks_solver* s, double* ms, int* launch
 miugks_status miugks_sweep_kernel_times(miugks_solver* s, double out[6])
 {
     if (!s || !out) return MIUGKS_EINVAL;
-    for (int k = 0; k < 2; ++k) {
-        out[3 * k] = s->timing ? s->t_sweepk[k] : -1.0;
-        out[3 * k + 1] = s->timing ? (double)s->n_sweepk[k] : 0.0;
-        out[3 * k + 2] = s->timing ? s->u_sweepk[k] : 0.0;
-        s->t_sweepk[k] = s->u_sweepk[k] = 0.0;
-        s->n_sweepk[k] = 0;
-    }
+    out[0] = s->timing ? s->t_sweepk : -1.0;
+    out[1] = s->timing ? (double)s->n_sweepk : 0.0;
+    out[2] = s->timing ? s->u_sweepk : 0.0;
+    out[3] = s->timing ? 0.0 : -1.0;
+    out[4] = out[5] = 0.0;
+    s->t_sweepk = s->u_sweepk = 0.0;
+    s->n_sweepk = 0;
     return MIUGKS_OK;
 }
 
@@ -1540,8 +1605,8 @@ miugks_status miugks_stage_flux(miugks_solver* s, double* R, double* phx, double
     HLevel& L0 = s->lev[0];
     if (R) CK(cudaMemcpyAsync(R, s->R, 4 * (size_t)L0.nc * sizeof(double), cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
-    if (phx) ST(to_host(s, phx, s->phx, 2 * (size_t)L0.nfx * s->nv));
-    if (phy) ST(to_host(s, phy, s->phy, 2 * (size_t)L0.nfy * s->nv));
+    if (phx) ST(rows_to_host(s, phx, s->phx, 2 * (size_t)L0.nfx));
+    if (phy) ST(rows_to_host(s, phy, s->phy, 2 * (size_t)L0.nfy));
     return MIUGKS_OK;
 }
 
@@ -1550,37 +1615,37 @@ miugks_status miugks_stage_sgs_micro(miugks_solver* s, int lev, const double* in
 {
     ST(check_level(s, lev));
     HLevel& Lv = s->lev[lev];
-    size_t n = 2 * (size_t)Lv.nc * s->nv;
+    size_t n = 2 * (size_t)Lv.nc;                    // rows of velocities
     CK(cudaMemcpyAsync(Lv.inv_tau, inv_tau, Lv.nc * sizeof(double), cudaMemcpyHostToDevice, s->st));
-    ST(to_device(s, Lv.r, r, n));
+    ST(rows_to_device(s, Lv.r, r, n));
     MicroArgs mi = micro_args(s, lev);
     if (s->mixed) {
         k_invD_from_itau<float><<<Lv.nc, 128, 0, s->st>>>(Lv.dev, s->vel, Lv.inv_tau, (float*)Lv.invD);
         CK(cudaGetLastError());
-        CK(launch_micro_sgs<float>(mi, sweep_plan(s, Lv), s->Zw, (float*)Lv.invD, (float*)Lv.r, (float*)Lv.dl, (float*)s->xcorner, s->st));
+        CK(launch_micro_sgs<float>(mi, sweep_plan(s, Lv), s->Zw, (float*)Lv.invD, (float*)Lv.r, (float*)Lv.dl, (float*)s->scratch, s->st));
     } else {
         k_invD_from_itau<double><<<Lv.nc, 128, 0, s->st>>>(Lv.dev, s->vel, Lv.inv_tau, (double*)Lv.invD);
         CK(cudaGetLastError());
-        CK(launch_micro_sgs<double>(mi, sweep_plan(s, Lv), s->Zw, (double*)Lv.invD, (double*)Lv.r, (double*)Lv.dl, (double*)s->xcorner,
+        CK(launch_micro_sgs<double>(mi, sweep_plan(s, Lv), s->Zw, (double*)Lv.invD, (double*)Lv.r, (double*)Lv.dl, (double*)s->scratch,
                                     s->st));
     }
-    return to_host(s, x, Lv.dl, n);
+    if (const miugks_status ts = sweep_status(s)) return ts;
+    return rows_to_host(s, x, Lv.dl, n);
 }
 
 miugks_status miugks_stage_apply_micro(miugks_solver* s, int lev, const double* inv_tau, const double* x, double* y)
 {
     ST(check_level(s, lev));
     HLevel& Lv = s->lev[lev];
-    size_t n = 2 * (size_t)Lv.nc * s->nv;
+    size_t n = 2 * (size_t)Lv.nc;                    // rows of velocities
     CK(cudaMemcpyAsync(Lv.inv_tau, inv_tau, Lv.nc * sizeof(double), cudaMemcpyHostToDevice, s->st));
-    ST(to_device(s, Lv.dl, x, n));
-    CK(cudaMemsetAsync(Lv.r, 0, n * s->fsz, s->st));
+    ST(rows_to_device(s, Lv.dl, x, n));
+    CK(cudaMemsetAsync(Lv.r, 0, n * s->ld * s->fsz, s->st));
     MicroArgs mi = micro_args(s, lev);
     if (s->mixed) CK(launch_micro_renew<float>(mi, s->Zw, (float*)Lv.dl, (float*)Lv.r, nullptr, 1, s->st));
     else CK(launch_micro_renew<double>(mi, s->Zw, (double*)Lv.dl, (double*)Lv.r, nullptr, 1, s->st));
-    std::vector<double> h(n);
-    ST(to_host(s, h.data(), Lv.r, n));
-    for (size_t q = 0; q < n; ++q) y[q] = -h[q];
+    ST(rows_to_host(s, y, Lv.r, n));
+    for (size_t q = 0; q < n * s->nv; ++q) y[q] = -y[q];
     return MIUGKS_OK;
 }
 
@@ -1598,11 +1663,7 @@ miugks_status miugks_stage_sgs_macro(miugks_solver* s, int lev, const double* W,
     ST(macro_stage(s, ma, Lv, 0, Lv.Wd, Lv.R, true));
     ST(macro_sgs(s, ma, Lv, -1));
     ST(to_host(s, dW, Lv.dW, n4));
-    double flag = 0.0;
-    CK(cudaMemcpyAsync(&flag, s->rms_out + 5, sizeof flag, cudaMemcpyDeviceToHost, s->st));
-    CK(cudaStreamSynchronize(s->st));
-    if (flag != 0.0) return fail(s, MIUGKS_ETIMEOUT, "a bounded wait of the macro sweep gave up");
-    return MIUGKS_OK;
+    return sweep_status(s);
 }
 
 miugks_status miugks_stage_resid_macro(miugks_solver* s, int lev, const double* W, const double* Wg, double* RE)
@@ -1707,9 +1768,12 @@ miugks_status adj_prepare(miugks_solver* s, int m)
         ST(dalloc(s, &A.Zb, (size_t)m * n));
         A.m = m;
     }
-    if (s->mixed) CK(launch_to_double<float>((const float*)s->f, A.f, n, s->st));
-    else CK(cudaMemcpyAsync(A.f, s->f, n * sizeof(double), cudaMemcpyDeviceToDevice, s->st));
-    CK(launch_moments<double>(L0.dev, s->vel, A.f, A.W, A.q, s->st));
+    const size_t rows = 2 * (size_t)L0.nc;
+    if (s->mixed) CK(launch_rows_to_double<float>((const float*)s->f, s->ld, A.f, s->nv, rows, s->st));
+    else CK(launch_rows_to_double<double>((const double*)s->f, s->ld, A.f, s->nv, rows, s->st));
+    VelDev packed = s->vel;                 // the adjoint's arrays are packed
+    packed.ld = s->nv;
+    CK(launch_moments<double>(L0.dev, packed, A.f, A.W, A.q, s->st));
     CK(launch_inv_tau(s->gas, A.W, L0.nc, A.itau, s->st));
     MacroArgs ma = macro_args(s, 0, 0.0);
     CK(launch_macro_gamma(ma, A.W, A.gx, A.gy, s->st));
@@ -2297,7 +2361,7 @@ miugks_status miugks_save(miugks_solver* s, const char* path)
     if (!s->initialised) return fail(s, MIUGKS_ESTATE, "save before init");
     const size_t n = 2 * (size_t)s->lev[0].nc * s->nv;
     std::vector<double> f(n);
-    ST(to_host(s, f.data(), s->f, n));
+    ST(rows_to_host(s, f.data(), s->f, 2 * (size_t)s->lev[0].nc));
     FILE* fp = std::fopen(path, "wb");
     if (!fp) return fail(s, MIUGKS_EINVAL, "cannot open %s for writing", path);
     const char magic[8] = {'M', 'I', 'U', 'G', 'K', 'S', 'v', '1'};

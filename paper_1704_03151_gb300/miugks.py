@@ -291,7 +291,7 @@ class Solver:
         self._check(self._lib.miugks_set_shock_capturing(self.h, 1 if on else 0))
 
     def set_sweep_split(self, mode):
-        """Evolution-sweep layout: "auto" (by level size), "split" or "wave" (same results)."""
+        """Evolution-sweep layout: "auto", "split" or "wave" (the same launches now)."""
         self._check(self._lib.miugks_set_sweep_split(self.h, {"auto": 0, "split": 1, "wave": 2}[mode]))
 
     def set_adaptive_ratio(self, ratio):
