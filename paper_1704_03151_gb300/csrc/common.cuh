@@ -23,7 +23,8 @@ struct BcDev { int type; double rho, u, v, t; };
 struct VelDev {
     int nu, nvv, nv;
     const double *u, *v, *w;     // per discrete velocity
-    const double *ua, *vb;       // per-axis nodes
+    const double *ua, *vb;       // per-axis nodes (ascending)
+    const double *wa, *wb;       // per-axis weights, w = wa wb
     const float *uf, *vf, *wf;   // u, v, w rounded to FP32 (for the mixed-precision kernels)
     double umax, vmax;           // largest |u|, |v|
     int ld;                      // row stride of per-velocity arrays: nv rounded up to a multiple of 16 (the tables

@@ -3,36 +3,16 @@
 // macroResidualCalc, microResidualDef) and the macroscopic residual R
 // (Eq. macroResidualDef), plus its RMS (Eq. Residual_Def).
 //
-// One CTA per face; threads stride over the discrete velocities, which are
-// contiguous in memory ([comp][cell][k]), so every load of f is coalesced.
-// The three velocity reductions a face needs (interface state W0; heat flux
-// and time slope; macroscopic flux) are deterministic block reductions.  The
-// equilibrium at the face is evaluated from separable per-axis exponential
-// tables (Nu + Nv exponentials per face instead of Nu * Nv).
+// One CTA per face; a thread keeps one velocity of the second axis and strides
+// over the first, so every load of f is coalesced and whatever depends on the
+// second axis only stays in registers.  Two passes over the velocities: the
+// first reconstructs the face values and takes their moments, the second forms
+// the flux and its moments.
 #include "kernels.cuh"
+#include <algorithm>
+#include <type_traits>
 
 namespace miugks {
-namespace cg = cooperative_groups;
-
-// Sum of N per-CTA totals over the CTAs of a cluster (one face split over its
-// CTAs by velocity), in rank order: every thread of every CTA gets the same
-// value.  slots: N doubles of this CTA's shared memory, one set per reduction.
-template <int N>
-__device__ __forceinline__ void cluster_total(cg::cluster_group& cl, double (&v)[N], double* slots)
-{
-    const int nb = (int)cl.num_blocks();
-    if (nb == 1) return;
-    if (threadIdx.x == 0)
-        #pragma unroll
-        for (int q = 0; q < N; ++q) slots[q] = v[q];
-    cl.sync();
-    #pragma unroll
-    for (int q = 0; q < N; ++q) {
-        double t = 0.0;
-        for (int r = 0; r < nb; ++r) t += cl.map_shared_rank(slots, r)[q];
-        v[q] = t;
-    }
-}
 
 __constant__ double c_series[5][28];   // power-series coefficients of the time integrals
 __constant__ float c_series_f[5][28];  // the same rounded to FP32
@@ -61,28 +41,6 @@ void upload_series_coefficients()
     for (int m = 0; m < 5; ++m)
         for (int n = 0; n < 28; ++n) cf[m][n] = (float)c[m][n];
     cudaMemcpyToSymbol(c_series_f, cf, sizeof cf);
-}
-
-__device__ __forceinline__ void time_coeffs_fast(double dt, double tau, double q[5])
-{
-    double x = dt / tau;
-    if (x < 1.0) {
-        double s[5];
-        #pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            double acc = c_series[m][27];
-            #pragma unroll
-            for (int n = 26; n >= 0; --n) acc = fma(acc, x, c_series[m][n]);
-            s[m] = acc;
-        }
-        q[0] = dt * s[0];
-        q[1] = dt * dt * s[1];
-        q[2] = dt * dt * s[2];
-        q[3] = dt * s[3];
-        q[4] = dt * dt * s[4];
-    } else {
-        time_coeffs(dt, tau, q);
-    }
 }
 
 // one of the five time integrals (series below x = dt/tau = 1, closed form above)
@@ -128,8 +86,8 @@ __device__ __forceinline__ float time_coeff_one_f(float dt, float tau, int m)
 // van Leer limited slope 2 s1 s2 / (s1 + s2) when s1 s2 > 0, else 0
 __device__ __forceinline__ double vl_limited(double s1, double s2)
 {
-    double p = s1 * s2;
-    return p > 0.0 ? 2.0 * p * rcp64(s1 + s2) : 0.0;
+    const double p = s1 * s2;      // (the sign is looked at in the bits: a comparison would take the FP64 pipe)
+    return __double_as_longlong(p) > 0 ? (p + p) * rcp64(s1 + s2) : 0.0;
 }
 __device__ __forceinline__ float vl_limited(float s1, float s2)
 {
@@ -137,49 +95,151 @@ __device__ __forceinline__ float vl_limited(float s1, float s2)
     return p > 0.0f ? __fdividef(2.0f * p, s1 + s2) : 0.0f;
 }
 
-// (a . psi) g split into the reduced components: b gM + a4 hM and b hM + a4 <xi^4>/4 gM
-template <typename F>
-__device__ __forceinline__ void slope_mom(const F* a, F u, F v, F gM, F hM, F xi4q, F& mG, F& mH)
+// Sums of N per-thread values over a warp: at every step a lane sends half of its
+// values and keeps the other half, so N values take about 1.4 N exchanges instead
+// of 5 N.  Afterwards the lane holds the sum of value `which` (none: which >= N).
+// FP32 values are float-float pairs throughout.
+template <int N>
+__device__ __forceinline__ double warp_sums(Acc<double> (&a)[N], int& which)
 {
-    F b = a[0] + a[1] * u + a[2] * v + F(0.5) * a[3] * (u * u + v * v);
-    mG = b * gM + a[3] * hM;
-    mH = b * hM + a[3] * xi4q * gM;
+    const int lane = threadIdx.x & 31;
+    double v[N];
+    #pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = a[q].s;
+    which = 0;
+    int n = N, mine = N;              // slots in use, and how many of this lane's hold a value
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int h = (n + 1) / 2;
+        const bool up = n > 1 && (lane & o);             // with one value left: a plain exchange
+        #pragma unroll
+        for (int q = 0; q < N; ++q) {
+            if (q >= h) break;
+            const double hi = n == 1 ? v[q] : q + h < n ? v[q + h] : 0.0;
+            const double r = __shfl_xor_sync(0xffffffffu, up ? v[q] : hi, o);
+            v[q] = (up ? hi : v[q]) + r;
+        }
+        which += up ? h : 0;
+        mine = up ? mine - h : min(mine, h);
+        n = h;
+    }
+    if (mine <= 0) which = N;
+    return v[0];
 }
+template <int N>
+__device__ __forceinline__ float2 warp_sums(Acc<float> (&a)[N], int& which)
+{
+    const int lane = threadIdx.x & 31;
+    float vh[N], vl[N];
+    #pragma unroll
+    for (int q = 0; q < N; ++q) { vh[q] = a[q].s; vl[q] = -a[q].c; }
+    which = 0;
+    int n = N, mine = N;              // slots in use, and how many of this lane's hold a value
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int h = (n + 1) / 2;
+        const bool up = n > 1 && (lane & o);             // with one value left: a plain exchange
+        #pragma unroll
+        for (int q = 0; q < N; ++q) {
+            if (q >= h) break;
+            const float th = n == 1 ? vh[q] : q + h < n ? vh[q + h] : 0.0f, tl = n == 1 ? vl[q] : q + h < n ? vl[q + h] : 0.0f;
+            const float rh = __shfl_xor_sync(0xffffffffu, up ? vh[q] : th, o), rl = __shfl_xor_sync(0xffffffffu, up ? vl[q] : tl, o);
+            float s, e;
+            two_sum(up ? th : vh[q], rh, s, e);
+            vl[q] = (up ? tl : vl[q]) + rl + e;
+            vh[q] = s;
+        }
+        which += up ? h : 0;
+        mine = up ? mine - h : min(mine, h);
+        n = h;
+    }
+    if (mine <= 0) which = N;
+    return make_float2(vh[0], vl[0]);
+}
+// ... and over the block: out[q] in shared memory, valid after the caller's next barrier
+template <int N>
+__device__ __forceinline__ void block_sums(Acc<double> (&a)[N], double* scratch, double* out)
+{
+    int which;
+    const double v = warp_sums<N>(a, which);
+    const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    if (which < N) scratch[warp * N + which] = v;        // (lanes with the same value agree)
+    __syncthreads();
+    if (threadIdx.x < N) {
+        double t = scratch[threadIdx.x];
+        for (int w = 1; w < nw; ++w) t += scratch[w * N + threadIdx.x];
+        out[threadIdx.x] = t;
+    }
+}
+template <int N>
+__device__ __forceinline__ void block_sums(Acc<float> (&a)[N], double* scratch, double* out)
+{
+    int which;
+    const float2 v = warp_sums<N>(a, which);
+    float2* fs = reinterpret_cast<float2*>(scratch);
+    const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    if (which < N) fs[warp * N + which] = v;
+    __syncthreads();
+    if (threadIdx.x < N) {
+        float2 t = fs[threadIdx.x];
+        for (int w = 1; w < nw; ++w) {
+            const float2 r = fs[w * N + threadIdx.x];
+            float s, e;
+            two_sum(t.x, r.x, s, e);
+            t = make_float2(s, t.y + r.y + e);
+        }
+        out[threadIdx.x] = (double)t.x + (double)t.y;
+    }
+}
+
+// Constants of the flux per node of the velocity axis normal to the face, and per
+// node of the tangential axis (k_face_flux, second pass)
+template <typename F> struct alignas(16) NormalNode { F un, E, P, C, Z, hZ, xZ, Fq, S, q5u; };
+template <typename F> struct alignas(16) TangentNode { F ut, h, E, Fq, S; };   // h = u_t / 2
 
 // Per-velocity arithmetic runs in F (FP64, or FP32 in the mixed form); the
 // velocity sums are FP64 (or Kahan-compensated FP32) per thread and combined in
 // FP64; the per-face scalars (interface state, slopes, time integrals) are FP64.
-// CACHE keeps the upwinded face values and slopes of every velocity in shared
-// memory between the three velocity passes; without it (a velocity grid too
-// large for shared memory in FP64) the later passes recompute them from f with
-// the same arithmetic.
 //
-// A face may be split over the CTAs of a cluster (launched with a cluster
-// dimension): each CTA takes a contiguous chunk of the velocities and caches
-// only its chunk, and the three velocity reductions add the CTAs' totals in
-// rank order through distributed shared memory.  Boundary faces and faces
-// inside a body are done by rank 0 alone.
+// What is done per velocity is kept small, since the kernel is bound by the issue
+// of its arithmetic (FP64: two lanes per clock and SM):
+//   * only the upwind side of a velocity is reconstructed (three cells of the
+//     four), with mirrored constants for the velocities that come from above;
+//   * the heat flux needs no pass of its own: it follows from moments about the
+//     mean velocity of the two cells, taken with the face values (about that
+//     velocity, not about zero, so that nothing cancels in a fast flow);
+//   * the compatibility sums of the equilibrium's slopes, sum w u_n psi (a.psi) g,
+//     are products of one-axis sums, because g, w and the powers of u and v
+//     separate: nu + nv terms by one warp instead of nu nv by all;
+//   * the equilibrium part of the flux is g times a polynomial whose coefficients
+//     depend on one axis each (NormalNode, TangentNode).
+// CACHE keeps the face values and slopes of every velocity in shared memory
+// between the passes; without it (a velocity grid too large for shared memory)
+// the second pass reconstructs again.
+// Per launch against three passes that reconstructed both sides of every velocity:
+// square cylinder (89x89) mixed 4.3 -> 2.1 ms, flat plate (48x48) mixed 0.73 ->
+// 0.51 ms, FP64 13.1 -> 4.8 ms, 64x64 cavity (32x32) mixed 131 -> 103 us, FP64 1.92
+// -> 0.72 ms, square cylinder at half size FP64 21.4 -> 10.1 ms.
 template <typename F, bool CACHE>
 __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceFluxArgs<F> A)
 {
     extern __shared__ double sm[];
-    cg::cluster_group cl = cg::this_cluster();
-    const int ncl = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const LevelDev& L = A.L;
     const VelDev& Vg = A.V;
-    const int nv = Vg.nv, tid = threadIdx.x, bs = blockDim.x;
+    const int nv = Vg.nv, nu = Vg.nu, nvv = Vg.nvv, tid = threadIdx.x, bs = blockDim.x;
     const size_t ld = Vg.ld;
-    const int axis = A.axis, fi = blockIdx.x / ncl;
-    const int chunk = (nv + ncl - 1) / ncl, kb = rank * chunk, ke = min(nv, kb + chunk);
+    const int axis = A.axis, fi = blockIdx.x;
     const int nx = L.nx, ny = L.ny;
     const size_t nc = L.nc, nf = axis == 0 ? L.nfx : L.nfy;
-    double* red = sm;                       // 32 * 8
-    double* par = red + 256;                // face scalars (FP64), [48]; cluster slots at 48..63
-    F* pf = reinterpret_cast<F*>(par + 64); // face constants in F, [64]
-    F* f0s = reinterpret_cast<F*>(par + 128);  // [2][chunk] (CACHE)
-    F* sgs = f0s + (CACHE ? 2 * chunk : 0); // [2][chunk] (CACHE)
-    F* Eu = sgs + (CACHE ? 2 * chunk : 0);  // [nu]
-    F* Ev = Eu + Vg.nu;                     // [nvv]
+    double* red = sm;                       // 32 * 9
+    double* par = red + 288;                // face scalars (FP64), [48]
+    double* tot = par + 48;                 // block sums, [16]
+    F* pf = reinterpret_cast<F*>(tot + 16); // face constants in F, [64]
+    NormalNode<F>* tn = reinterpret_cast<NormalNode<F>*>(pf + 64);   // per node of the first axis (or TangentNodes)
+    F* ta = reinterpret_cast<F*>(tn + nu);  // per node of the first axis: u - U_s, (u - U_s)^2 / 2, [nu][2]
+    F* wE = ta + 2 * nu;                    // exponentials per node, [nu] then [nvv]
+    F* f0s = wE + nu + nvv;                 // [2][nv] (CACHE)
+    F* sgs = f0s + 2 * nv;                  // [2][nv] (CACHE)
     const int i = axis == 0 ? fi % (nx + 1) : fi % nx;
     const int j = axis == 0 ? fi / (nx + 1) : fi / nx;
     const int bcid = (axis == 0 ? L.fbx : L.fby)[fi];
@@ -189,7 +249,6 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
     F* __restrict__ phH = A.ph + (nf + fi) * ld;
 
     if (bcid >= 0) {
-        if (rank != 0) return;
         // ---------------- boundary face: free transport of the face distribution
         int outsign, c;
         bface_side(L, axis, i, j, c, outsign);
@@ -234,7 +293,6 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
     }
 
     if (inactive_face(L, axis, i, j)) {   // inside a body: no flux
-        if (rank != 0) return;
         for (int k = tid; k < nv; k += bs) { phG[k] = F(0); phH[k] = F(0); }
         if (tid == 0)
             for (int m = 0; m < 4; ++m) A.Fm[4 * (size_t)fi + m] = 0.0;
@@ -244,18 +302,17 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
     // Face constants are computed once (by one thread or one lane each) and
     // broadcast through shared memory as F: an FP64 instruction occupies a
     // GB300 SM sub-partition for as long for one lane as for thirty-two.
-    const F* __restrict__ vu = VelT<F>::u(Vg);
-    const F* __restrict__ vv = VelT<F>::v(Vg);
     const F* __restrict__ vw = VelT<F>::w(Vg);
-    int cL, cR, cLL = -1, cRR = -1;
+    // a cell behind that does not exist is the upwind cell itself: its difference is zero, and so is the slope
+    int cL, cR, cLL, cRR;
     if (axis == 0) {
         cL = j * nx + i - 1; cR = cL + 1;
-        if (i - 1 > 0 && L.fbx[fi - 1] < 0) cLL = cL - 1;
-        if (i + 1 < nx && L.fbx[fi + 1] < 0) cRR = cR + 1;
+        cLL = i - 1 > 0 && L.fbx[fi - 1] < 0 ? cL - 1 : cL;
+        cRR = i + 1 < nx && L.fbx[fi + 1] < 0 ? cR + 1 : cR;
     } else {
         cL = (j - 1) * nx + i; cR = cL + nx;
-        if (j - 1 > 0 && L.fby[fi - nx] < 0) cLL = cL - nx;
-        if (j + 1 < ny && L.fby[fi + nx] < 0) cRR = cR + nx;
+        cLL = j - 1 > 0 && L.fby[fi - nx] < 0 ? cL - nx : cL;
+        cRR = j + 1 < ny && L.fby[fi + nx] < 0 ? cR + nx : cR;
     }
     // the face's mesh constants (kFluxGeo): par[32..40] in FP64, the first five also in F
     if (tid < kFluxGeo - 1) {
@@ -263,62 +320,84 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
         par[32 + tid] = gv;
         if (tid < 5) pf[tid] = (F)gv;
     }
+    // U_s, V_s: mean velocity of the two cells, rounded to FP32 (any value near the interface's serves)
+    if (tid >= 32 && tid < 34) {
+        const int m = tid - 31;
+        const double *wl = A.W + 4 * (size_t)cL, *wr = A.W + 4 * (size_t)cR;
+        pf[4 + m] = (F)(0.5f * ((float)wl[m] / (float)wl[0] + (float)wr[m] / (float)wr[0]));
+    }
     __syncthreads();
+    const F Us = pf[5], Vs = pf[6];
+    for (int a = tid; a < nu; a += bs) {
+        const F d = (F)Vg.ua[a] - Us;
+        ta[2 * a] = d;
+        ta[2 * a + 1] = F(0.5) * d * d;
+    }
+    __syncthreads();
+    // threads: columns tx of the second axis, rows ty of the first
+    const int bw = min(nvv, bs), rows = bs / bw, tx = tid % bw, ty = tid / bw;
+    // nodes ascend: the first nneg of the normal axis come from above, the last ones from below
+    const int nneg = Vg.nleave[0][axis], npos0 = (axis == 0 ? nu : nvv) - Vg.nleave[1][axis];
     const F r1 = pf[0], r2 = pf[1], r3 = pf[2], fhL = pf[3], fhR = pf[4];
-    // van Leer reconstruction and upwinding of velocity k: face value f0 and slope sg of G and H
-    auto recon = [&](int k, F (&f0)[2], F (&sg)[2]) {
-        const F un = axis == 0 ? vu[k] : vv[k];
+    const size_t oL = cL * ld, oR = cR * ld, oLL = cLL * ld, oRR = cRR * ld;
+    // face value f0 and slope sg of velocity k, reconstructed in its upwind cell (n: index on the normal axis)
+    auto recon = [&](int k, int n, F (&f0)[2], F (&sg)[2]) {
+        const bool neg = n < nneg;
+        const size_t om = neg ? oRR : oLL, o0 = neg ? oR : oL, op = neg ? oL : oR;
+        const F rm = neg ? -r3 : r1, rp = neg ? -r2 : r2, h = neg ? -fhR : fhL;
         #pragma unroll
         for (int cp = 0; cp < 2; ++cp) {
-            const F* fc = cp == 0 ? fG : fH;
-            F fL = fc[cL * ld + k], fR = fc[cR * ld + k];
-            F d2 = (fR - fL) * r2;
-            F sL = cLL >= 0 ? vl_limited((fL - fc[cLL * ld + k]) * r1, d2) : F(0);
-            F sR = cRR >= 0 ? vl_limited(d2, (fc[cRR * ld + k] - fR) * r3) : F(0);
-            F faceL = fL + sL * fhL, faceR = fR - sR * fhR;
-            if (un > F(0)) { f0[cp] = faceL; sg[cp] = sL; }
-            else if (un < F(0)) { f0[cp] = faceR; sg[cp] = sR; }
-            else { f0[cp] = F(0.5) * (faceL + faceR); sg[cp] = F(0.5) * (sL + sR); }
+            const F* fc = (cp == 0 ? fG : fH) + k;
+            const F fu = fc[o0], s1 = (fu - fc[om]) * rm, s2 = (fc[op] - fu) * rp;
+            sg[cp] = vl_limited(s1, s2);
+            f0[cp] = fu + sg[cp] * h;
         }
-    };
-    auto face_vals = [&](int k, F (&f0)[2], F (&sg)[2]) {
-        if constexpr (CACHE) {
-            const int e = k - kb;
-            f0[0] = f0s[e]; f0[1] = f0s[chunk + e]; sg[0] = sgs[e]; sg[1] = sgs[chunk + e];
-        } else {
-            recon(k, f0, sg);
+        if (n >= nneg && n < npos0) {            // u_n = 0: the mean of both sides
+            #pragma unroll
+            for (int cp = 0; cp < 2; ++cp) {
+                const F* fc = (cp == 0 ? fG : fH) + k;
+                const F fu = fc[oR], s = vl_limited((fc[oRR] - fu) * r3, (fu - fc[oL]) * r2);
+                f0[cp] = F(0.5) * (f0[cp] + (fu - s * fhR));
+                sg[cp] = F(0.5) * (sg[cp] + s);
+            }
         }
     };
 
-    // pass 1: reconstruction, upwinding, interface conservative variables
-    // (unrolled so that the loads of the next velocity are in flight with this one's arithmetic)
-    Acc<F> W0a[4];
-    #pragma unroll 2
-    for (int k = kb + tid; k < ke; k += bs) {
-        F f0[2], sg[2];
-        recon(k, f0, sg);
-        if constexpr (CACHE) {
-            const int e = k - kb;
-            f0s[e] = f0[0]; f0s[chunk + e] = f0[1];
-            sgs[e] = sg[0]; sgs[chunk + e] = sg[1];
+    // pass 1: reconstruction and moments about (U_s, V_s): 1, a, b, e; a e, b e; a^2, a b, b^2
+    // with (a, b) the shifted velocity and e its energy with the internal one
+    Acc<F> M[9];
+    if (ty < rows)
+        for (int b = tx; b < nvv; b += bw) {
+            const F db = (F)Vg.vb[b] - Vs, hb = F(0.5) * db * db;
+            #pragma unroll 2
+            for (int a = ty; a < nu; a += rows) {
+                const int k = a * nvv + b;
+                const F w = vw[k], da = ta[2 * a], ha = ta[2 * a + 1];
+                F f0[2], sg[2];
+                recon(k, axis == 0 ? a : b, f0, sg);
+                if constexpr (CACHE) {
+                    f0s[k] = f0[0]; f0s[nv + k] = f0[1];
+                    sgs[k] = sg[0]; sgs[nv + k] = sg[1];
+                }
+                const F g = w * f0[0], we = w * ((ha + hb) * f0[0] + f0[1]), ga = g * da, gb = g * db;
+                M[0].add(g); M[1].add(ga); M[2].add(gb); M[3].add(we);
+                M[4].add(we * da); M[5].add(we * db);
+                M[6].add(ga * da); M[7].add(ga * db); M[8].add(gb * db);
+            }
         }
-        const F w = vw[k], u = vu[k], v = vv[k], g = f0[0];
-        W0a[0].add(w * g); W0a[1].add(w * u * g); W0a[2].add(w * v * g);
-        W0a[3].add(w * (F(0.5) * (u * u + v * v) * g + f0[1]));
-    }
-    double W0[4];
-    block_total<4>(W0a, red, W0);
-    cluster_total<4>(cl, W0, par + 48);
+    block_sums<9>(M, red, tot);
+    __syncthreads();
     // face scalars, spread over the lanes of warp 0: lane 0 the collision time and
-    // time step, lanes 1 and 2 the left and right equilibrium slopes
-    if (tid < 3) {
-        double rho = W0[0], ir = rcp64(rho);
-        double U = W0[1] * ir, V = W0[2] * ir;
-        double lam = (kKint + 2) * rho * rcp64(4.0 * (W0[3] - 0.5 * (W0[1] * U + W0[2] * V)));
+    // time step, lanes 1 and 2 the left and right equilibrium slopes, lane 3 the heat flux
+    if (tid < 4) {
+        const double m0 = tot[0], m1 = tot[1], m2 = tot[2], m3 = tot[3], us = (double)Us, vs = (double)Vs;
+        const double ir = rcp64(m0), dx = m1 * ir, dy = m2 * ir;
+        const double U = us + dx, V = vs + dy;
+        const double lam = (0.25 * (kKint + 2)) * m0 * rcp64(m3 - 0.5 * (m1 * dx + m2 * dy));
         if (tid == 0) {
-            par[0] = rho; par[1] = U; par[2] = V; par[3] = lam;
-            if constexpr (sizeof(F) == 8) par[4] = tau_of(A.gas, rho, lam);
-            else par[4] = (double)tau_of_f(A.gas, (float)rho, (float)lam);
+            par[0] = m0; par[1] = U; par[2] = V; par[3] = lam;
+            if constexpr (sizeof(F) == 8) par[4] = tau_of(A.gas, m0, lam);
+            else par[4] = (double)tau_of_f(A.gas, (float)m0, (float)lam);
             par[5] = par[37];
             if (A.shock) {
                 double rl, ul, vl, ll, rr, ur, vr, lr;
@@ -327,11 +406,11 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
                 const double pl = rl / (2.0 * ll), pr = rr / (2.0 * lr);
                 par[4] += par[5] * fabs(pl - pr) / (pl + pr);
             }
-        } else {
+        } else if (tid < 3) {
             const double* Wc = A.W + 4 * (size_t)(tid == 1 ? cL : cR);
-            double hf, dw[4];
-            if constexpr (sizeof(F) == 8) hf = (tid == 1 ? 1.0 : -1.0) * ir * rcp64(tid == 1 ? par[35] : par[36]);
-            else hf = (tid == 1 ? 1.0 : -1.0) * ir * (tid == 1 ? par[39] : par[40]);
+            const double W0[4] = {m0, m1 + us * m0, m2 + vs * m0, m3 + us * m1 + vs * m2 + 0.5 * (us * us + vs * vs) * m0};
+            const double hf = (tid == 1 ? ir : -ir) * (tid == 1 ? par[39] : par[40]);
+            double dw[4];
             for (int m = 0; m < 4; ++m) dw[m] = (W0[m] - Wc[m]) * hf;
             if constexpr (sizeof(F) == 8) {
                 micro_slope(dw, U, V, lam, par + (tid == 1 ? 8 : 12));
@@ -340,207 +419,215 @@ __global__ void __launch_bounds__(256, sizeof(F) == 4 ? 4 : 2) k_face_flux(FaceF
                 micro_slope_t<float>(dwf, (float)U, (float)V, (float)lam, af);
                 for (int m = 0; m < 4; ++m) par[(tid == 1 ? 8 : 12) + m] = af[m];
             }
+        } else {
+            // moments about (U, V) = (U_s, V_s) + (dx, dy)
+            const double d2 = 0.5 * (dx * dx + dy * dy), es = m3 - dx * m1 - dy * m2 + d2 * m0;
+            par[6] = tot[4] - dx * tot[6] - dy * tot[7] + d2 * m1 - dx * es;
+            par[7] = tot[5] - dx * tot[7] - dy * tot[8] + d2 * m2 - dy * es;
         }
     }
     __syncthreads();
     {
-        // warp 0: constants of the equilibrium in F; the other warps: the per-axis exponentials
+        // warp 0: constants of the equilibrium in F, and one time integral per lane; the others: the exponentials
         const double rho0 = par[0], U0 = par[1], V0 = par[2], lam0 = par[3];
         if (tid < 32) {
             F val = F(0);
             if (tid < 8) val = (F)par[8 + tid];          // aL, aR
             else if (tid == 8) val = (F)U0;
             else if (tid == 9) val = (F)V0;
+            else if (tid == 14) val = (F)par[6];
+            else if (tid == 15) val = (F)par[7];
             else if constexpr (sizeof(F) == 8) {
                 if (tid == 10) val = rho0 * lam0 / kPi;
                 else if (tid == 11) val = kKint / (4.0 * lam0);
                 else if (tid == 12) val = kKint * (kKint + 2.0) / (16.0 * lam0 * lam0);
+                else if (tid == 13) val = (1.0 - A.gas.pr) * 4.0 * lam0 * lam0 / (5.0 * rho0);
+                else if (tid >= 16 && tid < 21) val = time_coeff_one(par[5], par[4], tid - 16) * par[38];   // q_i / dt
             } else {                                      // FP32 constants need no FP64 division
                 const float fl = (float)lam0;
                 if (tid == 10) val = (float)rho0 * fl * (float)(1.0 / kPi);
                 else if (tid == 11) val = (float)(kKint / 4.0) / fl;
                 else if (tid == 12) val = (float)(kKint * (kKint + 2.0) / 16.0) / (fl * fl);
+                else if (tid == 13) val = (float)((1.0 - A.gas.pr) * 0.8) * (fl * fl) / (float)rho0;
+                else if (tid >= 16 && tid < 21) val = (float)((double)time_coeff_one_f((float)par[5], (float)par[4], tid - 16) * par[38]);
             }
-            if (tid < 13) pf[8 + tid] = val;
+            if (tid == 21) val = (F)lam0;
+            if (tid < 22) pf[8 + tid] = val;
         } else {
-            for (int e = tid - 32; e < Vg.nu + Vg.nvv; e += bs - 32) {
-                const bool isu = e < Vg.nu;
-                const double d = isu ? Vg.ua[e] - U0 : Vg.vb[e - Vg.nu] - V0;
-                F ex;
+            for (int e = tid - 32; e < nu + nvv; e += bs - 32) {
+                const bool isu = e < nu;
+                const double d = isu ? Vg.ua[e] - U0 : Vg.vb[e - nu] - V0;
                 if constexpr (sizeof(F) == 8) {
-                    ex = exp(-lam0 * d * d);
+                    wE[e] = exp(-lam0 * d * d);
                 } else {
                     const float df = (float)d;
-                    ex = expf(-(float)lam0 * df * df);
+                    wE[e] = expf(-(float)lam0 * df * df);
                 }
-                (isu ? Eu[e] : Ev[e - Vg.nu]) = ex;
             }
         }
     }
     __syncthreads();
-    const F fU0 = pf[16], fV0 = pf[17], gnorm = pf[18], hfac = pf[19], xi4q = pf[20];
-    F aL[4], aR[4];
-    #pragma unroll
-    for (int m = 0; m < 4; ++m) { aL[m] = pf[8 + m]; aR[m] = pf[12 + m]; }
-
-    // velocity k = a * nvv + b of this thread, stepped by the block size without a division
-    const int ka0 = (kb + tid) / Vg.nvv, kb0 = kb + tid - ka0 * Vg.nvv;
-    const int sa = bs / Vg.nvv, sb = bs - sa * Vg.nvv;
-    // pass 2: heat flux of the interface distribution, compatibility moments for A
-    Acc<F> s6a[6];
-    for (int k = kb + tid, a = ka0, b = kb0; k < ke; k += bs, a += sa, b += sb) {
-        if (b >= Vg.nvv) { b -= Vg.nvv; ++a; }
-        const F u = vu[k], v = vv[k], w = vw[k];
-        F cx = u - fU0, cy = v - fV0, c2 = cx * cx + cy * cy;
-        F f0[2], sg[2];
-        face_vals(k, f0, sg);
-        F e = F(0.5) * c2 * f0[0] + f0[1];
-        s6a[0].add(w * cx * e);
-        s6a[1].add(w * cy * e);
-        F un = axis == 0 ? u : v;
-        if (un != F(0)) {
-            F gM = gnorm * Eu[a] * Ev[b], hM = gM * hfac, mG, mH;
-            slope_mom<F>(un > F(0) ? aL : aR, u, v, gM, hM, xi4q, mG, mH);
-            F wu = w * un;
-            s6a[2].add(wu * mG); s6a[3].add(wu * u * mG); s6a[4].add(wu * v * mG);
-            s6a[5].add(wu * (F(0.5) * (u * u + v * v) * mG + mH));
-        }
-    }
-    double s6[6];
-    block_total<6>(s6a, red, s6);
-    cluster_total<6>(cl, s6, par + 52);
-    // lane 0: time slope A from compatibility; lanes 1-5: one time integral each
-    if (tid < 6) {
-        const double rho0 = par[0], U0 = par[1], V0 = par[2], lam0 = par[3];
-        if (tid == 0) {
-            double dwt[4], ir = -rcp64(rho0);
-            for (int m = 0; m < 4; ++m) dwt[m] = s6[2 + m] * ir;
-            if constexpr (sizeof(F) == 8) {
-                micro_slope(dwt, U0, V0, lam0, par + 16);
-            } else {
-                float dwf[4] = {(float)dwt[0], (float)dwt[1], (float)dwt[2], (float)dwt[3]}, af[4];
-                micro_slope_t<float>(dwf, (float)U0, (float)V0, (float)lam0, af);
-                for (int m = 0; m < 4; ++m) par[16 + m] = af[m];
-            }
-            par[6] = s6[0]; par[7] = s6[1];
-        } else {
-            if constexpr (sizeof(F) == 8) par[20 + tid - 1] = time_coeff_one(par[5], par[4], tid - 1);
-            else par[20 + tid - 1] = time_coeff_one_f((float)par[5], (float)par[4], tid - 1);
-        }
-    }
-    __syncthreads();
+    const F fU0 = pf[16], fV0 = pf[17], gnorm = pf[18], hfac = pf[19], xi4q = pf[20], shk = pf[21], qx = pf[22], qy = pf[23];
+    const F q1 = pf[24], q2 = pf[25], q3 = pf[26], q4 = pf[27], q5 = pf[28], lam = pf[29];
+    // warp 0: one-axis sums N_i = sum w E u_n^i (i = 1..5, each side) and T_i = sum w E u_t^i (i = 0..4),
+    // then the compatibility sums and the time slope
     if (tid < 32) {
-        const double rho0 = par[0], lam0 = par[3];
-        F val = F(0);
-        if (tid < 4) val = (F)par[16 + tid];             // A
-        else if (tid < 9) val = (F)(par[20 + tid - 4] * par[38]);   // q_i / dt
-        else if (tid == 9) {
-            if constexpr (sizeof(F) == 8) val = (1.0 - A.gas.pr) * 4.0 * lam0 * lam0 / (5.0 * rho0);
-            else val = (float)((1.0 - A.gas.pr) * 0.8) * ((float)lam0 * (float)lam0) / (float)rho0;
+        const F* En = axis == 0 ? wE : wE + nu;
+        const F* Et = axis == 0 ? wE + nu : wE;
+        const int Nn = axis == 0 ? nu : nvv, Nt = axis == 0 ? nvv : nu;
+        Acc<F> T[15];
+        for (int n = tid; n < Nn; n += 32) {
+            const F u = (F)(axis == 0 ? Vg.ua : Vg.vb)[n];
+            F p = (F)(axis == 0 ? Vg.wa : Vg.wb)[n] * En[n] * u;
+            const bool neg = n < nneg;
+            #pragma unroll
+            for (int m = 0; m < 5; ++m) {
+                T[m].add(neg ? F(0) : p);
+                T[5 + m].add(neg ? p : F(0));
+                p *= u;
+            }
         }
-        else if (tid == 10) val = (F)par[6];
-        else if (tid == 11) val = (F)par[7];
-        else if (tid == 12) val = (F)(2.0 * lam0);
-        if (tid < 13) pf[24 + tid] = val;
+        for (int n = tid; n < Nt; n += 32) {
+            const F u = (F)(axis == 0 ? Vg.vb : Vg.ua)[n];
+            F p = (F)(axis == 0 ? Vg.wb : Vg.wa)[n] * Et[n];
+            #pragma unroll
+            for (int m = 0; m < 5; ++m) { T[10 + m].add(p); p *= u; }
+        }
+        int which;
+        const auto v = warp_sums<15>(T, which);
+        F* NT = pf + 40;                                         // N_1 .. N_5 of both sides, T_0 .. T_4
+        if (which < 15) {
+            if constexpr (sizeof(F) == 8) NT[which] = v;
+            else NT[which] = v.x + v.y;
+        }
+        __syncwarp();
+        // sums of u_n^i u_t^j (c + a_n u_n + a_t u_t + a_3 (u_n^2 + u_t^2) / 2) w u_n E E: one (side, i, j, c) per lane,
+        // lane 8 side + p: p 0 .. 4 with c = a_0 + a_3 K/(4 lambda) and (i, j) = 00, 10, 01, 20, 02; 5 with c = a_0; 6 a_3 alone
+        const int side = tid >> 3 & 1, p = tid & 7;
+        const F* as = pf + (side == 0 ? 8 : 12);
+        const F* N = NT + 5 * side;
+        const F* Tt = NT + 10;
+        const int ii = p == 1 ? 1 : p == 3 ? 2 : 0, jj = p == 2 ? 1 : p == 4 ? 2 : 0;
+        const F a3 = p == 6 ? F(0) : as[3], an = p == 6 ? F(0) : as[1 + axis], at = p == 6 ? F(0) : as[2 - axis];
+        const F c = p == 6 ? as[3] : p == 5 ? as[0] : fma(as[3], hfac, as[0]);
+        F S = (c * N[ii] + an * N[ii + 1] + F(0.5) * a3 * N[ii + 2]) * Tt[jj] + N[ii] * (at * Tt[jj + 1] + F(0.5) * a3 * Tt[jj + 2]);
+        S += __shfl_down_sync(0xffffffffu, S, 8);
+        // time slope A from -sum / rho, with g = rho lambda / pi E E
+        F dwt[4];
+        const F nrm = -lam * F(1.0 / kPi);
+        #pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const F x = __shfl_sync(0xffffffffu, S, m), s4 = __shfl_sync(0xffffffffu, S, 4), s5 = __shfl_sync(0xffffffffu, S, 5),
+                    s6 = __shfl_sync(0xffffffffu, S, 6);
+            dwt[m] = nrm * (m < 3 ? x : F(0.5) * (x + s4) + hfac * s5 + xi4q * s6);
+        }
+        const F d1 = axis == 0 ? dwt[1] : dwt[2], d2 = axis == 0 ? dwt[2] : dwt[1];
+        const F dw[4] = {dwt[0], d1, d2, dwt[3]};
+        F As[4];
+        micro_slope_t<F>(dw, fU0, fV0, lam, As);
+        if (tid == 0)
+            for (int m = 0; m < 4; ++m) pf[32 + m] = As[m];
     }
     __syncthreads();
-    F As[4];
-    #pragma unroll
-    for (int m = 0; m < 4; ++m) As[m] = pf[24 + m];
-    const F q1 = pf[28], q2 = pf[29], q3 = pf[30], q4 = pf[31], q5 = pf[32];
-    const F shk = pf[33], qx = pf[34], qy = pf[35], flam2 = pf[36];
-
-    // pass 3: time-averaged flux of every discrete velocity and its moments
-    Acc<F> Fa[4];
-    for (int k = kb + tid, a = ka0, b = kb0; k < ke; k += bs, a += sa, b += sb) {
-        if (b >= Vg.nvv) { b -= Vg.nvv; ++a; }
-        const F u = vu[k], v = vv[k], w = vw[k];
-        const F un = axis == 0 ? u : v;
-        F cx = u - fU0, cy = v - fV0, c2 = cx * cx + cy * cy;
-        F gM = gnorm * Eu[a] * Ev[b], hM = gM * hfac;
-        F Fq = shk * (cx * qx + cy * qy);
-        F gP = gM * (F(1) + Fq * (flam2 * c2 - F(4)));
-        F hP = hM * (F(1) + Fq * (flam2 * c2 - F(2)));
-        F mGa, mHa, mGA, mHA;
-        slope_mom<F>(un > F(0) ? aL : aR, u, v, gM, hM, xi4q, mGa, mHa);
-        slope_mom<F>(As, u, v, gM, hM, xi4q, mGA, mHA);
-        F f0[2], sg[2];
-        face_vals(k, f0, sg);
-        F pg = un * (q1 * gP + q2 * un * mGa + q3 * mGA + q4 * f0[0] + q5 * un * sg[0]);
-        F ph = un * (q1 * hP + q2 * un * mHa + q3 * mHA + q4 * f0[1] + q5 * un * sg[1]);
-        phG[k] = pg; phH[k] = ph;
-        Fa[0].add(w * pg); Fa[1].add(w * u * pg); Fa[2].add(w * v * pg);
-        Fa[3].add(w * (F(0.5) * (u * u + v * v) * pg + ph));
+    // nodes of the normal and the tangential axis
+    auto normal = [&](int n, NormalNode<F>& N) {
+        const F u = (F)(axis == 0 ? Vg.ua : Vg.vb)[n], c = u - (axis == 0 ? fU0 : fV0), qn = axis == 0 ? qx : qy;
+        const F* as = pf + (n < nneg ? 12 : 8);
+        const F an = as[1 + axis], at = as[2 - axis], a3 = as[3];
+        const F* As = pf + 32;
+        const F q2u = q2 * u;
+        N.un = u;
+        N.E = gnorm * (axis == 0 ? wE[n] : wE[nu + n]);
+        N.P = q1 + q2u * (as[0] + u * (an + F(0.5) * a3 * u)) + q3 * (As[0] + u * (As[1 + axis] + F(0.5) * As[3] * u));
+        N.C = q2u * at + q3 * As[2 - axis];
+        N.Z = q2u * a3 + q3 * As[3];
+        N.hZ = hfac * N.Z;
+        N.xZ = xi4q * N.Z;
+        N.Fq = q1 * shk * (c * qn);
+        N.S = F(2) * lam * (c * c) - F(4);
+        N.q5u = q5 * u;
+    };
+    auto tangent = [&](int n, TangentNode<F>& N) {
+        const F u = (F)(axis == 0 ? Vg.vb : Vg.ua)[n], c = u - (axis == 0 ? fV0 : fU0), qt = axis == 0 ? qy : qx;
+        N.ut = u;
+        N.h = F(0.5) * u;
+        N.E = axis == 0 ? wE[nu + n] : wE[n];
+        N.Fq = q1 * shk * (c * qt);
+        N.S = F(2) * lam * (c * c);
+    };
+    for (int a = tid; a < nu; a += bs) {
+        if (axis == 0) normal(a, tn[a]);
+        else tangent(a, reinterpret_cast<TangentNode<F>*>(tn)[a]);
     }
-    double Fm[4];
-    block_total<4>(Fa, red, Fm);
-    cluster_total<4>(cl, Fm, par + 58);
-    if (tid == 0 && rank == 0)
-        for (int m = 0; m < 4; ++m) A.Fm[4 * (size_t)fi + m] = Fm[m];
-    if (ncl > 1) cl.sync();   // the other CTAs' slots stay alive until every remote read is done
-}
+    __syncthreads();
 
-template <typename F>
-size_t face_flux_smem(const VelDev& V, bool cache, int ncl)
-{
-    const size_t chunk = ((size_t)V.nv + ncl - 1) / ncl;
-    return sizeof(double) * (256 + 128) + sizeof(F) * ((cache ? 4 * chunk : 0) + V.nu + V.nvv);
+    // pass 2: time-averaged flux of every discrete velocity and its moments
+    Acc<F> Fa[4];
+    auto sweep = [&](auto ax) {
+        constexpr int AX = decltype(ax)::value;
+        for (int b = tx; b < nvv; b += bw) {
+            NormalNode<F> N;
+            TangentNode<F> T;
+            if (AX == 0) tangent(b, T); else normal(b, N);
+            const F vb = (F)Vg.vb[b], hv2 = F(0.5) * vb * vb;
+            #pragma unroll 2
+            for (int a = ty; a < nu; a += rows) {
+                const int k = a * nvv + b;
+                const F w = vw[k];
+                if (AX == 0) N = tn[a];
+                else T = reinterpret_cast<const TangentNode<F>*>(tn)[a];
+                F f0[2], sg[2];
+                if constexpr (CACHE) {
+                    f0[0] = f0s[k]; f0[1] = f0s[nv + k]; sg[0] = sgs[k]; sg[1] = sgs[nv + k];
+                } else {
+                    recon(k, AX == 0 ? a : b, f0, sg);
+                }
+                const F gM = N.E * T.E, Fq = N.Fq + T.Fq, S = N.S + T.S;
+                const F Y = fma(Fq, S, fma(T.ut, fma(T.h, N.Z, N.C), N.P));
+                const F eG = gM * (Y + N.hZ), eH = gM * fma(hfac, fma(F(2), Fq, Y), N.xZ);
+                const F pg = N.un * fma(q4, f0[0], fma(N.q5u, sg[0], eG));
+                const F ph = N.un * fma(q4, f0[1], fma(N.q5u, sg[1], eH));
+                phG[k] = pg; phH[k] = ph;
+                const F u = AX == 0 ? N.un : T.ut, wg = w * pg;
+                Fa[0].add(wg); Fa[1].add(wg * u); Fa[2].add(wg * vb);
+                Fa[3].add(fma(wg, fma(F(0.5) * u, u, hv2), w * ph));
+            }
+        }
+    };
+    if (ty < rows) {
+        if (axis == 0) sweep(std::integral_constant<int, 0>());
+        else sweep(std::integral_constant<int, 1>());
+    }
+    block_sums<4>(Fa, red, tot);
+    if (tid < 4) A.Fm[4 * (size_t)fi + tid] = tot[tid];      // (written by this thread)
 }
 
 template <typename F>
 cudaError_t launch_face_flux(const FaceFluxArgs<F>& a, cudaStream_t st)
 {
     constexpr size_t kSmemMax = 227 * 1024;
-    // the cache pays while it leaves room for several CTAs per SM: a face is split
-    // over a cluster of 1, 2, 4 or 8 CTAs until each CTA's chunk fits in 64 KB;
-    // beyond that the recomputing variant (a few KB) is used
-    constexpr size_t kCacheMax = 64 * 1024;
-    int ncl = 1;
-    while (ncl < 8 && face_flux_smem<F>(a.V, true, ncl) > kCacheMax) ncl *= 2;
-    // In FP32 a face that needs a cluster for its cache (the 89^2 grid) runs faster as one CTA
-    // that recomputes the reconstruction in each pass (square cylinder: 8.7 against 11.8 ms of flux
-    // per iteration); with one CTA per face the cache wins (64^2 cavity 0.34 against 0.42 ms, flat
-    // plate 1.48 against 2.08 ms).  FP64 keeps the cluster split: recomputing costs FP64 issue.
-    const bool cache = face_flux_smem<F>(a.V, true, ncl) <= kCacheMax && (sizeof(F) == 8 || ncl == 1);
-    if (!cache) ncl = 1;
-    const size_t smem = face_flux_smem<F>(a.V, cache, ncl);
+    // the cache pays while it leaves room for two CTAs per SM; beyond that the face values are
+    // reconstructed again in the second pass (which costs a third of the arithmetic, where the split
+    // of a face over a cluster, each CTA caching its share, repeats the face's serial phases)
+    constexpr size_t kCacheMax = 110 * 1024;
+    const size_t base = sizeof(double) * (288 + 48 + 16) + sizeof(F) * (64 + 3 * (size_t)a.V.nu + a.V.nvv) +
+                        sizeof(NormalNode<F>) * (size_t)a.V.nu;
+    const size_t full = base + sizeof(F) * 4 * (size_t)a.V.nv;
+    const bool cache = full <= kCacheMax;
+    const size_t smem = cache ? full : base;
     if (smem > kSmemMax) return cudaErrorInvalidValue;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_face_flux<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kSmemMax);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_face_flux<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    auto kern = cache ? k_face_flux<F, true> : k_face_flux<F, false>;
+    if (smem > 47 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        attr_set = true;
     }
-    int nf = a.axis == 0 ? a.L.nfx : a.L.nfy;
-    // FP32 with a small velocity grid: 128 threads, so that more faces (CTAs) overlap their serial
-    // scalar phases on an SM (64^2 cavity, 32^2 velocities: 0.27 against 0.34 ms of flux per
-    // iteration); with 48^2 or more velocities 256 threads are faster (flat plate 1.48 against
-    // 1.72 ms, square cylinder 8.7 against 9.6 ms)
-    int threads = (a.V.nv / ncl < 256 || (sizeof(F) == 4 && a.V.nv / ncl <= 1536)) ? 128 : 256;
-    if (!cache) {
-        k_face_flux<F, false><<<nf, threads, smem, st>>>(a);
-        return cudaGetLastError();
-    }
-    if (ncl == 1) {
-        k_face_flux<F, true><<<nf, threads, smem, st>>>(a);
-        return cudaGetLastError();
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(nf * ncl), 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)ncl;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_face_flux<F, true>, a);
+    const int nf = a.axis == 0 ? a.L.nfx : a.L.nfy;
+    // whole rows of the second velocity axis, about 128 threads for a small velocity grid (more faces
+    // overlap their serial phases on an SM) and 256 for a large one
+    const int want = a.V.nv <= 1536 ? 128 : 256, rows = std::max(1, want / a.V.nvv);
+    const int threads = std::min(256, std::max(64, (rows * a.V.nvv + 31) / 32 * 32));
+    kern<<<nf, threads, smem, st>>>(a);
+    return cudaGetLastError();
 }
 template cudaError_t launch_face_flux<double>(const FaceFluxArgs<double>&, cudaStream_t);
 template cudaError_t launch_face_flux<float>(const FaceFluxArgs<float>&, cudaStream_t);

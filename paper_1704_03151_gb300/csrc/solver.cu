@@ -1076,6 +1076,8 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
         }
         if ((st = upload(s, (double**)&s->vel.ua, s->uah)) != MIUGKS_OK) break;
         if ((st = upload(s, (double**)&s->vel.vb, s->vbh)) != MIUGKS_OK) break;
+        if ((st = upload(s, (double**)&s->vel.wa, wa)) != MIUGKS_OK) break;
+        if ((st = upload(s, (double**)&s->vel.wb, wb)) != MIUGKS_OK) break;
         s->vel.nu = s->nu; s->vel.nvv = s->nvv; s->vel.nv = s->nv; s->vel.umax = s->umax; s->vel.vmax = s->vmax;
         s->vel.ld = s->ld;
         for (int p = 0; p < 2; ++p)
