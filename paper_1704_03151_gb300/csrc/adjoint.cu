@@ -213,13 +213,14 @@ __device__ __forceinline__ FaceGeo face_geo(const LevelDev& L, int axis, int fi)
 __device__ __forceinline__ void face_recon(const double* fc, size_t nv, int k, const FaceGeo& g, double un,
                                            double& f0, double& sg)
 {
-    double fL = fc[g.cL * nv + k], fR = fc[g.cR * nv + k];
-    double sL = g.cLL >= 0 ? adj_vl((fL - fc[g.cLL * nv + k]) * g.rLLL, (fR - fL) * g.rLR) : 0.0;
-    double sR = g.cRR >= 0 ? adj_vl((fR - fL) * g.rLR, (fc[g.cRR * nv + k] - fR) * g.rRRR) : 0.0;
-    double faceL = fL + sL * g.hL, faceR = fR - sR * g.hR;
-    if (un > 0) { f0 = faceL; sg = sL; }
-    else if (un < 0) { f0 = faceR; sg = sR; }
-    else { f0 = 0.5 * (faceL + faceR); sg = 0.5 * (sL + sR); }
+    // only the side the velocity comes from is reconstructed (both where it is zero)
+    const double fL = fc[g.cL * nv + k], fR = fc[g.cR * nv + k], d = (fR - fL) * g.rLR;
+    double sL = 0.0, sR = 0.0;
+    if (un >= 0 && g.cLL >= 0) sL = adj_vl((fL - fc[g.cLL * nv + k]) * g.rLLL, d);
+    if (un <= 0 && g.cRR >= 0) sR = adj_vl(d, (fc[g.cRR * nv + k] - fR) * g.rRRR);
+    if (un > 0) { f0 = fL + sL * g.hL; sg = sL; }
+    else if (un < 0) { f0 = fR - sR * g.hR; sg = sR; }
+    else { f0 = 0.5 * ((fL + sL * g.hL) + (fR - sR * g.hR)); sg = 0.5 * (sL + sR); }
 }
 
 template <int N>
@@ -1225,7 +1226,7 @@ __global__ void __launch_bounds__(256) k_adj_objective(AdjDev A, int obj, int bc
 __global__ void __launch_bounds__(256) k_adj_dtheta(AdjDev A, int bcid, const int* __restrict__ faces,
                                                      const double* __restrict__ lam_, double* __restrict__ part)
 {
-    __shared__ double red[kRed * 4];
+    __shared__ double red[kRed * 5];
     const LevelDev& L = A.L;
     const VelDev& Vg = A.V;
     const int nv = Vg.nv, tid = threadIdx.x, bs = blockDim.x, nx = L.nx;

@@ -211,38 +211,7 @@ template <> struct Acc<float> {
 };
 
 // ---------------------------------------------------------------------------
-// deterministic block reduction of N doubles (fixed tree order); every thread
-// receives the result.  scratch: at least 32 * N doubles of shared memory.
-template <int N>
-__device__ __forceinline__ void block_sum(double (&v)[N], double* scratch)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    #pragma unroll
-    for (int q = 0; q < N; ++q) {
-        double x = v[q];
-        #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        v[q] = x;
-    }
-    __syncthreads();
-    if (lane == 0) {
-        #pragma unroll
-        for (int q = 0; q < N; ++q) scratch[warp * N + q] = v[q];
-    }
-    __syncthreads();
-    #pragma unroll
-    for (int q = 0; q < N; ++q) {
-        double s = 0.0;
-        for (int w = 0; w < nw; ++w) s += scratch[w * N + q];
-        v[q] = s;
-    }
-    __syncthreads();
-}
-
-// Block reduction of per-thread velocity sums into FP64 totals, broadcast to
-// every thread.  FP64 form: FP64 shuffle tree per warp.  Mixed form: each warp
-// reduces its Kahan pairs as float-float numbers (error-free TwoSum in FP32),
-// then warp 0 alone adds the per-warp totals in FP64.  scratch: 32 * N doubles.
+// error-free sum of two floats: a + b = s + e
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
 {
     s = a + b;
@@ -250,45 +219,119 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
     e = (a - (s - bb)) + (b - bb);
 }
 
+// Sums of N per-thread values over a warp: at every step a lane sends half of its
+// values and keeps the other half, so N values take about 1.4 N exchanges instead
+// of 5 N.  Afterwards the lane holds the sum of value `which` (none: which >= N).
+// FP32 values are float-float pairs throughout.
+template <int N>
+__device__ __forceinline__ double warp_sums(Acc<double> (&a)[N], int& which)
+{
+    const int lane = threadIdx.x & 31;
+    double v[N];
+    #pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = a[q].s;
+    which = 0;
+    int n = N, mine = N;              // slots in use, and how many of this lane's hold a value
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int h = (n + 1) / 2;
+        const bool up = n > 1 && (lane & o);             // with one value left: a plain exchange
+        #pragma unroll
+        for (int q = 0; q < N; ++q) {
+            if (q >= h) break;
+            const double hi = n == 1 ? v[q] : q + h < n ? v[q + h] : 0.0;
+            const double r = __shfl_xor_sync(0xffffffffu, up ? v[q] : hi, o);
+            v[q] = (up ? hi : v[q]) + r;
+        }
+        which += up ? h : 0;
+        mine = up ? mine - h : min(mine, h);
+        n = h;
+    }
+    if (mine <= 0) which = N;
+    return v[0];
+}
+template <int N>
+__device__ __forceinline__ float2 warp_sums(Acc<float> (&a)[N], int& which)
+{
+    const int lane = threadIdx.x & 31;
+    float vh[N], vl[N];
+    #pragma unroll
+    for (int q = 0; q < N; ++q) { vh[q] = a[q].s; vl[q] = -a[q].c; }
+    which = 0;
+    int n = N, mine = N;              // slots in use, and how many of this lane's hold a value
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int h = (n + 1) / 2;
+        const bool up = n > 1 && (lane & o);             // with one value left: a plain exchange
+        #pragma unroll
+        for (int q = 0; q < N; ++q) {
+            if (q >= h) break;
+            const float th = n == 1 ? vh[q] : q + h < n ? vh[q + h] : 0.0f, tl = n == 1 ? vl[q] : q + h < n ? vl[q + h] : 0.0f;
+            const float rh = __shfl_xor_sync(0xffffffffu, up ? vh[q] : th, o), rl = __shfl_xor_sync(0xffffffffu, up ? vl[q] : tl, o);
+            float s, e;
+            two_sum(up ? th : vh[q], rh, s, e);
+            vl[q] = (up ? tl : vl[q]) + rl + e;
+            vh[q] = s;
+        }
+        which += up ? h : 0;
+        mine = up ? mine - h : min(mine, h);
+        n = h;
+    }
+    if (mine <= 0) which = N;
+    return make_float2(vh[0], vl[0]);
+}
+// deterministic block reduction of N doubles (fixed tree order); every thread
+// receives the result.  scratch: (warps + 1) * N doubles of shared memory.
+template <int N>
+__device__ __forceinline__ void block_sum(double (&v)[N], double* scratch)
+{
+    const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    Acc<double> a[N];
+    #pragma unroll
+    for (int q = 0; q < N; ++q) a[q].s = v[q];
+    int which;
+    const double x = warp_sums<N>(a, which);
+    __syncthreads();
+    if (which < N) scratch[warp * N + which] = x;        // (lanes with the same value agree)
+    __syncthreads();
+    // one thread per value adds the warps' sums (an FP64 addition costs a warp as much as 32 of them)
+    if (threadIdx.x < N) {
+        double t = scratch[threadIdx.x];
+        for (int w = 1; w < nw; ++w) t += scratch[w * N + threadIdx.x];
+        scratch[nw * N + threadIdx.x] = t;
+    }
+    __syncthreads();
+    #pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = scratch[nw * N + q];
+    __syncthreads();
+}
+
+// Block reduction of per-thread velocity sums into FP64 totals, broadcast to
+// every thread.  FP64 form: block_sum.  Mixed form: float-float pairs (error-free
+// TwoSum) within the warps and over them, one conversion to FP64 per value at the
+// end.  scratch: (warps + 1) * N doubles.
 template <int N>
 __device__ __forceinline__ void block_total(Acc<float> (&a)[N], double* scratch, double (&out)[N])
 {
-    // float-float pairs all the way; one conversion to FP64 per value at the end
-    // (an FP64 instruction costs a warp as much as thirty-two lanes of it)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    float* fs = reinterpret_cast<float*>(scratch);    // [32][N][2] per-warp pairs
-    #pragma unroll
-    for (int q = 0; q < N; ++q) {
-        float hi = a[q].s, lo = -a[q].c;
-        #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+    const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    float2* fs = reinterpret_cast<float2*>(scratch);
+    int which;
+    const float2 v = warp_sums<N>(a, which);
+    if (which < N) fs[warp * N + which] = v;
+    __syncthreads();
+    if (threadIdx.x < N) {
+        float2 t = fs[threadIdx.x];
+        for (int w = 1; w < nw; ++w) {
+            const float2 r = fs[w * N + threadIdx.x];
             float s, e;
-            two_sum(hi, h2, s, e);
-            lo = lo + l2 + e;
-            hi = s;
+            two_sum(t.x, r.x, s, e);
+            t = make_float2(s, t.y + r.y + e);
         }
-        if (lane == 0) { fs[(warp * N + q) * 2] = hi; fs[(warp * N + q) * 2 + 1] = lo; }
-    }
-    __syncthreads();
-    if (warp == 0) {
-        #pragma unroll
-        for (int q = 0; q < N; ++q) {
-            float hi = lane < nw ? fs[(lane * N + q) * 2] : 0.0f, lo = lane < nw ? fs[(lane * N + q) * 2 + 1] : 0.0f;
-            #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-                float s, e;
-                two_sum(hi, h2, s, e);
-                lo = lo + l2 + e;
-                hi = s;
-            }
-            if (lane == q) scratch[32 * N - N + q] = (double)hi + (double)lo;
-        }
+        scratch[nw * N + threadIdx.x] = (double)t.x + (double)t.y;
     }
     __syncthreads();
     #pragma unroll
-    for (int q = 0; q < N; ++q) out[q] = scratch[32 * N - N + q];
+    for (int q = 0; q < N; ++q) out[q] = scratch[nw * N + q];
     __syncthreads();
 }
 

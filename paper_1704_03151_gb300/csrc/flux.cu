@@ -95,68 +95,7 @@ __device__ __forceinline__ float vl_limited(float s1, float s2)
     return p > 0.0f ? __fdividef(2.0f * p, s1 + s2) : 0.0f;
 }
 
-// Sums of N per-thread values over a warp: at every step a lane sends half of its
-// values and keeps the other half, so N values take about 1.4 N exchanges instead
-// of 5 N.  Afterwards the lane holds the sum of value `which` (none: which >= N).
-// FP32 values are float-float pairs throughout.
-template <int N>
-__device__ __forceinline__ double warp_sums(Acc<double> (&a)[N], int& which)
-{
-    const int lane = threadIdx.x & 31;
-    double v[N];
-    #pragma unroll
-    for (int q = 0; q < N; ++q) v[q] = a[q].s;
-    which = 0;
-    int n = N, mine = N;              // slots in use, and how many of this lane's hold a value
-    #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int h = (n + 1) / 2;
-        const bool up = n > 1 && (lane & o);             // with one value left: a plain exchange
-        #pragma unroll
-        for (int q = 0; q < N; ++q) {
-            if (q >= h) break;
-            const double hi = n == 1 ? v[q] : q + h < n ? v[q + h] : 0.0;
-            const double r = __shfl_xor_sync(0xffffffffu, up ? v[q] : hi, o);
-            v[q] = (up ? hi : v[q]) + r;
-        }
-        which += up ? h : 0;
-        mine = up ? mine - h : min(mine, h);
-        n = h;
-    }
-    if (mine <= 0) which = N;
-    return v[0];
-}
-template <int N>
-__device__ __forceinline__ float2 warp_sums(Acc<float> (&a)[N], int& which)
-{
-    const int lane = threadIdx.x & 31;
-    float vh[N], vl[N];
-    #pragma unroll
-    for (int q = 0; q < N; ++q) { vh[q] = a[q].s; vl[q] = -a[q].c; }
-    which = 0;
-    int n = N, mine = N;              // slots in use, and how many of this lane's hold a value
-    #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int h = (n + 1) / 2;
-        const bool up = n > 1 && (lane & o);             // with one value left: a plain exchange
-        #pragma unroll
-        for (int q = 0; q < N; ++q) {
-            if (q >= h) break;
-            const float th = n == 1 ? vh[q] : q + h < n ? vh[q + h] : 0.0f, tl = n == 1 ? vl[q] : q + h < n ? vl[q + h] : 0.0f;
-            const float rh = __shfl_xor_sync(0xffffffffu, up ? vh[q] : th, o), rl = __shfl_xor_sync(0xffffffffu, up ? vl[q] : tl, o);
-            float s, e;
-            two_sum(up ? th : vh[q], rh, s, e);
-            vl[q] = (up ? tl : vl[q]) + rl + e;
-            vh[q] = s;
-        }
-        which += up ? h : 0;
-        mine = up ? mine - h : min(mine, h);
-        n = h;
-    }
-    if (mine <= 0) which = N;
-    return make_float2(vh[0], vl[0]);
-}
-// ... and over the block: out[q] in shared memory, valid after the caller's next barrier
+// Sums over the block: out[q] in shared memory, valid after the caller's next barrier
 template <int N>
 __device__ __forceinline__ void block_sums(Acc<double> (&a)[N], double* scratch, double* out)
 {

@@ -1116,35 +1116,123 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
     const VelDev& Vg = M.V;
     const int c = blockIdx.x, nx = L.nx, nv = Vg.ld, i = c % nx, j = c / nx;   // rows with their padding
     const size_t nc = L.nc;
-    const bool vec = sizeof(F) == 4 && (nv & 3) == 0;   // 16-byte accesses over four velocities
-    if (acc) {
-        if (vec) {
-            for (int cp = 0; cp < 2; ++cp)
-                for (int g = threadIdx.x; g < nv / 4; g += blockDim.x) {
-                    const size_t id = (cp * nc + c) * nv + 4 * g;
-                    F xa[4], aa[4];
-                    ld4(x + id, xa);
-                    ld4(acc + id, aa);
-                    #pragma unroll
-                    for (int q = 0; q < 4; ++q) aa[q] = aa[q] + xa[q];
-                    st4(acc + id, aa);
+    constexpr int V16 = 16 / (int)sizeof(F);
+    const bool inner = renew && !L.solid[c] && L.fbx[j * (nx + 1) + i] < 0 && L.fbx[j * (nx + 1) + i + 1] < 0 &&
+                       L.fby[j * nx + i] < 0 && L.fby[(j + 1) * nx + i] < 0;
+    if (inner) {
+        // A cell without boundary faces.
+        const F* __restrict__ vu = VelT<F>::u(Vg);
+        const F* __restrict__ vv = VelT<F>::v(Vg);
+        const F itau = (F)M.inv_tau[c], rdxi = (F)L.rdx[i], rdyj = (F)L.rdy[j];
+        const size_t hoff = nc * (size_t)nv, xrow = (size_t)nx * nv;
+        const F* xb = x + (size_t)c * nv;
+        F* rb = r + (size_t)c * nv;
+        F* ab = acc ? acc + (size_t)c * nv : nullptr;
+        if constexpr (sizeof(F) == 4) {
+            // FP32 is bound by memory: all four neighbours are read, so that every load can be issued at
+            // once (choosing the two that a velocity sees first made the square cylinder's renewals
+            // 16.0 -> 21.6 ms per three iterations)
+            for (int k0 = threadIdx.x * V16; k0 < nv; k0 += blockDim.x * V16) {
+                F u[V16], v[V16], cW[V16], cE[V16], cS[V16], cN[V16], dg[V16];
+                ld16(vu + k0, u);
+                ld16(vv + k0, v);
+                #pragma unroll
+                for (int q = 0; q < V16; ++q) {
+                    dg[q] = itau + geomD_r<F>(rdxi, rdyj, u[q], v[q]);
+                    cW[q] = min(-u[q], F(0)) * rdxi;
+                    cE[q] = min(u[q], F(0)) * rdxi;
+                    cS[q] = min(-v[q], F(0)) * rdyj;
+                    cN[q] = min(v[q], F(0)) * rdyj;
                 }
-        } else {
-            // four velocities a block apart per thread: coalesced, eight loads in flight
-            const int bs = blockDim.x;
-            for (int cp = 0; cp < 2; ++cp)
-                for (int k0 = threadIdx.x; k0 < nv; k0 += 4 * bs) {
-                    const size_t id0 = (cp * nc + c) * nv + k0;
-                    F xa[4], aa[4];
+                #pragma unroll
+                for (int cp = 0; cp < 2; ++cp) {
+                    const F* p = xb + cp * hoff + k0;
+                    F xc[V16], xw[V16], xe[V16], xs[V16], xn[V16], rr[V16], aa[V16];
+                    ld16(p, xc);
+                    ld16(p - nv, xw);
+                    ld16(p + nv, xe);
+                    ld16(p - xrow, xs);
+                    ld16(p + xrow, xn);
+                    ld16(rb + cp * hoff + k0, rr);
+                    if (ab) ld16(ab + cp * hoff + k0, aa);
                     #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (k0 + q * bs < nv) { xa[q] = x[id0 + q * bs]; aa[q] = acc[id0 + q * bs]; }
-                    #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (k0 + q * bs < nv) acc[id0 + q * bs] = aa[q] + xa[q];
+                    for (int q = 0; q < V16; ++q) {
+                        F a = dg[q] * xc[q];
+                        a += cW[q] * xw[q];
+                        a += cE[q] * xe[q];
+                        a += cS[q] * xs[q];
+                        a += cN[q] * xn[q];
+                        rr[q] = rr[q] - a;
+                        aa[q] = ab ? aa[q] + xc[q] : F(0);
+                    }
+                    st16(rb + cp * hoff + k0, rr);
+                    if (ab) st16(ab + cp * hoff + k0, aa);
                 }
+            }
+            return;
         }
+        // FP64 is bound by its arithmetic: of its four neighbours a velocity sees the two it comes from, and
+        // the other two are neither read nor multiplied.  Where the velocities of an access (16 bytes) come
+        // from the same sides, which their index tells, the access is one group; else one by one.
+        // (64x64 cavity with 32x32 velocities 252 -> 158 us on the finest level, half-size square cylinder
+        // 22.0 -> 16.2 ms per two iterations)
+        const int nvv = Vg.nvv, nun = Vg.nleave[0][0], nvn = Vg.nleave[0][1];
+        for (int k0 = threadIdx.x * V16; k0 < Vg.nv; k0 += blockDim.x * V16) {
+            const int a = k0 / nvv, b = k0 - a * nvv;
+            if (b + V16 <= nvv && (b >= nvn || b + V16 <= nvn)) {
+                const F* pu = xb + k0 + (a < nun ? (long)nv : -(long)nv);
+                const F* pv = xb + k0 + (b < nvn ? (long)xrow : -(long)xrow);
+                F u[V16], v[V16], xc[2][V16], xu[2][V16], xv[2][V16], rr[2][V16], aa[2][V16];
+                #pragma unroll
+                for (int cp = 0; cp < 2; ++cp) {
+                    ld16(xb + cp * hoff + k0, xc[cp]);
+                    ld16(pu + cp * hoff, xu[cp]);
+                    ld16(pv + cp * hoff, xv[cp]);
+                    ld16(rb + cp * hoff + k0, rr[cp]);
+                    if (ab) ld16(ab + cp * hoff + k0, aa[cp]);
+                }
+                ld16(vu + k0, u);
+                ld16(vv + k0, v);
+                #pragma unroll
+                for (int q = 0; q < V16; ++q) {
+                    const F du = fabs(u[q]) * rdxi, dv = fabs(v[q]) * rdyj, dg = itau + (du + dv);
+                    #pragma unroll
+                    for (int cp = 0; cp < 2; ++cp) {
+                        rr[cp][q] -= fma(-dv, xv[cp][q], fma(-du, xu[cp][q], dg * xc[cp][q]));
+                        if (ab) aa[cp][q] += xc[cp][q];
+                    }
+                }
+                #pragma unroll
+                for (int cp = 0; cp < 2; ++cp) {
+                    st16(rb + cp * hoff + k0, rr[cp]);
+                    if (ab) st16(ab + cp * hoff + k0, aa[cp]);
+                }
+            } else {
+                #pragma unroll 1
+                for (int k = k0; k < min(k0 + V16, Vg.nv); ++k) {
+                    const F u = vu[k], v = vv[k], du = fabs(u) * rdxi, dv = fabs(v) * rdyj, dg = itau + (du + dv);
+                    const long ou = u < F(0) ? (long)nv : -(long)nv, ov = v < F(0) ? (long)xrow : -(long)xrow;
+                    for (int cp = 0; cp < 2; ++cp) {
+                        const F* p = xb + cp * hoff + k;
+                        rb[cp * hoff + k] -= fma(-dv, p[ov], fma(-du, p[ou], dg * p[0]));
+                        if (ab) ab[cp * hoff + k] += p[0];
+                    }
+                }
+            }
+        }
+        return;
     }
+    if (acc)
+        for (int cp = 0; cp < 2; ++cp)
+            for (int k0 = threadIdx.x * V16; k0 < nv; k0 += blockDim.x * V16) {
+                const size_t id = (cp * nc + c) * nv + k0;
+                F xa[V16], aa[V16];
+                ld16(x + id, xa);
+                ld16(acc + id, aa);
+                #pragma unroll
+                for (int q = 0; q < V16; ++q) aa[q] += xa[q];
+                st16(acc + id, aa);
+            }
     if (!renew || L.solid[c]) return;   // a body keeps a zero residual
     BFace bf[4];
     int nb = side_faces(L, i, j, 2, bf);
@@ -1177,80 +1265,6 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
     __syncthreads();
     F rho[4] = {srho[0], srho[1], srho[2], srho[3]};
     const F itau = sgeo[0], rdxi = sgeo[1], rdyj = sgeo[2];
-    if (vec && nb == 0) {
-        // interior cell: four velocities per thread, both components, 16-byte accesses
-        for (int g = threadIdx.x; g < nv / 4; g += blockDim.x) {
-            F u[4], v[4], cW[4], cE[4], cS[4], cN[4], dg[4];
-            ld4(vu + 4 * g, u);
-            ld4(vv + 4 * g, v);
-            #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                dg[q] = itau + geomD_r<F>(rdxi, rdyj, u[q], v[q]);
-                cW[q] = Dface<F>(0, -1, rdxi, u[q], v[q]);
-                cE[q] = Dface<F>(0, 1, rdxi, u[q], v[q]);
-                cS[q] = Dface<F>(1, -1, rdyj, u[q], v[q]);
-                cN[q] = Dface<F>(1, 1, rdyj, u[q], v[q]);
-            }
-            #pragma unroll
-            for (int cp = 0; cp < 2; ++cp) {
-                const size_t id = (cp * nc + c) * nv + 4 * g;
-                F xc[4], xw[4], xe[4], xs[4], xn[4], rr[4];
-                ld4(x + id, xc);
-                ld4(x + id - nv, xw);
-                ld4(x + id + nv, xe);
-                ld4(x + id - (size_t)nx * nv, xs);
-                ld4(x + id + (size_t)nx * nv, xn);
-                ld4(r + id, rr);
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    F a = dg[q] * xc[q];
-                    a += cW[q] * xw[q];
-                    a += cE[q] * xe[q];
-                    a += cS[q] * xs[q];
-                    a += cN[q] * xn[q];
-                    rr[q] = rr[q] - a;
-                }
-                st4(r + id, rr);
-            }
-        }
-        return;
-    }
-    if (nb == 0) {
-        // interior cell, any velocity count: four velocities a block apart per thread, so
-        // that every access is coalesced and 24 loads are in flight per thread (one
-        // velocity at a time leaves the cell's two DRAM streams latency-bound)
-        const int bs = blockDim.x;
-        for (int cp = 0; cp < 2; ++cp) {
-            const F* xb = x + cp * nc * nv;
-            F* rb = r + cp * nc * nv;
-            for (int k0 = threadIdx.x; k0 < nv; k0 += 4 * bs) {
-                F xc[4], xw[4], xe[4], xs[4], xn[4], rr[4];
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int k = k0 + q * bs;
-                    if (k < nv) {
-                        const size_t id = (size_t)c * nv + k;
-                        xc[q] = xb[id]; xw[q] = xb[id - nv]; xe[q] = xb[id + nv];
-                        xs[q] = xb[id - (size_t)nx * nv]; xn[q] = xb[id + (size_t)nx * nv]; rr[q] = rb[id];
-                    }
-                }
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int k = k0 + q * bs;
-                    if (k < nv) {
-                        const F u = vu[k], v = vv[k];
-                        F a = (itau + geomD_r<F>(rdxi, rdyj, u, v)) * xc[q];
-                        a += Dface<F>(0, -1, rdxi, u, v) * xw[q];
-                        a += Dface<F>(0, 1, rdxi, u, v) * xe[q];
-                        a += Dface<F>(1, -1, rdyj, u, v) * xs[q];
-                        a += Dface<F>(1, 1, rdyj, u, v) * xn[q];
-                        rb[(size_t)c * nv + k] = rr[q] - a;
-                    }
-                }
-            }
-        }
-        return;
-    }
     // interior neighbours (faces without a BC id)
     const bool hw = L.fbx[j * (nx + 1) + i] < 0, he = L.fbx[j * (nx + 1) + i + 1] < 0;
     const bool hs = L.fby[j * nx + i] < 0, hn = L.fby[(j + 1) * nx + i] < 0;
@@ -1302,77 +1316,59 @@ template <typename F>
 __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F* __restrict__ f, const F* __restrict__ df,
                                                         double* __restrict__ W, double* __restrict__ q)
 {
+    // Two passes over f + df: its moments, then, about the velocity they give, the heat flux, which also
+    // commits f + df.  W and q depend on the committed f alone, so that a state read back gives the same.
     __shared__ double red[32 * 4];
-    const int c = blockIdx.x, nv = Vg.nv;
-    const size_t nc = L.nc, ld = Vg.ld;
     __shared__ F sUV[2];
+    __shared__ int sok;
+    const int c = blockIdx.x, nv = Vg.nv, bs = blockDim.x;
+    const size_t nc = L.nc, ld = Vg.ld;
     F* fG = f + (size_t)c * ld;
     F* fH = f + (nc + c) * ld;
+    const F* dG = df ? df + (size_t)c * ld : nullptr;
+    const F* dH = df ? df + (nc + c) * ld : nullptr;
     const F* __restrict__ vu = VelT<F>::u(Vg);
     const F* __restrict__ vv = VelT<F>::v(Vg);
     const F* __restrict__ vw = VelT<F>::w(Vg);
-    __shared__ int sok;
-    // Each thread takes four velocities a block apart per round and issues all their
-    // loads before the arithmetic (the summation order is that of k = tid, tid + bs, ...).
-    const int bs = blockDim.x;
-    Acc<F> sa[4];
-    for (int k0 = threadIdx.x; k0 < nv; k0 += 4 * bs) {
-        F g[4], h[4];
+    // four velocities a block apart per round, their loads issued before the arithmetic
+    auto load = [&](int k0, bool with, F (&g)[4], F (&h)[4]) {
         #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = k0 + q * bs;
+        for (int t = 0; t < 4; ++t) {
+            const int k = k0 + t * bs;
+            g[t] = h[t] = F(0);
             if (k < nv) {
-                g[q] = fG[k]; h[q] = fH[k];
-                if (df) {
-                    g[q] = g[q] + df[(size_t)c * ld + k];
-                    h[q] = h[q] + df[(nc + c) * ld + k];
+                g[t] = fG[k]; h[t] = fH[k];
+                if (with) { g[t] += dG[k]; h[t] += dH[k]; }
+            }
+        }
+    };
+    double s[4];
+    auto moments = [&](bool with) {
+        Acc<F> sa[4];
+        for (int k0 = threadIdx.x; k0 < nv; k0 += 4 * bs) {
+            F g[4], h[4];
+            load(k0, with, g, h);
+            #pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int k = k0 + t * bs;
+                if (k < nv) {
+                    const F w = vw[k], u = vu[k], v = vv[k], wg = w * g[t], gu = wg * u, gv = wg * v;
+                    sa[0].add(wg); sa[1].add(gu); sa[2].add(gv);
+                    sa[3].add(fma(w, h[t], F(0.5) * fma(gu, u, gv * v)));
                 }
             }
         }
-        #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = k0 + q * bs;
-            if (k < nv) {
-                const F u = vu[k], v = vv[k], w = vw[k];
-                sa[0].add(w * g[q]); sa[1].add(w * u * g[q]); sa[2].add(w * v * g[q]);
-                sa[3].add(w * (F(0.5) * (u * u + v * v) * g[q] + h[q]));
-            }
-        }
-    }
-    double s[4];
-    block_total<4>(sa, red, s);
+        block_total<4>(sa, red, s);
+    };
+    moments(df != nullptr);
+    bool commit = df != nullptr;
     if (df) {
         // commit f + df, unless it would leave the cell with non-positive density or
         // internal energy: then the cell keeps f and its moments are those of f
         if (threadIdx.x == 0) sok = s[0] > 0.0 && s[3] * s[0] - 0.5 * (s[1] * s[1] + s[2] * s[2]) > 0.0;
         __syncthreads();
-        if (sok) {
-            for (int k0 = threadIdx.x; k0 < nv; k0 += 4 * bs) {
-                F g[4], h[4], dg[4], dh[4];
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int k = k0 + q * bs;
-                    if (k < nv) {
-                        g[q] = fG[k]; h[q] = fH[k];
-                        dg[q] = df[(size_t)c * ld + k]; dh[q] = df[(nc + c) * ld + k];
-                    }
-                }
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int k = k0 + q * bs;
-                    if (k < nv) { fG[k] = g[q] + dg[q]; fH[k] = h[q] + dh[q]; }
-                }
-            }
-        } else {
-            Acc<F> sb[4];
-            for (int k = threadIdx.x; k < nv; k += blockDim.x) {
-                const F g = fG[k], h = fH[k], u = vu[k], v = vv[k], w = vw[k];
-                sb[0].add(w * g); sb[1].add(w * u * g); sb[2].add(w * v * g);
-                sb[3].add(w * (F(0.5) * (u * u + v * v) * g + h));
-            }
-            block_total<4>(sb, red, s);
-        }
-        __syncthreads();
+        commit = sok;
+        if (!commit) moments(false);
     }
     if (threadIdx.x == 0) {
         const double ir = rcp64(s[0]);
@@ -1384,17 +1380,16 @@ __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F
     Acc<F> ta[2];
     for (int k0 = threadIdx.x; k0 < nv; k0 += 4 * bs) {
         F g[4], h[4];
+        load(k0, commit, g, h);
         #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (k0 + q * bs < nv) { g[q] = fG[k0 + q * bs]; h[q] = fH[k0 + q * bs]; }
-        #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = k0 + q * bs;
+        for (int t = 0; t < 4; ++t) {
+            const int k = k0 + t * bs;
             if (k < nv) {
-                F cx = vu[k] - fU, cy = vv[k] - fV;
-                F e = F(0.5) * (cx * cx + cy * cy) * g[q] + h[q];
-                ta[0].add(vw[k] * cx * e);
-                ta[1].add(vw[k] * cy * e);
+                if (commit) { fG[k] = g[t]; fH[k] = h[t]; }
+                const F cx = vu[k] - fU, cy = vv[k] - fV;
+                const F we = vw[k] * fma(F(0.5) * fma(cx, cx, cy * cy), g[t], h[t]);
+                ta[0].add(we * cx);
+                ta[1].add(we * cy);
             }
         }
     }
@@ -1411,7 +1406,8 @@ template <typename F>
 cudaError_t launch_update_moments(const LevelDev& L, const VelDev& V, F* f, const F* df, double* W, double* q,
                                   cudaStream_t st)
 {
-    k_update_moments<F><<<L.nc, V.nv >= 256 ? 256 : 128, 0, st>>>(L, V, f, df, W, q);
+    // FP64: fewer warps per cell, so that fewer repeat the reductions in the FP64 pipe
+    k_update_moments<F><<<L.nc, V.nv >= (sizeof(F) == 8 ? 2048 : 256) ? 256 : 128, 0, st>>>(L, V, f, df, W, q);
     return cudaGetLastError();
 }
 template <typename F>
