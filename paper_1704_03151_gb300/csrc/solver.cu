@@ -1944,8 +1944,10 @@ miugks_status sum_parts(miugks_solver* s, int nblk, int m, double* out)
 
 miugks_status vdots_n(miugks_solver* s, const double* Vb, int m, size_t n, const double* w, double* out)
 {
-    CK(launch_multi_dot(Vb, m, n, w, s->adj.part, kDotBlocks, s->st));
-    return sum_parts(s, kDotBlocks, m, out);
+    // at least 512 values per block: the partial sums go to the host
+    const int nblk = (int)std::min<size_t>(kDotBlocks, (n + 511) / 512);
+    CK(launch_multi_dot(Vb, m, n, w, s->adj.part, nblk, s->st));
+    return sum_parts(s, nblk, m, out);
 }
 
 miugks_status vdots(miugks_solver* s, const double* Vb, int m, const double* w, double* out)
