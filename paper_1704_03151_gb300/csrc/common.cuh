@@ -110,44 +110,6 @@ __device__ __forceinline__ float tau_of_f(const GasDev& g, float rho, float lam)
     return (float)g.mu_ref * powf(T, (float)g.omega) / (0.5f * rho * T);
 }
 
-// Time integrals of the UGKS integral solution over [0, dt] (x = dt/tau):
-// q[0..4] multiply g0, u_n a g0, A g0, f0, u_n sigma.  Series in x below 1.
-__device__ __forceinline__ void time_coeffs(double dt, double tau, double q[5])
-{
-    double x = dt / tau;
-    if (x < 1.0) {
-        // Horner-free explicit sums of the power series, terms x^n / n!
-        double pn = 1.0;             // x^n / n!
-        double s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0;
-        #pragma unroll 1
-        for (int n = 0; n < 26; ++n) {
-            double sg = (n & 1) ? -1.0 : 1.0;
-            s4 += sg * pn / (n + 1);                      // (-1)^n x^n/(n+1)!
-            // m = n + 1 terms use x^{m-1}/(m-1)! = pn
-            int m = n + 1;
-            s5 += -sg * pn / (m + 1);                     // (-1)^m m x^{m-1}/(m+1)! = (-1)^m x^{m-1}/((m+1) (m-1)!)
-            if (m >= 2) s2 += -sg * (1.0 - m) * pn / ((double)m * (m + 1));
-            double pn1 = pn * x / (n + 1);                // x^{n+1}/(n+1)!
-            // n+1 >= 1 terms of q1, q3
-            s1 += sg * pn1 / (n + 2);                     // (-1)^{n+2} x^{n+1}/(n+2)!
-            s3 += sg * pn1 / ((double)(n + 2) * (n + 3));
-            pn = pn1;
-        }
-        q[0] = dt * s1;
-        q[1] = dt * dt * s2;
-        q[2] = dt * dt * s3;
-        q[3] = dt * s4;
-        q[4] = dt * dt * s5;
-    } else {
-        double e = exp(-x), E1 = -expm1(-x);
-        q[0] = dt - tau * E1;
-        q[1] = -tau * dt * (1.0 + e) + 2.0 * tau * tau * E1;
-        q[2] = 0.5 * dt * dt - tau * dt + tau * tau * E1;
-        q[3] = tau * E1;
-        q[4] = tau * dt * e - tau * tau * E1;
-    }
-}
-
 // moments dw (already divided by rho) -> slope coefficients of a Maxwellian at (U, V, lam)
 template <typename T>
 __device__ __forceinline__ void micro_slope_t(const T dw[4], T U, T V, T lam, T a[4])
@@ -180,13 +142,6 @@ __device__ __forceinline__ double rcp64(double x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"((float)x));
     const double y = (double)s, e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
-}
-
-template <typename T>
-__device__ __forceinline__ T van_leer(T s1, T s2)
-{
-    T p = s1 * s2;
-    return p > T(0) ? T(2) * p / (s1 + s2) : T(0);
 }
 
 // ---------------------------------------------------------------------------

@@ -30,8 +30,6 @@
 #include <array>
 #include <type_traits>
 
-namespace cg = cooperative_groups;
-
 namespace miugks {
 
 // asynchronous 4- or 8-byte global -> shared copies (LDGSTS), completed per commit group
@@ -45,11 +43,6 @@ __device__ __forceinline__ void cp_async_elem(F* sdst, const F* gsrc)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gsrc) : "memory");
 }
 // (1/V) sum over the faces with u_n > 0 of u_n S = |u|/dx + |v|/dy
-template <typename F>
-__device__ __forceinline__ F geomD(const LevelDev& L, int i, int j, F u, F v)
-{
-    return fabs(u) * (F)L.rdx[i] + fabs(v) * (F)L.rdy[j];
-}
 template <typename F>
 __device__ __forceinline__ F geomD_r(F rdxi, F rdyj, F u, F v)
 {
@@ -229,27 +222,6 @@ __device__ __forceinline__ int side_faces(const LevelDev& L, int i, int j, int s
     if (side != 0 && e >= 0) bf[n++] = {e, 0, 1, L.rdx[i]};
     if (side != 0 && no >= 0) bf[n++] = {no, 1, 1, L.rdy[j]};
     return n;
-}
-
-// four consecutive values through 16-byte accesses (16-byte aligned for float, 32 for double)
-__device__ __forceinline__ void ld4(const float* p, float (&v)[4])
-{
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-}
-__device__ __forceinline__ void ld4(const double* p, double (&v)[4])
-{
-    const double2 t0 = *reinterpret_cast<const double2*>(p), t1 = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = t0.x; v[1] = t0.y; v[2] = t1.x; v[3] = t1.y;
-}
-__device__ __forceinline__ void st4(float* p, const float (&v)[4])
-{
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ void st4(double* p, const double (&v)[4])
-{
-    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
-    *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
 }
 
 // ---------------------------------------------------------------------------
