@@ -1550,9 +1550,8 @@ cudaError_t launch_multi_dot(const double* Vb, int m, size_t n, const double* w,
                              cudaStream_t st)
 {
     // Short vectors (the inner, macroscopic basis) would spend one block reduction after another on the
-    // m products: a CTA each.  Long ones are bound by memory, and one CTA per range reads w once.
-    // (inner basis
-    // of 32x32 cells, 4096 values: 19 -> 5 us on average, the adjoint solve there 0.93 -> 0.81 s)
+    // m products: a CTA each (32x32 cells, 4096 values: 19 -> 5 us on average, the adjoint solve there
+    // 0.93 -> 0.81 s).  From 2 MB on the products are bound by memory and the reductions do not show.
     const dim3 grid((unsigned)nblk, n < (1u << 18) ? (unsigned)m : 1u);
     k_multi_dot<<<grid, 256, 0, st>>>(Vb, m, n, w, part);
     return cudaGetLastError();
