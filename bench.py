@@ -245,15 +245,15 @@ def measure(precision, steps, warmup, world, rank, dev, with_e2e=True, with_ttr=
     return out
 
 
-# Dominant kernel of the step (largest share of the ncu launch list): the
-# prediction smoother's LU-SGS sweep, k_macro_sgs, on the finest level.
+# The kernel with the step's longest dependency chain: the prediction
+# smoother's LU-SGS sweep, k_macro_sgs, on the finest level.
 # Algorithmic bytes per cell and launch: reads W, R (4 doubles each), the
 # inverse diagonal (1), the Gamma of the faces (2 per cell), writes dW and W
 # (4 each): 19 doubles = 152 B.
 MACRO_BYTES_PER_CELL = 152.0
 # DRAM bytes (read + write) of one finest-level k_macro_sgs<float> launch from
-# the ncu capture summarised in profiles/k_macro_sgs_cavity64_v32_mixed.md
-MACRO_TRAFFIC_MIXED = 1.796352e6
+# the ncu capture summarised in profiles/k_kernels_cavity64_v32_mixed.md
+MACRO_TRAFFIC_MIXED = 0.91e6
 
 
 def macro_roofline(m, precision):
@@ -263,7 +263,8 @@ def macro_roofline(m, precision):
     return {"bound": "hbm", "kernel": "k_macro_sgs (finest level)", "achieved": gbs, "peak": hpeak, "unit": "GB/s",
             "frac": gbs / hpeak, "traffic": MACRO_TRAFFIC_MIXED if precision == "mixed" else None,
             "peak_source": hsrc, "launch_ms": m["macro_ms_per_launch"],
-            "limiter": "dependency chain: %d anti-diagonals per sweep, one halo exchange each" % (NX + NY - 1)}
+            "limiter": "dependency chain: %d anti-diagonals per sweep, strips of grid lines hand edge values on" %
+                       (NX + NY - 1)}
 
 
 def flux_roofline(m, precision, nx=None, ny=None, nv=None, traffic=None):
@@ -406,15 +407,15 @@ def measure_plate(steps, warmup):
 SWEEP_VALUES_PER_CV = 5
 # DRAM bytes per cell-velocity pair of the flat plate's finest-level sweep
 # kernels (mixed), from the ncu captures summarised in
-# profiles/k_sgs_plate128x96_v48_mixed.md (forward and backward launches)
-SWEEP_TRAFFIC_PER_CV = {"lines": 30.2, "wave": 29.8}
+# profiles/k_kernels_plate128x96_v48_mixed.md (forward and backward launches)
+SWEEP_TRAFFIC_PER_CV = {"wave": 21.8}
 # DRAM bytes (read + written) of one launch of the flat plate's face-flux kernel
-# (mixed, x-faces), from the ncu capture in profiles/k_face_flux_plate128x96_v48_mixed.md
-FLUX_TRAFFIC_PLATE_MIXED = 417.3e6
+# (mixed, x-faces), from the ncu capture in profiles/k_kernels_plate128x96_v48_mixed.md
+FLUX_TRAFFIC_PLATE_MIXED = 421.2e6
 # the same for one launch of the square cylinder's face flux (mixed, x-faces): the ncu capture of the half-size
-# case (80x60 cells, 4,860 x-faces, 580.9 MB; profiles/k_face_flux_square80x60_v89_mixed.md) scaled by the
+# case (80x60 cells, 4,860 x-faces, 631.1 MB; profiles/k_kernels_square80x60_v89_mixed.md) scaled by the
 # faces of the full case (19,320), since each face reads its cells' rows and writes its own fluxes
-FLUX_TRAFFIC_SQUARE_MIXED = 580.9e6 * 19320 / 4860
+FLUX_TRAFFIC_SQUARE_MIXED = 631.1e6 * 19320 / 4860
 
 
 def sweep_roofline(sk, precision):
@@ -423,13 +424,13 @@ def sweep_roofline(sk, precision):
     size = 4 if precision == "mixed" else 8
     hpeak, hsrc = hbm_peak()
     out = {}
-    for name in ("lines", "wave"):
+    for name in ("wave",):
         ms, n, units = sk[name]
         if n <= 0 or ms <= 0:
             continue
         gbs = SWEEP_VALUES_PER_CV * size * units / (ms * 1e-3) / 1e9
         tr = SWEEP_TRAFFIC_PER_CV[name]
-        out[name] = {"bound": "hbm", "kernel": "k_sgs_lines" if name == "lines" else "k_sgs_wave",
+        out[name] = {"bound": "hbm", "kernel": "k_sgs_wave",
                      "achieved": gbs, "peak": hpeak, "unit": "GB/s", "frac": gbs / hpeak,
                      "traffic": None if tr is None else tr * units / n, "peak_source": hsrc,
                      "launch_ms": ms / n, "cv_per_launch": units / n}
