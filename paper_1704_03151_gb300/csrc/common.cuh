@@ -264,7 +264,7 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double* scratch)
 // Block reduction of per-thread velocity sums into FP64 totals, broadcast to
 // every thread.  FP64 form: block_sum.  Mixed form: float-float pairs (error-free
 // TwoSum) within the warps and over them, one conversion to FP64 per value at the
-// end.  scratch: (warps + 1) * N doubles.
+// end; at most eight warps.  scratch: (warps + 1) * N doubles.
 template <int N>
 __device__ __forceinline__ void block_total(Acc<float> (&a)[N], double* scratch, double (&out)[N])
 {
@@ -275,14 +275,19 @@ __device__ __forceinline__ void block_total(Acc<float> (&a)[N], double* scratch,
     if (which < N) fs[warp * N + which] = v;
     __syncthreads();
     if (threadIdx.x < N) {
-        float2 t = fs[threadIdx.x];
-        for (int w = 1; w < nw; ++w) {
-            const float2 r = fs[w * N + threadIdx.x];
-            float s, e;
-            two_sum(t.x, r.x, s, e);
-            t = make_float2(s, t.y + r.y + e);
-        }
-        scratch[nw * N + threadIdx.x] = (double)t.x + (double)t.y;
+        // the warps' pairs (at most eight) as a tree, 4, 2 and 1 apart
+        float2 t[8];
+        #pragma unroll
+        for (int w = 0; w < 8; ++w) t[w] = w < nw ? fs[w * N + threadIdx.x] : make_float2(0.0f, 0.0f);
+        #pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+            #pragma unroll
+            for (int w = 0; w < o; ++w) {
+                float s, e;
+                two_sum(t[w].x, t[w + o].x, s, e);
+                t[w] = make_float2(s, t[w].y + t[w + o].y + e);
+            }
+        scratch[nw * N + threadIdx.x] = (double)t[0].x + (double)t[0].y;
     }
     __syncthreads();
     #pragma unroll

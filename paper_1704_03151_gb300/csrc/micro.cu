@@ -1290,6 +1290,8 @@ __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F
 {
     // Two passes over f + df: its moments, then, about the velocity they give, the heat flux, which also
     // commits f + df.  W and q depend on the committed f alone, so that a state read back gives the same.
+    // FP64 is bound by its products and shares their factors; in the mixed form each term keeps its own
+    // products and roundings, which the prediction amplifies from a marginally stable start.
     __shared__ double red[32 * 4];
     __shared__ F sUV[2];
     __shared__ int sok;
@@ -1324,9 +1326,15 @@ __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F
             for (int t = 0; t < 4; ++t) {
                 const int k = k0 + t * bs;
                 if (k < nv) {
-                    const F w = vw[k], u = vu[k], v = vv[k], wg = w * g[t], gu = wg * u, gv = wg * v;
-                    sa[0].add(wg); sa[1].add(gu); sa[2].add(gv);
-                    sa[3].add(fma(w, h[t], F(0.5) * fma(gu, u, gv * v)));
+                    const F w = vw[k], u = vu[k], v = vv[k];
+                    if constexpr (sizeof(F) == 8) {
+                        const F wg = w * g[t], gu = wg * u, gv = wg * v;
+                        sa[0].add(wg); sa[1].add(gu); sa[2].add(gv);
+                        sa[3].add(fma(w, h[t], F(0.5) * fma(gu, u, gv * v)));
+                    } else {
+                        sa[0].add(w * g[t]); sa[1].add(w * u * g[t]); sa[2].add(w * v * g[t]);
+                        sa[3].add(w * (F(0.5) * (u * u + v * v) * g[t] + h[t]));
+                    }
                 }
             }
         }
@@ -1359,9 +1367,15 @@ __global__ void __launch_bounds__(256) k_update_moments(LevelDev L, VelDev Vg, F
             if (k < nv) {
                 if (commit) { fG[k] = g[t]; fH[k] = h[t]; }
                 const F cx = vu[k] - fU, cy = vv[k] - fV;
-                const F we = vw[k] * fma(F(0.5) * fma(cx, cx, cy * cy), g[t], h[t]);
-                ta[0].add(we * cx);
-                ta[1].add(we * cy);
+                if constexpr (sizeof(F) == 8) {
+                    const F we = vw[k] * fma(F(0.5) * fma(cx, cx, cy * cy), g[t], h[t]);
+                    ta[0].add(we * cx);
+                    ta[1].add(we * cy);
+                } else {
+                    const F e = F(0.5) * (cx * cx + cy * cy) * g[t] + h[t];
+                    ta[0].add(vw[k] * cx * e);
+                    ta[1].add(vw[k] * cy * e);
+                }
             }
         }
     }
