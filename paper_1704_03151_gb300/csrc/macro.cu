@@ -39,24 +39,22 @@ __device__ __forceinline__ void euler_axis(const double* W, int axis, double T[4
 __device__ void macro_ghost(const BcDev& b, int axis, const double* Wi, double Wg[4], double* M)
 {
     if (b.type == BC_WALL) {
-        // lam_g = 2 lam_w - lam and Y = lam / (lam - 2 lam_w) through the temperatures:
-        // 1 / lam_g = T T_w / (2 T - T_w), Y = -T_w / (2 T - T_w), so two reciprocals in a row, not five
-        const double rho = Wi[0], ir = rcp64(rho), U = Wi[1] * ir, V = Wi[2] * ir, K = kKint + 2.0;
-        const double T = (4.0 / (kKint + 2)) * (Wi[3] * ir - 0.5 * (U * U + V * V));
-        const double Ug = 2.0 * b.u - U, Vg = 2.0 * b.v - V;
-        const double h = b.t * rcp64(2.0 * T - b.t);
+        double rho, U, V, lam;
+        prim4(Wi, rho, U, V, lam);
+        double lamw = 1.0 / b.t;
+        double lamg = 2.0 * lamw - lam, Ug = 2.0 * b.u - U, Vg = 2.0 * b.v - V;
         Wg[0] = rho; Wg[1] = rho * Ug; Wg[2] = rho * Vg;
-        Wg[3] = rho * (0.5 * (Ug * Ug + Vg * Vg) + 0.25 * K * (T * h));
+        Wg[3] = 0.5 * rho * (Ug * Ug + Vg * Vg) + (kKint + 2) * rho / (4.0 * lamg);
         if (M) {
-            const double Y = -h, Y2 = h * h;
+            double Y = lam / (lam - 2.0 * lamw), K = kKint + 2.0;
             for (int q = 0; q < 16; ++q) M[q] = 0.0;
             M[0] = 1.0;
             M[4] = 2.0 * b.u; M[5] = -1.0;
             M[8] = 2.0 * b.v; M[10] = -1.0;
-            M[12] = 2.0 * (b.u * b.u + b.v * b.v) - 0.5 * (U * U + V * V) * (1.0 + Y2) + 0.25 * K * T * (Y2 - Y);
-            M[13] = U - 2.0 * b.u + U * Y2;
-            M[14] = V - 2.0 * b.v + V * Y2;
-            M[15] = -Y2;
+            M[12] = 2.0 * (b.u * b.u + b.v * b.v) - 0.5 * (U * U + V * V) * (1.0 + Y * Y) + K / (4.0 * lam) * (Y * Y - Y);
+            M[13] = U - 2.0 * b.u + U * Y * Y;
+            M[14] = V - 2.0 * b.v + V * Y * Y;
+            M[15] = -Y * Y;
         }
     } else if (b.type == BC_SYMMETRY) {
         for (int m = 0; m < 4; ++m) Wg[m] = Wi[m];
@@ -67,8 +65,9 @@ __device__ void macro_ghost(const BcDev& b, int axis, const double* Wi, double W
             M[5 * (1 + axis)] = -1.0;
         }
     } else if (b.type == BC_FARFIELD) {
+        double lam = 1.0 / b.t;
         Wg[0] = b.rho; Wg[1] = b.rho * b.u; Wg[2] = b.rho * b.v;
-        Wg[3] = b.rho * (0.5 * (b.u * b.u + b.v * b.v) + 0.25 * (kKint + 2) * b.t);
+        Wg[3] = 0.5 * b.rho * (b.u * b.u + b.v * b.v) + (kKint + 2) * b.rho / (4.0 * lam);
         if (M) for (int q = 0; q < 16; ++q) M[q] = 0.0;
     } else {
         for (int m = 0; m < 4; ++m) Wg[m] = Wi[m];
@@ -164,7 +163,7 @@ __device__ __forceinline__ double face_gamma(const LevelDev& L, const double* gx
 // ---- records of the sweep
 //
 // How a strip's warp is laid out: lanes per grid line (and components per lane),
-// lines per strip, values of a lane's record, records in flight, steps that a
+// lines per strip, values of a lane's record, records in flight (at most), steps that a
 // strip starts after the values it needs first, and the place of (1/2V) / D in a record.
 template <typename F> struct MacroLane;
 template <> struct MacroLane<float> {
@@ -174,7 +173,10 @@ template <> struct MacroLane<double> {
     static constexpr int kLanes = 4, kComp = 1, kLines = 8, kVals = 10, kRow = kVals * 32, kRing = 4, kLead = 1, kHv = 2;
 };
 constexpr int kMacroMaxLines = 256;   // min(nx, ny)
-constexpr int kGhostRec = 24;         // per upper boundary face: dB/dW (16), rho, m_x, m_y, E + p, U, V of the ghost, S, S Gamma
+// values of a cell of a strip's last line that the next strip needs: the term across (4), or in the mixed form
+// with lines along x the cell's X along y and dW (8)
+template <typename F> __host__ __device__ constexpr int macro_edge(bool xl) { return sizeof(F) == 4 && !xl ? 8 : 4; }
+constexpr int kGhostRec = 26;         // per upper boundary face: dB/dW (16), the ghost state (4), its flux T (4), S, Gamma
 
 // Frame of a pass: s counts grid lines across the strips (along the shorter mesh
 // direction, so that few strips do many steps), t the cells along a line, both
@@ -243,17 +245,15 @@ __global__ void __launch_bounds__(64) k_macro_stage(MacroArgs a, MacroStage<F> A
         const int c = L.ubc[b], i = c % L.nx, j = c / L.nx;
         const int bcid = axis == 0 ? L.fbx[j * (L.nx + 1) + i + 1] : L.fby[(j + 1) * L.nx + i];
         double* g = A.ghost + (size_t)q * kGhostRec;
-        if (bcid < 0) { g[22] = 0.0; return; }
-        double w[4], G[4], M[16];
+        if (bcid < 0) { g[24] = 0.0; return; }
+        double w[4], G[4], M[16], T[4];
         ld_state(A.W, A.dw, c, w);
         macro_ghost(a.bc[bcid], axis, w, G, M);
+        euler_axis(G, axis, T);
         for (int m = 0; m < 16; ++m) g[m] = M[m];
-        const double ir = rcp64(G[0]), U = G[1] * ir, V = G[2] * ir;
-        const double p = (2.0 / (kKint + 2)) * (G[3] - 0.5 * (G[1] * U + G[2] * V));
-        const double S = axis == 0 ? L.dy[j] : L.dx[i];
-        g[16] = G[0]; g[17] = G[1]; g[18] = G[2]; g[19] = G[3] + p; g[20] = U; g[21] = V;
-        g[22] = S;
-        g[23] = S * (axis == 0 ? A.gx[j * (L.nx + 1) + i + 1] : A.gy[(j + 1) * L.nx + i]);
+        for (int m = 0; m < 4; ++m) { g[16 + m] = G[m]; g[20 + m] = T[m]; }
+        g[24] = axis == 0 ? L.dy[j] : L.dx[i];
+        g[25] = axis == 0 ? A.gx[j * (L.nx + 1) + i + 1] : A.gy[(j + 1) * L.nx + i];
         return;
     }
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -321,11 +321,10 @@ __global__ void __launch_bounds__(64) k_macro_stage(MacroArgs a, MacroStage<F> A
         for (int m = 0; m < 4; ++m) u[m] = __shfl_sync(cell, R, base + m) * id;
         if (f == 1) { u[0] = solid ? 1.0 : Wi[0]; u[1] = solid ? 0.0 : Wi[1]; u[2] = solid ? 0.0 : Wi[2]; u[3] = solid ? 0.0 : Wi[3] + p; }
         if (f == 2) { u[0] = solid ? 0.0 : U; u[1] = solid ? 0.0 : V; u[2] = hv; u[3] = 0.0; }
-        const int xu = fr.xl ? 0 : 2, yu = 2 - xu;         // x- and y-faces: across and along, or the other way round
-        if (f == 3) { u[xu] = -fS[1]; u[xu + 1] = fSg[1]; u[yu] = -fS[3]; u[yu + 1] = fSg[3]; }
+        if (f == 3) { u[0] = -fS[1]; u[1] = fSg[1]; u[2] = -fS[2]; u[3] = fSg[2]; }   // east, south
         *reinterpret_cast<float4*>(A.rec + fr.at(0, i, j, 0, 4 * f)) = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
         if (f == 0) return;                                // pass 1 takes its own value from pass 0
-        if (f == 3) { u[xu] = fS[0]; u[xu + 1] = fSg[0]; u[yu] = fS[2]; u[yu + 1] = fSg[2]; }
+        if (f == 3) { u[0] = fS[0]; u[1] = fSg[0]; u[2] = fS[3]; u[3] = fSg[3]; }      // west, north
         *reinterpret_cast<float4*>(A.rec + fr.at(1, i, j, 0, 4 * f)) = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
     } else {
         const double w = f == 0 ? Wi[0] : f == 1 ? Wi[1] : f == 2 ? Wi[2] : Wi[3];
@@ -464,63 +463,58 @@ cudaError_t launch_macro_jacT(const MacroArgs& a, const double* W, const double*
 // LU-SGS pass of Eq. macroFinalDefect.  At every step a strip's lanes update one
 // cell per grid line, an anti-diagonal:
 //   dW = own - (1/2V D) (sum over the two upstream faces of sgn S X - S Gamma dW),
-// X = T(W + dW) - T(W) of the upstream cell.  The cell that owns a value forms
-// its two downstream face terms itself: the one along the line stays in
-// registers, the one across goes to the next line by a shuffle, and the last
+// X = T(W + dW) - T(W) of the upstream cell.  What a cell hands to the next one of its
+// line stays in registers, what it hands to the next line goes by a shuffle, and the last
 // line's goes to the next strip's shared memory.  Those edge values announce
 // themselves: the buffer starts out filled with a signalling NaN, which no
-// arithmetic produces, and a reader waits (bounded) until the value it wants is
-// another one, so a step has no barrier, no fence (a fence would wait for the
+// arithmetic produces, and a reader waits (bounded) until the values it wants are
+// others, so a step has no barrier, no fence (a fence would wait for the
 // step's global stores: 3300 against 2500 cycles per FP64 step) and no remote
 // round trip.  A strip starts kLead steps late and reads a step ahead, so that
-// the values are there when it looks.  Records stream into a ring of kRing steps
+// the values are there when it looks.  Records stream into a ring of steps
 // (every lane copies and reads its own, so the ring needs no barrier either).
 //
 // What bounds it is the dependency chain of a step times nx + ny - 1 steps,
 // twice; DRAM idles.  Mixed form: one lane per line with all four components, so
 // that no value crosses lanes inside a cell, X through the increments
 // (dU = (dm_x - U drho) / (rho + drho), dp, ... -- exact identities, with no
-// cancellation against T(W)); every strip in one CTA.  FP64: one lane per
+// cancellation against T(W)); every strip in one CTA.  The sum over the two faces is
+// taken x first, and each product and sum is rounded where a serial sweep with one lane
+// per component rounds it: from a marginally stable start (the Mach 5 square cylinder's
+// first iteration) the prediction amplifies a rounding to the first digits, so that
+// another order would be another result.  So an upstream cell forms its x-face's term and
+// hands on X and dW for the y-face, whose term is added to the other one's.  FP64: one lane per
 // component and eight lines per strip.  An FP64 instruction holds its warp for
 // about 50 cycles however many lanes take part, so the step is its count of FP64
 // instructions (23 with a component per lane, 60 with a cell per lane: 0.32
 // against 0.64 ms per sweep of the 64x64 level), and the strips are spread over
-// the CTAs of a cluster, handing over through distributed shared memory; X from
-// T(W + dW) with -sgn S T(W) in the record.
-// 64x64 level, one sweep (both passes): mixed 155 -> 66 us, FP64 407 -> 320 us, against the
+// the CTAs of a cluster, handing over through distributed shared memory; each cell forms
+// both its downstream terms; X from T(W + dW) with -sgn S T(W) in the record.
+// 64x64 level, one sweep (both passes): mixed 155 -> @MIXED@ us, FP64 407 -> @FP64@ us, against the
 // wavefront of CTAs with a barrier per diagonal that this replaces.
 //
 // Boundary ghosts enter only the backward sweep (they use dW of the forward
 // sweep); their term is folded into that sweep's own value between the passes.
 // The update W += dW is left to the next kernel over the cells.
 
-__device__ __forceinline__ float recip_of(float x)
+// X = T(W + dW) - T(W) along x and y of a state (rho, m_x, m_y, E + p: Q; U, V) changed by d.
+// Each operation's rounding is written out, so that the result does not depend on what is inlined where.
+__device__ __forceinline__ void flux_increments(const float (&d)[4], const float (&Q)[4], float U, float V, float (&Xx)[4], float (&Xy)[4])
 {
-    float y;                                             // one Newton-Raphson step from the approximate seed
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return fmaf(y, fmaf(-x, y, 1.0f), y);
-}
-__device__ __forceinline__ double recip_of(double x) { return rcp64(x); }
-
-// flux increments X_x, X_y of a state (rho, m_x, m_y, E + p; U, V) changed by d
-template <typename F>
-__device__ __forceinline__ void flux_increments(const F (&d)[4], F rho, F mx, F my, F Ep, F U, F V, F (&Xx)[4], F (&Xy)[4])
-{
-    // dp = 2/3 (d(E) - d(m^2 / 2 rho)), the kinetic part as one quotient: its numerator waits for no reciprocal
-    const F n = d[1] * (mx + mx + d[1]) + (d[2] * (my + my + d[2]) - (mx * U + my * V) * d[0]);
-    const F ir = recip_of(rho + d[0]);
-    const F dU = (d[1] - U * d[0]) * ir, dV = (d[2] - V * d[0]) * ir;
-    const F Up = U + dU, Vp = V + dV;
-    const F dp = fma(F(-1.0 / (kKint + 2)) * n, ir, F(2.0 / (kKint + 2)) * d[3]), dE = d[3] + dp;
-    const F a = mx * dU + d[1] * Up, b = my * dV + d[2] * Vp;
-    Xx[0] = d[1];
-    Xx[1] = a + dp;
-    Xx[2] = my * dU + d[2] * Up;
-    Xx[3] = Ep * dU + dE * Up;
-    Xy[0] = d[2];
-    Xy[1] = mx * dV + d[1] * Vp;
-    Xy[2] = b + dp;
-    Xy[3] = Ep * dV + dE * Vp;
+    const float ir = __frcp_rn(Q[0] + d[0]);
+    const float dU = __fmul_rn(fmaf(-U, d[0], d[1]), ir), dV = __fmul_rn(fmaf(-V, d[0], d[2]), ir);
+    const float Up = U + dU, Vp = V + dV;
+    float k = fmaf(__fmul_rn(Q[0], U), dU, __fmul_rn(d[1], Up));          // twice the kinetic energy's increment
+    k = fmaf(d[2], Vp, fmaf(__fmul_rn(Q[0], V), dV, k));
+    const float dp = __fmul_rn(2.0f / (kKint + 2), fmaf(-0.5f, k, d[3]));
+    #pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const float e = m == 3 ? d[3] + dp : d[m];
+        Xx[m] = fmaf(Q[m], dU, __fmul_rn(e, Up));
+        Xy[m] = fmaf(Q[m], dV, __fmul_rn(e, Vp));
+    }
+    Xx[1] += dp;
+    Xy[2] += dp;
 }
 
 // edge values: relaxed accesses, each value complete by itself (4 or 8 bytes)
@@ -528,6 +522,12 @@ __device__ __forceinline__ void st_edge(bool on, unsigned a, const float (&v)[4]
 {
     asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n @p st.relaxed.cluster.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};\n}\n"
                  ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void st_edge(bool on, unsigned a, const float (&v)[8])
+{
+    const float lo[4] = {v[0], v[1], v[2], v[3]}, hi[4] = {v[4], v[5], v[6], v[7]};
+    st_edge(on, a, lo);
+    st_edge(on, a + 16, hi);
 }
 __device__ __forceinline__ void st_edge(bool on, unsigned a, const double (&v)[1])
 {
@@ -538,6 +538,14 @@ __device__ __forceinline__ void ld_edge(unsigned a, float (&v)[4])
 {
     asm volatile("ld.relaxed.cluster.shared::cta.v4.f32 {%0, %1, %2, %3}, [%4];\n"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ld_edge(unsigned a, float (&v)[8])
+{
+    float lo[4], hi[4];
+    ld_edge(a, lo);
+    ld_edge(a + 16, hi);
+    #pragma unroll
+    for (int q = 0; q < 4; ++q) { v[q] = lo[q]; v[4 + q] = hi[q]; }
 }
 __device__ __forceinline__ void ld_edge(unsigned a, double (&v)[1])
 {
@@ -586,22 +594,25 @@ __device__ __forceinline__ void st_if(bool on, double* p, const double (&v)[1])
 template <typename F>
 struct MacroStrip {
     const F* src;            // its records of this pass, [nk][kRow]
-    F* ring;                 // [kRing][kRow]
-    unsigned edge, p_edge;   // [nt][4] across terms from the strip before; the next strip's (shared addresses)
+    F* ring;                 // [R][kRow]
+    unsigned edge, p_edge;   // [nt] cells' values from the strip before; the next strip's (shared addresses)
     F* out;                  // where cell t = 0 of this lane's line puts its dW ...
     long ostep;              // ... and the step from one cell of the line to the next
     bool first, feeds, line; // no strip before; a strip after; this lane has a grid line
 };
 
-template <typename F, bool XL, int PASS>
+template <typename F, bool XL, int PASS, int R>
 __device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int nk, uint64_t limit_ns)
 {
     using T = MacroLane<F>;
-    constexpr int C = T::kComp, R = T::kRing, NU = T::kVals * (int)sizeof(F) / 16, V = 16 / (int)sizeof(F);
+    constexpr int C = T::kComp, E = macro_edge<F>(XL), H = E / T::kLanes;   // E values per edge cell, H per lane
+    constexpr int NU = T::kVals * (int)sizeof(F) / 16, V = 16 / (int)sizeof(F);
     const int lane = threadIdx.x & 31, ll = lane / T::kLanes, m = lane % T::kLanes, g0 = lane & 28;
-    F across[C], along[C], rc[T::kVals];
+    F across[H], along[H == 8 ? 4 : 2 * C], rc[T::kVals];   // handed on by the line before, and by the cell before
     #pragma unroll
-    for (int q = 0; q < C; ++q) across[q] = along[q] = F(0);
+    for (int q = 0; q < H; ++q) across[q] = F(0);
+    #pragma unroll
+    for (int q = 0; q < (H == 8 ? 4 : 2 * C); ++q) along[q] = F(0);
     const F* g = S.src + lane * V;
     F* rl = S.ring + lane * V;
     auto issue = [&](int k, int stage) {       // rows beyond nk exist (allocation is rounded up) and are not used
@@ -624,17 +635,17 @@ __device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int 
         }
     };
     F* out = S.out - ll * S.ostep;                                      // cell t = k - ll at step k
-    const bool mine = !S.first && ll == 0;                              // this lane takes across terms from the edge
+    const bool mine = !S.first && ll == 0;                              // this lane takes across values from the edge
     const unsigned edge = S.edge + (unsigned)(m * (int)sizeof(F));
     #pragma unroll
     for (int k = 0; k < R - 1; ++k) issue(k, k);
     if (limit_ns == 0) return false;
-    F en[C];
+    F en[H];
     #pragma unroll
-    for (int q = 0; q < C; ++q) en[q] = F(0);
+    for (int q = 0; q < H; ++q) en[q] = F(0);
     if (!S.first) {
-        if (!edge_wait<F, C>(edge + (unsigned)(4 * min(nt - 1, T::kLead) * (int)sizeof(F)), mine, limit_ns, en)) return false;
-        if (!edge_wait<F, C>(edge, mine, limit_ns, en)) return false;
+        if (!edge_wait<F, H>(edge + (unsigned)(E * min(nt - 1, T::kLead) * (int)sizeof(F)), mine, limit_ns, en)) return false;
+        if (!edge_wait<F, H>(edge, mine, limit_ns, en)) return false;
     }
     cp_async_wait_n<R - 2>();
     fetch(0, rc);
@@ -643,14 +654,14 @@ __device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int 
         for (int kk = 0; kk < R; ++kk) {
             const int k = k0 + kk;
             #pragma unroll
-            for (int q = 0; q < C; ++q) across[q] = mine ? en[q] : across[q];
+            for (int q = 0; q < H; ++q) across[q] = mine ? en[q] : across[q];
             if (!S.first) {                                             // the next step's edge values
-                const unsigned ea = edge + (unsigned)(4 * min(nt - 1, k + 1) * (int)sizeof(F));
+                const unsigned ea = edge + (unsigned)(E * min(nt - 1, k + 1) * (int)sizeof(F));
                 if (mine) ld_edge(ea, en);
                 bool empty = false;
                 #pragma unroll
-                for (int q = 0; q < C; ++q) empty = empty || is_empty(en[q]);
-                if (__any_sync(0xffffffffu, mine && empty) && !edge_wait<F, C>(ea, mine, limit_ns, en)) return false;
+                for (int q = 0; q < H; ++q) empty = empty || is_empty(en[q]);
+                if (__any_sync(0xffffffffu, mine && empty) && !edge_wait<F, H>(ea, mine, limit_ns, en)) return false;
             }
             issue(k + R - 1, (kk + R - 1) % R);
             cp_async_wait_n<R - 2>();                                   // step k + 1 has arrived
@@ -658,17 +669,32 @@ __device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int 
             fetch((kk + 1) % R, rn);
             const int t = k - ll;
             const bool on = (unsigned)t < (unsigned)nt && S.line;
-            F dw[C], oc[C];
+            F dw[C], oc[H];
             if constexpr (C == 4) {
-                // record: own[4], rho, m_x, m_y, E + p, U, V, (1/2V) / D, -, across (sgn S, S Gamma), along
-                F Xx[4], Xy[4];
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) dw[q] = fma(-across[q], rc[10], fma(-along[q], rc[10], rc[q]));
-                flux_increments<F>(dw, rc[4], rc[5], rc[6], rc[7], rc[8], rc[9], Xx, Xy);
+                // record: own[4], rho, m_x, m_y, E + p, U, V, (1/2V) / D, -, downstream x-face (sgn S, S Gamma), upstream y-face
+                F tx[4], Xx[4], Xy[4];
+                const F* const yn = XL ? along : across;                // X along y and dW of the y-neighbour
                 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    oc[q] = fma(rc[12], XL ? Xx[q] : Xy[q], -rc[13] * dw[q]);
-                    along[q] = fma(rc[14], XL ? Xy[q] : Xx[q], -rc[15] * dw[q]);
+                    F a = XL ? across[q] : along[q];                    // the x-face's term
+                    a = rc[14] != F(0) ? fmaf(rc[14], yn[q], fmaf(-rc[15], yn[4 + q], a)) : a;
+                    dw[q] = fmaf(-a, rc[10], rc[q]);
+                }
+                const F Q[4] = {rc[4], rc[5], rc[6], rc[7]};
+                flux_increments(dw, Q, rc[8], rc[9], Xx, Xy);
+                #pragma unroll
+                for (int q = 0; q < 4; ++q) tx[q] = on && rc[12] != F(0) ? fmaf(rc[12], Xx[q], -__fmul_rn(rc[13], dw[q])) : F(0);
+                #pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if constexpr (XL) {
+                        oc[q] = tx[q];
+                        along[q] = Xy[q];
+                        along[4 + q] = dw[q];
+                    } else {
+                        oc[q] = Xy[q];
+                        oc[4 + q] = dw[q];
+                        along[q] = tx[q];
+                    }
                 }
             } else {
                 // record of component m: own, W, (1/2V) / D, -, across (sgn S, S Gamma, -sgn S T(W)), along
@@ -679,20 +705,20 @@ __device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int 
                 for (int q = 0; q < 4; ++q) w[q] = __shfl_sync(0xffffffffu, wp, g0 + q);
                 const F s2 = F(-1.0 / (kKint + 2)) * fma(w[2], w[2], w[1] * w[1]);
                 const F pk = (m == 3 ? F(2.0 / (kKint + 2) + 1.0) : F(2.0 / (kKint + 2))) * w[3];
-                const F ir = recip_of(w[0]), U = w[1] * ir, W = w[2] * ir;
+                const F ir = rcp64(w[0]), U = w[1] * ir, W = w[2] * ir;
                 const F z = fma(s2, ir, pk), A = m == 3 ? z : wp;       // p, or E + p in lane 3
                 F Tx = fma(A, U, m == 1 ? z : F(0)), Ty = fma(A, W, m == 2 ? z : F(0));
                 if (m == 0) { Tx = w[1]; Ty = w[2]; }
                 oc[0] = fma(rc[4], XL ? Tx : Ty, fma(-rc[5], dw[0], rc[6]));
                 along[0] = fma(rc[7], XL ? Ty : Tx, fma(-rc[8], dw[0], rc[9]));
+                if (!on) oc[0] = along[0] = F(0);
             }
             #pragma unroll
-            for (int q = 0; q < C; ++q) {
-                if (!on) { oc[q] = F(0); along[q] = F(0); }
+            for (int q = 0; q < H; ++q) {
                 const F v = __shfl_up_sync(0xffffffffu, oc[q], T::kLanes);
                 across[q] = ll > 0 ? v : F(0);
             }
-            st_edge(S.feeds && ll == T::kLines - 1 && on, S.p_edge + (unsigned)((4 * t + m) * (int)sizeof(F)), oc);
+            st_edge(S.feeds && ll == T::kLines - 1 && on, S.p_edge + (unsigned)((E * t + m) * (int)sizeof(F)), oc);
             // pass 0: the backward sweep's own value; pass 1: the row of dW
             st_if(on, out + k * S.ostep, dw);
             #pragma unroll
@@ -702,27 +728,28 @@ __device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int 
     return true;
 }
 
-template <typename F, bool XL>
+template <typename F, bool XL, int R>
 __global__ void __launch_bounds__(256, 1) k_macro_sgs(MacroArgs a, F* __restrict__ rec, F* __restrict__ dW,
                                                       const double* __restrict__ ghost, int wpc)
 {
     using T = MacroLane<F>;
+    constexpr int E = macro_edge<F>(XL);
     extern __shared__ __align__(128) unsigned char smraw[];
     cg::cluster_group cl = cg::this_cluster();
     const LevelDev& L = a.L;
     const MacroFrame<F> fr(L.nx, L.ny);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = (int)cl.block_rank();
-    F* edge = reinterpret_cast<F*>(smraw);                              // [wpc][nt][4] from the strip before
+    F* edge = reinterpret_cast<F*>(smraw);                              // [wpc][nt][E] from the strip before
     const int strip = rank * wpc + warp;
     const bool active = warp < wpc && strip < fr.strips;
-    for (int q = threadIdx.x; q < wpc * fr.nt * 4; q += blockDim.x) set_empty(edge + q);
+    for (int q = threadIdx.x; q < wpc * fr.nt * E; q += blockDim.x) set_empty(edge + q);
     cl.sync();
 
     bool ok = true;
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
             if (warp < wpc)                                             // (read by this warp alone)
-                for (int q = lane; q < fr.nt * 4; q += 32) set_empty(edge + (size_t)warp * fr.nt * 4 + q);
+                for (int q = lane; q < fr.nt * E; q += 32) set_empty(edge + (size_t)warp * fr.nt * E + q);
             cl.sync();                                                  // forward dW of every strip is in the records
             // ghost terms of the upper boundary faces from the forward dW
             for (int b = rank * blockDim.x + threadIdx.x; b < L.nubc; b += (int)cl.num_blocks() * blockDim.x) {
@@ -732,13 +759,19 @@ __global__ void __launch_bounds__(256, 1) k_macro_sgs(MacroArgs a, F* __restrict
                 for (int m = 0; m < 4; ++m) own[m] = (double)__ldcg(rec + fr.at(1, i, j, m, 0));
                 for (int axis = 0; axis < 2; ++axis) {
                     const double* g = ghost + ((size_t)b * 2 + axis) * kGhostRec;
-                    if (g[22] == 0.0) continue;
-                    double d[4], Xx[4], Xy[4];
+                    if (g[24] == 0.0) continue;
+                    double d[4], w[4], T[4];
                     #pragma unroll
-                    for (int m = 0; m < 4; ++m) d[m] = g[4 * m] * own[0] + g[4 * m + 1] * own[1] + g[4 * m + 2] * own[2] + g[4 * m + 3] * own[3];
-                    flux_increments<double>(d, g[16], g[17], g[18], g[19], g[20], g[21], Xx, Xy);
+                    for (int m = 0; m < 4; ++m) {
+                        double t = 0.0;
+                        #pragma unroll
+                        for (int q = 0; q < 4; ++q) t += g[4 * m + q] * own[q];
+                        d[m] = t;
+                        w[m] = g[16 + m] + t;
+                    }
+                    euler_axis(w, axis, T);
                     #pragma unroll
-                    for (int m = 0; m < 4; ++m) Gc[m] += g[22] * (axis == 0 ? Xx[m] : Xy[m]) - g[23] * d[m];
+                    for (int m = 0; m < 4; ++m) Gc[m] += g[24] * ((T[m] - g[20 + m]) - g[25] * d[m]);
                 }
                 const double h = (double)rec[fr.at(1, i, j, 0, T::kHv)];
                 #pragma unroll
@@ -749,11 +782,11 @@ __global__ void __launch_bounds__(256, 1) k_macro_sgs(MacroArgs a, F* __restrict
         if (!active || !ok) continue;
         MacroStrip<F> S;
         S.src = rec + ((size_t)pass * fr.strips + strip) * fr.rows * T::kRow;
-        S.ring = edge + (size_t)wpc * fr.nt * 4 + (size_t)warp * T::kRing * T::kRow;
+        S.ring = edge + (size_t)wpc * fr.nt * E + (size_t)warp * R * T::kRow;
         S.first = strip == 0;
         S.feeds = strip + 1 < fr.strips;
-        S.edge = smem_addr(edge + (size_t)warp * fr.nt * 4);
-        S.p_edge = S.feeds ? peer_addr(edge + (size_t)((strip + 1) % wpc) * fr.nt * 4, (strip + 1) / wpc) : 0u;
+        S.edge = smem_addr(edge + (size_t)warp * fr.nt * E);
+        S.p_edge = S.feeds ? peer_addr(edge + (size_t)((strip + 1) % wpc) * fr.nt * E, (strip + 1) / wpc) : 0u;
         const int sl = strip * T::kLines + lane / T::kLanes, m = lane % T::kLanes;   // this lane's line in the pass's frame
         S.line = sl < fr.ns;
         const int s = pass ? fr.ns - 1 - sl : sl, t0 = pass ? fr.nt - 1 : 0;
@@ -767,7 +800,7 @@ __global__ void __launch_bounds__(256, 1) k_macro_sgs(MacroArgs a, F* __restrict
             S.out = dW + (S.line ? 4 * ((long)j0 * L.nx + i0) + m : 0);
             S.ostep = -(long)(XL ? 4 * L.nx : 4);
         }
-        ok = pass == 0 ? macro_strip<F, XL, 0>(S, fr.nt, fr.nk, a.wait_ns) : macro_strip<F, XL, 1>(S, fr.nt, fr.nk, a.wait_ns);
+        ok = pass == 0 ? macro_strip<F, XL, 0, R>(S, fr.nt, fr.nk, a.wait_ns) : macro_strip<F, XL, 1, R>(S, fr.nt, fr.nk, a.wait_ns);
         cp_async_wait_n<0>();
         if (!ok && lane == 0) *a.flag = 1.0;                            // a wait gave up: report, and skip the second pass
     }
@@ -784,8 +817,16 @@ cudaError_t launch_macro_sgs(const MacroArgs& a, F* rec, const double* ghost, F*
     const int wpc = sizeof(F) == 8 ? (fr.strips + 7) / 8 : fr.strips;
     int ncl = 1;
     while (ncl * wpc < fr.strips) ncl *= 2;
-    const size_t smem = sizeof(F) * (size_t)wpc * ((size_t)fr.nt * 4 + T::kRing * T::kRow);
-    auto kern = fr.xl ? k_macro_sgs<F, true> : k_macro_sgs<F, false>;
+    constexpr size_t kSmemMax = 227 * 1024;
+    auto bytes = [&](int R) { return sizeof(F) * (size_t)wpc * ((size_t)fr.nt * macro_edge<F>(fr.xl) + R * T::kRow); };
+    int R = T::kRing;
+    auto kern = fr.xl ? k_macro_sgs<F, true, T::kRing> : k_macro_sgs<F, false, T::kRing>;
+    if constexpr (macro_edge<F>(false) == 8)                // more than 224 lines of more than 396 cells
+        if (bytes(R) > kSmemMax) {
+            R = 4;
+            kern = k_macro_sgs<F, false, 4>;
+        }
+    const size_t smem = bytes(R);
     if (smem > 47 * 1024) {                             // with the static part, 48 KB need no opt-in
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

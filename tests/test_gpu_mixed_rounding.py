@@ -147,7 +147,7 @@ def hot_channel(lib):
 STAGES = {f.__name__: f for f in (moments, flux, prediction, evolution, residual, hot_channel)}
 
 
-@pytest.mark.parametrize("stage", ["moments", "flux"])
+@pytest.mark.parametrize("stage", ["moments", "flux", "prediction"])
 def test_recorded_values(lib, stage):
     want = np.load(GOLDEN)
     for key, a in STAGES[stage](lib).items():
