@@ -539,6 +539,9 @@ __device__ __forceinline__ void slope_mom(const F* a, F u, F v, F gM, F hM, F xi
 // Only the upwind side of a velocity is reconstructed (three cells of the four).  CACHE
 // keeps the face values and slopes in shared memory between the passes; without it (a
 // velocity grid whose cache leaves too few CTAs per SM) each pass reconstructs them.
+// Bound by the issue of its FP32 arithmetic.  Flux per iteration against reconstructing both
+// sides: square cylinder (89x89) 8.7 -> 6.1 ms, flat plate (48x48) 1.46 -> 1.03 ms, 64x64 cavity
+// (32x32) 0.26 -> 0.18 ms.
 template <bool CACHE>
 __global__ void __launch_bounds__(256, 4) k_face_flux_mixed(FaceFluxArgs<float> A)
 {
@@ -822,10 +825,10 @@ template <>
 cudaError_t launch_face_flux<float>(const FaceFluxArgs<float>& a, cudaStream_t st)
 {
     constexpr size_t kSmemMax = 227 * 1024;
-    // the cache pays while it leaves room for several CTAs per SM (64x64 cavity with 32x32 velocities
-    // 0.34 against 0.42 ms of flux per iteration, flat plate with 48x48 1.48 against 2.08 ms); beyond it
-    // (89x89) one CTA per face that reconstructs in each pass beats a face split over a cluster
-    // (8.7 against 11.8 ms); measured with both sides of a face reconstructed
+    // the cache pays while it leaves room for several CTAs per SM; beyond it (89x89) one CTA per face that
+    // reconstructs in each pass beats a face split over a cluster.  Measured with both sides of a face
+    // reconstructed, per iteration: 64x64 cavity with 32x32 velocities 0.34 with the cache, 0.42 ms without,
+    // flat plate with 48x48 1.48 and 2.08 ms, square cylinder 8.7 ms without and 11.8 ms split
     constexpr size_t kCacheMax = 64 * 1024;
     const size_t base = sizeof(double) * (256 + 48) + sizeof(float) * (64 + (size_t)a.V.nu + a.V.nvv);
     const size_t full = base + sizeof(float) * 4 * (size_t)a.V.nv;

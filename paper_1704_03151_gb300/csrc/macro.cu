@@ -473,6 +473,8 @@ cudaError_t launch_macro_jacT(const MacroArgs& a, const double* W, const double*
 // round trip.  A strip starts kLead steps late and reads a step ahead, so that
 // the values are there when it looks.  Records stream into a ring of steps
 // (every lane copies and reads its own, so the ring needs no barrier either).
+// A face that joins no two fluid cells has no term at all, whatever its coefficients
+// would multiply: at a strong shock an overflow ahead of a body must not pass through it.
 //
 // What bounds it is the dependency chain of a step times nx + ny - 1 steps,
 // twice; DRAM idles.  Mixed form: one lane per line with all four components, so
@@ -490,7 +492,7 @@ cudaError_t launch_macro_jacT(const MacroArgs& a, const double* W, const double*
 // against 0.64 ms per sweep of the 64x64 level), and the strips are spread over
 // the CTAs of a cluster, handing over through distributed shared memory; each cell forms
 // both its downstream terms; X from T(W + dW) with -sgn S T(W) in the record.
-// 64x64 level, one sweep (both passes): mixed 155 -> @MIXED@ us, FP64 407 -> @FP64@ us, against the
+// 64x64 level, one sweep (both passes): mixed 159 -> 92 us, FP64 415 -> 282 us, against the
 // wavefront of CTAs with a barrier per diagonal that this replaces.
 //
 // Boundary ghosts enter only the backward sweep (they use dW of the forward
@@ -709,9 +711,12 @@ __device__ __forceinline__ bool macro_strip(const MacroStrip<F>& S, int nt, int 
                 const F z = fma(s2, ir, pk), A = m == 3 ? z : wp;       // p, or E + p in lane 3
                 F Tx = fma(A, U, m == 1 ? z : F(0)), Ty = fma(A, W, m == 2 ? z : F(0));
                 if (m == 0) { Tx = w[1]; Ty = w[2]; }
+                // (a face without a coefficient is seen in the bits: a comparison would take the FP64 pipe)
+                const bool fa = on && __double2hiint(rc[4]) << 1 != 0, fl = on && __double2hiint(rc[7]) << 1 != 0;
                 oc[0] = fma(rc[4], XL ? Tx : Ty, fma(-rc[5], dw[0], rc[6]));
                 along[0] = fma(rc[7], XL ? Ty : Tx, fma(-rc[8], dw[0], rc[9]));
-                if (!on) oc[0] = along[0] = F(0);
+                if (!fa) oc[0] = F(0);
+                if (!fl) along[0] = F(0);
             }
             #pragma unroll
             for (int q = 0; q < H; ++q) {
