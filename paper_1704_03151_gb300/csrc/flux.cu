@@ -599,7 +599,8 @@ __global__ void __launch_bounds__(256, 4) k_face_flux_mixed(FaceFluxArgs<float> 
     const F* __restrict__ gL = fG + cL * ld;
     const F* __restrict__ hL = fH + cL * ld;
     const int oR = (cR - cL) * Vg.ld, oLL = cLL >= 0 ? -oR : 0, oRR = cRR >= 0 ? 2 * oR : oR;
-    // face value f0 and slope sg of G and H of velocity k, reconstructed in its upwind cell (van Leer)
+    // face value f0 and slope sg of G and H of velocity k, reconstructed in its upwind cell (van Leer); the sum of the
+    // slopes is rounded once, the inner product fused into it, where the value is kept, and from both products else
     auto recon = [&](int k, F (&f0)[2], F (&sg)[2]) {
         const F un = axis == 0 ? vu[k] : vv[k];
         const bool neg = un < F(0);
@@ -609,7 +610,7 @@ __global__ void __launch_bounds__(256, 4) k_face_flux_mixed(FaceFluxArgs<float> 
         for (int cp = 0; cp < 2; ++cp) {
             const F* fc = (cp == 0 ? gL : hL) + k;
             const F fu = fc[o0], d1 = fu - fc[om], d2 = fc[op] - fu, s1 = __fmul_rn(d1, rm), s2 = __fmul_rn(d2, rp);
-            sg[cp] = vl_limited(s1, s2, fmaf(d2, rp, s1));
+            sg[cp] = vl_limited(s1, s2, CACHE ? fmaf(d2, rp, s1) : s1 + s2);
             f0[cp] = fmaf(sg[cp], h, fu);
         }
         if (un == F(0)) {                        // the mean of both sides
@@ -617,7 +618,7 @@ __global__ void __launch_bounds__(256, 4) k_face_flux_mixed(FaceFluxArgs<float> 
             for (int cp = 0; cp < 2; ++cp) {
                 const F* fc = (cp == 0 ? gL : hL) + k;
                 const F fu = fc[oR], d1 = fc[oRR] - fu, d2 = fu - fc[0], s1 = __fmul_rn(d1, r3), s2 = __fmul_rn(d2, r2);
-                const F s = vl_limited(s1, s2, fmaf(d2, r2, s1));
+                const F s = vl_limited(s1, s2, CACHE ? fmaf(d2, r2, s1) : s1 + s2);
                 f0[cp] = F(0.5) * (f0[cp] + fmaf(-s, fhR, fu));
                 sg[cp] = F(0.5) * (sg[cp] + s);
             }

@@ -88,6 +88,8 @@ def flux(lib):
     for name, c in (("box", box(4, 3, (W, S, F, O), 17, 13, vmax=15.0)), ("body", body())):
         R, px, py = fast_flow(lib, c).stage_flux()
         out.update({name + "_R": R, name + "_x": px, name + "_y": py})
+    # too many velocities for the cache between the passes: the residual holds the sums of every flux
+    out["large_R"] = fast_flow(lib, box(3, 2, (W, S, F, O), 63, 64, vmax=15.0)).stage_flux()[0]
     return out
 
 
