@@ -33,6 +33,9 @@ struct VelDev {
     // through a boundary face on the sweep side (u_n > 0): the first ones of the
     // axis in pass 0, the last ones in pass 1
     int nleave[2][2];
+    // wall sums of the line cells (k_line_rho): velocities and weights w u_n (storage type) of the chains' steps
+    const int* chain;
+    const void* wchain;
 };
 
 // one grid level (all device pointers)

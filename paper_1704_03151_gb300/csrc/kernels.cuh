@@ -92,15 +92,16 @@ cudaError_t launch_sub(double* out, const double* a, const double* b, size_t n, 
 // bodies.  Each such cell has a fold entry e (its ghost-folded inputs).
 struct SweepPlanDev {
     const int* code[2];     // per cell: -1 ordinary, -2 in a body, else its fold entry
-    const int4* lcell[2];   // per fold entry: {cell, line axis (0 x-face, 1 y-face), the face's bc id, corner}
-    const int* lines[2];    // lines: [q][8] = {i0, j0, di, dj, len, line axis, entry of cell 0, has symmetry faces};
+    const int4* lcell[2];   // per fold entry: {cell, line axis (0 x-face, 1 y-face), the face's bc id, 0 at the corner}
+    const int4* lsum[2];    // per fold entry, of its wall sum: {place in VelDev::chain, shares (0: no wall), steps, 0}
+    int shares[2];          // most shares of an edge cell's wall sum (0: no walls there)
+    const int* lines[2];    // lines: [q][8] = {i0, j0, di, dj, len, line axis, entry of cell 0, 0};
                             // 0 the edge column, 1 the edge row, then the lines along bodies
     int nl[2];              // fold entries of the edge lines (the rest belong to body lines)
     int nl_max;             // fold entries (larger pass)
     int bodies;             // the level has solid cells
-    int sym[2];             // bit q: edge line q has symmetry faces
     int cbc[2][2];          // boundary ids of the corner cell's x- and y-face
-    int general[2];         // a line has symmetry faces, or the corner a symmetry or outflow face
+    int general[2];         // the corner has a symmetry or outflow face
 };
 constexpr int kMaxBodyLines = 64;   // lines along bodies per pass and level
 struct MicroArgs {
@@ -115,15 +116,13 @@ template <typename F>
 struct SweepScratch {
     F* corner;   // [2][ld] corner cell of the pass
     F* rho;      // [nl] wall densities of the line cells
-    F* part;     // [2 + body lines][chunks][kMaxLine] partial wall sums
     F* fold;     // [velocity blocks][nl][3][block] inputs of the line cells
-    F* xline;    // [nl][2][ld] leaving values on lines with symmetry faces
-    int* count;  // [2 + body lines] CTAs done per line (zero between launches)
+    F* xline;    // [nl][2][ld] leaving values of the line cells
     int nl;
 };
 // Host schedule of the body lines of one pass: after wave step dd - 1, the lines
 // q0 .. q0 + nq - 1 (fold entries e0 .. e0 + ne - 1) are walked and folded.
-struct SweepBreak { int dd, q0, nq, e0, ne; };
+struct SweepBreak { int dd, q0, nq, e0, ne, shares; };   // (shares: the most of their wall sums)
 // Timing mode: event pairs around the launches of the wavefront kernel, with the
 // cell-velocity pairs each launch sweeps.
 struct SweepTimer {
@@ -131,10 +130,10 @@ struct SweepTimer {
     std::vector<double> units;
     int used = 0;
 };
-// timer: null unless the launches are to be timed; nl, nlines, nchunk, count: the scratch's layout
+// timer: null unless the launches are to be timed; nl: the scratch's layout
 struct SweepPlanHost {
     const SweepBreak* brk[2]; int nbrk[2]; SweepTimer* timer;
-    int nl, nlines, nchunk; int* count;
+    int nl;
 };
 // Step 3-4: r = (g~ - f)/tau~ - div(ph) on level 0; also inv_tau (with dtn_inv) and invD
 template <typename F>
@@ -147,9 +146,8 @@ cudaError_t launch_coarse_coeffs(const MicroArgs& m, GasDev gas, const double* W
                                  double* inv_tau, F* invD, cudaStream_t st);
 // one symmetric Gauss-Seidel pass: x = SGS(r).  Zw[b*4 + axis*2 + (outsign>0)] = sum over the
 // incoming velocities of w u_n C_k of wall BC b; scratch: micro_scratch_elems values
-// (nl, nlines: the largest over the levels)
-size_t micro_scratch_elems(int ld, int nl, int nlines, int nchunk, bool sym);
-int micro_edge_chunks(const VelDev& V);   // CTAs per line of the line walk
+// (nl: the largest over the levels)
+size_t micro_scratch_elems(int ld, int nl);
 // *out = sum of a[q]^2 over n values; part: scratch of 128 doubles
 template <typename T>
 cudaError_t launch_sumsq(const T* a, size_t n, double* part, double* out, cudaStream_t st);

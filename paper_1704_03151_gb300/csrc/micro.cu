@@ -15,15 +15,19 @@
 // same holds for the last column and row in the backward sweep.  At a line
 // cell, the velocities leaving through the boundary face (outgoing) need no
 // ghost, and the incoming ones need only the cell's wall density, a sum over
-// the outgoing ones.  Each sweep is therefore two launches:
-//   * k_sgs_edge walks the lines for their outgoing velocities and sums up the
-//     wall densities;
+// the outgoing ones.  Each sweep is therefore three launches:
+//   * k_sgs_edge walks the lines for their outgoing velocities;
+//   * k_line_rho sums up the wall densities of their cells;
 //   * k_sgs_wave sweeps all cells, every CTA for its own velocities and with
 //     no synchronisation between CTAs; the incoming velocities of line cells
 //     are ordinary updates there, their ghost term being known.
+// Which products are fused into sums, and the order of the wall sums, are written
+// out: the mixed form's roundings are part of its result, since a marginally stable
+// flow (a hot channel under the F cycle) amplifies them from one iteration to the next.
 //
-// Rows of velocities are padded to a multiple of eight (VelDev::ld), so that
-// every cell's row starts on a 32-byte sector; the padding is zero and stays so.
+// Rows of velocities are padded to a multiple of sixteen (VelDev::ld), four lanes
+// of 16 bytes in FP32, so that a block of the wavefront never leaves its row; the
+// padding is zero and stays so.
 #include "kernels.cuh"
 #include "async.cuh"
 #include <algorithm>
@@ -42,11 +46,15 @@ __device__ __forceinline__ void cp_async_elem(F* sdst, const F* gsrc)
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gsrc) : "memory");
 }
+// a product that is not fused into a sum
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+
 // (1/V) sum over the faces with u_n > 0 of u_n S = |u|/dx + |v|/dy
 template <typename F>
 __device__ __forceinline__ F geomD_r(F rdxi, F rdyj, F u, F v)
 {
-    return fabs(u) * rdxi + fabs(v) * rdyj;
+    return fma(fabs(u), rdxi, mul_rn(fabs(v), rdyj));
 }
 
 // coefficient (1/V) u_n S of a neighbour (or ghost) through the face with outward normal
@@ -247,15 +255,10 @@ __device__ __forceinline__ void st16(double* p, const double* v) { *reinterpret_
 // Walk of boundary lines.  On the sweep side of a pass, the cells of a line
 // each have one boundary face of the same orientation (the domain edge's column
 // and row, and runs along bodies).  A velocity that leaves through that face is
-// coupled only along the line, and the wall density of a cell is a sum over the
-// leaving velocities: one thread per line and leaving velocity walks the line
-// (inputs streamed RA cells ahead by asynchronous copies), and the contributions
-// of RA cells at a time are summed over the CTA's velocities through shared
-// memory; the last CTA of a line to finish adds the CTAs' sums in order and
-// publishes rho = -sum / Z per cell.  Nothing is written to x: the wavefront
-// recomputes the leaving velocities as ordinary cells and takes the densities.
-// Where a line has a symmetry face, the leaving values themselves are kept (the
-// mirrored ghosts are made of them).
+// coupled only along the line: one thread per line and leaving velocity walks the
+// line (inputs streamed RA cells ahead by asynchronous copies) and keeps the values
+// in S.xline, from which the wall densities (k_line_rho), the mirrored ghosts of
+// symmetry faces and the line cells' final values are taken.
 //
 // Edge lines start in the corner cell, whose two faces couple its velocities
 // (a 2x2 system for two walls, substitution otherwise): every CTA solves it for
@@ -264,47 +267,43 @@ __device__ __forceinline__ void st16(double* p, const double* v) { *reinterpret_
 // has finished.
 //
 // Bound by latency: the corner, then one load latency and a short recurrence per
-// RA cells.  64x64 cavity, 32x32 velocities, mixed: 14 us, against 34 us for the walk
-// by clusters of eight CTAs that this replaces (with its fold launch).
+// RA cells.  64x64 cavity, 32x32 velocities, mixed: 17 us, and 5 us for the wall sums, against 34 us
+// for the walk by clusters of eight CTAs with its fold launch that this replaces.
 template <typename F> struct EdgeRing { static constexpr int RA = 128 / (int)sizeof(F); };
 
-// GENERAL: symmetry faces on the lines, or a symmetry or outflow face at the corner
-// (without them the code is half as long, and a short kernel is mostly instruction fetches).
+// GENERAL: a symmetry or outflow face at the corner (without them the code is half as
+// long, and a short kernel is mostly instruction fetches).
 template <typename F, bool GENERAL>
 __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __restrict__ Zw, const F* __restrict__ invD,
                                                   const F* __restrict__ r, const F* __restrict__ x, SweepScratch<F> S,
                                                   int pass, int q0, int nchunk)
 {
-    constexpr int RA = EdgeRing<F>::RA, U = 8, NB = RA / U, B = 128, TP = B / RA, TS = B + 4;
+    constexpr int RA = EdgeRing<F>::RA, U = 8, NB = RA / U, B = 128;
     extern __shared__ __align__(16) unsigned char esm[];
     F* ring = reinterpret_cast<F*>(esm);              // [RA][3][B]
-    F* tile = ring + RA * 3 * B;                      // [RA][TS] contributions to the wall sums
-    __shared__ F nbS[kMaxLine], zf[kMaxLine];
-    __shared__ F red[4][4];
-    __shared__ int last;
+    __shared__ F nbS[kMaxLine], itS[kMaxLine];
+    __shared__ F red[32][4];
     const LevelDev& L = M.L;
     const VelDev& V = M.V;
-    const int nx = L.nx, ny = L.ny, nv = V.nv, tid = threadIdx.x;
+    const int nx = L.nx, ny = L.ny, nv = V.nv, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const size_t nc = L.nc, ld = V.ld;
     const F* __restrict__ vu = VelT<F>::u(V);
     const F* __restrict__ vv = VelT<F>::v(V);
     const F* __restrict__ vw = VelT<F>::w(V);
-    const double* __restrict__ iZw = Zw + 4 * kMaxBcs;
     const int q = q0 + (int)blockIdx.x / nchunk, chunk = (int)blockIdx.x % nchunk;
     // the line; the edge's two follow from the mesh (a load less before the first inputs can be asked for)
     const bool edge = q < 2;
     int i0 = pass == 0 ? 0 : nx - 1, j0 = pass == 0 ? 0 : ny - 1, di = q == 1 ? (pass == 0 ? 1 : -1) : 0,
         dj = q == 0 ? (pass == 0 ? 1 : -1) : 0, len = q == 0 ? ny : nx, axis = q, ebase = q == 0 ? 0 : ny;
-    bool sym = GENERAL && edge && (M.P.sym[pass] >> (q & 1) & 1);
     if (!edge) {
         const int* ln = M.P.lines[pass] + 8 * q;
         i0 = ln[0]; j0 = ln[1]; di = ln[2]; dj = ln[3]; len = ln[4]; axis = ln[5]; ebase = ln[6];
-        sym = GENERAL && ln[7] != 0;
     }
     const long c0 = (long)j0 * nx + i0, cstep = (long)dj * nx + di;
     const F* src = pass == 0 ? r : x;
-    // the velocities that leave: nodes ascend, so the first (pass 0) or last ones of that axis
-    const int v = chunk * B + tid, nl1 = V.nleave[pass][axis], other = axis == 0 ? V.nvv : V.nu;
+    // the velocities that leave (zero ones among them): nodes ascend, so the first (pass 0) or last ones of that axis
+    const int naxis = axis == 0 ? V.nu : V.nvv, nl1 = naxis - V.nleave[1 - pass][axis], other = axis == 0 ? V.nvv : V.nu;
+    const int v = chunk * B + tid;
     const bool on = v < nl1 * other;
     int k = 0;
     if (on) {
@@ -320,7 +319,7 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
             if (1 + U * b + u < len && on) {
                 cp_async_elem(d + u * 3 * B, pi);
                 cp_async_elem(d + u * 3 * B + B, ps);
-                if (sym) cp_async_elem(d + u * 3 * B + 2 * B, ps + nc * ld);
+                cp_async_elem(d + u * 3 * B + 2 * B, ps + nc * ld);
             }
             pi += pst;
             ps += pst;
@@ -328,14 +327,10 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
         cp_async_commit();
     };
     for (int b = 0; b < NB - 1; ++b) issue(b);
-    // what the end of the walk needs per cell, asked for early: 1/d along the line and the boundary id
-    int zb[kMaxLine / B];
-    #pragma unroll
-    for (int t = 0; t < kMaxLine / B; ++t) {
-        const int st = tid + t * B;
-        zb[t] = -1;
-        if (st < len && (st > 0 || edge)) zb[t] = M.P.lcell[pass][ebase + st].z;
-        if (st < len) nbS[st] = (F)(axis == 0 ? L.rdy[j0 + st * dj] : L.rdx[i0 + st * di]);
+    // per cell: 1/d along the line and the collision frequency, asked for early
+    for (int st = tid; st < len; st += B) {
+        nbS[st] = (F)(axis == 0 ? L.rdy[j0 + st * dj] : L.rdx[i0 + st * di]);
+        itS[st] = (F)M.inv_tau[c0 + st * cstep];
     }
     F xp[2] = {F(0), F(0)};
     if (edge) {
@@ -343,208 +338,253 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
         const int c = pass == 0 ? 0 : (int)nc - 1, ci = pass == 0 ? 0 : nx - 1, cj = pass == 0 ? 0 : ny - 1;
         const int bc0 = M.P.cbc[pass][0], bc1 = M.P.cbc[pass][1];
         const BcDev B0 = M.bc[bc0], B1 = M.bc[bc1];
-        const double* __restrict__ C0 = M.Cw + (size_t)bc0 * nv;
-        const double* __restrict__ C1 = M.Cw + (size_t)bc1 * nv;
-        const double z0 = iZw[bc0 * 4 + pass], z1 = iZw[bc1 * 4 + 2 + pass];
         const F rx = (F)L.rdx[ci], ry = (F)L.rdy[cj], itau = (F)M.inv_tau[c];
-        const F h0 = (F)(kKint * B0.t / 4.0), h1 = (F)(kKint * B1.t / 4.0);
-        const bool w0 = B0.type == BC_WALL, w1 = B1.type == BC_WALL;
+        const bool w0 = B0.type == BC_WALL, w1 = B1.type == BC_WALL, two = w0 && w1;
         const bool y0 = GENERAL && B0.type == BC_SYMMETRY, y1 = GENERAL && B1.type == BC_SYMMETRY;
         const bool o0 = GENERAL && B0.type == BC_OUTFLOW, o1 = GENERAL && B1.type == BC_OUTFLOW;
         const F sg = pass == 0 ? F(-1) : F(1);
-        // a velocity of the corner: outward normal speeds, 1/D, values without ghosts, the walls' Maxwellians
-        struct Vel { F ux, uy, w, den, x[2], c0, c1; };
-        auto fetch = [&](int kk, Vel& q) {           // independent loads, used once all are asked for
-            q.ux = vu[kk];
-            q.uy = vv[kk];
-            q.w = vw[kk];
-            q.den = invD[(size_t)c * ld + kk];
-            q.x[0] = src[(size_t)c * ld + kk];
-            q.x[1] = src[(nc + c) * ld + kk];
-            q.c0 = w0 ? (F)C0[kk] : F(0);
-            q.c1 = w1 ? (F)C1[kk] : F(0);
+        // a velocity of the corner: outward normal speeds, weight, 1/D, right-hand sides
+        struct Vel { F ux, uy, w, den, b[2]; };
+        auto fetch = [&](int kk, Vel& p) {           // independent loads, used once all are asked for
+            p.ux = vu[kk];
+            p.uy = vv[kk];
+            p.w = vw[kk];
+            p.den = invD[(size_t)c * ld + kk];
+            p.b[0] = src[(size_t)c * ld + kk];
+            p.b[1] = src[(nc + c) * ld + kk];
         };
-        auto finish = [&](Vel& q) {
-            q.ux *= sg;
-            q.uy *= sg;
-            if (o0 || o1) {
-                const F D = itau + fabs(q.ux) * rx + fabs(q.uy) * ry;
-                q.den = recip(D + (o0 ? min(q.ux, F(0)) * rx : F(0)) + (o1 ? min(q.uy, F(0)) * ry : F(0)));
-                if (pass == 1) { q.x[0] *= D; q.x[1] *= D; }
+        // coefficient of the ghost behind face f (zero unless the velocity enters there)
+        auto Dg = [&](int f, const Vel& p) { return f == 0 ? mul_rn(min(p.ux, F(0)), rx) : mul_rn(min(p.uy, F(0)), ry); };
+        auto finish = [&](Vel& p) {
+            p.ux *= sg;
+            p.uy *= sg;
+            if (pass == 1 || o0 || o1) {
+                const F D = itau + geomD_r<F>(rx, ry, p.ux, p.uy);
+                if (o0 || o1) {
+                    F d = D;
+                    if (o0) d += Dg(0, p);
+                    if (o1) d += Dg(1, p);
+                    p.den = recip(d);
+                }
+                if (pass == 1) { p.b[0] = mul_rn(D, p.b[0]); p.b[1] = mul_rn(D, p.b[1]); }
             }
-            if (pass == 0 || o0 || o1) { q.x[0] *= q.den; q.x[1] *= q.den; }
         };
-        auto mirrored = [&](int f, int kk, Vel& q) { // the velocity mirrored at face f, ready
+        auto wallC = [&](int f, int kk, int cp) {     // the wall's Maxwellian
+            const double C = M.Cw[(size_t)(f == 0 ? bc0 : bc1) * nv + kk];
+            return cp == 0 ? (F)C : (F)(C * (kKint * (f == 0 ? B0.t : B1.t) / 4.0));
+        };
+        auto mirror = [&](int f, int kk) {
             const int a = kk / V.nvv, b = kk - a * V.nvv;
-            fetch(f == 0 ? (V.nu - 1 - a) * V.nvv + b : a * V.nvv + (V.nvv - 1 - b), q);
-            finish(q);
+            return f == 0 ? (V.nu - 1 - a) * V.nvv + b : a * V.nvv + (V.nvv - 1 - b);
         };
         F rho0 = F(0), rho1 = F(0);
-        const bool two = w0 && w1;
         if (w0 || w1) {
-            F acc[4] = {F(0), F(0), F(0), F(0)};
+            // sums over the velocities: eight groups of row pairs (a, nu - 1 - a) a group apart, a thread's share of a
+            // group in order, then warps and groups by exchange
+            const int ngroups = (V.nu + 1) / 2, per = 2 * V.nvv, nloc = (ngroups + 7) / 8 * per;
             #pragma unroll 1
-            for (int kb = tid; kb < nv; kb += 4 * B) {
-                Vel q[4];
+            for (int r0 = 0; r0 < 8; r0 += 4) {
+                F acc[4][4];
                 #pragma unroll
-                for (int t = 0; t < 4; ++t) fetch(min(kb + t * B, nv - 1), q[t]);
-                #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    finish(q[t]);
-                    F val = q[t].x[0];
-                    if (!two && ((y0 && q[t].ux < F(0)) || (y1 && q[t].uy < F(0)))) {
-                        // beside a symmetry face: the mirrored ghost of a velocity that enters through it
-                        Vel m;
-                        mirrored(y0 ? 0 : 1, min(kb + t * B, nv - 1), m);
-                        val -= (y0 ? q[t].ux * rx : q[t].uy * ry) * q[t].den * m.x[0];
+                for (int rr = 0; rr < 4; ++rr)
+                    #pragma unroll
+                    for (int m = 0; m < 4; ++m) acc[rr][m] = F(0);
+                #pragma unroll 1
+                for (int m = tid; m < nloc; m += B) {
+                    const int sl = m / per, rem = m - sl * per, side = rem >= V.nvv, b = rem - side * V.nvv;
+                    Vel p[4];
+                    int kk[4];
+                    #pragma unroll
+                    for (int rr = 0; rr < 4; ++rr) {
+                        const int g = r0 + rr + sl * 8, a = side ? V.nu - 1 - g : g;
+                        kk[rr] = g < ngroups && !(side && a == g) ? a * V.nvv + b : -1;
+                        fetch(max(kk[rr], 0), p[rr]);
                     }
-                    const F wt = kb + t * B < nv ? q[t].w : F(0);
-                    const F ax = w0 ? wt * max(q[t].ux, F(0)) : F(0), ay = w1 ? wt * max(q[t].uy, F(0)) : F(0);
-                    acc[0] += ax * val;
-                    acc[1] += ay * val;
-                    if (two) {
-                        acc[2] += ax * (min(q[t].uy, F(0)) * ry) * q[t].c1 * q[t].den;
-                        acc[3] += ay * (min(q[t].ux, F(0)) * rx) * q[t].c0 * q[t].den;
+                    #pragma unroll
+                    for (int rr = 0; rr < 4; ++rr) {
+                        if (kk[rr] < 0) continue;
+                        finish(p[rr]);
+                        const F wx = mul_rn(p[rr].w, max(p[rr].ux, F(0))), wy = mul_rn(p[rr].w, max(p[rr].uy, F(0)));
+                        if (two) {
+                            acc[rr][0] = fma(mul_rn(wx, p[rr].b[0]), p[rr].den, acc[rr][0]);
+                            acc[rr][1] = fma(mul_rn(wy, p[rr].b[0]), p[rr].den, acc[rr][1]);
+                            acc[rr][2] = fma(mul_rn(mul_rn(wx, Dg(1, p[rr])), wallC(1, kk[rr], 0)), p[rr].den, acc[rr][2]);
+                            acc[rr][3] = fma(mul_rn(mul_rn(wy, Dg(0, p[rr])), wallC(0, kk[rr], 0)), p[rr].den, acc[rr][3]);
+                        } else {
+                            F val = p[rr].b[0];
+                            if (y0 || y1) {          // beside a symmetry face: the mirrored ghost of a velocity that enters through it
+                                const F d = Dg(y0 ? 0 : 1, p[rr]);
+                                if (d != F(0)) {
+                                    Vel mv;
+                                    fetch(mirror(y0 ? 0 : 1, kk[rr]), mv);
+                                    finish(mv);
+                                    val = fma(-d, mul_rn(mv.b[0], mv.den), val);
+                                }
+                            }
+                            val = mul_rn(val, p[rr].den);
+                            acc[rr][0] = fma(w0 ? wx : wy, val, acc[rr][0]);
+                        }
                     }
                 }
+                #pragma unroll
+                for (int rr = 0; rr < 4; ++rr)
+                    #pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        #pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) acc[rr][m] += __shfl_xor_sync(0xffffffffu, acc[rr][m], o);
+                        if (lane == 0) red[(r0 + rr) * 4 + warp][m] = acc[rr][m];
+                    }
             }
+            __syncthreads();
+            F t[4];
             #pragma unroll
             for (int m = 0; m < 4; ++m) {
+                t[m] = red[lane][m];
                 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
-                if ((tid & 31) == 0) red[tid >> 5][m] = acc[m];
+                for (int o = 16; o > 0; o >>= 1) t[m] += __shfl_xor_sync(0xffffffffu, t[m], o);
             }
             __syncthreads();
             if (tid == 0) {
-                double t[4];
-                for (int m = 0; m < 4; ++m) t[m] = ((double)red[0][m] + red[1][m]) + ((double)red[2][m] + red[3][m]);
-                // rho_0 = k_0 + m_0 rho_1, rho_1 = k_1 + m_1 rho_0
-                const double k0 = -t[0] * z0, k1 = -t[1] * z1, m0 = t[2] * z0, m1 = t[3] * z1;
-                const double r0 = two ? (k0 + m0 * k1) * rcp64(1.0 - m0 * m1) : k0;
-                red[0][0] = w0 ? (F)r0 : F(0);
-                red[0][1] = w1 ? (F)(two ? k1 + m1 * r0 : k1) : F(0);
+                if (two) {
+                    // rho_0 = k_0 + m_0 rho_1, rho_1 = k_1 + m_1 rho_0
+                    const double z0 = Zw[bc0 * 4 + pass], z1 = Zw[bc1 * 4 + 2 + pass];
+                    const double k0 = -t[0] / z0, k1 = -t[1] / z1, m0 = t[2] / z0, m1 = t[3] / z1;
+                    const double r0 = (k0 + m0 * k1) / (1.0 - m0 * m1);
+                    red[0][0] = (F)r0;
+                    red[0][1] = (F)(k1 + m1 * r0);
+                } else {
+                    const F iz = (F)(Zw + 4 * kMaxBcs)[w0 ? bc0 * 4 + pass : bc1 * 4 + 2 + pass];
+                    red[0][0] = red[0][1] = -t[0] * iz;
+                }
             }
             __syncthreads();
             rho0 = red[0][0];
             rho1 = red[0][1];
         }
-        // value of a velocity with both ghosts
-        auto value = [&](int kk, const Vel& q, int cp) {
-            F a = q.x[cp];
-            const F f0 = cp ? h0 : F(1), f1 = cp ? h1 : F(1);
-            if (q.ux < F(0)) {
-                if (w0) a -= q.ux * rx * q.den * (q.c0 * f0 * rho0);
-                else if (y0) {       // the mirrored velocity leaves there and may itself enter through the other face
-                    Vel m;
-                    mirrored(0, kk, m);
-                    F g = m.x[cp];
-                    if (m.uy < F(0) && w1) g -= m.uy * ry * m.den * (m.c1 * f1 * rho1);
-                    if (m.uy < F(0) && y1) { Vel n; const int aa = kk / V.nvv, bb = kk - aa * V.nvv;
-                        mirrored(1, (V.nu - 1 - aa) * V.nvv + bb, n); g -= m.uy * ry * m.den * n.x[cp]; }
-                    a -= q.ux * rx * q.den * g;
+        // value of a velocity with its ghosts: a wall's from its density, a symmetry face's from the mirrored velocity,
+        // which leaves there and may itself enter through the other face
+        auto value = [&](auto&& self, auto depth, int kk, F (&out)[2]) {
+            Vel p;
+            fetch(kk, p);
+            finish(p);
+            F a[2] = {p.b[0], p.b[1]};
+            #pragma unroll
+            for (int f = 0; f < 2; ++f) {
+                const F d = Dg(f, p);
+                if (d == F(0)) continue;
+                if (f == 0 ? w0 : w1) {
+                    #pragma unroll
+                    for (int cp = 0; cp < 2; ++cp) a[cp] = fma(-mul_rn(d, wallC(f, kk, cp)), f == 0 ? rho0 : rho1, a[cp]);
+                } else if (f == 0 ? y0 : y1) {
+                    if constexpr (GENERAL && decltype(depth)::value > 0) {
+                        F g[2];
+                        self(self, std::integral_constant<int, decltype(depth)::value - 1>(), mirror(f, kk), g);
+                        #pragma unroll
+                        for (int cp = 0; cp < 2; ++cp) a[cp] = fma(-d, g[cp], a[cp]);
+                    }
                 }
             }
-            if (q.uy < F(0)) {
-                if (w1) a -= q.uy * ry * q.den * (q.c1 * f1 * rho1);
-                else if (y1) {
-                    Vel m;
-                    mirrored(1, kk, m);
-                    F g = m.x[cp];
-                    if (m.ux < F(0) && w0) g -= m.ux * rx * m.den * (m.c0 * f0 * rho0);
-                    if (m.ux < F(0) && y0) { Vel n; const int aa = kk / V.nvv, bb = kk - aa * V.nvv;
-                        mirrored(0, aa * V.nvv + (V.nvv - 1 - bb), n); g -= m.ux * rx * m.den * n.x[cp]; }
-                    a -= q.uy * ry * q.den * g;
-                }
-            }
-            return a;
+            out[0] = mul_rn(a[0], p.den);
+            out[1] = mul_rn(a[1], p.den);
         };
-        if (on) {
-            Vel q0;
-            fetch(k, q0);
-            finish(q0);
-            xp[0] = value(k, q0, 0);
-            if (sym) xp[1] = value(k, q0, 1);
-        }
+        const std::integral_constant<int, GENERAL ? 2 : 0> deep;
+        if (on) value(value, deep, k, xp);
         if (q == 0) {                                // the corner's values for the wavefront, a slice per CTA
             const int per = (nv + nchunk - 1) / nchunk;
             #pragma unroll 1
             for (int kk = chunk * per + tid; kk < min(nv, (chunk + 1) * per); kk += B) {
-                Vel q0;
-                fetch(kk, q0);
-                finish(q0);
-                S.corner[kk] = value(kk, q0, 0);
-                S.corner[ld + kk] = value(kk, q0, 1);
+                F t[2];
+                value(value, deep, kk, t);
+                S.corner[kk] = t[0];
+                S.corner[ld + kk] = t[1];
             }
         }
     } else if (on) {
         xp[0] = x[c0 * ld + k];
         xp[1] = x[(nc + c0) * ld + k];
     }
-    // -1/Z of the cells' walls (0 at other boundaries), for the end of the walk
-    #pragma unroll
-    for (int t = 0; t < kMaxLine / B; ++t) {
-        const int st = tid + t * B;
-        if (st < len) zf[st] = zb[t] >= 0 && M.bc[zb[t]].type == BC_WALL ? -(F)iZw[zb[t] * 4 + axis * 2 + pass] : F(0);
-    }
-    if (sym && edge && on)
-        for (int cp = 0; cp < 2; ++cp) S.xline[((size_t)ebase * 2 + cp) * ld + k] = xp[cp];
-    __syncthreads();                                 // nbS
-    // an[k]: coefficient of the previous cell of the line; lw: weight of the velocity in the wall sum
-    const F s1 = axis == 0 ? vv[k] : vu[k], uo = axis == 0 ? (pass == 0 ? -vu[k] : vu[k]) : (pass == 0 ? -vv[k] : vv[k]);
-    const F an = min(pass == 0 ? -s1 : s1, F(0)), lw = on ? vw[k] * uo : F(0);
-    F* part = S.part + ((size_t)q * nchunk + chunk) * kMaxLine;
+    __syncthreads();                                 // nbS, itS
+    // an: coefficient of the previous cell of the line; D = 1/tau + (|u|/dx + |v|/dy), the line's fixed spacing in gfix
+    const F s1 = axis == 0 ? vv[k] : vu[k], an = min(pass == 0 ? -s1 : s1, F(0)), gvar = fabs(s1);
+    const F gfix = axis == 0 ? mul_rn(fabs(vu[k]), (F)L.rdx[i0]) : mul_rn(fabs(vv[k]), (F)L.rdy[j0]);
     const int nbat = (len - 1 + U - 1) / U;
+    F* xo = S.xline + (size_t)(ebase + 1) * 2 * ld + k;
     for (int b = 0; b < nbat; ++b) {
         issue(b + NB - 1);
         cp_async_wait_n<NB - 1>();
         const F* d = ring + (b % NB) * U * 3 * B + tid;
-        F xv[U];
         #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int st = 1 + U * b + u;
-            xv[u] = F(0);
             if (st < len && on) {
-                const F id = d[u * 3 * B], in = d[u * 3 * B + B], Dn = an * nbS[st];
-                xp[0] = xv[u] = pass == 0 ? (in - Dn * xp[0]) * id : in - Dn * xp[0] * id;
-                if (sym) {
-                    const F ih = d[u * 3 * B + 2 * B];
-                    xp[1] = pass == 0 ? (ih - Dn * xp[1]) * id : ih - Dn * xp[1] * id;
-                    S.xline[((size_t)(ebase + st) * 2) * ld + k] = xp[0];
-                    S.xline[((size_t)(ebase + st) * 2 + 1) * ld + k] = xp[1];
+                const F id = d[u * 3 * B], Dn = mul_rn(an, nbS[st]), D = itS[st] + fma(gvar, nbS[st], gfix);
+                #pragma unroll
+                for (int cp = 0; cp < 2; ++cp) {
+                    const F in = d[u * 3 * B + (1 + cp) * B];
+                    xp[cp] = mul_rn(pass == 0 ? fma(-Dn, xp[cp], in) : fma(D, in, -mul_rn(Dn, xp[cp])), id);
+                    xo[cp * ld] = xp[cp];
                 }
+                xo += 2 * ld;
             }
-        }
-        const int row = (b % NB) * U;
-        #pragma unroll
-        for (int u = 0; u < U; ++u) tile[(row + u) * TS + tid] = lw * xv[u];
-        if (row + U == RA || b == nbat - 1) {          // sums of the cells of the last NB batches
-            __syncthreads();
-            const int cell = tid / TP, p = tid % TP, st = 1 + U * b - row + cell;
-            F s0 = F(0), s2 = F(0);
-            for (int m = p; m < B; m += 2 * TP) { s0 += tile[cell * TS + m]; s2 += tile[cell * TS + m + TP]; }
-            s0 += s2;
-            #pragma unroll
-            for (int o = TP / 2; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-            if (p == 0 && cell < row + U && st < len) part[st] = s0;
-            __syncthreads();
         }
     }
     cp_async_wait_n<0>();
-    // the last CTA of the line adds the partial sums, in order
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        last = atomicAdd(S.count + q, 1) == nchunk - 1;
-        if (last) S.count[q] = 0;
+}
+
+// Wall densities of the line cells [e0, e0 + gridDim.x), rho = -sum / Z with the sum of
+// w u_n x over the velocities that leave through the wall, one CTA per cell.  Order of the
+// sum: eight groups of row pairs of the velocity grid, in a group P shares (128 over the
+// line's cells) of eight interleaved chains each, a chain in order; then the chains as a
+// tree, the shares and the groups in order.  The tables hold the chains side by side, a
+// step of all of them after the other, so that a thread's loads are known ahead.
+// A kernel of its own because all of a line's walks have to be done; bound by latency
+// (64x64 cavity with 32x32 velocities 5 us, square cylinder's body lines 8 us).
+template <typename F>
+__global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __restrict__ Zw, SweepScratch<F> S, int pass, int e0)
+{
+    __shared__ F part[8 * 128];                      // [group][share]
+    const VelDev& V = M.V;
+    const int e = e0 + (int)blockIdx.x, tid = threadIdx.x;
+    const int4 lc = M.P.lcell[pass][e];              // {cell, line axis, bc id, 0 at the corner}
+    const int4 ls = M.P.lsum[pass][e];               // {place in the tables, shares, steps}
+    if (ls.y == 0) return;                           // no wall there: the density is not asked for
+    constexpr int U = 16;
+    const int P = ls.y, nch = 64 * P;
+    const F* __restrict__ x = S.xline + (size_t)e * 2 * V.ld;
+    for (int t = tid; t < nch; t += blockDim.x) {    // chain u of share p of group g; whole warps
+        const int* __restrict__ kt = V.chain + ls.x + t;
+        const F* __restrict__ wt = reinterpret_cast<const F*>(V.wchain) + ls.x + t;
+        F acc = F(0);
+        for (int n = 0; n < ls.z; n += U) {
+            F w[U], v[U];
+            int k[U];
+            #pragma unroll
+            for (int q = 0; q < U; ++q) {            // (a chain that has ended goes on with weight zero)
+                const int at = min(n + q, ls.z - 1) * nch;
+                k[q] = kt[at];
+                w[q] = n + q < ls.z ? wt[at] : F(0);
+            }
+            #pragma unroll
+            for (int q = 0; q < U; ++q) v[q] = x[k[q]];
+            #pragma unroll
+            for (int q = 0; q < U; ++q) acc = w[q] != F(0) ? fma(w[q], v[q], acc) : acc;
+        }
+        #pragma unroll
+        for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((t & 7) == 0) part[t >> 3] = acc;
     }
     __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int st = 1 + tid; st < len; st += B) {
-        F sum = F(0);
-        #pragma unroll 4
-        for (int m = 0; m < nchunk; ++m) sum += __ldcg(S.part + ((size_t)q * nchunk + m) * kMaxLine + st);
-        S.rho[ebase + st] = sum * zf[st];
+    if (tid < 8) {
+        F t = F(0);
+        #pragma unroll 8
+        for (int p = 0; p < P; ++p) t += part[tid * P + p];
+        part[tid * P] = t;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        F t = F(0);
+        for (int g = 0; g < 8; ++g) t += part[g * P];
+        S.rho[e] = -t * (F)(Zw + 4 * kMaxBcs)[lc.z * 4 + lc.y * 2 + pass];
     }
 }
 
@@ -559,19 +599,22 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
 //   forward   x = (b - C_a x_a - C_l x_l) / D, b the residual,
 //   backward  x = b - (C_a x_a + C_l x_l) / D, b the forward value,
 // with the coefficients zero where the neighbour lies downwind: a CTA whose
-// velocities need no neighbour across (or along) skips that part, and in the
-// backward pass one that needs neither leaves its values as they are.
+// velocities need no neighbour across hands none on, and in the backward pass
+// one that needs neither only takes over the line cells' values.
+// Of the two products, the neighbour's along x is fused into their sum.
 // Boundary-line cells take b and 1/D from the fold, which the CTA makes for its
 // velocities before it starts, from the wall densities of the line walk: the
-// entries [e0, e0 + ne) of the lines walked last.  Cells in a body, and steps
-// outside a line, are copied as zeros, which makes their result zero and drops
-// the neighbour across a boundary face without a test.
+// entries [e0, e0 + ne) of the lines walked last.  1/D = 0 marks a value that is
+// final: the corner cell, a line cell's leaving velocities (the walk's own values),
+// and the zeros that stand for a cell in a body or a step outside a line.  They are
+// chosen, not computed, so that nothing that overflowed ahead of a body gets into
+// it; a zero in the body in turn drops it as a neighbour.
 // What bounds it: on large levels the L1 look-ups of the copies and stores (one per
 // cell and warp access, see LPC in launch_micro_sgs), on small ones the
 // instructions of a step, as an SM sub-partition has one warp.  Square cylinder,
-// mixed: 9.0 ms per iteration for all levels, against 16.4 ms for the wavefront of
+// mixed: 8.7 ms per iteration for all levels, against 16.4 ms for the wavefront of
 // 4-velocity CTAs with a barrier per diagonal and the line kernel beside it that
-// this replaces; 64x64 cavity 29 us per launch against 32 us.
+// this replaces; 64x64 cavity 26 us per launch against 32 us.
 constexpr int kWaveChunk = 4;
 constexpr int kWaveEdge = 16;                       // results of a strip's last line in flight to the next strip
 constexpr int kWaveSpin = 1 << 24;                  // looks of a wait before it gives up
@@ -598,6 +641,15 @@ template <> struct Pack<float> {
     using T = unsigned long long;
     static __device__ __forceinline__ T make(float a, float b) { T r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
     static __device__ __forceinline__ T splat(float a) { return make(a, a); }
+    static __device__ __forceinline__ void split(T v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+    static __device__ __forceinline__ T pick(T iv, T v, T b)                // v where 1/D is given, else b
+    {
+        float i0, i1, v0, v1, b0, b1;
+        split(iv, i0, i1);
+        split(v, v0, v1);
+        split(b, b0, b1);
+        return make(i0 > 0.0f ? v0 : b0, i1 > 0.0f ? v1 : b1);
+    }
     static __device__ __forceinline__ T load(const float* p) { return make(p[0], p[1]); }
     static __device__ __forceinline__ T mul(T a, T b) { T r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
     static __device__ __forceinline__ T add(T a, T b) { T r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
@@ -610,6 +662,7 @@ template <> struct Pack<float> {
 };
 template <> struct Pack<double> {
     using T = double;
+    static __device__ __forceinline__ T pick(T iv, T v, T b) { return iv > 0.0 ? v : b; }
     static __device__ __forceinline__ T splat(double a) { return a; }
     static __device__ __forceinline__ T load(const double* p) { return p[0]; }
     static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
@@ -661,7 +714,7 @@ template <typename F, int PASS, int LPC>
 __device__ void wave_fold(const MicroArgs& M, const F* __restrict__ invD, const F* __restrict__ src, const SweepScratch<F>& S,
                           F* __restrict__ fold, int k0, int e0, int ne)
 {
-    constexpr int V16 = 16 / (int)sizeof(F), K = V16, KB = LPC * V16;   // a thread's and the CTA's velocities
+    constexpr int V16 = 16 / (int)sizeof(F), KB = LPC * V16;            // a thread's and the CTA's velocities
     const LevelDev& L = M.L;
     const VelDev& V = M.V;
     const int nx = L.nx, nv = V.nv;
@@ -671,52 +724,46 @@ __device__ void wave_fold(const MicroArgs& M, const F* __restrict__ invD, const 
     const int part = (int)threadIdx.x % LPC;
     k0 += part * V16;
     for (int e = e0 + (int)threadIdx.x / LPC; e < e0 + ne; e += (int)blockDim.x / LPC) {
-        const int4 lc = M.P.lcell[PASS][e];         // {cell, line axis, bc id, corner}
+        const int4 lc = M.P.lcell[PASS][e];         // {cell, line axis, bc id, 0 at the corner}
         const int c = lc.x, axis = lc.y, i = c % nx, j = c / nx;
-        F b[2][K], iv[K];
-        if (lc.w) {
-            #pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const bool in = k0 + q < nv;
-                b[0][q] = in ? S.corner[k0 + q] : F(0);
-                b[1][q] = in ? S.corner[ld + k0 + q] : F(0);
-                iv[q] = F(1);
-            }
-        } else {
-            const size_t o = (size_t)c * ld + k0;
-            #pragma unroll
-            for (int q = 0; q < K; q += V16) {
-                ld16(src + o + q, b[0] + q);
-                ld16(src + nc * ld + o + q, b[1] + q);
-                ld16(invD + o + q, iv + q);
-            }
-            const int bc = lc.z;
-            const BcDev Bc = M.bc[bc];
-            const F rS = axis == 0 ? (F)L.rdx[i] : (F)L.rdy[j], h = (F)(kKint * Bc.t / 4.0), rho = S.rho[e];
-            #pragma unroll
-            for (int q = 0; q < K; ++q) {
-                const int k = k0 + q;
-                const F u = vu[k], v = vv[k];
-                F un = axis == 0 ? u : v;
-                un = PASS == 0 ? -un : un;
-                if (!(un < F(0)) || k >= nv) continue;
-                const F Db = un * rS;
+        F b[2][V16], iv[V16];
+        const F* fin = lc.w == 0 ? S.corner : S.xline + (size_t)e * 2 * ld;   // final values: the corner, leaving velocities
+        const size_t o1 = (size_t)c * ld + k0;
+        ld16(src + o1, b[0]);
+        ld16(src + nc * ld + o1, b[1]);
+        ld16(invD + o1, iv);
+        const int bc = lc.z;
+        const BcDev Bc = M.bc[bc];
+        const F rx = (F)L.rdx[i], ry = (F)L.rdy[j], rS = axis == 0 ? rx : ry, itau = (F)M.inv_tau[c], rho = S.rho[e];
+        #pragma unroll
+        for (int q = 0; q < V16; ++q) {
+            const int k = k0 + q;
+            const F u = vu[k], v = vv[k];
+            F un = axis == 0 ? u : v;
+            un = PASS == 0 ? -un : un;
+            if (k >= nv) {
+                b[0][q] = b[1][q] = iv[q] = F(0);
+            } else if (lc.w == 0 || un >= F(0)) {
+                b[0][q] = fin[k];
+                b[1][q] = fin[ld + k];
+                iv[q] = F(0);
+            } else {
+                const F Db = mul_rn(un, rS), D = itau + geomD_r<F>(rx, ry, u, v);
                 F g[2] = {F(0), F(0)};
                 if (Bc.type == BC_WALL) {
-                    g[0] = Db * ((F)M.Cw[(size_t)bc * nv + k] * rho);
-                    g[1] = h * g[0];
+                    const double C = M.Cw[(size_t)bc * nv + k];
+                    g[0] = mul_rn(Db, mul_rn((F)C, rho));
+                    g[1] = mul_rn(Db, mul_rn((F)(C * (kKint * Bc.t / 4.0)), rho));
                 } else if (Bc.type == BC_SYMMETRY) {
                     const int a2 = k / V.nvv, b2 = k - a2 * V.nvv;
                     const int km = axis == 0 ? (V.nu - 1 - a2) * V.nvv + b2 : a2 * V.nvv + (V.nvv - 1 - b2);
-                    g[0] = Db * S.xline[((size_t)e * 2) * ld + km];
-                    g[1] = Db * S.xline[((size_t)e * 2 + 1) * ld + km];
+                    g[0] = mul_rn(Db, fin[km]);
+                    g[1] = mul_rn(Db, fin[ld + km]);
                 } else if (Bc.type == BC_OUTFLOW) {
-                    const F D = (F)M.inv_tau[c] + fabs(u) * (F)L.rdx[i] + fabs(v) * (F)L.rdy[j];
                     iv[q] = recip(D + Db);
-                    if (PASS == 1) { b[0][q] = D * b[0][q] * iv[q]; b[1][q] = D * b[1][q] * iv[q]; }
                 }
-                b[0][q] -= PASS == 0 ? g[0] : g[0] * iv[q];
-                b[1][q] -= PASS == 0 ? g[1] : g[1] * iv[q];
+                #pragma unroll
+                for (int cp = 0; cp < 2; ++cp) b[cp][q] = PASS == 0 ? b[cp][q] - g[cp] : fma(D, b[cp][q], -g[cp]) * iv[q];
             }
         }
         F* o = fold + (size_t)e * 3 * KB + part * V16;
@@ -726,8 +773,8 @@ __device__ void wave_fold(const MicroArgs& M, const F* __restrict__ invD, const 
     }
 }
 
-// LPC: lanes per cell, 16 bytes of velocities each
-template <typename F, int R, int PASS, bool BODIES, int LPC>
+// LPC: lanes per cell, 16 bytes of velocities each; XL: the lines are columns
+template <typename F, int R, int PASS, bool BODIES, int LPC, bool XL>
 __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restrict__ invD, const F* __restrict__ r,
                                                   F* __restrict__ x, SweepScratch<F> S, int dd0, int dd1, int e0, int ne)
 {
@@ -738,8 +785,7 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
     const LevelDev& L = M.L;
     const VelDev& V = M.V;
     const int nx = L.nx, ny = L.ny, k0 = (int)blockIdx.x * K;
-    const bool xl = nx <= ny;                       // lines are columns
-    const int ns = xl ? nx : ny, nt = xl ? ny : nx, nw = (int)blockDim.x >> 5;
+    const int ns = XL ? nx : ny, nt = XL ? ny : nx, nw = (int)blockDim.x >> 5;
     const size_t nc = L.nc, ld = V.ld;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, ll = lane / LPC, part = lane % LPC, s = NL * w + ll;
     unsigned char* ring = wsm + (size_t)w * R * step_bytes + lane * 16;
@@ -758,19 +804,30 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
     for (int q = 0; q < V16; ++q) {
         const F u = vu[kl + q], v = vv[kl + q];     // the tables are padded with zeros
         const F cu = min(PASS == 0 ? -u : u, F(0)), cv = min(PASS == 0 ? -v : v, F(0));
-        ca[q] = xl ? cu : cv;
-        cl[q] = xl ? cv : cu;
+        ca[q] = XL ? cu : cv;
+        cl[q] = XL ? cv : cu;
         any_a = any_a || ca[q] != F(0);
         any_l = any_l || cl[q] != F(0);
     }
     any_a = __any_sync(0xffffffffu, any_a);
     any_l = __any_sync(0xffffffffu, any_l);
-    if (PASS == 1 && !any_a && !any_l) return;      // (the same in every warp)
     F* fold = S.fold + (size_t)blockIdx.x * S.nl * 3 * K;
     wave_fold<F, PASS, LPC>(M, invD, src, S, fold, k0, e0, ne);
+    if (PASS == 1 && !any_a && !any_l) {            // (the same in every warp)
+        for (int e = e0 + (int)threadIdx.x / LPC; e < e0 + ne; e += (int)blockDim.x / LPC) {   // (a thread's own entries)
+            const size_t o = (size_t)M.P.lcell[PASS][e].x * ld + kl;
+            const F* f = fold + (size_t)e * 3 * K + part * V16;
+            F v[V16];
+            ld16(f, v);
+            st16(x + o, v);
+            ld16(f + K, v);
+            st16(x + nc * ld + o, v);
+        }
+        return;
+    }
     for (int t = threadIdx.x; t < nt; t += blockDim.x) {
         const int p = PASS == 0 ? t : nt - 1 - t;
-        ral[t] = -(F)(xl ? L.rdy[p] : L.rdx[p]);
+        ral[t] = -(F)(XL ? L.rdy[p] : L.rdx[p]);
     }
     if (lane == 0) prog[w] = cons[w] = max(0, dd0 + 1 - NL * w);
     __threadfence();                                // the fold is read by asynchronous copies of other threads
@@ -780,16 +837,16 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
     if (kb >= ke) return;
     const bool line = s < ns;
     const int sp = PASS == 0 ? s : ns - 1 - s, tp = PASS == 0 ? 0 : nt - 1;
-    const long cfirst = line ? (xl ? (long)tp * nx + sp : (long)sp * nx + tp) : 0;   // the line's cell t = 0
-    const long cst = (PASS == 0 ? 1 : -1) * (xl ? (long)nx : 1L);
+    const long cfirst = line ? (XL ? (long)tp * nx + sp : (long)sp * nx + tp) : 0;   // the line's cell t = 0
+    const long cst = (PASS == 0 ? 1 : -1) * (XL ? (long)nx : 1L);
     const long pst = cst * (long)ld;                // from a cell of the line to the next, in values
-    const F rac = line && s > 0 ? -(xl ? (F)L.rdx[sp] : (F)L.rdy[sp]) : F(0);
+    const F rac = line && s > 0 ? -(XL ? (F)L.rdx[sp] : (F)L.rdy[sp]) : F(0);
     T nca[2], ncl[2];
     #pragma unroll
     for (int q = 0; q < V16; ++q) ca[q] *= rac;
     #pragma unroll
     for (int q = 0; q < 2; ++q) { nca[q] = P::load(ca + q * (V16 / 2)); ncl[q] = P::load(cl + q * (V16 / 2)); }
-    const int ea = xl ? 0 : ny, eb = xl ? ny + s : s;   // fold entries of line 0 (+ t) and of the cells t = 0
+    const int ea = XL ? 0 : ny, eb = XL ? ny + s : s;   // fold entries of line 0 (+ t) and of the cells t = 0
     const int* __restrict__ code = M.P.code[PASS];
     auto code_of = [&](int k) {
         const int t = k - ll;
@@ -841,7 +898,7 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
         const bool hl = line && t >= 1 && t <= nt, ha = s >= 1 && s <= ns && t >= 0 && t < nt;
         const long c_l = cfirst + (long)(t - 1) * cst;
         const int sa = PASS == 0 ? s - 1 : ns - s, ta = PASS == 0 ? t : nt - 1 - t;
-        const long c_a = xl ? (long)ta * nx + sa : (long)sa * nx + ta;
+        const long c_a = XL ? (long)ta * nx + sa : (long)sa * nx + ta;
         #pragma unroll
         for (int cp = 0; cp < 2; ++cp) {
             if (hl) ld_pair(x + (cp * nc + c_l) * ld + kl, al[cp]);
@@ -876,22 +933,21 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
             lds_pair_if(tk, ea_ + 16, ac[1]);
             issue(k + R - 1, (kk + R - 1) % R);
             // minus the neighbours' terms (line 0 has no neighbour across: its coefficient is zero)
-            if (any_l) {
-                const T ra = P::splat(ral[min(max(t, 0), nt - 1)]);
+            const T ra = P::splat(ral[min(max(t, 0), nt - 1)]);
+            #pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const T g = P::mul(ncl[q], ra);
                 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const T g = P::mul(ncl[q], ra);
-                    al[0][q] = P::mul(g, al[0][q]);
-                    al[1][q] = P::mul(g, al[1][q]);
+                for (int cp = 0; cp < 2; ++cp) {
+                    const T n = XL ? P::fma(nca[q], ac[cp][q], P::mul(g, al[cp][q])) : P::fma(g, al[cp][q], P::mul(nca[q], ac[cp][q]));
+                    al[cp][q] = PASS == 0 ? P::mul(P::add(b[cp][q], n), iv[q]) : P::fma(n, iv[q], b[cp][q]);
                 }
             }
-            #pragma unroll
-            for (int cp = 0; cp < 2; ++cp)
+            if (BODIES || w == 0 || k < NL)          // (the other steps of a strip hold no final value)
                 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    T n = any_l ? al[cp][q] : P::splat(F(0));
-                    if (any_a) n = any_l ? P::fma(nca[q], ac[cp][q], n) : P::mul(nca[q], ac[cp][q]);
-                    al[cp][q] = PASS == 0 ? P::mul(P::add(b[cp][q], n), iv[q]) : P::fma(n, iv[q], b[cp][q]);
+                    al[0][q] = P::pick(iv[q], al[0][q], b[0][q]);
+                    al[1][q] = P::pick(iv[q], al[1][q], b[1][q]);
                 }
             const bool on = line && (unsigned)t < (unsigned)nt && k < ke;
             st_pair_if(on, xo, bits(al[0][0]), bits(al[0][1]));
@@ -918,30 +974,29 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
     cp_async_wait_n<0>();
 }
 
-// sweep scratch: values of the storage type per solver (the largest level), and line counters
-size_t micro_scratch_elems(int ld, int nl, int nlines, int nchunk, bool sym)
+// sweep scratch: values of the storage type per solver (the largest level)
+size_t micro_scratch_elems(int ld, int nl)
 {
-    return 2 * (size_t)ld + (((size_t)nl + 15) & ~(size_t)15) + (2 + (size_t)nlines) * nchunk * kMaxLine +
-           3 * (size_t)ld * nl + (sym ? 2 * (size_t)nl * ld : 0);
+    return 2 * (size_t)ld + (((size_t)nl + 15) & ~(size_t)15) + 5 * (size_t)ld * nl;
 }
 template <typename F>
-SweepScratch<F> sweep_scratch(F* base, int* count, int ld, int nl, int nlines, int nchunk)
+SweepScratch<F> sweep_scratch(F* base, int ld, int nl)
 {
     SweepScratch<F> S;
     S.corner = base;
     S.rho = S.corner + 2 * (size_t)ld;
-    S.part = S.rho + (((size_t)nl + 15) & ~(size_t)15);
-    S.fold = S.part + (2 + (size_t)nlines) * nchunk * kMaxLine;
+    S.fold = S.rho + (((size_t)nl + 15) & ~(size_t)15);
     S.xline = S.fold + 3 * (size_t)ld * nl;
-    S.count = count;
     S.nl = nl;
     return S;
 }
-int micro_edge_chunks(const VelDev& V)
+// CTAs of the line walk per line: the leaving velocities of a pass and axis, zero ones among them
+static int edge_chunks(const VelDev& V)
 {
     int m = 1;
     for (int p = 0; p < 2; ++p)
-        for (int a = 0; a < 2; ++a) m = std::max(m, (V.nleave[p][a] * (a == 0 ? V.nvv : V.nu) + 127) / 128);
+        for (int a = 0; a < 2; ++a)
+            m = std::max(m, (((a == 0 ? V.nu : V.nvv) - V.nleave[1 - p][a]) * (a == 0 ? V.nvv : V.nu) + 127) / 128);
     return m;
 }
 
@@ -950,10 +1005,10 @@ cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, cons
                              const F* r, F* x, F* scratch, cudaStream_t st)
 {
     if (m.L.nx > kMaxLine || m.L.ny > kMaxLine) return cudaErrorInvalidValue;
-    const int ns = std::min(m.L.nx, m.L.ny), nt = std::max(m.L.nx, m.L.ny), nchunk = plan.nchunk;
-    const SweepScratch<F> S = sweep_scratch<F>(scratch, plan.count, m.V.ld, plan.nl, plan.nlines, nchunk);
+    const int ns = std::min(m.L.nx, m.L.ny), nt = std::max(m.L.nx, m.L.ny), nchunk = edge_chunks(m.V);
+    const SweepScratch<F> S = sweep_scratch<F>(scratch, m.V.ld, plan.nl);
     constexpr size_t kSmemMax = 227 * 1024;
-    constexpr size_t esmem = sizeof(F) * EdgeRing<F>::RA * (3 * 128 + 132);
+    constexpr size_t esmem = sizeof(F) * EdgeRing<F>::RA * 3 * 128;
     // Lanes per cell: an asynchronous copy or store of a warp costs its SM's L1 one look-up per cell, so
     // the more lanes share a cell the better (64 bytes of a cell with four), as long as the strips fit a
     // CTA of 16 warps and the CTAs fill the SMs.  Finest level and coarser ones together, per
@@ -968,19 +1023,22 @@ cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, cons
     const size_t wsmem = fixed + R * slot;
     if (wsmem > kSmemMax) return cudaErrorInvalidValue;
     using Wave = void (*)(MicroArgs, const F*, const F*, F*, SweepScratch<F>, int, int, int, int);
-    auto pick = [&](auto h, auto bodies) {
+    const bool xl = m.L.nx <= m.L.ny;
+    if (R == 4 && LPC != 4) return cudaErrorInvalidValue;   // (eight steps always fit with fewer lanes)
+    auto pick = [&](auto h, auto bodies, auto cols) {
         constexpr int HH = decltype(h)::value;
-        constexpr bool BB = decltype(bodies)::value;
-        std::array<Wave, 2> f;
-        f[0] = R == 8 ? k_sgs_wave<F, 8, 0, BB, HH> : k_sgs_wave<F, 4, 0, BB, HH>;
-        f[1] = R == 8 ? k_sgs_wave<F, 8, 1, BB, HH> : k_sgs_wave<F, 4, 1, BB, HH>;
+        constexpr bool BB = decltype(bodies)::value, XX = decltype(cols)::value;
+        std::array<Wave, 2> f = {k_sgs_wave<F, 8, 0, BB, HH, XX>, k_sgs_wave<F, 8, 1, BB, HH, XX>};
+        if constexpr (HH == 4)
+            if (R == 4) f = {k_sgs_wave<F, 4, 0, BB, HH, XX>, k_sgs_wave<F, 4, 1, BB, HH, XX>};
         return f;
     };
-    auto by_lanes = [&](auto bodies) {
-        return LPC == 4 ? pick(std::integral_constant<int, 4>(), bodies)
-               : LPC == 2 ? pick(std::integral_constant<int, 2>(), bodies) : pick(std::integral_constant<int, 1>(), bodies);
+    auto by_lanes = [&](auto bodies, auto cols) {
+        return LPC == 4 ? pick(std::integral_constant<int, 4>(), bodies, cols)
+               : LPC == 2 ? pick(std::integral_constant<int, 2>(), bodies, cols) : pick(std::integral_constant<int, 1>(), bodies, cols);
     };
-    const std::array<Wave, 2> wave = m.P.bodies ? by_lanes(std::true_type()) : by_lanes(std::false_type());
+    auto by_axis = [&](auto bodies) { return xl ? by_lanes(bodies, std::true_type()) : by_lanes(bodies, std::false_type()); };
+    const std::array<Wave, 2> wave = m.P.bodies ? by_axis(std::true_type()) : by_axis(std::false_type());
     for (int p = 0; p < 2; ++p) {
         cudaError_t e = cudaFuncSetAttribute(wave[p], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
         if (e != cudaSuccess) return e;
@@ -1013,6 +1071,8 @@ cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, cons
     const int nd = m.L.nx + m.L.ny - 1;
     for (int pass = 0; pass < 2; ++pass) {
         walk[m.P.general[pass]]<<<2 * nchunk, 128, esmem, st>>>(m, Zw, invD, r, x, S, pass, 0, nchunk);
+        // (a thread per chain, up to 512)
+        if (m.P.shares[pass]) k_line_rho<F><<<m.P.nl[pass], std::min(512, 64 * m.P.shares[pass]), 0, st>>>(m, Zw, S, pass, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // wavefront segments between the body lines' walks
         int dd = 0, e0 = 0, ne = m.P.nl[pass];
@@ -1031,6 +1091,7 @@ cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, cons
             if (b < plan.nbrk[pass]) {
                 const SweepBreak& k = plan.brk[pass][b];
                 walk[m.P.general[pass]]<<<k.nq * nchunk, 128, esmem, st>>>(m, Zw, invD, r, x, S, pass, 2 + k.q0, nchunk);
+                if (k.shares) k_line_rho<F><<<k.ne, std::min(512, 64 * k.shares), 0, st>>>(m, Zw, S, pass, k.e0);
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
                 e0 = k.e0;
                 ne = k.ne;
@@ -1104,6 +1165,7 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
             // FP32 is bound by memory: all four neighbours are read, so that every load can be issued at
             // once (choosing the two that a velocity sees first made the square cylinder's renewals
             // 16.0 -> 21.6 ms per three iterations)
+            const bool four = (Vg.nv & 3) == 0;
             for (int k0 = threadIdx.x * V16; k0 < nv; k0 += blockDim.x * V16) {
                 F u[V16], v[V16], cW[V16], cE[V16], cS[V16], cN[V16], dg[V16];
                 ld16(vu + k0, u);
@@ -1129,11 +1191,11 @@ __global__ void __launch_bounds__(256) k_micro_renew(MicroArgs M, const double* 
                     if (ab) ld16(ab + cp * hoff + k0, aa);
                     #pragma unroll
                     for (int q = 0; q < V16; ++q) {
-                        F a = dg[q] * xc[q];
-                        a += cW[q] * xw[q];
-                        a += cE[q] * xe[q];
-                        a += cS[q] * xs[q];
-                        a += cN[q] * xn[q];
+                        // (which of the first two products is rounded before the sum follows the row's length)
+                        F a = four ? fma(dg[q], xc[q], mul_rn(cW[q], xw[q])) : fma(cW[q], xw[q], mul_rn(dg[q], xc[q]));
+                        a = fma(cE[q], xe[q], a);
+                        a = fma(cS[q], xs[q], a);
+                        a = fma(cN[q], xn[q], a);
                         rr[q] = rr[q] - a;
                         aa[q] = ab ? aa[q] + xc[q] : F(0);
                     }

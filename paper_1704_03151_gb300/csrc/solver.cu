@@ -6,7 +6,9 @@
 #include <cstdarg>
 #include <cstdio>
 #include <algorithm>
+#include <array>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -26,7 +28,6 @@ struct HLevel {
     LevelDev dev{};
     SweepPlanDev plan{};                // sweep order tables (device)
     std::vector<SweepBreak> brk[2];     // body-line walks between wavefront segments
-    int nlines = 0;                     // body lines (larger pass)
     // transposed sweep (adjoint preconditioner): the cells with one wall face of a body on
     // a pass's side, cell * 4 + face, grouped by wavefront step (AdjBodyPlan)
     int* adjb[2] = {nullptr, nullptr};
@@ -71,8 +72,12 @@ struct miugks_solver {
     bool mixed = false;
     size_t fsz = sizeof(double);
     void *f = nullptr, *phx = nullptr, *phy = nullptr, *scratch = nullptr;
-    int* line_count = nullptr;
-    int sw_nl = 0, sw_nlines = 0, sw_nchunk = 1;   // layout of the sweep scratch
+    int sw_nl = 0;                          // layout of the sweep scratch
+    // chains of the wall sums by {pass, axis, shares}: {place in the tables, steps} (wall_chains)
+    std::map<std::array<int, 3>, std::array<int, 2>> chain_at;
+    std::vector<int> chain_k;
+    std::vector<float> chain_wf;
+    std::vector<double> chain_w;
     double* fgeo[2] = {nullptr, nullptr};   // finest level: mesh constants of the interface flux per face
     double *W = nullptr, *q = nullptr, *R = nullptr, *Fx = nullptr, *Fy = nullptr;
     double *rms_part = nullptr, *rms_out = nullptr;
@@ -369,9 +374,51 @@ SweepPlanHost sweep_plan(const miugks_solver* s, const HLevel& Lv)
 {
     SweepPlanHost h{};
     for (int p = 0; p < 2; ++p) { h.brk[p] = Lv.brk[p].data(); h.nbrk[p] = (int)Lv.brk[p].size(); }
-    h.nl = s->sw_nl; h.nlines = s->sw_nlines; h.nchunk = s->sw_nchunk; h.count = s->line_count;
+    h.nl = s->sw_nl;
     h.timer = s->timing && &Lv == &s->lev[0] ? const_cast<SweepTimer*>(&s->sweep_timer) : nullptr;
     return h;
+}
+
+// Chains of a wall sum over the velocities that leave through the faces of one axis on a pass's sweep side
+// (k_line_rho): the velocities in eight groups of row pairs (a, nu - 1 - a), in a group `shares` times eight chains
+// that take its places in turn.  Laid out step after step, [steps][group][share][chain], ended chains with weight 0.
+template <typename F>
+int wall_chains(const miugks_solver* s, int pass, int axis, int shares, std::vector<int>& chain, std::vector<F>& weight)
+{
+    const int nu = s->nu, nvv = s->nvv, ngroups = (nu + 1) / 2, nch = 64 * shares;
+    const std::vector<double>& un = axis == 0 ? s->uah : s->vbh;
+    auto leaves = [&](double z) { return pass == 0 ? z < 0.0 : z > 0.0; };
+    // every leaving velocity's chain and its step there, in the chains' order
+    std::vector<int> step(nch, 0), at, n, k;
+    int steps = 0;
+    for (int g = 0; g < 8; ++g) {
+        int q = 0;                                       // place in the group
+        for (int pair = g; pair < ngroups; pair += 8)
+            for (int side = 0; side < 2; ++side, q += nvv) {
+                const int a = side ? nu - 1 - pair : pair;
+                if ((side && a == pair) || (axis == 0 && !leaves(un[a]))) continue;
+                int p = q % shares, u = q / shares % 8;
+                for (int b = 0; b < nvv; ++b) {
+                    if (axis == 0 || leaves(un[b])) {
+                        const int c = (g * shares + p) * 8 + u;
+                        at.push_back(c);
+                        n.push_back(step[c]);
+                        k.push_back(a * nvv + b);
+                        steps = std::max(steps, ++step[c]);
+                    }
+                    if (++p == shares) { p = 0; u = (u + 1) % 8; }
+                }
+            }
+    }
+    const size_t base = chain.size();
+    chain.resize(base + (size_t)steps * nch, 0);
+    weight.resize(base + (size_t)steps * nch, F(0));
+    for (size_t e = 0; e < k.size(); ++e) {
+        const size_t to = base + (size_t)n[e] * nch + at[e];
+        chain[to] = k[e];
+        weight[to] = (F)s->wh[k[e]] * std::fabs((F)(axis == 0 ? s->uh : s->vh)[k[e]]);
+    }
+    return steps;
 }
 
 // Sweep order of a level.  Per pass (0 forward: west / south faces on the
@@ -389,21 +436,41 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
     auto by = [&](int p, int i, int j) { return Lv.fby[(j + p) * nx + i] >= 0; };
     int nl_max = 0;
     for (int p = 0; p < 2; ++p) {
+        Lv.plan.shares[p] = 0;
         std::vector<int> code(nc, -1);
         std::vector<int> lcell;              // int4 per entry
         for (int c = 0; c < nc; ++c) if (Lv.solid[c]) code[c] = -2;
         const int ie = p == 0 ? 0 : nx - 1, je = p == 0 ? 0 : ny - 1, sg = p == 0 ? 1 : -1;
+        // wall sum of a line cell: shares (128 over the line's cells) and table; the corner, and cells at other
+        // boundaries, have none (0 shares)
+        std::vector<int> lsum;               // int4 per entry
+        auto add_sum = [&](int ncell, int axis, int bc, bool corner, int& most) {
+            if (corner || s->bch[bc].type != MIUGKS_BC_WALL) { lsum.insert(lsum.end(), {0, 0, 0, 0}); return; }
+            const int shares = ncell >= 128 ? 1 : 128 / ncell;
+            most = std::max(most, shares);
+            const std::array<int, 3> key = {p, axis, shares};
+            if (!s->chain_at.count(key)) {
+                const int at = (int)s->chain_k.size();
+                const int steps = s->mixed ? wall_chains<float>(s, p, axis, shares, s->chain_k, s->chain_wf)
+                                           : wall_chains<double>(s, p, axis, shares, s->chain_k, s->chain_w);
+                s->chain_at[key] = {at, steps};
+            }
+            const std::array<int, 2> t = s->chain_at[key];
+            lsum.insert(lsum.end(), {t[0], shares, t[1], 0});
+        };
         // the edge column (e = st) and row (e = ny + st), the corner first
         for (int st = 0; st < ny; ++st) {
             int i = ie, j = je + sg * st, c = j * nx + i;
             if (Lv.solid[c]) return fail(s, MIUGKS_EINVAL, "level with %dx%d cells: the cells on the domain edge must be fluid", nx, ny);
-            lcell.insert(lcell.end(), {c, 0, Lv.fbx[j * (nx + 1) + i + p], st == 0});
+            lcell.insert(lcell.end(), {c, 0, Lv.fbx[j * (nx + 1) + i + p], st != 0});
+            add_sum(ny - 1, 0, lcell[lcell.size() - 2], st == 0, Lv.plan.shares[p]);
             code[c] = st;
         }
         for (int st = 0; st < nx; ++st) {
             int i = ie + sg * st, j = je, c = j * nx + i;
             if (Lv.solid[c]) return fail(s, MIUGKS_EINVAL, "level with %dx%d cells: the cells on the domain edge must be fluid", nx, ny);
-            lcell.insert(lcell.end(), {c, 1, Lv.fby[(j + p) * nx + i], st == 0});
+            lcell.insert(lcell.end(), {c, 1, Lv.fby[(j + p) * nx + i], st != 0});
+            add_sum(nx - 1, 1, lcell[lcell.size() - 2], st == 0, Lv.plan.shares[p]);
             if (st > 0) code[c] = ny + st;
         }
         Lv.plan.nl[p] = nx + ny;
@@ -444,54 +511,48 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
         }
         std::stable_sort(runs.begin(), runs.end(), [](const Run& x, const Run& y) { return x.dd < y.dd; });
         if ((int)runs.size() > kMaxBodyLines) return fail(s, MIUGKS_EINVAL, "too many body lines (%d > %d)", (int)runs.size(), kMaxBodyLines);
-        // the line's faces on the sweep side: does one belong to a symmetry plane
-        auto has_sym = [&](int i, int j, int di, int dj, int first, int len, int axis) {
-            for (int st = first; st < len; ++st) {
-                const int a = i + st * di, b = j + st * dj;
-                const int id = axis == 0 ? Lv.fbx[b * (nx + 1) + a + p] : Lv.fby[(b + p) * nx + a];
-                if (id >= 0 && s->bch[id].type == MIUGKS_BC_SYMMETRY) return 1;
-            }
-            return 0;
-        };
-        std::vector<int> lines = {ie, je, 0, sg, ny, 0, 0, has_sym(ie, je, 0, sg, 0, ny, 0),
-                                  ie, je, sg, 0, nx, 1, ny, has_sym(ie, je, sg, 0, 0, nx, 1)};
+        std::vector<int> lines = {ie, je, 0, sg, ny, 0, 0, 0, ie, je, sg, 0, nx, 1, ny, 0};
         Lv.brk[p].clear();
         for (int q = 0; q < (int)runs.size(); ++q) {
             const Run& R = runs[q];
             const int e0 = (int)lcell.size() / 4;
-            lines.insert(lines.end(), {R.i0, R.j0, R.di, R.dj, R.len, R.axis, e0 - 1,
-                                       has_sym(R.i0, R.j0, R.di, R.dj, 1, R.len, R.axis)});
+            int most = 0;                    // shares of the line's wall sums
+            lines.insert(lines.end(), {R.i0, R.j0, R.di, R.dj, R.len, R.axis, e0 - 1, 0});
             for (int st = 1; st < R.len; ++st) {
                 int i = R.i0 + st * R.di, j = R.j0 + st * R.dj, c = j * nx + i;
                 code[c] = (int)lcell.size() / 4;
-                lcell.insert(lcell.end(), {c, R.axis, R.axis == 0 ? Lv.fbx[j * (nx + 1) + i + p] : Lv.fby[(j + p) * nx + i], 0});
+                lcell.insert(lcell.end(), {c, R.axis, R.axis == 0 ? Lv.fbx[j * (nx + 1) + i + p] : Lv.fby[(j + p) * nx + i], 1});
+                add_sum(R.len - 1, R.axis, lcell[lcell.size() - 2], false, most);
             }
             const int ne = (int)lcell.size() / 4 - e0;
             if (!Lv.brk[p].empty() && Lv.brk[p].back().dd == R.dd) {
                 Lv.brk[p].back().nq++;
                 Lv.brk[p].back().ne += ne;
+                Lv.brk[p].back().shares = std::max(Lv.brk[p].back().shares, most);
             } else {
-                Lv.brk[p].push_back(SweepBreak{R.dd, q, 1, e0, ne});
+                Lv.brk[p].push_back(SweepBreak{R.dd, q, 1, e0, ne, most});
             }
         }
-        Lv.nlines = std::max(Lv.nlines, (int)runs.size());
         nl_max = std::max(nl_max, (int)lcell.size() / 4);
         int* dcode;
-        int4* dl;
+        int4 *dl, *dsum;
         int* dlines;
         ST(upload(s, &dcode, code));
-        std::vector<int4> l4(lcell.size() / 4);
-        for (size_t e = 0; e < l4.size(); ++e) l4[e] = make_int4(lcell[4 * e], lcell[4 * e + 1], lcell[4 * e + 2], lcell[4 * e + 3]);
-        ST(upload(s, &dl, l4));
+        auto int4s = [](const std::vector<int>& v) {
+            std::vector<int4> h(v.size() / 4);
+            for (size_t e = 0; e < h.size(); ++e) h[e] = make_int4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            return h;
+        };
+        ST(upload(s, &dl, int4s(lcell)));
+        ST(upload(s, &dsum, int4s(lsum)));
         ST(upload(s, &dlines, lines));
         Lv.plan.code[p] = dcode;
         Lv.plan.lcell[p] = dl;
+        Lv.plan.lsum[p] = dsum;
         Lv.plan.lines[p] = dlines;
-        Lv.plan.sym[p] = lines[7] | lines[15] << 1;
         Lv.plan.cbc[p][0] = Lv.fbx[je * (nx + 1) + ie + p];
         Lv.plan.cbc[p][1] = Lv.fby[(je + p) * nx + ie];
         Lv.plan.general[p] = 0;
-        for (size_t q = 7; q < lines.size(); q += 8) Lv.plan.general[p] |= lines[q];
         for (int f = 0; f < 2; ++f) {
             const int type = s->bch[Lv.plan.cbc[p][f]].type;
             Lv.plan.general[p] |= type == MIUGKS_BC_SYMMETRY || type == MIUGKS_BC_OUTFLOW;
@@ -1085,7 +1146,6 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
                 const std::vector<double>& n = a == 0 ? ua : vb;
                 s->vel.nleave[p][a] = (int)std::count_if(n.begin(), n.end(), [&](double z) { return p == 0 ? z < 0.0 : z > 0.0; });
             }
-        if (st != MIUGKS_OK) break;
         if ((st = upload(s, &s->bc, s->bch)) != MIUGKS_OK) break;
         s->Cwh.assign((size_t)n_bcs * s->nv, 0.0);
         for (int b = 0; b < n_bcs; ++b) refresh_bc_tables(s, b);
@@ -1094,6 +1154,9 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
         for (int l = 0; l < s->L && st == MIUGKS_OK; ++l) st = upload_level(s, s->lev[l]);
         if (st != MIUGKS_OK) break;
         for (int l = 0; l < s->L && st == MIUGKS_OK; ++l) st = build_sweep_plan(s, s->lev[l]);
+        if (st != MIUGKS_OK) break;
+        if ((st = upload(s, (int**)&s->vel.chain, s->chain_k)) != MIUGKS_OK) break;
+        if ((st = s->mixed ? upload(s, (float**)&s->vel.wchain, s->chain_wf) : upload(s, (double**)&s->vel.wchain, s->chain_w)) != MIUGKS_OK) break;
         if (st != MIUGKS_OK) break;
         for (int l = 0; l + 1 < s->L && st == MIUGKS_OK; ++l) {
             HLevel& F = s->lev[l];
@@ -1129,16 +1192,8 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
         if ((st = dalloc(s, &s->rms_out, 8)) != MIUGKS_OK) break;
         if ((st = dalloc(s, &s->nrm, 129)) != MIUGKS_OK) break;
         if (cudaMemset(s->rms_out, 0, 8 * sizeof(double)) != cudaSuccess) { st = fail(s, MIUGKS_ECUDA, "cudaMemset"); break; }
-        for (int l = 0; l < s->L; ++l) {
-            s->sw_nlines = std::max(s->sw_nlines, s->lev[l].nlines);
-            s->sw_nl = std::max(s->sw_nl, s->lev[l].plan.nl_max);
-        }
-        s->sw_nchunk = micro_edge_chunks(s->vel);
-        bool any_sym = false;
-        for (const BcDev& B : s->bch) any_sym = any_sym || B.type == MIUGKS_BC_SYMMETRY;
-        if ((st = falloc(s, &s->scratch, micro_scratch_elems(s->ld, s->sw_nl, s->sw_nlines, s->sw_nchunk, any_sym))) != MIUGKS_OK) break;
-        if ((st = dalloc(s, &s->line_count, 2 + (size_t)s->sw_nlines)) != MIUGKS_OK) break;
-        if (cudaMemsetAsync(s->line_count, 0, (2 + (size_t)s->sw_nlines) * sizeof(int), s->st) != cudaSuccess) { st = fail(s, MIUGKS_ECUDA, "cudaMemset"); break; }
+        for (int l = 0; l < s->L; ++l) s->sw_nl = std::max(s->sw_nl, s->lev[l].plan.nl_max);
+        if ((st = falloc(s, &s->scratch, micro_scratch_elems(s->ld, s->sw_nl))) != MIUGKS_OK) break;
         // smallest interior physical time step (for the numerical time step)
         s->dtp_min = 1e300;
         for (int i = 1; i < L0.nx; ++i) s->dtp_min = std::fmin(s->dtp_min, opts->cfl * std::fmin(L0.dx[i - 1], L0.dx[i]) / s->umax);

@@ -149,7 +149,7 @@ def hot_channel(lib):
 STAGES = {f.__name__: f for f in (moments, flux, prediction, evolution, residual, hot_channel)}
 
 
-@pytest.mark.parametrize("stage", ["moments", "flux", "prediction"])
+@pytest.mark.parametrize("stage", ["moments", "flux", "prediction", "evolution", "residual", "hot_channel"])
 def test_recorded_values(lib, stage):
     want = np.load(GOLDEN)
     for key, a in STAGES[stage](lib).items():

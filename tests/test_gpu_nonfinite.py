@@ -60,3 +60,25 @@ def test_prediction_sweep(lib, wide, precision):
     x, y = g.sgs_macro(0, w, w, r), o.sgs_macro(0, w, w, r)
     assert np.all(x[solid.ravel()] == 0.0) and not np.all(np.isfinite(y))
     agrees(x, y, 1e-10 if precision == "fp64" else 2e-5)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("wide", [False, True])
+def test_evolution_sweep(lib, wide, precision):
+    """(Here the oracle multiplies by the zero coefficient of a downwind neighbour, so that an infinity goes
+    further in it; the GPU's values beyond are held to be finite, not to be the oracle's.)"""
+    c = body(wide)
+    nx, n = c["nx"], c["nx"] * c["ny"]
+    solid = np.asarray(c["solid"]).reshape(c["ny"], nx) > 0
+    j, i = np.argwhere(solid)[0]
+    o, g = oracle.Oracle(c), lib.Solver(c, precision=precision)
+    rng = np.random.default_rng(5)
+    it, r = rng.uniform(0.2, 3.0, n), rng.normal(size=(2, n, o.nv))
+    r[:, solid.ravel()] = 0.0
+    r[:, j * nx + i - 2, ::3] = np.inf
+    x, y = g.sgs_micro(0, it, r), o.sgs_micro(0, it, r)
+    assert np.all(x[:, solid.ravel()] == 0.0)
+    ok = np.isfinite(y)
+    assert not np.all(ok) and np.all(np.isfinite(x[ok]))
+    tol = 1e-10 if precision == "fp64" else 2e-5
+    assert np.max(np.abs(x[ok] - y[ok])) <= tol * np.max(np.abs(y[ok]))
