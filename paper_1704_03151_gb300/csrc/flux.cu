@@ -810,7 +810,7 @@ cudaError_t launch_face_flux<double>(const FaceFluxArgs<double>& a, cudaStream_t
     if (smem > kSmemMax) return cudaErrorInvalidValue;
     auto kern = cache ? k_face_flux<true> : k_face_flux<false>;
     if (smem > 47 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_shared_memory((const void*)kern);
         if (e != cudaSuccess) return e;
     }
     const int nf = a.axis == 0 ? a.L.nfx : a.L.nfy;
@@ -838,7 +838,7 @@ cudaError_t launch_face_flux<float>(const FaceFluxArgs<float>& a, cudaStream_t s
     if (smem > kSmemMax) return cudaErrorInvalidValue;
     auto kern = cache ? k_face_flux_mixed<true> : k_face_flux_mixed<false>;
     if (smem > 47 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_shared_memory((const void*)kern);
         if (e != cudaSuccess) return e;
     }
     const int nf = a.axis == 0 ? a.L.nfx : a.L.nfy;

@@ -5,6 +5,12 @@
 
 namespace miugks {
 
+// Let kernel `kern` (a __global__ function) be launched with as much dynamic shared memory
+// as its static part leaves of a block's limit.  The limit belongs to the function, not to
+// a solver, so it is raised once per device and never lowered: solvers of different
+// sizes in several host threads launch the same kernel.
+cudaError_t allow_shared_memory(const void* kern);
+
 template <typename F>
 struct FaceFluxArgs {
     LevelDev L; VelDev V; GasDev gas;

@@ -833,7 +833,7 @@ cudaError_t launch_macro_sgs(const MacroArgs& a, F* rec, const double* ghost, F*
         }
     const size_t smem = bytes(R);
     if (smem > 47 * 1024) {                             // with the static part, 48 KB need no opt-in
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_shared_memory((const void*)kern);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};

@@ -1040,14 +1040,14 @@ cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, cons
     auto by_axis = [&](auto bodies) { return xl ? by_lanes(bodies, std::true_type()) : by_lanes(bodies, std::false_type()); };
     const std::array<Wave, 2> wave = m.P.bodies ? by_axis(std::true_type()) : by_axis(std::false_type());
     for (int p = 0; p < 2; ++p) {
-        cudaError_t e = cudaFuncSetAttribute(wave[p], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
+        const cudaError_t e = allow_shared_memory((const void*)wave[p]);
         if (e != cudaSuccess) return e;
     }
     using Edge = void (*)(MicroArgs, const double*, const F*, const F*, const F*, SweepScratch<F>, int, int, int);
     const Edge walk[2] = {k_sgs_edge<F, false>, k_sgs_edge<F, true>};
     cudaError_t e = cudaSuccess;
     for (int g = 0; g < 2; ++g)
-        if ((e = cudaFuncSetAttribute(walk[g], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esmem)) != cudaSuccess) return e;
+        if ((e = allow_shared_memory((const void*)walk[g])) != cudaSuccess) return e;
     // timing mode: an event pair around a launch, with the cell-velocity pairs it sweeps
     auto timed = [&](double units, auto&& launch) {
         SweepTimer* T = plan.timer;

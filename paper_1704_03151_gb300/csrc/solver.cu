@@ -9,11 +9,32 @@
 #include <array>
 #include <cstring>
 #include <map>
+#include <mutex>
+#include <set>
 #include <string>
 #include <vector>
 
 #include "../../include/miugks.h"
 #include "kernels.cuh"
+
+namespace miugks {
+cudaError_t allow_shared_memory(const void* kern)
+{
+    static std::mutex lock;
+    static std::set<std::pair<const void*, int>> done;       // (one entry per kernel and device)
+    int dev = 0, most = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> hold(lock);
+    if (done.count({kern, dev})) return cudaSuccess;
+    if ((e = cudaFuncGetAttributes(&a, kern)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+    if (e == cudaSuccess) done.insert({kern, dev});
+    return e;
+}
+} // namespace miugks
 
 using namespace miugks;
 
