@@ -200,11 +200,12 @@ struct alignas(16) TangentNode { double ut, h, E, Fq, S; };   // h = u_t / 2
 //     depend on one axis each (NormalNode, TangentNode).
 // CACHE keeps the face values and slopes of every velocity in shared memory
 // between the passes; without it (a velocity grid too large for shared memory)
-// the second pass reconstructs again.
+// the second pass reconstructs again.  Without TABLES (a first axis of more than
+// about 2,200 nodes) the node constants are formed where they are used, too.
 // Per launch against three passes that reconstructed both sides of every velocity: flat
 // plate (48x48) 13.1 -> 4.8 ms, 64x64 cavity (32x32) 1.92 -> 0.72 ms, square cylinder at
 // half size (89x89) 21.4 -> 10.1 ms.
-template <bool CACHE>
+template <bool CACHE, bool TABLES>
 __global__ void __launch_bounds__(256, 2) k_face_flux(FaceFluxArgs<double> A)
 {
     using F = double;
@@ -220,10 +221,10 @@ __global__ void __launch_bounds__(256, 2) k_face_flux(FaceFluxArgs<double> A)
     double* par = red + 288;                // face scalars, [48]
     double* tot = par + 48;                 // block sums, [16]
     F* pf = tot + 16;                       // face constants, [64]
-    NormalNode* tn = reinterpret_cast<NormalNode*>(pf + 64);   // per node of the first axis (or TangentNodes)
-    F* ta = reinterpret_cast<F*>(tn + nu);  // per node of the first axis: u - U_s, (u - U_s)^2 / 2, [nu][2]
-    F* wE = ta + 2 * nu;                    // exponentials per node, [nu] then [nvv]
-    F* f0s = wE + nu + nvv;                 // [2][nv] (CACHE)
+    F* wE = pf + 64;                        // exponentials per node, [nu] then [nvv], to an even number
+    NormalNode* tn = reinterpret_cast<NormalNode*>(wE + ((nu + nvv + 1) & ~1));   // per node of the first axis (or TangentNodes)
+    F* ta = reinterpret_cast<F*>(tn + (TABLES ? nu : 0));   // per node of the first axis: u - U_s, (u - U_s)^2 / 2, [nu][2]
+    F* f0s = ta + (TABLES ? 2 * nu : 0);    // [2][nv] (CACHE)
     F* sgs = f0s + 2 * nv;                  // [2][nv] (CACHE)
     const int i = axis == 0 ? fi % (nx + 1) : fi % nx;
     const int j = axis == 0 ? fi / (nx + 1) : fi / nx;
@@ -263,12 +264,11 @@ __global__ void __launch_bounds__(256, 2) k_face_flux(FaceFluxArgs<double> A)
     }
     __syncthreads();
     const F Us = pf[5], Vs = pf[6];
-    for (int a = tid; a < nu; a += bs) {
-        const F d = (F)Vg.ua[a] - Us;
-        ta[2 * a] = d;
-        ta[2 * a + 1] = F(0.5) * d * d;
+    auto shifted = [&](int a, F& d, F& h) { d = Vg.ua[a] - Us; h = F(0.5) * d * d; };
+    if constexpr (TABLES) {
+        for (int a = tid; a < nu; a += bs) shifted(a, ta[2 * a], ta[2 * a + 1]);
+        __syncthreads();
     }
-    __syncthreads();
     // threads: columns tx of the second axis, rows ty of the first
     const int bw = min(nvv, bs), rows = bs / bw, tx = tid % bw, ty = tid / bw;
     // nodes ascend: the first nneg of the normal axis come from above, the last ones from below
@@ -307,7 +307,10 @@ __global__ void __launch_bounds__(256, 2) k_face_flux(FaceFluxArgs<double> A)
             #pragma unroll 2
             for (int a = ty; a < nu; a += rows) {
                 const int k = a * nvv + b;
-                const F w = vw[k], da = ta[2 * a], ha = ta[2 * a + 1];
+                const F w = vw[k];
+                F da, ha;
+                if constexpr (TABLES) { da = ta[2 * a]; ha = ta[2 * a + 1]; }
+                else shifted(a, da, ha);
                 F f0[2], sg[2];
                 recon(k, axis == 0 ? a : b, f0, sg);
                 if constexpr (CACHE) {
@@ -466,11 +469,13 @@ __global__ void __launch_bounds__(256, 2) k_face_flux(FaceFluxArgs<double> A)
         N.Fq = q1 * shk * (c * qt);
         N.S = F(2) * lam * (c * c);
     };
-    for (int a = tid; a < nu; a += bs) {
-        if (axis == 0) normal(a, tn[a]);
-        else tangent(a, reinterpret_cast<TangentNode*>(tn)[a]);
+    if constexpr (TABLES) {
+        for (int a = tid; a < nu; a += bs) {
+            if (axis == 0) normal(a, tn[a]);
+            else tangent(a, reinterpret_cast<TangentNode*>(tn)[a]);
+        }
+        __syncthreads();
     }
-    __syncthreads();
 
     // pass 2: time-averaged flux of every discrete velocity and its moments
     Acc<F> Fa[4];
@@ -485,8 +490,14 @@ __global__ void __launch_bounds__(256, 2) k_face_flux(FaceFluxArgs<double> A)
             for (int a = ty; a < nu; a += rows) {
                 const int k = a * nvv + b;
                 const F w = vw[k];
-                if (AX == 0) N = tn[a];
-                else T = reinterpret_cast<const TangentNode*>(tn)[a];
+                if constexpr (!TABLES) {
+                    if (AX == 0) normal(a, N);
+                    else tangent(a, T);
+                } else if (AX == 0) {
+                    N = tn[a];
+                } else {
+                    T = reinterpret_cast<const TangentNode*>(tn)[a];
+                }
                 F f0[2], sg[2];
                 if constexpr (CACHE) {
                     f0[0] = f0s[k]; f0[1] = f0s[nv + k]; sg[0] = sgs[k]; sg[1] = sgs[nv + k];
@@ -803,12 +814,13 @@ cudaError_t launch_face_flux<double>(const FaceFluxArgs<double>& a, cudaStream_t
     // reconstructed again in the second pass (which costs a third of the arithmetic, where the split
     // of a face over a cluster, each CTA caching its share, repeats the face's serial phases)
     constexpr size_t kCacheMax = 110 * 1024;
-    const size_t base = sizeof(double) * (288 + 48 + 16 + 64 + 3 * (size_t)a.V.nu + a.V.nvv) + sizeof(NormalNode) * (size_t)a.V.nu;
+    const size_t nodes = sizeof(double) * (288 + 48 + 16 + 64 + (((size_t)a.V.nu + a.V.nvv + 1) & ~(size_t)1));
+    const size_t base = nodes + (sizeof(double) * 2 + sizeof(NormalNode)) * (size_t)a.V.nu;
     const size_t full = base + sizeof(double) * 4 * (size_t)a.V.nv;
-    const bool cache = full <= kCacheMax;
-    const size_t smem = cache ? full : base;
+    const bool cache = full <= kCacheMax, tables = base <= kSmemMax;
+    const size_t smem = cache ? full : tables ? base : nodes;
     if (smem > kSmemMax) return cudaErrorInvalidValue;
-    auto kern = cache ? k_face_flux<true> : k_face_flux<false>;
+    auto kern = cache ? k_face_flux<true, true> : tables ? k_face_flux<false, true> : k_face_flux<false, false>;
     if (smem > 47 * 1024) {
         const cudaError_t e = allow_shared_memory((const void*)kern);
         if (e != cudaSuccess) return e;
