@@ -84,8 +84,8 @@ __device__ __forceinline__ float time_coeff_one_f(float dt, float tau, int m)
 // van Leer limited slope 2 s1 s2 / (s1 + s2) when s1 s2 > 0, else 0
 __device__ __forceinline__ double vl_limited(double s1, double s2)
 {
-    const double p = s1 * s2;      // (the sign is looked at in the bits: a comparison would take the FP64 pipe)
-    return __double_as_longlong(p) > 0 ? (p + p) * rcp64(s1 + s2) : 0.0;
+    const double p = s1 * s2;      // p > 0 is looked at in the bits (a comparison would take the FP64 pipe); a NaN is not > 0
+    return (unsigned long long)(__double_as_longlong(p) - 1) < 0x7ff0000000000000ull ? (p + p) * rcp64(s1 + s2) : 0.0;
 }
 // (sum: s1 + s2, as the caller rounds it)
 __device__ __forceinline__ float vl_limited(float s1, float s2, float sum)
