@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(256, 2) k_face_flux(FaceFluxArgs<double> A)
     if (tid >= 32 && tid < 34) {
         const int m = tid - 31;
         const double *wl = A.W + 4 * (size_t)cL, *wr = A.W + 4 * (size_t)cR;
-        pf[4 + m] = (F)(0.5f * ((float)wl[m] / (float)wl[0] + (float)wr[m] / (float)wr[0]));
+        pf[4 + m] = (F)(float)(0.5 * (wl[m] * rcp64(wl[0]) + wr[m] * rcp64(wr[0])));
     }
     __syncthreads();
     const F Us = pf[5], Vs = pf[6];

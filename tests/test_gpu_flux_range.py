@@ -2,7 +2,8 @@
 
 A NaN in one cell reaches the cells that share a face with it and no others: the
 limiter gives a face beyond them no slope, as the oracle's does (the iteration
-then reports divergence instead of spreading it).  Bounds as for the other fluxes."""
+then reports divergence instead of spreading it).  And in FP64 densities far
+outside FP32's range are ordinary numbers.  Bounds as for the other fluxes."""
 import numpy as np
 import pytest
 
@@ -39,3 +40,13 @@ def test_nan_stays_beside_its_cell(lib, precision):
         ok = np.isfinite(b)
         assert not np.all(ok) and np.array_equal(np.isfinite(a), ok)
         assert np.max(np.abs(a[ok] - b[ok])) <= (1e-10 if precision == "fp64" else 2e-5) * np.max(np.abs(b[ok]))
+
+
+@pytest.mark.parametrize("scale", [1e-100, 1e-60, 1e-20, 1e20, 1e60])
+def test_densities_outside_single_precision(lib, scale):
+    o, g, f = state(lib, "fp64")
+    o.set_f(f * scale)
+    g.set_f(f * scale)
+    for a, b in zip(g.stage_flux(), o.stage_flux()):
+        assert np.all(np.isfinite(a))
+        assert np.max(np.abs(a - b)) <= 1e-10 * np.max(np.abs(b))
