@@ -186,9 +186,9 @@ miugks_status miugks_set_sweep_split(miugks_solver *s, int mode);
  * nothing where it is continuous.  The adjoint (which does not differentiate
  * this term) returns MIUGKS_EINVAL while it is on. */
 miugks_status miugks_set_shock_capturing(miugks_solver *s, int on);
-/* Bound of the prediction smoother's device waits (in the sweep of Eq.
- * macroFinalDefect a strip of grid lines waits for the values of the strip
- * before it): a wait that has not completed after `seconds` (default 0.2, at
+/* Bound of the smoothers' device waits (in the sweeps of Eqs. macroFinalDefect
+ * and microFinalDefect a strip of grid lines waits for the values of the strip
+ * before it, in the latter also for room to hand its own on): a wait that has not completed after `seconds` (default 0.2, at
  * most 10) gives up, the kernel drains its copies in flight and returns, and the
  * next miugks_step / miugks_wait returns MIUGKS_ETIMEOUT (sticky for the
  * solver).  0 makes every sweep give up before its first step, without testing

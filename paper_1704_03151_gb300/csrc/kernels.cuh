@@ -115,6 +115,7 @@ struct MicroArgs {
     const double* inv_tau;                 // [nc] collision frequency (+ 1/dt_n)
     SweepPlanDev P;
     double* flag;                          // set to 1 when a bounded device wait gave up
+    unsigned long long wait_ns;            // bound of the wavefront's waits between strips (ns of global time)
 };
 // Scratch of the sweeps, kept per solver and sized for its largest level
 // (micro_scratch_elems); laid out by launch_micro_sgs.

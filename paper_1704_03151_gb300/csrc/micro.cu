@@ -617,16 +617,22 @@ __global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __r
 // this replaces; 64x64 cavity 26 us per launch against 32 us.
 constexpr int kWaveChunk = 4;
 constexpr int kWaveEdge = 16;                       // results of a strip's last line in flight to the next strip
-constexpr int kWaveSpin = 1 << 24;                  // looks of a wait before it gives up
 
-__device__ __forceinline__ bool wave_wait(const int* flag, int need)
+// false once limit_ns of global time (or kWaitRounds looks) have gone by
+__device__ __forceinline__ bool wave_wait(const int* flag, int need, uint64_t limit_ns)
 {
     const unsigned a = smem_addr(flag);
-    for (int it = 0; it < kWaveSpin; ++it) {
+    uint64_t t0 = 0;
+    for (int it = 0; it < kWaitRounds; ++it) {
         int v;
         asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];\n" : "=r"(v) : "r"(a) : "memory");
         if (v >= need) return true;
         __nanosleep(20);                             // (a spinning strip takes issue slots from the working ones)
+        if ((it & 31) == 31) {
+            const uint64_t t = global_ns();
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > limit_ns) return false;
+        }
     }
     return false;
 }
@@ -793,6 +799,10 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
     F* ral = reinterpret_cast<F*>(edges + (size_t)nw * kWaveEdge * ebytes);     // [nt] -1/d along the lines
     int* prog = reinterpret_cast<int*>(ral + nt);                               // per strip: edge values there
     int* cons = prog + nw;                                                      // per strip: edge values taken
+    if (M.wait_ns == 0) {                           // gives up before its first step
+        if (threadIdx.x == 0) *M.flag = 1.0;
+        return;
+    }
     const F* src = PASS == 0 ? r : x;
     const F* __restrict__ vu = VelT<F>::u(V);
     const F* __restrict__ vv = VelT<F>::v(V);
@@ -917,8 +927,8 @@ __global__ void __launch_bounds__(512) k_sgs_wave(MicroArgs M, const F* __restri
             if (kk % kWaveChunk == 0) {
                 const int kn = min(k + kWaveChunk, ke);
                 bool got = true;
-                if (takes) got = wave_wait(prog + w, min(nt, kn));
-                if (feeds) got = got && wave_wait(cons + w + 1, min(nt, kn - (NL - 1)) - kWaveEdge);
+                if (takes) got = wave_wait(prog + w, min(nt, kn), M.wait_ns);
+                if (feeds) got = got && wave_wait(cons + w + 1, min(nt, kn - (NL - 1)) - kWaveEdge, M.wait_ns);
                 if (!__all_sync(0xffffffffu, got)) { if (lane == 0) *M.flag = 1.0; cp_async_wait_n<0>(); return; }
             }
             cp_async_wait_n<R - 2>();

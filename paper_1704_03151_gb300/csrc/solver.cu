@@ -112,7 +112,7 @@ struct miugks_solver {
     std::vector<unsigned char> adapt_log = std::vector<unsigned char>(4096);
     double* nrm = nullptr;                      // device: 128 partial sums and the total
     bool shock = false;                         // pressure-jump collision time at interior faces
-    unsigned long long wait_ns = 200000000ull;  // bound of the prediction sweep's device waits
+    unsigned long long wait_ns = 200000000ull;  // bound of the sweeps' device waits
     // timing mode: the finest level's wavefront launches; totals since the last read
     SweepTimer sweep_timer;
     double t_sweepk = 0, u_sweepk = 0;
@@ -388,7 +388,7 @@ miugks_status upload_level(miugks_solver* s, HLevel& Lv)
 
 MicroArgs micro_args(miugks_solver* s, int l)
 {
-    return MicroArgs{s->lev[l].dev, s->vel, s->bc, s->Cw, s->lev[l].inv_tau, s->lev[l].plan, s->rms_out + 5};
+    return MicroArgs{s->lev[l].dev, s->vel, s->bc, s->Cw, s->lev[l].inv_tau, s->lev[l].plan, s->rms_out + 5, s->wait_ns};
 }
 
 SweepPlanHost sweep_plan(const miugks_solver* s, const HLevel& Lv)
