@@ -373,7 +373,8 @@ miugks_status upload_level(miugks_solver* s, HLevel& Lv)
     Lv.dev = LevelDev{Lv.nx, Lv.ny, Lv.nc, Lv.nfx, Lv.nfy, xn, yn, xc, yc, dx, dy, fbx, fby, rdx, rdy, solid,
                       ubcd, (int)ubc.size()};
     size_t n4 = 4 * (size_t)Lv.nc, nf = 2 * (size_t)Lv.nc * s->ld;
-    ST(dalloc(s, &Lv.Wn, n4)); ST(dalloc(s, &Lv.Wc, n4)); ST(dalloc(s, &Lv.Rc, n4)); ST(dalloc(s, &Lv.P, n4));
+    ST(dalloc(s, &Lv.Wn, n4)); ST(dalloc(s, &Lv.Wc, n4)); ST(dalloc(s, &Lv.P, n4));
+    if (&Lv != &s->lev[0]) ST(dalloc(s, &Lv.Rc, n4));        // (the finest level's residual is the solver's R)
     ST(dalloc(s, &Lv.R, n4)); ST(dalloc(s, &Lv.dW, n4)); ST(dalloc(s, &Lv.Wt, n4));
     ST(dalloc(s, &Lv.gx, (size_t)Lv.nfx)); ST(dalloc(s, &Lv.gy, (size_t)Lv.nfy));
     ST(dalloc(s, &Lv.idiag, (size_t)Lv.nc)); // records, ghosts and the state's other buffer (16-byte aligned parts of one block)
