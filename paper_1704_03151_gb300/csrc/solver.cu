@@ -1140,9 +1140,9 @@ miugks_status miugks_create(const miugks_mesh* mesh, const miugks_vgrid* vg, con
         }
         if (st != MIUGKS_OK) break;
         if (mesh->nx > kMaxLine || mesh->ny > kMaxLine) { st = bad("nx and ny are limited to 512"); break; }
-        // chain kernel capacity: velocities per CTA of the 8-CTA cluster
-        int nloc = (((s->nu + 1) / 2 + 7) / 8) * 2 * s->nvv;
-        if (nloc > 8 * 256) { st = bad("velocity grid too large for the boundary-line kernel (%d local > 2048)", nloc); break; }
+        // the velocity grids that are taken: at most 2048 velocities in each of the eight groups of row pairs (wall_chains)
+        const int nloc = (((s->nu + 1) / 2 + 7) / 8) * 2 * s->nvv;
+        if (nloc > 2048) { st = bad("velocity grid too large (%d velocities in a group of row pairs, at most 2048)", nloc); break; }
         // device data (on the caller's stream, or the legacy default stream when none is given)
         upload_series_coefficients();
         {
