@@ -231,12 +231,14 @@ std::vector<double> flux_face_geometry(const HLevel& L, int axis, double cfl, do
 }
 
 // per-velocity array of count elements of the solver's storage type
-// (zeroed: the padding of the rows of velocities is zero and stays so)
+// (rows of velocities: their padding is zero and stays so; the rest, and the sweeps' scratch, is written before it is read)
 miugks_status falloc(miugks_solver* s, void** p, size_t count)
 {
     if (s->mixed) ST(dalloc(s, (float**)p, count));
     else ST(dalloc(s, (double**)p, count));
-    if (s->ld != s->nv) CK(cudaMemsetAsync(*p, 0, count * s->fsz, s->st));
+    if (s->ld == s->nv) return MIUGKS_OK;
+    if (count % s->ld) CK(cudaMemsetAsync(*p, 0, count * s->fsz, s->st));
+    else CK(cudaMemset2DAsync((char*)*p + s->nv * s->fsz, s->ld * s->fsz, 0, (s->ld - s->nv) * s->fsz, count / s->ld, s->st));
     return MIUGKS_OK;
 }
 
@@ -410,8 +412,10 @@ int wall_chains(const miugks_solver* s, int pass, int axis, int shares, std::vec
     const int nu = s->nu, nvv = s->nvv, ngroups = (nu + 1) / 2, nch = 64 * shares;
     const std::vector<double>& un = axis == 0 ? s->uah : s->vbh;
     auto leaves = [&](double z) { return pass == 0 ? z < 0.0 : z > 0.0; };
-    // every leaving velocity's chain and its step there, in the chains' order
-    std::vector<int> step(nch, 0), at, n, k;
+    const size_t base = chain.size(), most = (size_t)((ngroups + 7) / 8 * 2 * nvv + 8 * shares - 1) / (8 * shares);
+    chain.resize(base + most * nch, 0);
+    weight.resize(base + most * nch, F(0));
+    std::vector<int> step(nch, 0);
     int steps = 0;
     for (int g = 0; g < 8; ++g) {
         int q = 0;                                       // place in the group
@@ -421,25 +425,20 @@ int wall_chains(const miugks_solver* s, int pass, int axis, int shares, std::vec
                 if ((side && a == pair) || (axis == 0 && !leaves(un[a]))) continue;
                 int p = q % shares, u = q / shares % 8;
                 for (int b = 0; b < nvv; ++b) {
-                    if (axis == 0 || leaves(un[b])) {
-                        const int c = (g * shares + p) * 8 + u;
-                        at.push_back(c);
-                        n.push_back(step[c]);
-                        k.push_back(a * nvv + b);
+                    const double z = un[axis == 0 ? a : b];
+                    if (leaves(z)) {
+                        const int c = (g * shares + p) * 8 + u, k = a * nvv + b;
+                        const size_t to = base + (size_t)step[c] * nch + c;
+                        chain[to] = k;
+                        weight[to] = (F)s->wh[k] * std::fabs((F)z);
                         steps = std::max(steps, ++step[c]);
                     }
                     if (++p == shares) { p = 0; u = (u + 1) % 8; }
                 }
             }
     }
-    const size_t base = chain.size();
-    chain.resize(base + (size_t)steps * nch, 0);
-    weight.resize(base + (size_t)steps * nch, F(0));
-    for (size_t e = 0; e < k.size(); ++e) {
-        const size_t to = base + (size_t)n[e] * nch + at[e];
-        chain[to] = k[e];
-        weight[to] = (F)s->wh[k[e]] * std::fabs((F)(axis == 0 ? s->uh : s->vh)[k[e]]);
-    }
+    chain.resize(base + (size_t)steps * nch);
+    weight.resize(base + (size_t)steps * nch);
     return steps;
 }
 
