@@ -1026,6 +1026,7 @@ cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, cons
     // 64x64 cavity with 32x32 velocities (64 CTAs with four lanes) 0.62 / 0.57 / 0.63 ms.
     constexpr int V16 = 16 / (int)sizeof(F);
     const int LPC = ns <= 128 && m.V.ld / (4 * V16) > 128 ? 4 : ns <= 256 ? 2 : 1;
+    if (m.V.ld % (LPC * V16)) return cudaErrorInvalidValue;   // a block of velocities would leave its row
     const int nblk = m.V.ld / (LPC * V16), nw = (ns * LPC + 31) / 32;
     // ring depth: eight steps in flight where they fit, else four
     const size_t fixed = (size_t)nw * kWaveEdge * 32 * LPC + sizeof(F) * nt + 2 * sizeof(int) * nw + 16, slot = (size_t)nw * 1536;
