@@ -247,10 +247,10 @@ def measure(precision, steps, warmup, world, rank, dev, with_e2e=True, with_ttr=
 
 # The kernel with the step's longest dependency chain: the prediction
 # smoother's LU-SGS sweep, k_macro_sgs, on the finest level.
-# Algorithmic bytes per cell and launch: reads W, R (4 doubles each), the
-# inverse diagonal (1), the Gamma of the faces (2 per cell), writes dW and W
-# (4 each): 19 doubles = 152 B.
-MACRO_BYTES_PER_CELL = 152.0
+# Algorithmic bytes per cell and launch: the records of both passes are read
+# (16 floats, or 4 x 10 doubles, each) and two rows of dW written (4 values
+# each; the state's update and the records are k_macro_stage's).
+MACRO_BYTES_PER_CELL = {"mixed": 160.0, "fp64": 704.0}
 # DRAM bytes (read + write) of one finest-level k_macro_sgs<float> launch from
 # the ncu capture summarised in profiles/k_kernels_cavity64_v32_mixed.md
 MACRO_TRAFFIC_MIXED = 0.91e6
@@ -259,7 +259,7 @@ MACRO_TRAFFIC_MIXED = 0.91e6
 def macro_roofline(m, precision):
     t = m["macro_ms_per_launch"] * 1e-3
     hpeak, hsrc = hbm_peak()
-    gbs = MACRO_BYTES_PER_CELL * NX * NY / t / 1e9
+    gbs = MACRO_BYTES_PER_CELL["mixed" if precision == "mixed" else "fp64"] * NX * NY / t / 1e9
     return {"bound": "hbm", "kernel": "k_macro_sgs (finest level)", "achieved": gbs, "peak": hpeak, "unit": "GB/s",
             "frac": gbs / hpeak, "traffic": MACRO_TRAFFIC_MIXED if precision == "mixed" else None,
             "peak_source": hsrc, "launch_ms": m["macro_ms_per_launch"],
@@ -408,14 +408,14 @@ SWEEP_VALUES_PER_CV = 5
 # DRAM bytes per cell-velocity pair of the flat plate's finest-level sweep
 # kernels (mixed), from the ncu captures summarised in
 # profiles/k_kernels_plate128x96_v48_mixed.md (forward and backward launches)
-SWEEP_TRAFFIC_PER_CV = {"wave": 21.8}
+SWEEP_TRAFFIC_PER_CV = {"wave": 22.0}
 # DRAM bytes (read + written) of one launch of the flat plate's face-flux kernel
 # (mixed, x-faces), from the ncu capture in profiles/k_kernels_plate128x96_v48_mixed.md
-FLUX_TRAFFIC_PLATE_MIXED = 421.2e6
+FLUX_TRAFFIC_PLATE_MIXED = 417.5e6
 # the same for one launch of the square cylinder's face flux (mixed, x-faces): the ncu capture of the half-size
-# case (80x60 cells, 4,860 x-faces, 631.1 MB; profiles/k_kernels_square80x60_v89_mixed.md) scaled by the
+# case (80x60 cells, 4,860 x-faces, 647.8 MB; profiles/k_kernels_square80x60_v89_mixed.md) scaled by the
 # faces of the full case (19,320), since each face reads its cells' rows and writes its own fluxes
-FLUX_TRAFFIC_SQUARE_MIXED = 631.1e6 * 19320 / 4860
+FLUX_TRAFFIC_SQUARE_MIXED = 647.8e6 * 19320 / 4860
 
 
 def sweep_roofline(sk, precision):
@@ -965,18 +965,18 @@ def count_launches():
     """Kernel launches of one outer iteration of the workload, following the
     library's launch sequence (every launch is one of this library's kernels;
     memsets and copies are not counted).  Matches the ncu launch list of the
-    same workload (134 per iteration for 3 levels)."""
+    same workload (117 per iteration for 3 levels)."""
     L, nu1, nu2, nuc = LEVELS, 2, 1, 4
-    macro_sweep = 2            # per-diagonal record kernel + cluster sweep
-    micro_sweep = 6            # boundary-line chain, line fold and wavefront, forward and backward
+    macro_sweep = 1
+    micro_sweep = 6            # line walk, wall sums and wavefront, forward and backward
     n = 2 + 1 + 2              # Step 1: two face-flux launches, cell residual, RMS (partial + final)
     for l in range(L):         # Step 2: FAS
         coarsest = l == L - 1
         npre = nuc if coarsest else nu1
-        n += 2 + 1             # Gamma and inverse diagonal, forcing
+        n += 1 + 1             # Gamma, forcing with the first sweep's records
         n += npre * macro_sweep + (npre - 1 if coarsest else npre)
         if not coarsest:
-            n += 2 + 1 + 1 + nu2 * (1 + macro_sweep)   # restrictions, difference, prolongation, post-smoothing
+            n += 1 + 1 + nu2 * (1 + macro_sweep)   # restriction, prolongation, post-smoothing
     n += 1                     # the predicted state (FAS result, or W^n where it is unphysical)
     n += 1 + 2 * (L - 1)       # Steps 3-4: micro residual; per coarse level restriction + coefficients
     for l in range(L):         # Step 5: CS
