@@ -1022,8 +1022,8 @@ cudaError_t launch_micro_sgs(const MicroArgs& m, const SweepPlanHost& plan, cons
     // Lanes per cell: an asynchronous copy or store of a warp costs its SM's L1 one look-up per cell, so
     // the more lanes share a cell the better (64 bytes of a cell with four), as long as the strips fit a
     // CTA of 16 warps and the CTAs fill the SMs.  Finest level and coarser ones together, per
-    // iteration, 1 / 2 / 4 lanes: square cylinder mixed 21.5 / 12.8 / 9.0 ms, plate mixed 2.9 / 2.0 / 1.7 ms;
-    // 64x64 cavity with 32x32 velocities (64 CTAs with four lanes) 0.62 / 0.57 / 0.63 ms.
+    // iteration, 1 / 2 / 4 lanes: square cylinder mixed 21.5 / 12.6 / 8.7 ms, plate mixed 2.8 / 2.0 / 1.6 ms;
+    // 64x64 cavity with 32x32 velocities (64 CTAs with four lanes) 0.55 / 0.53 / 0.58 ms.
     constexpr int V16 = 16 / (int)sizeof(F);
     const int LPC = ns <= 128 && m.V.ld / (4 * V16) > 128 ? 4 : ns <= 256 ? 2 : 1;
     if (m.V.ld % (LPC * V16)) return cudaErrorInvalidValue;   // a block of velocities would leave its row

@@ -384,8 +384,12 @@ miugks_status upload_level(miugks_solver* s, HLevel& Lv)
     ST(dalloc(s, &Lv.T, nrec + ngh + n4));
     Lv.ghost = Lv.T + nrec;
     Lv.Wd = Lv.ghost + ngh;
-    ST(falloc(s, &Lv.r, nf)); ST(falloc(s, &Lv.df, nf)); ST(falloc(s, &Lv.dl, nf));
-    ST(falloc(s, &Lv.invD, (size_t)Lv.nc * s->ld)); ST(dalloc(s, &Lv.inv_tau, (size_t)Lv.nc));
+    // (one block for the arrays of rows: an allocation and a clearing of the padding each would take longer)
+    ST(falloc(s, &Lv.r, 3 * nf + nf / 2));
+    Lv.df = (char*)Lv.r + nf * s->fsz;
+    Lv.dl = (char*)Lv.df + nf * s->fsz;
+    Lv.invD = (char*)Lv.dl + nf * s->fsz;
+    ST(dalloc(s, &Lv.inv_tau, (size_t)Lv.nc));
     return MIUGKS_OK;
 }
 
