@@ -534,9 +534,10 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
 // Wall densities of the line cells [e0, e0 + gridDim.x), rho = -sum / Z with the sum of
 // w u_n x over the velocities that leave through the wall, one CTA per cell.  Order of the
 // sum: eight groups of row pairs of the velocity grid, in a group P shares (128 over the
-// line's cells) of eight interleaved chains each, a chain in order; then the chains as a
-// tree, the shares and the groups in order.  The tables hold the chains side by side, a
-// step of all of them after the other, so that a thread's loads are known ahead.
+// line's cells, in FP64 eight, less those without a velocity) of eight interleaved chains
+// each, a chain in order; then the chains as a tree, the shares and the groups in order.
+// The tables hold the chains side by side, a step of all of them after the other, so that
+// a thread's loads are known ahead.
 // A kernel of its own because all of a line's walks have to be done; bound by latency
 // (64x64 cavity with 32x32 velocities 5 us, square cylinder's body lines 8 us).
 template <typename F>
@@ -548,30 +549,60 @@ __global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __r
     const int4 lc = M.P.lcell[pass][e];              // {cell, line axis, bc id, 0 at the corner}
     const int4 ls = M.P.lsum[pass][e];               // {place in the tables, shares, steps}
     if (ls.y == 0) return;                           // no wall there: the density is not asked for
-    constexpr int U = 16;
+    constexpr int U = sizeof(F) == 8 ? 4 : 16;       // (512 threads in FP64: chains of a few steps)
     const int P = ls.y, nch = 64 * P;
+    const F iz = (F)(Zw + 4 * kMaxBcs)[lc.z * 4 + lc.y * 2 + pass];
     const F* __restrict__ x = S.xline + (size_t)e * 2 * V.ld;
-    for (int t = tid; t < nch; t += blockDim.x) {    // chain u of share p of group g; whole warps
-        const int* __restrict__ kt = V.chain + ls.x + t;
-        const F* __restrict__ wt = reinterpret_cast<const F*>(V.wchain) + ls.x + t;
-        F acc = F(0);
-        for (int n = 0; n < ls.z; n += U) {
-            F w[U], v[U];
-            int k[U];
-            #pragma unroll
-            for (int q = 0; q < U; ++q) {            // (a chain that has ended goes on with weight zero)
-                const int at = min(n + q, ls.z - 1) * nch;
-                k[q] = kt[at];
-                w[q] = n + q < ls.z ? wt[at] : F(0);
-            }
-            #pragma unroll
-            for (int q = 0; q < U; ++q) v[q] = x[k[q]];
-            #pragma unroll
-            for (int q = 0; q < U; ++q) acc = w[q] != F(0) ? fma(w[q], v[q], acc) : acc;
-        }
+    const int* __restrict__ chain = V.chain + ls.x;
+    const F* __restrict__ weight = reinterpret_cast<const F*>(V.wchain) + ls.x;
+    auto finish = [&](int t, F acc) {                // the tree over the eight chains of share t / 8
         #pragma unroll
         for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if ((t & 7) == 0) part[t >> 3] = acc;
+    };
+    if (nch <= (int)blockDim.x) {                    // a long chain per thread: its steps' loads in flight together
+        if (tid < nch) {                             // (whole warps)
+            F acc = F(0);
+            for (int n = 0; n < ls.z; n += U) {
+                F w[U], v[U];
+                int k[U];
+                #pragma unroll
+                for (int q = 0; q < U; ++q) {        // (a chain that has ended goes on with weight zero)
+                    const int at = min(n + q, ls.z - 1) * nch + tid;
+                    k[q] = chain[at];
+                    w[q] = n + q < ls.z ? weight[at] : F(0);
+                }
+                #pragma unroll
+                for (int q = 0; q < U; ++q) v[q] = x[k[q]];
+                #pragma unroll
+                for (int q = 0; q < U; ++q) acc = w[q] != F(0) ? fma(w[q], v[q], acc) : acc;
+            }
+            finish(tid, acc);
+        }
+    } else {                                         // many short ones: eight chains' loads together
+        constexpr int G = 8;
+        for (int t0 = tid; t0 < nch; t0 += G * blockDim.x) {
+            F acc[G];
+            #pragma unroll
+            for (int g = 0; g < G; ++g) acc[g] = F(0);
+            for (int n = 0; n < ls.z; ++n) {
+                F w[G], v[G];
+                int k[G];
+                #pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const int t = t0 + g * (int)blockDim.x, at = n * nch + min(t, nch - 1);
+                    k[g] = chain[at];
+                    w[g] = t < nch ? weight[at] : F(0);
+                }
+                #pragma unroll
+                for (int g = 0; g < G; ++g) v[g] = x[k[g]];
+                #pragma unroll
+                for (int g = 0; g < G; ++g) acc[g] = w[g] != F(0) ? fma(w[g], v[g], acc[g]) : acc[g];
+            }
+            #pragma unroll
+            for (int g = 0; g < G; ++g)
+                if (t0 + g * (int)blockDim.x < nch) finish(t0 + g * (int)blockDim.x, acc[g]);   // (whole warps)
+        }
     }
     __syncthreads();
     if (tid < 8) {
@@ -584,7 +615,7 @@ __global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __r
     if (tid == 0) {
         F t = F(0);
         for (int g = 0; g < 8; ++g) t += part[g * P];
-        S.rho[e] = -t * (F)(Zw + 4 * kMaxBcs)[lc.z * 4 + lc.y * 2 + pass];
+        S.rho[e] = -t * iz;
     }
 }
 

@@ -94,8 +94,8 @@ struct miugks_solver {
     size_t fsz = sizeof(double);
     void *f = nullptr, *phx = nullptr, *phy = nullptr, *scratch = nullptr;
     int sw_nl = 0;                          // layout of the sweep scratch
-    // chains of the wall sums by {pass, axis, shares}: {place in the tables, steps} (wall_chains)
-    std::map<std::array<int, 3>, std::array<int, 2>> chain_at;
+    // chains of the wall sums by {pass, axis, shares}: {place in the tables, steps, shares left} (wall_chains)
+    std::map<std::array<int, 3>, std::array<int, 3>> chain_at;
     std::vector<int> chain_k;
     std::vector<float> chain_wf;
     std::vector<double> chain_w;
@@ -410,40 +410,55 @@ SweepPlanHost sweep_plan(const miugks_solver* s, const HLevel& Lv)
 // Chains of a wall sum over the velocities that leave through the faces of one axis on a pass's sweep side
 // (k_line_rho): the velocities in eight groups of row pairs (a, nu - 1 - a), in a group `shares` times eight chains
 // that take its places in turn.  Laid out step after step, [steps][group][share][chain], ended chains with weight 0.
+// A share without a velocity is left out: it would add an exact zero, and a line of a few cells, with up to 128 shares,
+// has mostly such (level of 2x1 cells, 48x13 velocities: the launch took 93 us with all of them).
+// Returns {steps, shares that are left}.
 template <typename F>
-int wall_chains(const miugks_solver* s, int pass, int axis, int shares, std::vector<int>& chain, std::vector<F>& weight)
+std::array<int, 2> wall_chains(const miugks_solver* s, int pass, int axis, int shares, std::vector<int>& chain,
+                               std::vector<F>& weight)
 {
-    const int nu = s->nu, nvv = s->nvv, ngroups = (nu + 1) / 2, nch = 64 * shares;
+    const int nu = s->nu, nvv = s->nvv, ngroups = (nu + 1) / 2;
     const std::vector<double>& un = axis == 0 ? s->uah : s->vbh;
-    auto leaves = [&](double z) { return pass == 0 ? z < 0.0 : z > 0.0; };
+    auto each = [&](auto&& take) {                       // take(group, share, chain, velocity, weight), in order
+        for (int g = 0; g < 8; ++g) {
+            int q = 0;                                   // place in the group
+            for (int pair = g; pair < ngroups; pair += 8)
+                for (int side = 0; side < 2; ++side, q += nvv) {
+                    const int a = side ? nu - 1 - pair : pair;
+                    if (side && a == pair) continue;
+                    int p = q % shares, u = q / shares % 8;
+                    for (int b = 0; b < nvv; ++b) {
+                        const double z = un[axis == 0 ? a : b];
+                        if (pass == 0 ? z < 0.0 : z > 0.0) take(g, p, u, a * nvv + b, (F)s->wh[a * nvv + b] * std::fabs((F)z));
+                        if (++p == shares) { p = 0; u = (u + 1) % 8; }
+                    }
+                }
+        }
+    };
+    std::vector<int> place(8 * shares, -1);              // of a share among its group's that are left
+    each([&](int g, int p, int, int, F) { place[g * shares + p] = 0; });
+    int left = 1;
+    for (int g = 0; g < 8; ++g) {
+        int n = 0;
+        for (int p = 0; p < shares; ++p) if (place[g * shares + p] == 0) place[g * shares + p] = n++;
+        left = std::max(left, n);
+    }
+    const int nch = 64 * left;
     const size_t base = chain.size(), most = (size_t)((ngroups + 7) / 8 * 2 * nvv + 8 * shares - 1) / (8 * shares);
     chain.resize(base + most * nch, 0);
     weight.resize(base + most * nch, F(0));
     std::vector<int> step(nch, 0);
     int steps = 0;
-    for (int g = 0; g < 8; ++g) {
-        int q = 0;                                       // place in the group
-        for (int pair = g; pair < ngroups; pair += 8)
-            for (int side = 0; side < 2; ++side, q += nvv) {
-                const int a = side ? nu - 1 - pair : pair;
-                if ((side && a == pair) || (axis == 0 && !leaves(un[a]))) continue;
-                int p = q % shares, u = q / shares % 8;
-                for (int b = 0; b < nvv; ++b) {
-                    const double z = un[axis == 0 ? a : b];
-                    if (leaves(z)) {
-                        const int c = (g * shares + p) * 8 + u, k = a * nvv + b;
-                        const size_t to = base + (size_t)step[c] * nch + c;
-                        chain[to] = k;
-                        weight[to] = (F)s->wh[k] * std::fabs((F)z);
-                        steps = std::max(steps, ++step[c]);
-                    }
-                    if (++p == shares) { p = 0; u = (u + 1) % 8; }
-                }
-            }
-    }
+    each([&](int g, int p, int u, int k, F w) {
+        const int c = (g * left + place[g * shares + p]) * 8 + u;
+        const size_t to = base + (size_t)step[c] * nch + c;
+        chain[to] = k;
+        weight[to] = w;
+        steps = std::max(steps, ++step[c]);
+    });
     chain.resize(base + (size_t)steps * nch);
     weight.resize(base + (size_t)steps * nch);
-    return steps;
+    return {steps, left};
 }
 
 // Sweep order of a level.  Per pass (0 forward: west / south faces on the
@@ -466,22 +481,23 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
         std::vector<int> lcell;              // int4 per entry
         for (int c = 0; c < nc; ++c) if (Lv.solid[c]) code[c] = -2;
         const int ie = p == 0 ? 0 : nx - 1, je = p == 0 ? 0 : ny - 1, sg = p == 0 ? 1 : -1;
-        // wall sum of a line cell: shares (128 over the line's cells) and table; the corner, and cells at other
+        // wall sum of a line cell: shares (128 over the line's cells in the mixed form) and table; the corner, and cells at other
         // boundaries, have none (0 shares)
         std::vector<int> lsum;               // int4 per entry
         auto add_sum = [&](int ncell, int axis, int bc, bool corner, int& most) {
             if (corner || s->bch[bc].type != MIUGKS_BC_WALL) { lsum.insert(lsum.end(), {0, 0, 0, 0}); return; }
-            const int shares = ncell >= 128 ? 1 : 128 / ncell;
-            most = std::max(most, shares);
+            // (FP64: eight, with which every chain has a thread of its own and is short)
+            const int shares = !s->mixed ? 8 : ncell >= 128 ? 1 : 128 / ncell;
             const std::array<int, 3> key = {p, axis, shares};
             if (!s->chain_at.count(key)) {
                 const int at = (int)s->chain_k.size();
-                const int steps = s->mixed ? wall_chains<float>(s, p, axis, shares, s->chain_k, s->chain_wf)
-                                           : wall_chains<double>(s, p, axis, shares, s->chain_k, s->chain_w);
-                s->chain_at[key] = {at, steps};
+                const std::array<int, 2> n = s->mixed ? wall_chains<float>(s, p, axis, shares, s->chain_k, s->chain_wf)
+                                                      : wall_chains<double>(s, p, axis, shares, s->chain_k, s->chain_w);
+                s->chain_at[key] = {at, n[0], n[1]};
             }
-            const std::array<int, 2> t = s->chain_at[key];
-            lsum.insert(lsum.end(), {t[0], shares, t[1], 0});
+            const std::array<int, 3> t = s->chain_at[key];
+            most = std::max(most, t[2]);
+            lsum.insert(lsum.end(), {t[0], t[2], t[1], 0});
         };
         // the edge column (e = st) and row (e = ny + st), the corner first
         for (int st = 0; st < ny; ++st) {
