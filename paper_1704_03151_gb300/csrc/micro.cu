@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
     extern __shared__ __align__(16) unsigned char esm[];
     F* ring = reinterpret_cast<F*>(esm);              // [RA][3][B]
     __shared__ F nbS[kMaxLine], itS[kMaxLine];
-    __shared__ F red[32][4];
+    __shared__ F red[sizeof(F) == 4 ? 32 : 4][4];
     const LevelDev& L = M.L;
     const VelDev& V = M.V;
     const int nx = L.nx, ny = L.ny, nv = V.nv, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -343,8 +343,10 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
         const bool y0 = GENERAL && B0.type == BC_SYMMETRY, y1 = GENERAL && B1.type == BC_SYMMETRY;
         const bool o0 = GENERAL && B0.type == BC_OUTFLOW, o1 = GENERAL && B1.type == BC_OUTFLOW;
         const F sg = pass == 0 ? F(-1) : F(1);
-        // a velocity of the corner: outward normal speeds, weight, 1/D, right-hand sides
-        struct Vel { F ux, uy, w, den, b[2]; };
+        // a velocity of the corner: outward normal speeds, weight, 1/D, right-hand sides, the walls' Maxwellians
+        struct Vel { F ux, uy, w, den, b[2]; double C[2]; };
+        const double* __restrict__ C0 = M.Cw + (size_t)bc0 * nv;
+        const double* __restrict__ C1 = M.Cw + (size_t)bc1 * nv;
         auto fetch = [&](int kk, Vel& p) {           // independent loads, used once all are asked for
             p.ux = vu[kk];
             p.uy = vv[kk];
@@ -352,6 +354,8 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
             p.den = invD[(size_t)c * ld + kk];
             p.b[0] = src[(size_t)c * ld + kk];
             p.b[1] = src[(nc + c) * ld + kk];
+            p.C[0] = w0 ? C0[kk] : 0.0;
+            p.C[1] = w1 ? C1[kk] : 0.0;
         };
         // coefficient of the ghost behind face f (zero unless the velocity enters there)
         auto Dg = [&](int f, const Vel& p) { return f == 0 ? mul_rn(min(p.ux, F(0)), rx) : mul_rn(min(p.uy, F(0)), ry); };
@@ -369,9 +373,8 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
                 if (pass == 1) { p.b[0] = mul_rn(D, p.b[0]); p.b[1] = mul_rn(D, p.b[1]); }
             }
         };
-        auto wallC = [&](int f, int kk, int cp) {     // the wall's Maxwellian
-            const double C = M.Cw[(size_t)(f == 0 ? bc0 : bc1) * nv + kk];
-            return cp == 0 ? (F)C : (F)(C * (kKint * (f == 0 ? B0.t : B1.t) / 4.0));
+        auto wallC = [&](int f, const Vel& p, int cp) {
+            return cp == 0 ? (F)p.C[f] : (F)(p.C[f] * (kKint * (f == 0 ? B0.t : B1.t) / 4.0));
         };
         auto mirror = [&](int f, int kk) {
             const int a = kk / V.nvv, b = kk - a * V.nvv;
@@ -379,87 +382,88 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
         };
         F rho0 = F(0), rho1 = F(0);
         if (w0 || w1) {
-            // sums over the velocities: eight groups of row pairs (a, nu - 1 - a) a group apart, a thread's share of a
-            // group in order, then warps and groups by exchange
-            const int ngroups = (V.nu + 1) / 2, per = 2 * V.nvv, nloc = (ngroups + 7) / 8 * per;
-            #pragma unroll 1
-            for (int r0 = 0; r0 < 8; r0 += 4) {
-                F acc[4][4];
+            // sums over the velocities: in the mixed form eight groups of row pairs (a, nu - 1 - a) a group apart, a
+            // thread's share of a group in order, then warps and groups by exchange; in FP64, where the groups'
+            // exchanges would take longer than the sums, a thread's velocities, then warps.  At a time RB velocities,
+            // their loads in flight together.
+            constexpr bool GROUPS = sizeof(F) == 4;
+            constexpr int RB = GROUPS ? 8 : 4, NA = GROUPS ? 8 : 1;
+            const int ngroups = (V.nu + 1) / 2, per = 2 * V.nvv, nloc = GROUPS ? (ngroups + 7) / 8 * per : nv;
+            const double z0 = w0 ? Zw[bc0 * 4 + pass] : 0.0, z1 = w1 ? Zw[bc1 * 4 + 2 + pass] : 0.0;
+            const F iz = (F)(Zw + 4 * kMaxBcs)[w0 ? bc0 * 4 + pass : bc1 * 4 + 2 + pass];
+            F acc[NA][4];
+            #pragma unroll
+            for (int rr = 0; rr < NA; ++rr)
                 #pragma unroll
-                for (int rr = 0; rr < 4; ++rr)
-                    #pragma unroll
-                    for (int m = 0; m < 4; ++m) acc[rr][m] = F(0);
-                #pragma unroll 1
-                for (int m = tid; m < nloc; m += B) {
-                    const int sl = m / per, rem = m - sl * per, side = rem >= V.nvv, b = rem - side * V.nvv;
-                    Vel p[4];
-                    int kk[4];
-                    #pragma unroll
-                    for (int rr = 0; rr < 4; ++rr) {
-                        const int g = r0 + rr + sl * 8, a = side ? V.nu - 1 - g : g;
-                        kk[rr] = g < ngroups && !(side && a == g) ? a * V.nvv + b : -1;
-                        fetch(max(kk[rr], 0), p[rr]);
-                    }
-                    #pragma unroll
-                    for (int rr = 0; rr < 4; ++rr) {
-                        if (kk[rr] < 0) continue;
-                        finish(p[rr]);
-                        const F wx = mul_rn(p[rr].w, max(p[rr].ux, F(0))), wy = mul_rn(p[rr].w, max(p[rr].uy, F(0)));
-                        if (two) {
-                            acc[rr][0] = fma(mul_rn(wx, p[rr].b[0]), p[rr].den, acc[rr][0]);
-                            acc[rr][1] = fma(mul_rn(wy, p[rr].b[0]), p[rr].den, acc[rr][1]);
-                            acc[rr][2] = fma(mul_rn(mul_rn(wx, Dg(1, p[rr])), wallC(1, kk[rr], 0)), p[rr].den, acc[rr][2]);
-                            acc[rr][3] = fma(mul_rn(mul_rn(wy, Dg(0, p[rr])), wallC(0, kk[rr], 0)), p[rr].den, acc[rr][3]);
-                        } else {
-                            F val = p[rr].b[0];
-                            if (y0 || y1) {          // beside a symmetry face: the mirrored ghost of a velocity that enters through it
-                                const F d = Dg(y0 ? 0 : 1, p[rr]);
-                                if (d != F(0)) {
-                                    Vel mv;
-                                    fetch(mirror(y0 ? 0 : 1, kk[rr]), mv);
-                                    finish(mv);
-                                    val = fma(-d, mul_rn(mv.b[0], mv.den), val);
-                                }
-                            }
-                            val = mul_rn(val, p[rr].den);
-                            acc[rr][0] = fma(w0 ? wx : wy, val, acc[rr][0]);
-                        }
-                    }
+                for (int m = 0; m < 4; ++m) acc[rr][m] = F(0);
+            #pragma unroll 1
+            for (int m = tid; m < nloc; m += GROUPS ? B : RB * B) {
+                const int sl = m / per, rem = m - sl * per, side = rem >= V.nvv, b = rem - side * V.nvv;
+                Vel p[RB];
+                int kk[RB];
+                #pragma unroll
+                for (int rr = 0; rr < RB; ++rr) {
+                    const int g = rr + sl * 8, a = side ? V.nu - 1 - g : g;
+                    if (GROUPS) kk[rr] = g < ngroups && !(side && a == g) ? a * V.nvv + b : -1;
+                    else kk[rr] = m + rr * B < nv ? m + rr * B : -1;
+                    fetch(max(kk[rr], 0), p[rr]);
                 }
                 #pragma unroll
-                for (int rr = 0; rr < 4; ++rr)
-                    #pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        #pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) acc[rr][m] += __shfl_xor_sync(0xffffffffu, acc[rr][m], o);
-                        if (lane == 0) red[(r0 + rr) * 4 + warp][m] = acc[rr][m];
+                for (int rr = 0; rr < RB; ++rr) {
+                    if (kk[rr] < 0) continue;
+                    F* s = acc[GROUPS ? rr : 0];
+                    finish(p[rr]);
+                    const F wx = mul_rn(p[rr].w, max(p[rr].ux, F(0))), wy = mul_rn(p[rr].w, max(p[rr].uy, F(0)));
+                    if (two) {
+                        s[0] = fma(mul_rn(wx, p[rr].b[0]), p[rr].den, s[0]);
+                        s[1] = fma(mul_rn(wy, p[rr].b[0]), p[rr].den, s[1]);
+                        s[2] = fma(mul_rn(mul_rn(wx, Dg(1, p[rr])), wallC(1, p[rr], 0)), p[rr].den, s[2]);
+                        s[3] = fma(mul_rn(mul_rn(wy, Dg(0, p[rr])), wallC(0, p[rr], 0)), p[rr].den, s[3]);
+                    } else {
+                        F val = p[rr].b[0];
+                        if (y0 || y1) {              // beside a symmetry face: the mirrored ghost of a velocity that enters through it
+                            const F d = Dg(y0 ? 0 : 1, p[rr]);
+                            if (d != F(0)) {
+                                Vel mv;
+                                fetch(mirror(y0 ? 0 : 1, kk[rr]), mv);
+                                finish(mv);
+                                val = fma(-d, mul_rn(mv.b[0], mv.den), val);
+                            }
+                        }
+                        val = mul_rn(val, p[rr].den);
+                        s[0] = fma(w0 ? wx : wy, val, s[0]);
                     }
+                }
             }
+            #pragma unroll
+            for (int rr = 0; rr < NA; ++rr)
+                #pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    #pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) acc[rr][m] += __shfl_xor_sync(0xffffffffu, acc[rr][m], o);
+                    if (lane == 0) red[rr * 4 + warp][m] = acc[rr][m];
+                }
             __syncthreads();
             F t[4];
             #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                t[m] = red[lane][m];
+                t[m] = red[lane % (4 * NA)][m];
                 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) t[m] += __shfl_xor_sync(0xffffffffu, t[m], o);
+                for (int o = 2 * NA; o > 0; o >>= 1) t[m] += __shfl_xor_sync(0xffffffffu, t[m], o);
             }
-            __syncthreads();
-            if (tid == 0) {
-                if (two) {
-                    // rho_0 = k_0 + m_0 rho_1, rho_1 = k_1 + m_1 rho_0
-                    const double z0 = Zw[bc0 * 4 + pass], z1 = Zw[bc1 * 4 + 2 + pass];
-                    const double k0 = -t[0] / z0, k1 = -t[1] / z1, m0 = t[2] / z0, m1 = t[3] / z1;
-                    const double r0 = (k0 + m0 * k1) / (1.0 - m0 * m1);
-                    red[0][0] = (F)r0;
-                    red[0][1] = (F)(k1 + m1 * r0);
-                } else {
-                    const F iz = (F)(Zw + 4 * kMaxBcs)[w0 ? bc0 * 4 + pass : bc1 * 4 + 2 + pass];
-                    red[0][0] = red[0][1] = -t[0] * iz;
-                }
+            // (the same in every thread)
+            if (two) {
+                // rho_0 = k_0 + m_0 rho_1, rho_1 = k_1 + m_1 rho_0; lane 0 .. 3 of a warp divides for k_0, k_1, m_0, m_1
+                const F tl = (lane & 3) == 0 ? -t[0] : (lane & 3) == 1 ? -t[1] : (lane & 3) == 2 ? t[2] : t[3];
+                const double d = (double)tl / (lane & 1 ? z1 : z0);
+                const double k0 = __shfl_sync(0xffffffffu, d, 0), k1 = __shfl_sync(0xffffffffu, d, 1);
+                const double m0 = __shfl_sync(0xffffffffu, d, 2), m1 = __shfl_sync(0xffffffffu, d, 3);
+                const double r0 = (k0 + m0 * k1) / (1.0 - m0 * m1);
+                rho0 = (F)r0;
+                rho1 = (F)(k1 + m1 * r0);
+            } else {
+                rho0 = rho1 = -t[0] * iz;
             }
-            __syncthreads();
-            rho0 = red[0][0];
-            rho1 = red[0][1];
         }
         // value of a velocity with its ghosts: a wall's from its density, a symmetry face's from the mirrored velocity,
         // which leaves there and may itself enter through the other face
@@ -474,7 +478,7 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
                 if (d == F(0)) continue;
                 if (f == 0 ? w0 : w1) {
                     #pragma unroll
-                    for (int cp = 0; cp < 2; ++cp) a[cp] = fma(-mul_rn(d, wallC(f, kk, cp)), f == 0 ? rho0 : rho1, a[cp]);
+                    for (int cp = 0; cp < 2; ++cp) a[cp] = fma(-mul_rn(d, wallC(f, p, cp)), f == 0 ? rho0 : rho1, a[cp]);
                 } else if (f == 0 ? y0 : y1) {
                     if constexpr (GENERAL && decltype(depth)::value > 0) {
                         F g[2];
