@@ -475,6 +475,8 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
     auto bx = [&](int p, int i, int j) { return Lv.fbx[j * (nx + 1) + i + p] >= 0; };
     auto by = [&](int p, int i, int j) { return Lv.fby[(j + p) * nx + i] >= 0; };
     int nl_max = 0;
+    std::vector<int> tables;             // of both passes, one block on the device
+    std::vector<size_t> at[2];           // places of lcell, lsum, lines and code
     for (int p = 0; p < 2; ++p) {
         Lv.plan.shares[p] = 0;
         std::vector<int> code(nc, -1);
@@ -490,10 +492,10 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
             const int shares = !s->mixed ? 8 : ncell >= 128 ? 1 : 128 / ncell;
             const std::array<int, 3> key = {p, axis, shares};
             if (!s->chain_at.count(key)) {
-                const int at = (int)s->chain_k.size();
+                const int place = (int)s->chain_k.size();
                 const std::array<int, 2> n = s->mixed ? wall_chains<float>(s, p, axis, shares, s->chain_k, s->chain_wf)
                                                       : wall_chains<double>(s, p, axis, shares, s->chain_k, s->chain_w);
-                s->chain_at[key] = {at, n[0], n[1]};
+                s->chain_at[key] = {place, n[0], n[1]};
             }
             const std::array<int, 3> t = s->chain_at[key];
             most = std::max(most, t[2]);
@@ -575,22 +577,11 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
             }
         }
         nl_max = std::max(nl_max, (int)lcell.size() / 4);
-        int* dcode;
-        int4 *dl, *dsum;
-        int* dlines;
-        ST(upload(s, &dcode, code));
-        auto int4s = [](const std::vector<int>& v) {
-            std::vector<int4> h(v.size() / 4);
-            for (size_t e = 0; e < h.size(); ++e) h[e] = make_int4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-            return h;
-        };
-        ST(upload(s, &dl, int4s(lcell)));
-        ST(upload(s, &dsum, int4s(lsum)));
-        ST(upload(s, &dlines, lines));
-        Lv.plan.code[p] = dcode;
-        Lv.plan.lcell[p] = dl;
-        Lv.plan.lsum[p] = dsum;
-        Lv.plan.lines[p] = dlines;
+        for (std::vector<int>* v : {&lcell, &lsum, &lines, &code}) {
+            at[p].push_back(tables.size());
+            tables.insert(tables.end(), v->begin(), v->end());
+        }
+        tables.resize((tables.size() + 3) / 4 * 4);          // (16-byte aligned entries in the next pass)
         Lv.plan.cbc[p][0] = Lv.fbx[je * (nx + 1) + ie + p];
         Lv.plan.cbc[p][1] = Lv.fby[(je + p) * nx + ie];
         Lv.plan.general[p] = 0;
@@ -598,6 +589,14 @@ miugks_status build_sweep_plan(miugks_solver* s, HLevel& Lv)
             const int type = s->bch[Lv.plan.cbc[p][f]].type;
             Lv.plan.general[p] |= type == MIUGKS_BC_SYMMETRY || type == MIUGKS_BC_OUTFLOW;
         }
+    }
+    int* dt;
+    ST(upload(s, &dt, tables));
+    for (int p = 0; p < 2; ++p) {
+        Lv.plan.lcell[p] = reinterpret_cast<int4*>(dt + at[p][0]);
+        Lv.plan.lsum[p] = reinterpret_cast<int4*>(dt + at[p][1]);
+        Lv.plan.lines[p] = dt + at[p][2];
+        Lv.plan.code[p] = dt + at[p][3];
     }
     Lv.plan.nl_max = nl_max;
     Lv.plan.bodies = Lv.nfluid != Lv.nc;
