@@ -99,7 +99,7 @@ cudaError_t launch_sub(double* out, const double* a, const double* b, size_t n, 
 struct SweepPlanDev {
     const int* code[2];     // per cell: -1 ordinary, -2 in a body, else its fold entry
     const int4* lcell[2];   // per fold entry: {cell, line axis (0 x-face, 1 y-face), the face's bc id, 0 at the corner}
-    const int4* lsum[2];    // per fold entry, of its wall sum: {place in VelDev::chain, shares (0: no wall), steps, 0}
+    const int4* lsum[2];    // per fold entry, of its wall sum: {place in VelDev::chain, shares (0: no wall), steps, 1: many short chains}
     int shares[2];          // most shares of an edge cell's wall sum (0: no walls there)
     const int* lines[2];    // lines: [q][8] = {i0, j0, di, dj, len, line axis, entry of cell 0, 0};
                             // 0 the edge column, 1 the edge row, then the lines along bodies

@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __r
     const VelDev& V = M.V;
     const int e = e0 + (int)blockIdx.x, tid = threadIdx.x;
     const int4 lc = M.P.lcell[pass][e];              // {cell, line axis, bc id, 0 at the corner}
-    const int4 ls = M.P.lsum[pass][e];               // {place in the tables, shares, steps}
+    const int4 ls = M.P.lsum[pass][e];               // {place in the tables, shares, steps, short chains}
     if (ls.y == 0) return;                           // no wall there: the density is not asked for
     constexpr int U = sizeof(F) == 8 ? 4 : 16;       // (512 threads in FP64: chains of a few steps)
     const int P = ls.y, nch = 64 * P;
@@ -564,15 +564,17 @@ __global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __r
         for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if ((t & 7) == 0) part[t >> 3] = acc;
     };
-    if (nch <= (int)blockDim.x) {                    // a long chain per thread: its steps' loads in flight together
-        if (tid < nch) {                             // (whole warps)
+    // U steps of a chain or one step of G chains at a time, their loads in flight together
+    constexpr int G = 8;
+    if (ls.w == 0) {
+        for (int t = tid; t < nch; t += blockDim.x) {    // (whole warps)
             F acc = F(0);
             for (int n = 0; n < ls.z; n += U) {
                 F w[U], v[U];
                 int k[U];
                 #pragma unroll
                 for (int q = 0; q < U; ++q) {        // (a chain that has ended goes on with weight zero)
-                    const int at = min(n + q, ls.z - 1) * nch + tid;
+                    const int at = min(n + q, ls.z - 1) * nch + t;
                     k[q] = chain[at];
                     w[q] = n + q < ls.z ? weight[at] : F(0);
                 }
@@ -581,10 +583,9 @@ __global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __r
                 #pragma unroll
                 for (int q = 0; q < U; ++q) acc = w[q] != F(0) ? fma(w[q], v[q], acc) : acc;
             }
-            finish(tid, acc);
+            finish(t, acc);
         }
-    } else {                                         // many short ones: eight chains' loads together
-        constexpr int G = 8;
+    } else {
         for (int t0 = tid; t0 < nch; t0 += G * blockDim.x) {
             F acc[G];
             #pragma unroll
