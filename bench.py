@@ -411,11 +411,11 @@ SWEEP_VALUES_PER_CV = 5
 SWEEP_TRAFFIC_PER_CV = {"wave": 22.0}
 # DRAM bytes (read + written) of one launch of the flat plate's face-flux kernel
 # (mixed, x-faces), from the ncu capture in profiles/k_kernels_plate128x96_v48_mixed.md
-FLUX_TRAFFIC_PLATE_MIXED = 417.5e6
+FLUX_TRAFFIC_PLATE_MIXED = 415.9e6
 # the same for one launch of the square cylinder's face flux (mixed, x-faces): the ncu capture of the half-size
-# case (80x60 cells, 4,860 x-faces, 647.8 MB; profiles/k_kernels_square80x60_v89_mixed.md) scaled by the
+# case (80x60 cells, 4,860 x-faces, 644.1 MB; profiles/k_kernels_square80x60_v89_mixed.md) scaled by the
 # faces of the full case (19,320), since each face reads its cells' rows and writes its own fluxes
-FLUX_TRAFFIC_SQUARE_MIXED = 647.8e6 * 19320 / 4860
+FLUX_TRAFFIC_SQUARE_MIXED = 644.1e6 * 19320 / 4860
 
 
 def sweep_roofline(sk, precision):

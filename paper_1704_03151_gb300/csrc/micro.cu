@@ -267,8 +267,10 @@ __device__ __forceinline__ void st16(double* p, const double* v) { *reinterpret_
 // has finished.
 //
 // Bound by latency: the corner, then one load latency and a short recurrence per
-// RA cells.  64x64 cavity, 32x32 velocities, mixed: 17 us, and 5 us for the wall sums, against 34 us
-// for the walk by clusters of eight CTAs with its fold launch that this replaces.
+// RA cells.  64x64 cavity, 32x32 velocities, mixed: 11 us, and 6 us for the wall sums, against 34 us
+// for the walk by clusters of eight CTAs with its fold launch that this replaces (17 us with the
+// corner's sums in two rounds of loads and its divisions in one thread).  Levels of 20x8 cells and
+// less, 47x13 velocities, FP64: 17 us and 6 us, against 27 us and 7 us.
 template <typename F> struct EdgeRing { static constexpr int RA = 128 / (int)sizeof(F); };
 
 // GENERAL: a symmetry or outflow face at the corner (without them the code is half as
@@ -543,7 +545,8 @@ __global__ void __launch_bounds__(128) k_sgs_edge(MicroArgs M, const double* __r
 // The tables hold the chains side by side, a step of all of them after the other, so that
 // a thread's loads are known ahead.
 // A kernel of its own because all of a line's walks have to be done; bound by latency
-// (64x64 cavity with 32x32 velocities 5 us, square cylinder's body lines 8 us).
+// (mixed: 64x64 cavity with 32x32 velocities 6 us, square cylinder's body lines 8 us; FP64:
+// square cylinder at half size 9 us, against 22 us with as many shares as the mixed form).
 template <typename F>
 __global__ void __launch_bounds__(512) k_line_rho(MicroArgs M, const double* __restrict__ Zw, SweepScratch<F> S, int pass, int e0)
 {

@@ -411,7 +411,7 @@ SweepPlanHost sweep_plan(const miugks_solver* s, const HLevel& Lv)
 // (k_line_rho): the velocities in eight groups of row pairs (a, nu - 1 - a), in a group `shares` times eight chains
 // that take its places in turn.  Laid out step after step, [steps][group][share][chain], ended chains with weight 0.
 // A share without a velocity is left out: it would add an exact zero, and a line of a few cells, with up to 128 shares,
-// has mostly such (level of 2x1 cells, 48x13 velocities: the launch took 93 us with all of them).
+// has mostly such (levels of 20x8 cells and less, 47x13 velocities, FP64: 53 us per launch with all of them, 6 us now).
 // Returns {steps, shares that are left}.
 template <typename F>
 std::array<int, 2> wall_chains(const miugks_solver* s, int pass, int axis, int shares, std::vector<int>& chain,
